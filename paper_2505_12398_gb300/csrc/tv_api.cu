@@ -66,6 +66,8 @@ constexpr unsigned kPathFlags = TV_FLAG_UNFUSED | TV_FLAG_CLUSTER | TV_FLAG_PERS
 
 enum Path { kPathThree = 0, kPathCluster = 1, kPathPersistent = 2 };
 
+size_t logit_bytes(const tv_handle* h) { return h->dtype == TV_BF16 ? 2 : 4; }
+
 FlowPlan flow_plan(const tv_handle* h, int R, int B) {
   return tv_flow_plan(R, B, h->vocab, h->smem_per_sm, h->smem_per_block, h->flow_force[0],
                       h->flow_force[1],
@@ -86,7 +88,7 @@ constexpr int kClusterMaxRows = 128;
 Path choose_path(const tv_handle* h, int B, int R, FusedPlan* plan) {
   if ((h->vocab % 8) != 0 || (h->flags & TV_FLAG_UNFUSED)) return kPathThree;
   if (h->flags & TV_FLAG_CLUSTER) {
-    *plan = tv_fused_plan(B, R, h->vocab, h->sm_count, h->smem_per_sm, h->smem_per_block,
+    *plan = tv_fused_plan(B, R, h->vocab, (int)logit_bytes(h), h->sm_count, h->smem_per_sm, h->smem_per_block,
                           h->force_ncw, h->force_c, h->force_stages);
     return plan->ok ? kPathCluster : kPathThree;
   }
@@ -97,7 +99,7 @@ Path choose_path(const tv_handle* h, int B, int R, FusedPlan* plan) {
     // tree, exchanging partials through distributed shared memory, is faster
     // (V = 32000, EAGLE-shaped trees: 13-22 % less time at 16 to 2048 trees;
     // the persistent kernel is faster from V = 128256 and on deep trees)
-    *plan = tv_fused_plan(B, R, h->vocab, h->sm_count, h->smem_per_sm, h->smem_per_block,
+    *plan = tv_fused_plan(B, R, h->vocab, (int)logit_bytes(h), h->sm_count, h->smem_per_sm, h->smem_per_block,
                           h->force_ncw, h->force_c, h->force_stages);
     if (plan->ok) return kPathCluster;
   }
@@ -209,8 +211,6 @@ bool capturing(cudaStream_t st) {
 
 bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
-size_t logit_bytes(const tv_handle* h) { return h->dtype == TV_BF16 ? 2 : 4; }
-
 int check_call(const tv_handle* h, int B, int N, const void* parents, const void* tokens,
                const void* logits, const void* drafts, float temperature,
                const void* uniforms, const void* out_path, const void* out_len,
@@ -272,7 +272,7 @@ int verify_impl(tv_handle* h, int B, int N, const int32_t* parents, const int32_
     // graph must not replay it: under capture, a handle that chose the path
     // itself uses the cluster path (else the three-kernel one)
     if ((h->flags & TV_FLAG_PERSISTENT) || row_stats) return TV_ERR_INVALID_ARG;
-    plan = tv_fused_plan(B, N + 1, h->vocab, h->sm_count, h->smem_per_sm, h->smem_per_block,
+    plan = tv_fused_plan(B, N + 1, h->vocab, (int)logit_bytes(h), h->sm_count, h->smem_per_sm, h->smem_per_block,
                          h->force_ncw, h->force_c, h->force_stages);
     path = plan.ok ? kPathCluster : kPathThree;
   }

@@ -16,14 +16,7 @@
 namespace tvk {
 namespace fused {
 
-// A CTA of the cluster kernel has NCW consumer warps (4 or 8) and one producer
-// warp; its ring stages hold 3 * NCW KB: a target + draft slice of 512 * NCW
-// tokens (bf16), or a target-only slice of 1536 * NCW tokens.  (The
-// persistent kernel sizes its stages itself, tv_flow.cu.)
-constexpr int kMaxStages = 8;
-constexpr int kMaxCluster = 8;
 constexpr int kTileElems = 256;       // one warp x 8 elements
-__host__ __device__ constexpr int stage_bytes(int ncw) { return 3072 * ncw; }
 
 enum : int { kJobStats = 1, kJobPass = 2, kJobBonusLeaf = 3, kJobBonusRes = 4, kJobDone = 5 };
 enum : uint8_t { kAlive = 0, kRejected = 1, kPruned = 2 };
@@ -43,16 +36,12 @@ struct Ctl {
   uint32_t bad;        // TV_STATUS_* bits
   int accepted;        // accepted node (-1: invalid tree)
   float S;             // result of the last pass
-  int bonus_y;
   float bmargin;       // margin of the bonus draw (out_margin[b][1])
   // serial control state (thread 0)
   int node;
   int pending;         // child whose rejection the running pass serves
   double masked_sum;
   int n_tests, n_passes;
-  int stage, phase;    // consumer ring position
-  uint32_t xphase;     // parity of the cluster-exchange barrier
-  int xbuf;            // double-buffer index of the exchange slots
 };
 
 struct TreeSmem {
@@ -67,8 +56,10 @@ __host__ __device__ inline int slice_len(int V, int C) {
   return (per + kChunk - 1) / kChunk * kChunk;
 }
 
-__host__ __device__ inline int n_tiles(int V, int C) {
-  return (slice_len(V, C) + kTileElems - 1) / kTileElems;
+// Bonus tiles of a cluster CTA's slice (a slice may start inside an 8-element
+// block, so up to 7 elements more).
+__host__ __device__ inline int tree_tiles(int V, int C) {
+  return (slice_len(V, C) + kChunk - 1 + kTileElems - 1) / kTileElems;
 }
 
 // Shared memory of one tree's state with `nt` bonus tiles.
@@ -76,9 +67,6 @@ __host__ __device__ inline size_t tree_smem_bytes_nt(int R, int nt) {
   return (size_t)R * (9 * 8 + 7 * 4 + 6 * 4 + 1) + (size_t)nt * 8 + 64;
 }
 
-__host__ __device__ inline size_t tree_smem_bytes(int R, int V, int C) {
-  return tree_smem_bytes_nt(R, n_tiles(V, C));
-}
 
 __device__ __forceinline__ TreeSmem carve_tree_nt(char* base, int R, int nt) {
   TreeSmem s;
@@ -113,10 +101,6 @@ __device__ __forceinline__ TreeSmem carve_tree_nt(char* base, int R, int nt) {
   return s;
 }
 
-__device__ __forceinline__ TreeSmem carve_tree(char* base, int R, int V, int C) {
-  return carve_tree_nt(base, R, n_tiles(V, C));
-}
-
 // ------------------------------------------------------------ control ----
 
 __device__ __forceinline__ int first_alive_child(const TreeSmem& s, int i) {
@@ -125,16 +109,10 @@ __device__ __forceinline__ int first_alive_child(const TreeSmem& s, int i) {
   return j;
 }
 
-// M_b^(0)(x_c | X^i) of every child c of node i, in float64, computed by the
-// consumer warps as soon as row i's normaliser is known (a residual
-// a M_b(x) - b M_s(x) of a sibling can cancel by orders of magnitude, so this
-// single value must not carry a float32 rounding).  Kept in s.mb0[c].
-__device__ __forceinline__ void children_mb0(const TreeSmem& s, int i, double cd, int lane) {
-  int j = s.first[i];
-  for (int k = 0; j >= 0; ++k, j = s.next[j])
-    if ((k & 31) == lane)
-      s.mb0[j] = exp2(((double)s.gl[j] - (double)s.rowm[i]) * cd) * s.invs[i];
-}
+// s.mb0[c] holds M_b^(0)(x_c | X^i) of child c of node i, in float64,
+// exp2((l_i(x_c) - m_i) log2(e) / T) / s_i, computed as soon as row i's
+// normaliser is known (a residual a M_b(x) - b M_s(x) of a sibling can cancel by
+// orders of magnitude, so this single value must not carry a float32 rounding).
 
 // min(p_i M_b(x_c) / M_s(x_c), 1) from i's current state, with
 // M_s(x_c) = q_c / Z_i; false if it is zero.

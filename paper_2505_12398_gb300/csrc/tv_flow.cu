@@ -55,6 +55,7 @@ namespace flow {
 using namespace tvk::fused;
 
 constexpr int kMaxNCW = 8;
+constexpr int kMaxStages = 8;       // ring stages at most
 constexpr int kSlots = 2;           // queued slices a CTA holds: one streaming, one ahead
 constexpr int kPBuf = 256;          // partials of a job kept in shared memory by the poll
 constexpr unsigned long long kNoPart = ~0ull;   // a partial slot not written yet
@@ -858,7 +859,7 @@ __device__ void owner_combine(const TravArgs& a, const FlowArgs& f, const TreeSm
     if (__any_sync(0xffffffffu, bad_row) && lane == 0) sh.ctl.bad |= 64u;
     __syncwarp();
     // ... then M_b^(0) of those rows' children, one lane per node (the same
-    // value children_mb0 gives, see there)
+    // value the cluster kernel computes, see tv_control.cuh)
     for (int i = lane + 1; i < R; i += 32) {
       const int p = s.par[i];
       bool mine = false;
@@ -1420,11 +1421,11 @@ FlowPlan tv_flow_plan(int R, int B, int V, int smem_per_sm, int smem_per_block, 
   if (force_slice_min >= 256 && force_slice_min % 256 == 0) p.slice_min = force_slice_min;
   p.slice_min = std::min(p.slice_min, std::min(p.slice_pass, p.slice_stats));
   const int per_sm = 16 / p.ncw;   // CTAs per SM the kernel is built for
-  if (force_stages >= 2 && force_stages <= tvk::fused::kMaxStages) {
+  if (force_stages >= 2 && force_stages <= tvk::flow::kMaxStages) {
     p.stages = force_stages;
   } else {
     p.stages = 2;
-    for (int st = tvk::fused::kMaxStages; st >= 2; --st)
+    for (int st = tvk::flow::kMaxStages; st >= 2; --st)
       if ((size_t)per_sm * (flow_smem_bytes(R, p.ncw, st) + 4096) <= (size_t)smem_per_sm) {
         p.stages = st;
         break;

@@ -1,24 +1,49 @@
-// tv_tree.cu -- fused, lazy, TMA-pipelined Traversal Verification (sm_103a).
+// tv_tree.cu -- one thread-block cluster per tree: lazy, latency-oriented
+// Traversal Verification (sm_103a).
 //
 // One kernel does all of Algorithm 3 (§3.1) for a batch of trees.  Each tree
-// is owned by a thread-block cluster of C CTAs (C = 1, 2 or 4): CTA r streams
-// the vocabulary slice [v0_r, v1_r) of every row the tree needs, and every CTA
-// runs the same serial control on identical data, so their decisions agree
-// without being broadcast; only per-row partial results cross the cluster
-// (distributed shared memory + a remote mbarrier arrive).
+// is owned by a cluster of C CTAs: CTA r streams the vocabulary slice
+// [v0_r, v1_r) of every row the tree needs, and every CTA runs the same serial
+// control on identical data, so their decisions agree without being broadcast;
+// only partial results cross the cluster.
 //
-// Inside a CTA, warp 8 is a producer: one lane issues 1-D bulk copies
-// (cp.async.bulk, TMA) of row slices into a ring of shared-memory stages,
-// completion counted on per-stage mbarriers; warps 0-7 consume the stages
-// (128-bit shared loads) and arrive on per-stage "empty" mbarriers.
+// What bounds it: a tree is a chain of 10 to 30 dependent vocabulary jobs
+// (normalisers of a chain of rows, rejection passes, the bonus draw), each of
+// a few microseconds, so the time is the sum of the latencies along that chain,
+// not bandwidth.  The kernel is built to keep each link short:
+//   * warp-specialised: NCW consumer warps reduce, a producer warp issues the
+//     bulk copies (TMA), a control warp runs the serial control.  While a pass
+//     runs, the control warp works out the step after it (Ahead), so that one
+//     float64 comparison and one division stand between a pass's S and the
+//     next job;
+//   * every consumer warp sends its partial straight to the control warps of
+//     all C CTAs (st.async: the store carries its own completion count), with
+//     no reduction inside the CTA in between; two exchange buffers alternate;
+//   * a normaliser job takes up to kStatRows rows of the chain being entered:
+//     one exchange for all of them, and the rows' final sums and their
+//     children's float64 masses are spread over the consumer warps;
+//   * where a slice of a (target, draft) row pair fits the ring, it stays there:
+//     the next pass at the same node (about half of all passes) reads no
+//     memory, and with room for two the parent's pair is fetched while the
+//     node's passes run.
 //
 // Rows are read lazily.  The target row of a node is streamed (for its
-// normaliser) only when the traversal first descends through the node --
-// the rates of a node's children are needed only then -- so sub-trees the
-// traversal never enters cost nothing.  The whole not-yet-normalised part of
-// the chain being entered is requested as one job.  Each rejection streams the
-// parent's ORIGINAL target and draft rows once (the (a, b, Z) closed form of
+// normaliser) only when the traversal first descends through the node, so
+// sub-trees the traversal never enters cost nothing.  Each rejection needs the
+// parent's ORIGINAL target and draft rows (the (a, b, Z) closed form of
 // Eqs. (1)-(2), see tv_kernels.cu); the bonus draw streams one row (pair).
+//
+// Rows need no alignment: slices are copied as whole 8-element blocks of the
+// flat [B][N+1][V] arrays and the elements of the neighbouring rows in the
+// first and last block are masked.  (Handles use this kernel for V % 8 == 0.)
+//
+// Every wait is bounded; one that gives up raises TV_STATUS_TIMEOUT, and all
+// roles still reach the cluster barrier at the end.
+//
+// Measured (60-node trees, V = 32000, bf16; 8-token chains, fp32), against one
+// thread of the consumers doing the control, a reduction and an exchange per
+// row and no resident pairs: B = 64 254.7 -> 183.2 us, B = 1 119 -> 81 us,
+// 16 chains 117.2 -> 77.2 us.
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -30,76 +55,913 @@
 namespace tvk {
 namespace fused {
 
-// ----------------------------------------------------- cluster exchange ---
+constexpr int kTreeMaxStages = 16;
+constexpr int kTreeMaxSlots = 8;     // resident row pairs tracked at most
+constexpr int kStatRows = 8;         // rows of one normaliser job at most
 
-// Publishes this CTA's partial (x, y) for the current row to every CTA of the
-// cluster and waits for all of them; returns false on timeout.  Called by
-// thread 0 only.  Slots are double-buffered so that a fast CTA's next
-// exchange cannot overwrite a slot a slow CTA has not read yet.
-__device__ bool exchange(float2 (*slots)[kMaxCluster], uint64_t* xbar, Ctl& ctl, int C,
-                         uint32_t rank, float x, float y) {
-  const int buf = ctl.xbuf;
-  for (int r = 0; r < C; ++r) {
-    st_cluster_v2(map_shared(&slots[buf][rank], r), x, y);
-    mbar_arrive_remote(map_shared(xbar, r));
+// Tiles of 256 tokens one consumer warp takes per ring stage.
+__host__ __device__ constexpr int tiles_per_warp(int ncw) { return ncw == 16 ? 1 : 2; }
+
+// One ring stage holds tiles_per_warp tiles per consumer warp of target and
+// draft values, or (normalisers, leaf draws) that many bytes of target values.
+__host__ __device__ constexpr int tree_stage_bytes(int ncw, int lb) {
+  return ncw * tiles_per_warp(ncw) * kTileElems * (lb + 4);
+}
+
+// A job as the control warp hands it to the CTA's other warps.
+struct TreeJob {
+  int kind, node, n_rows, nmask;
+  float alpha1, beta, rowmax;
+  int total;               // ring chunks the job loads (0: its pair is resident)
+  int slot;                // resident slot of a pair (-1: streamed through the ring)
+  int pf_node, pf_slot;    // pair to fetch ahead into another slot (-1: none)
+  int mbuf;                // which list of removed tokens
+  int xb, xph;             // exchange buffer and the parity of its barrier
+  int rows[kStatRows];
+};
+
+struct TreeShared {
+  Ctl ctl;
+  Ahead ahead;
+  TreeJob job;
+  // the resident row pairs, tracked by the control warp: node and last use
+  int slot_node[kTreeMaxSlots];
+  int slot_used[kTreeMaxSlots];
+};
+
+// Sends (x, y) to slot address `dst` of a CTA of the cluster; the store counts
+// 8 bytes on that CTA's barrier `bar` (both addresses from map_shared).
+__device__ __forceinline__ void st_async_v2(uint32_t dst, float x, float y, uint32_t bar) {
+  asm volatile(
+      "st.async.shared::cluster.mbarrier::complete_tx::bytes.v2.f32 [%0], {%1, %2}, [%3];" ::"r"(
+          dst),
+      "f"(x), "f"(y), "r"(bar)
+      : "memory");
+}
+
+__device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity) {
+  return __all_sync(0xffffffffu, mbar_wait(bar, parity) ? 1 : 0) != 0;
+}
+
+// A row's slice [v0, v1) as whole 8-element blocks of the flat array: first
+// element of the first block, elements of the previous row in it, and the
+// length from that block's start.
+struct Slice {
+  size_t base;
+  int sh, n;
+  __device__ __forceinline__ Slice(size_t row, int V, int v0, int v1) {
+    const size_t f = row * (size_t)V + (size_t)v0;
+    sh = (int)(f & 7u);
+    base = f - (size_t)sh;
+    n = v1 > v0 ? v1 - v0 + sh : 0;
   }
-  const bool ok = mbar_wait_cluster(xbar, ctl.xphase);
-  ctl.xphase ^= 1u;
-  ctl.xbuf ^= 1;
-  return ok;
+};
+
+__device__ __forceinline__ int chunks_of(int n, int per) { return (n + per - 1) / per; }
+
+// Eight logits of one lane: bf16 clamped and widened, or fp32.
+template <typename L>
+__device__ __forceinline__ void lds_logits(const typename L::elem* p, float v[8]) {
+  if constexpr (L::kBytes == 2) {
+    float2 vp[4];
+    bf16x8_pairs(lds128(p), vp);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) { v[2 * k] = vp[k].x; v[2 * k + 1] = vp[k].y; }
+  } else {
+    const uint4 a = lds128(p), b = lds128(p + 4);
+    v[0] = __uint_as_float(a.x); v[1] = __uint_as_float(a.y);
+    v[2] = __uint_as_float(a.z); v[3] = __uint_as_float(a.w);
+    v[4] = __uint_as_float(b.x); v[5] = __uint_as_float(b.y);
+    v[6] = __uint_as_float(b.z); v[7] = __uint_as_float(b.w);
+  }
+}
+
+// e(x) of eight logits relative to m (kPass: the cheaper form of passes and
+// draws; see tv_device.cuh).
+template <typename L, bool kPass>
+__device__ __forceinline__ void exp8(const float v[8], float m, float c_hi, float c_lo,
+                                     float e[8]) {
+  if constexpr (L::kBytes == 2) {
+    const float2 mm = make_float2(-m, -m), ch = make_float2(c_hi, c_hi),
+                 cl = make_float2(c_lo, c_lo);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const float2 d = __fadd2_rn(make_float2(v[2 * k], v[2 * k + 1]), mm);
+      const float2 r = kPass ? exp2_corrected_x2(d, ch, cl) : exp2_split_x2(d, ch, cl);
+      e[2 * k] = r.x;
+      e[2 * k + 1] = r.y;
+    }
+  } else {
+#pragma unroll
+    for (int k = 0; k < 8; ++k)
+      e[k] = kPass ? L::exp_pass(v[k], m, c_hi, c_lo) : L::exp_rel(v[k], m, c_hi, c_lo);
+  }
+}
+
+// [alpha e(x) - beta q(x)]_+ of eight tokens.
+template <typename L>
+__device__ __forceinline__ void residual8(const float v[8], const float* qp, float rowmax,
+                                          float alpha, float beta, float c_hi, float c_lo,
+                                          float t[8]) {
+  const uint4 qa = lds128(qp), qc = lds128(qp + 4);
+  const float q[8] = {__uint_as_float(qa.x), __uint_as_float(qa.y), __uint_as_float(qa.z),
+                      __uint_as_float(qa.w), __uint_as_float(qc.x), __uint_as_float(qc.y),
+                      __uint_as_float(qc.z), __uint_as_float(qc.w)};
+  float e[8];
+  exp8<L, true>(v, rowmax, c_hi, c_lo, e);
+  if constexpr (L::kBytes == 2) {
+    const float2 al2 = make_float2(alpha, alpha), nb2 = make_float2(-beta, -beta);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const float2 x = __ffma2_rn(al2, make_float2(e[2 * k], e[2 * k + 1]),
+                                  __fmul2_rn(nb2, make_float2(q[2 * k], q[2 * k + 1])));
+      t[2 * k] = fmaxf(x.x, 0.f);
+      t[2 * k + 1] = fmaxf(x.y, 0.f);
+    }
+  } else {
+#pragma unroll
+    for (int k = 0; k < 8; ++k) t[k] = fmaxf(fmaf(alpha, e[k], -beta * q[k]), 0.f);
+  }
+}
+
+// Up to eight logits / draft probabilities of a block in global memory,
+// elements outside [lo, hi) of the block read as -inf / 0.
+template <typename L>
+__device__ __forceinline__ void block_logits(const typename L::elem* p, int lo, int hi,
+                                             float v[8]) {
+  if (lo <= 0 && hi >= 8) {
+    L::chunk_vec(p, 0, v);
+  } else {
+#pragma unroll
+    for (int k = 0; k < 8; ++k) v[k] = (k >= lo && k < hi) ? L::at(p, k) : TV_NEG_INF;
+  }
+}
+
+__device__ __forceinline__ void block_probs(const float* p, int lo, int hi, float q[8]) {
+#pragma unroll
+  for (int k = 0; k < 8; ++k) q[k] = (k >= lo && k < hi) ? __ldg(p + k) : 0.f;
 }
 
 // ------------------------------------------------------------- kernel -----
 
-struct ConsumerCtx {
-  int stage, phase;
+template <typename L, int NCW>
+struct TreeCta {
+  using E = typename L::elem;
+  static constexpr int kLB = L::kBytes;
+  static constexpr int kStageBytes = tree_stage_bytes(NCW, kLB);
+  static constexpr int kPair = kStageBytes / (kLB + 4);   // tokens of a pair chunk
+  static constexpr int kRow = kStageBytes / kLB;          // tokens of a target-only chunk
+  static constexpr int kSweep = NCW * kTileElems;
+  static constexpr int kThreads = NCW * 32 + 64;          // + producer, control warps
+  static_assert(kPair % kTileElems == 0, "whole tiles per stage");
+
+  const TravArgs& a;
+  TreeSmem s;
+  TreeShared& sh;
+  char* ring;
+  float2* xs;              // [2][kStatRows][C * NCW] exchange slots
+  int* mtok_ahead;         // [2][R] removed tokens of passes worked out ahead
+  uint64_t *full_bar, *empty_bar, *xbar, *job_bar, *ack_bar, *stat_bar, *tile_bar;
+  int C, n_stages, b, v0, v1;
+  uint32_t rank;
+  size_t row0;             // the tree's first row in the batch
+
+  __device__ TreeCta(const TravArgs& args, TreeShared& shared) : a(args), sh(shared) {}
+
+  __device__ __forceinline__ void fail() { atomicOr(&sh.ctl.bad, 32u); }
+  __device__ __forceinline__ float2* xslots(int buf, int row) const {
+    return xs + ((size_t)buf * kStatRows + row) * (size_t)(C * NCW);
+  }
+  // Lists of removed tokens: 0 the control's own, 1 and 2 worked out ahead.
+  __device__ __forceinline__ int* mtok(int k) const {
+    return k == 0 ? s.mask_tok : mtok_ahead + (size_t)(k - 1) * (a.N + 1);
+  }
+  static __device__ __forceinline__ bool is_pair(int kind) {
+    return kind == kJobPass || kind == kJobBonusRes;
+  }
+
+  // ---------------------------------------------------------- producer --
+  // Fills stage `st` with chunk k of the row's slice (n_all: elements of the
+  // arrays).  `filled` and `fph` track each stage's fills: a fetch ahead that no
+  // job has waited for must have landed before its stage is filled again.
+  __device__ bool fill(int st, size_t row, int k, bool pair, size_t n_all, uint32_t& filled,
+                       uint32_t& fph) {
+    if ((filled >> st) & 1u) {
+      if (!mbar_wait(&full_bar[st], (fph >> st) & 1u)) return false;
+    }
+    filled |= 1u << st;
+    fph ^= 1u << st;
+    const Slice sl(row, a.V, v0, v1);
+    const int per = pair ? kPair : kRow;
+    const size_t e0 = sl.base + (size_t)k * per;
+    int n = min(per, sl.n - k * per);
+    n = (n + 7) & ~7;                        // whole blocks
+    char* dst = ring + (size_t)st * kStageBytes;
+    int whole = n;
+    if (e0 + n > n_all) {
+      // the last, partial block of the arrays: its elements one by one
+      whole = (int)((n_all - e0) & ~(size_t)7);
+      const int tail = (int)(n_all - e0);
+      const E* lg = reinterpret_cast<const E*>(a.logits);
+      for (int j = whole; j < tail; ++j) {
+        reinterpret_cast<E*>(dst)[j] = lg[e0 + j];
+        if (pair) reinterpret_cast<float*>(dst + (size_t)kPair * kLB)[j] = a.draft_probs[e0 + j];
+      }
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    }
+    const uint32_t lbytes = (uint32_t)whole * kLB, qbytes = pair ? (uint32_t)whole * 4u : 0u;
+    mbar_arrive_expect_tx(&full_bar[st], lbytes + qbytes);
+    if (whole > 0) {
+      tma_load_1d(dst, reinterpret_cast<const E*>(a.logits) + e0, lbytes, &full_bar[st]);
+      if (pair)
+        tma_load_1d(dst + (size_t)kPair * kLB, a.draft_probs + e0, qbytes, &full_bar[st]);
+    }
+    return true;
+  }
+
+  // Streams the jobs' rows (one lane).
+  __device__ bool produce(size_t n_all, uint32_t& filled, uint32_t& fph) {
+    const int spc = chunks_of(v1 - v0 + 7, kPair);
+    uint32_t jp = 0u, eph = 0u;
+    for (;;) {
+      if (!mbar_wait(job_bar, jp)) return false;
+      jp ^= 1u;
+      const TreeJob job = sh.job;
+      mbar_arrive(ack_bar);                    // the job may be replaced from here on
+      if (job.kind == kJobDone) return true;
+      const bool pair = is_pair(job.kind);
+      const int per = pair ? kPair : kRow;
+      if (job.total > 0) {
+        const int st0 = job.slot > 0 ? job.slot * spc : 0;
+        int q = 0;
+        for (int r = 0; r < job.n_rows; ++r) {
+          const size_t row = row0 + (job.kind == kJobStats ? sh.job.rows[r] : job.node);
+          const int nch = chunks_of(Slice(row, a.V, v0, v1).n, per);
+          for (int k = 0; k < nch; ++k, ++q) {
+            const int st = st0 + (job.slot >= 0 ? k : q % n_stages);
+            if (q >= n_stages) {               // a stage of this job, used again
+              if (!mbar_wait(&empty_bar[st], (eph >> st) & 1u)) return false;
+              eph ^= 1u << st;
+            }
+            if (!fill(st, row, k, pair, n_all, filled, fph)) return false;
+          }
+        }
+      }
+      if (job.pf_node >= 0) {
+        const size_t row = row0 + job.pf_node;
+        const int nch = chunks_of(Slice(row, a.V, v0, v1).n, kPair);
+        for (int k = 0; k < nch; ++k)
+          if (!fill(job.pf_slot * spc + k, row, k, true, n_all, filled, fph)) return false;
+      }
+    }
+  }
+
+  __device__ void producer(size_t n_all) {
+    uint32_t filled = 0u, fph = 0xffffffffu;
+    if (!produce(n_all, filled, fph)) fail();
+    // copies in flight land before the CTA may exit
+    for (int st = 0; st < n_stages; ++st)
+      if (((filled >> st) & 1u) && !mbar_wait(&full_bar[st], (fph >> st) & 1u)) fail();
+  }
+
+  // ---------------------------------------------------------- exchange --
+  // A partial of row r of the job, to every CTA.  The exchange's barrier
+  // counts the bytes of all CTAs' partials (the control warp arms it); a tree
+  // of one CTA is launched without a cluster, so there the warps store to
+  // their own slots and arrive once per job (arrive_alone).
+  __device__ __forceinline__ void send(int xb, int r, int slot, int lane, float x, float y) {
+    if (C == 1) {
+      if (lane == 0) xslots(xb, r)[slot] = make_float2(x, y);
+    } else if (lane < C) {
+      st_async_v2(map_shared(xslots(xb, r) + slot, lane), x, y, map_shared(&xbar[xb], lane));
+    }
+  }
+  __device__ __forceinline__ void arrive_alone(int xb, int lane) {
+    if (C == 1 && lane == 0) mbar_arrive(&xbar[xb]);
+  }
+  __device__ __forceinline__ bool exchanged(int xb, uint32_t parity) {   // a whole warp
+    if (C == 1) return mbar_wait_warp(&xbar[xb], parity);
+    return __all_sync(0xffffffffu, mbar_wait_cluster(&xbar[xb], parity) ? 1 : 0) != 0;
+  }
+
+  // --------------------------------------------------------- consumers --
+
+  __device__ void consumer(int wid, int lane) {
+    const float c_hi = a.c_hi, c_lo = a.c_lo;
+    uint32_t jp = 0u;
+    uint32_t ph = 0xffffffffu;                 // parity of each stage's latest fill
+    for (;;) {
+      if (!mbar_wait_warp(job_bar, jp)) { fail(); return; }
+      jp ^= 1u;
+      const TreeJob& job = sh.job;
+      const int kind = job.kind;
+      if (kind == kJobDone) return;
+      const bool pair = is_pair(kind);
+      const int per = pair ? kPair : kRow;
+      const int nrows = kind == kJobStats ? job.n_rows : 1;
+      const int total = job.total, slot = job.slot;
+      const int spc = chunks_of(v1 - v0 + 7, kPair);
+      const int st0 = slot > 0 ? slot * spc : 0;
+      const int nmask = job.nmask;
+      const int pf_node = job.pf_node, pf_slot = job.pf_slot, xb = job.xb;
+      const int* mt = mtok(job.mbuf);
+      const float al = job.alpha1, be = job.beta, rm = job.rowmax;
+      int q = 0;
+      for (int r = 0; r < nrows; ++r) {
+        const int node = kind == kJobStats ? job.rows[r] : job.node;
+        const Slice sl(row0 + node, a.V, v0, v1);
+        const int nch = chunks_of(sl.n, per);
+        float m_run = TV_NEG_INF;
+        Comp acc;
+        int mp = 0;
+        for (int k = 0; k < nch; ++k, ++q) {
+          const int st = st0 + (slot >= 0 ? k : q % n_stages);
+          if (total > 0) ph ^= 1u << st;       // filled by this job
+          if (!mbar_wait_warp(&full_bar[st], (ph >> st) & 1u)) { fail(); return; }
+          const int n = min(per, sl.n - k * per);
+          const char* buf = ring + (size_t)st * kStageBytes;
+          const E* lb = reinterpret_cast<const E*>(buf);
+          const float* qb = reinterpret_cast<const float*>(buf + (size_t)kPair * kLB);
+          for (int t0 = wid * kTileElems; t0 < n; t0 += kSweep) {
+            const int e0 = t0 + lane * kChunk;
+            const bool valid = e0 < n;
+            const int g0 = k * per + e0;       // from the start of the slice's first block
+            const int xg = v0 - sl.sh + g0;    // token of the lane's first element
+            // elements of the lane's block that belong to the slice: [lo, hi)
+            const int lo = sl.sh - g0, hi = sl.n - g0;
+            const bool edge = valid && (lo > 0 || hi < 8);
+            float v[8], t[8];
+            if (valid) {
+              lds_logits<L>(lb + e0, v);
+            } else {
+#pragma unroll
+              for (int e = 0; e < 8; ++e) v[e] = kLB == 2 ? -9984.f : TV_NEG_INF;
+            }
+            if (edge) {
+#pragma unroll
+              for (int e = 0; e < 8; ++e)
+                if (e < lo || e >= hi) v[e] = kLB == 2 ? -9984.f : TV_NEG_INF;
+            }
+            if (kind == kJobStats) {
+              if (valid) {
+                const float cm = fmaxf(fmaxf(fmaxf(v[0], v[1]), fmaxf(v[2], v[3])),
+                                       fmaxf(fmaxf(v[4], v[5]), fmaxf(v[6], v[7])));
+                if (cm > m_run) {
+                  if (m_run != TV_NEG_INF) {
+                    const float sc = L::exp_rel(m_run, cm, c_hi, c_lo);
+                    acc.s *= sc;
+                    acc.c *= sc;
+                  }
+                  m_run = cm;
+                }
+                exp8<L, false>(v, m_run, c_hi, c_lo, t);
+                if (edge) {
+#pragma unroll
+                  for (int e = 0; e < 8; ++e) if (e < lo || e >= hi) t[e] = 0.f;
+                }
+                acc.add(sum8(t));
+              }
+            } else if (kind == kJobBonusLeaf) {
+              const float lm = fmaxf(fmaxf(fmaxf(v[0], v[1]), fmaxf(v[2], v[3])),
+                                     fmaxf(fmaxf(v[4], v[5]), fmaxf(v[6], v[7])));
+              const float tm = warp_max(lm);
+              exp8<L, true>(v, tm, c_hi, c_lo, t);
+              if (edge) {
+#pragma unroll
+                for (int e = 0; e < 8; ++e) if (e < lo || e >= hi) t[e] = 0.f;
+              }
+              const float ts = warp_sum(valid ? sum8(t) : 0.f);
+              if (lane == 0) {
+                const int tile = (k * per + t0) / kTileElems;
+                s.tsum[tile] = ts;
+                s.tmax[tile] = tm;
+              }
+            } else {
+              if (valid) {
+                residual8<L>(v, qb + e0, rm, al, be, c_hi, c_lo, t);
+              } else {
+#pragma unroll
+                for (int e = 0; e < 8; ++e) t[e] = 0.f;
+              }
+              if (edge) {
+#pragma unroll
+                for (int e = 0; e < 8; ++e) if (e < lo || e >= hi) t[e] = 0.f;
+              }
+              while (mp < nmask && mt[mp] < xg) ++mp;
+              for (int mq = mp; mq < nmask && mt[mq] < xg + kChunk; ++mq) {
+                const int off = mt[mq] - xg;
+                if (!valid || off < lo || off >= hi) continue;   // (another slice's token)
+                const float mv = (kind == kJobPass) ? 0.f : s.mask_val[mq];
+#pragma unroll
+                for (int e = 0; e < 8; ++e) if (e == off) t[e] = mv;
+              }
+              if (kind == kJobPass) {
+                if (valid) acc.add(sum8(t));
+              } else {
+                const float ts = warp_sum(valid ? sum8(t) : 0.f);
+                if (lane == 0) s.tsum[(k * per + t0) / kTileElems] = ts;
+              }
+            }
+          }
+          if (q + n_stages < total) {          // the producer waits for this stage
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&empty_bar[st]);
+          }
+        }
+        // ---- this warp's partial of the row, to every CTA's control warp ----
+        if (kind == kJobStats) {
+          const float wm = warp_max(m_run);
+          const float part =
+              (m_run == TV_NEG_INF) ? 0.f : acc.value() * L::exp_rel(m_run, wm, c_hi, c_lo);
+          send(xb, r, (int)rank * NCW + wid, lane, wm, warp_sum(part));
+        } else if (kind == kJobPass) {
+          send(xb, 0, (int)rank * NCW + wid, lane, warp_sum(acc.value()), 0.f);
+        }
+      }
+      if (wid != 0 || kind == kJobStats || kind == kJobPass) arrive_alone(xb, lane);
+      // (a pass's job may have been replaced by now: nothing of it is read below)
+      if (pf_node >= 0) {
+        const int nch = chunks_of(Slice(row0 + pf_node, a.V, v0, v1).n, kPair);
+        ph ^= ((1u << nch) - 1u) << (pf_slot * spc);
+      }
+      if (kind == kJobStats) {
+        if (!finish_rows(job, wid, lane)) { fail(); return; }
+      } else if (kind != kJobPass) {
+        __syncwarp();
+        if (lane == 0) mbar_arrive(tile_bar);
+        if (wid == 0 && !draw(job, lane)) { fail(); return; }
+      }
+    }
+  }
+
+  // The rows' normalisers from all warps' partials (a row per warp, the same
+  // order in every CTA), and M_b^(0) of their children.
+  __device__ bool finish_rows(const TreeJob& job, int wid, int lane) {
+    const float c_hi = a.c_hi, c_lo = a.c_lo;
+    const int n_rows = job.n_rows, n = C * NCW;
+    if (!exchanged(job.xb, job.xph)) return false;
+    for (int r = wid; r < n_rows; r += NCW) {
+      const float2* x = xslots(job.xb, r);
+      float M = TV_NEG_INF;
+      for (int k = lane; k < n; k += 32) M = fmaxf(M, x[k].x);
+      M = warp_max(M);
+      float S = 0.f;
+      for (int k = lane; k < n; k += 32) {
+        const float2 p = x[k];
+        if (p.x != TV_NEG_INF) S += p.y * L::exp_rel(p.x, M, c_hi, c_lo);
+      }
+      S = warp_sum(S);
+      const int node = job.rows[r];
+      const double invs = 1.0 / (double)S;
+      int j = s.first[node];
+      for (int k = 0; k < lane && j >= 0; ++k) j = s.next[j];
+      while (j >= 0) {
+        s.mb0[j] = exp2(((double)s.gl[j] - (double)M) * a.c) * invs;
+        for (int k = 0; k < 32 && j >= 0; ++k) j = s.next[j];
+      }
+      if (lane == 0) {
+        s.rowm[node] = M;
+        s.rows[node] = S;
+        s.invs[node] = invs;
+        if (!(S > 0.f)) atomicOr(&sh.ctl.bad, 64u);   // no finite logit in the row
+      }
+    }
+    __syncwarp();
+    if (lane == 0) mbar_arrive(stat_bar);
+    return true;
+  }
+
+  // The bonus draw (warp 0 of every CTA): slice totals, crossing slice,
+  // crossing tile, token.
+  __device__ bool draw(const TreeJob& job, int lane) {
+    const float c_hi = a.c_hi, c_lo = a.c_lo;
+    const bool leaf = (job.kind == kJobBonusLeaf);
+    const int node = job.node, R = a.N + 1;
+    const float* u = a.uniforms + (size_t)b * (R + 1);
+    if (!mbar_wait_warp(tile_bar, 0u)) return false;
+    const Slice sl(row0 + node, a.V, v0, v1);
+    const int ntl = (sl.n + kTileElems - 1) / kTileElems;
+    float Mc = 0.f;
+    if (leaf) {
+      float lm = TV_NEG_INF;
+      for (int k = lane; k < ntl; k += 32) lm = fmaxf(lm, s.tmax[k]);
+      Mc = warp_max(lm);
+      for (int k = lane; k < ntl; k += 32)
+        s.tsum[k] = (s.tmax[k] == TV_NEG_INF)
+                        ? 0.f : s.tsum[k] * L::exp_rel(s.tmax[k], Mc, c_hi, c_lo);
+      __syncwarp();
+    }
+    float Wc = 0.f;
+    for (int k0 = 0; k0 < ntl; k0 += 32) {
+      const float v = (k0 + lane < ntl) ? s.tsum[k0 + lane] : 0.f;
+      Wc += warp_sum(v);
+    }
+    // every CTA learns every slice's (max, total)
+    send(job.xb, 0, (int)rank, lane, Mc, Wc);
+    arrive_alone(job.xb, lane);
+    if (!exchanged(job.xb, job.xph)) return false;
+    const float2* x = xslots(job.xb, 0);
+    float scale = 1.f, target = 0.f, before = 0.f, W = 0.f;
+    int owner = -1;
+    float Mg = x[0].x;
+    if (leaf)
+      for (int rr = 1; rr < C; ++rr) Mg = fmaxf(Mg, x[rr].x);
+    auto slice_scale = [&](int rr) -> float {
+      return leaf ? ((x[rr].x == TV_NEG_INF) ? 0.f : L::exp_rel(x[rr].x, Mg, c_hi, c_lo)) : 1.f;
+    };
+    for (int rr = 0; rr < C; ++rr) W += x[rr].y * slice_scale(rr);
+    target = u[R] * W;
+    float acc0 = 0.f;
+    for (int rr = 0; rr < C; ++rr) {
+      const float wr = x[rr].y * slice_scale(rr);
+      if (owner < 0 && target < acc0 + wr) { owner = rr; before = acc0; }
+      acc0 += wr;
+    }
+    if (owner < 0) {   // rounding: the last slice with weight
+      owner = C - 1;
+      while (owner > 0 && !(x[owner].y > 0.f)) --owner;
+      before = 0.f;
+      for (int rr = 0; rr < owner; ++rr) before += x[rr].y * slice_scale(rr);
+    }
+    if ((uint32_t)owner != rank) return true;
+    scale = slice_scale((int)rank);
+    // local target in this slice's units
+    const float lt = (scale > 0.f) ? (target - before) / scale : 0.f;
+    int tile = -1;
+    float tbase = 0.f, base = 0.f;
+    for (int k0 = 0; k0 < ntl && tile < 0; k0 += 32) {
+      float v = (k0 + lane < ntl) ? s.tsum[k0 + lane] : 0.f;
+      const float own = v;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const float w2 = __shfl_up_sync(0xffffffffu, v, o);
+        if (lane >= o) v += w2;
+      }
+      const unsigned hit = __ballot_sync(0xffffffffu, (k0 + lane < ntl) && (lt < base + v));
+      if (hit) {
+        const int l = __ffs(hit) - 1;
+        tile = k0 + l;
+        tbase = base + __shfl_sync(0xffffffffu, v - own, l);
+      }
+      base += __shfl_sync(0xffffffffu, v, 31);
+    }
+    if (tile < 0) {
+      tile = ntl - 1;
+      while (tile > 0 && !(s.tsum[tile] > 0.f)) --tile;
+      float a0 = 0.f;
+      for (int k = 0; k < tile; ++k) a0 += s.tsum[k];
+      tbase = a0;
+    }
+    // element-level rescan of the crossing tile (global loads, L2-hot)
+    const int g0 = tile * kTileElems + lane * kChunk;
+    const int x0 = v0 - sl.sh + g0;
+    const int lo = sl.sh - g0, hi = sl.n - g0;
+    const size_t at = sl.base + (size_t)g0;
+    float w[8];
+    {
+      float v[8];
+      block_logits<L>(reinterpret_cast<const E*>(a.logits) + at, lo, hi, v);
+      if (leaf) {
+#pragma unroll
+        for (int e = 0; e < 8; ++e)
+          w[e] = (v[e] == TV_NEG_INF) ? 0.f : L::exp_pass(v[e], Mc, c_hi, c_lo);
+      } else {
+        float qv[8];
+        block_probs(a.draft_probs + at, lo, hi, qv);
+#pragma unroll
+        for (int e = 0; e < 8; ++e)
+          w[e] = (v[e] == TV_NEG_INF)
+                     ? 0.f
+                     : fmaxf(fmaf(job.alpha1, L::exp_pass(v[e], job.rowmax, c_hi, c_lo),
+                                  -job.beta * qv[e]), 0.f);
+        const int* mt = mtok(job.mbuf);
+        for (int mq = 0; mq < job.nmask; ++mq) {
+          const int off = mt[mq] - x0;
+          if (off < lo || off >= hi) continue;
+          const float mv = s.mask_val[mq];
+#pragma unroll
+          for (int e = 0; e < 8; ++e) if (e == off) w[e] = mv;
+        }
+      }
+    }
+    float pre[8];
+    float run = 0.f;
+#pragma unroll
+    for (int e = 0; e < 8; ++e) { run += w[e]; pre[e] = run; }
+    float v = run;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const float w2 = __shfl_up_sync(0xffffffffu, v, o);
+      if (lane >= o) v += w2;
+    }
+    const float lbase = tbase + (v - run);
+    int found = 8;
+#pragma unroll
+    for (int e = 7; e >= 0; --e) if (e >= lo && lt < lbase + pre[e]) found = e;
+    const unsigned hit = __ballot_sync(0xffffffffu, found < 8);
+    // the draw's margin (kernel sums), in this slice's units, then relative to
+    // the total
+    float clo = lbase, chi = lbase;
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+      if (e == found) chi = lbase + pre[e];
+      if (e + 1 == found) clo = lbase + pre[e];
+    }
+    const float my_margin = fminf(lt - clo, chi - lt) * scale / W;
+    int yy;
+    float bm = 0.f;
+    if (hit) {
+      const int l = __ffs(hit) - 1;
+      yy = x0 - lane * kChunk + l * kChunk + __shfl_sync(0xffffffffu, found, l);
+      bm = __shfl_sync(0xffffffffu, my_margin, l);
+    } else {
+      int last = -1;
+#pragma unroll
+      for (int e = 0; e < 8; ++e) if (w[e] > 0.f) last = x0 + e;
+      const unsigned any = __ballot_sync(0xffffffffu, last >= 0);
+      yy = any ? __shfl_sync(0xffffffffu, last, 31 - __clz(any)) : v1 - 1;
+    }
+    if (lane == 0) {
+      a.out_bonus[b] = yy;
+      if (a.out_margin) a.out_margin[2 * (size_t)b + 1] = bm;
+    }
+    return true;
+  }
+
+  // ----------------------------------------------------------- control --
+  // Lane 0: completes the job's ring, slot and exchange fields and publishes it.
+  __device__ bool publish(const Job& j, int mbuf, int n_slots, int xk, int jobs) {
+    TreeJob& t = sh.job;
+    // the producer has copied the job before (the consumers have finished it)
+    if (jobs > 0 && !mbar_wait(ack_bar, (uint32_t)(jobs - 1) & 1u)) return false;
+    t.kind = j.kind;
+    t.pf_node = -1;
+    if (j.kind != kJobDone) {
+      t.node = j.node;
+      t.nmask = j.nmask;
+      t.alpha1 = j.alpha1;
+      t.beta = j.beta;
+      t.rowmax = j.rowmax;
+      t.mbuf = mbuf;
+      t.xb = xk & 1;
+      t.xph = (xk >> 1) & 1;
+      t.slot = -1;
+      int n_rows = 1;
+      uint32_t bytes;
+      if (is_pair(j.kind)) {
+        const int nch = chunks_of(Slice(row0 + j.node, a.V, v0, v1).n, kPair);
+        t.total = nch;
+        if (n_slots > 0) {
+          int at = -1, old = 0;
+          for (int k = 0; k < n_slots; ++k) {
+            if (sh.slot_node[k] == j.node) at = k;
+            if (sh.slot_used[k] < sh.slot_used[old]) old = k;
+          }
+          if (at >= 0) t.total = 0;
+          else at = old;
+          t.slot = at;
+          sh.slot_node[at] = j.node;
+          sh.slot_used[at] = jobs + 1;
+          // the parent's pair, for the pass there that a rejection of this node
+          // leads to (unless the traversal goes down into another child first)
+          if (j.kind == kJobPass && n_slots > 1 && j.node != 0 && !a.token_level) {
+            const int g = s.par[j.node];
+            bool have = false;
+            for (int k = 0; k < n_slots; ++k) have |= sh.slot_node[k] == g;
+            if (!have) {
+              int o2 = at == 0 ? 1 : 0;
+              for (int k = 0; k < n_slots; ++k)
+                if (k != at && sh.slot_used[k] < sh.slot_used[o2]) o2 = k;
+              t.pf_node = g;
+              t.pf_slot = o2;
+              sh.slot_node[o2] = g;
+              sh.slot_used[o2] = jobs + 1;
+            }
+          }
+        }
+        bytes = (j.kind == kJobPass) ? (uint32_t)(C * NCW) * 8u : (uint32_t)C * 8u;
+      } else {
+        // target rows only: through the whole ring
+        for (int k = 0; k < n_slots; ++k) sh.slot_node[k] = -1;
+        int total = 0;
+        if (j.kind == kJobStats) {
+          n_rows = min(j.n_rows, kStatRows);
+          for (int r = 0; r < n_rows; ++r) {
+            t.rows[r] = s.job_rows[r];
+            total += chunks_of(Slice(row0 + s.job_rows[r], a.V, v0, v1).n, kRow);
+          }
+          bytes = (uint32_t)(n_rows * C * NCW) * 8u;
+        } else {
+          total = chunks_of(Slice(row0 + j.node, a.V, v0, v1).n, kRow);
+          bytes = (uint32_t)C * 8u;
+        }
+        t.total = total;
+      }
+      t.n_rows = n_rows;
+      if (C > 1) mbar_arrive_expect_tx(&xbar[xk & 1], bytes);
+    }
+    mbar_arrive(job_bar);
+    return true;
+  }
+
+  __device__ void control(int lane) {
+    const int R = a.N + 1;
+    const float* u = a.uniforms + (size_t)b * (R + 1);
+    // resident row pairs the ring has room for (0: pairs are streamed)
+    const int n_slots = min(n_stages / chunks_of(v1 - v0 + 7, kPair), kTreeMaxSlots);
+    if (lane < kTreeMaxSlots) { sh.slot_node[lane] = -1; sh.slot_used[lane] = 0; }
+    __syncwarp();
+    Ctl& ctl = sh.ctl;
+    Ahead& ah = sh.ahead;
+    int xk = 0, jobs = 0, mnext = 1;     // exchanges, jobs, next list of removed tokens
+    uint32_t stat_ph = 0u;               // parity of stat_bar
+    int ok = 1;
+    if (lane == 0) {
+      if (ctl.job.kind != kJobDone) advance(s, ctl, u, a.token_level != 0);
+      ok = publish(ctl.job, 0, n_slots, xk, jobs) ? 1 : 0;
+      ah.ok = 0;
+      if (ctl.job.kind == kJobPass && !a.token_level) prepare_ahead(s, ctl, ah, mtok(mnext));
+    }
+    for (;;) {
+      ++jobs;
+      __syncwarp();
+      ok = __shfl_sync(0xffffffffu, ok, 0);
+      if (!ok) { fail(); return; }
+      const int kind = ctl.job.kind;
+      if (kind == kJobDone) return;
+      float S = 0.f;
+      bool got;
+      if (kind == kJobStats) {
+        got = mbar_wait_warp(stat_bar, stat_ph);
+      } else {
+        got = exchanged(xk & 1, (uint32_t)(xk >> 1) & 1u);
+      }
+      if (!got) { fail(); return; }
+      if (kind == kJobPass) {
+        const float2* x = xslots(xk & 1, 0);
+        for (int k = lane; k < C * NCW; k += 32) S += x[k].x;
+        S = warp_sum(S);
+      }
+      ++xk;
+      if (kind == kJobStats) stat_ph ^= 1u;
+      if (lane == 0) {
+        if (kind == kJobBonusLeaf || kind == kJobBonusRes) {
+          ctl.job.kind = kJobDone;
+          ok = publish(ctl.job, 0, n_slots, xk, jobs) ? 1 : 0;
+        } else {
+          if (kind == kJobPass) ctl.S = S;
+          bool fast = false;
+          if (kind == kJobPass && ah.ok) {
+            // the next step was worked out while the pass ran: decide, publish,
+            // then update the state
+            const double Sd = (double)S + s.p[ah.i] * ctl.masked_sum;
+            if (Sd > 1e-300) {
+              fast = true;
+              const double D = Sd + ah.omp;
+              Job jf;
+              jf.n_rows = 1;
+              jf.kind = kJobPass;
+              bool accept, first = true;
+              if (ah.mode == 1) {
+                accept = (double)u[ah.c2] * D < ah.X;
+                if (accept) {
+                  jf.kind = kJobBonusLeaf;
+                  jf.node = ah.c2;
+                  jf.nmask = 0;
+                } else {
+                  const double invD = 1.0 / D;
+                  jf.node = ah.i;
+                  jf.nmask = ah.nmask;
+                  jf.alpha1 = (float)(ah.ainvs * invD);
+                  jf.beta = (float)(ah.beta * invD + ah.invZn);
+                  jf.rowmax = s.rowm[ah.i];
+                }
+              } else {
+                accept = (double)u[ah.i] * D < Sd;
+                if (accept) {
+                  first = false;              // the residual draw needs the new state
+                } else {
+                  jf.node = ah.g;
+                  jf.nmask = ah.nmask;
+                  jf.alpha1 = ah.alpha1_g;
+                  jf.beta = ah.beta_g;
+                  jf.rowmax = ah.rowmax_g;
+                }
+              }
+              if (first) ok = publish(jf, mnext, n_slots, xk, jobs) ? 1 : 0;
+              control_step_ahead(s, ctl, ah, accept);
+              if (!first) ok = publish(ctl.job, 0, n_slots, xk, jobs) ? 1 : 0;
+              else mnext = 3 - mnext;         // that list is in use now
+            }
+          }
+          if (!fast) {
+            if (*(volatile uint32_t*)&ctl.bad & (32u | 64u)) ctl.job.kind = kJobDone;
+            else advance(s, ctl, u, a.token_level != 0);
+            ok = publish(ctl.job, 0, n_slots, xk, jobs) ? 1 : 0;
+          }
+          ah.ok = 0;
+          if (ctl.job.kind == kJobPass && !a.token_level) prepare_ahead(s, ctl, ah, mtok(mnext));
+        }
+      }
+    }
+  }
+
+  // Writes the tree's outputs (control warp of rank 0).
+  __device__ void outputs(int lane) {
+    const int R = a.N + 1, N = a.N;
+    const Ctl& ctl = sh.ctl;
+    const float* u = a.uniforms + (size_t)b * (R + 1);
+    const bool ok = (ctl.bad & (15u | 32u | 64u)) == 0u;
+    for (int k = lane; k < N; k += 32) a.out_path[(size_t)b * N + k] = -1;
+    if (a.out_node_p)
+      for (int i = lane; i < R; i += 32)
+        a.out_node_p[row0 + i] = ok ? s.dbgp[i] : __int_as_float(0x7fc00000);
+    __syncwarp();
+    if (lane != 0) return;
+    const int acc_node = ok ? ctl.accepted : -1;
+    if (acc_node >= 0) {
+      int depth = 0;
+      for (int j = acc_node; j != 0; j = s.par[j]) ++depth;
+      int k = depth - 1;
+      for (int j = acc_node; j != 0; j = s.par[j]) a.out_path[(size_t)b * N + (k--)] = j;
+      a.out_accept_len[b] = depth;
+    } else {
+      a.out_accept_len[b] = -1;
+      a.out_bonus[b] = -1;
+    }
+    if (a.out_stats) {
+      int distinct = 0;
+      for (int i = 0; i < R; ++i) distinct += (s.npass[i] > 0);
+      int normalised = 0;
+      for (int i = 0; i < R; ++i) normalised += (s.rows[i] > 0.f);
+      int32_t* o = a.out_stats + (size_t)b * 5;
+      o[0] = ok ? ctl.n_tests : 0;
+      o[1] = ok ? ctl.n_passes : 0;
+      o[2] = ok ? distinct : 0;
+      o[3] = (acc_node >= 0 && s.first[acc_node] < 0) ? 1 : 0;
+      o[4] = ok ? normalised : 0;
+    }
+    if (a.out_margin) {
+      // the bonus margin was written by the CTA that drew the bonus
+      const float nan = __int_as_float(0x7fc00000);
+      a.out_margin[2 * (size_t)b] = acc_node >= 0 ? test_margin_serial(s.dbgp, u, R) : nan;
+      if (acc_node < 0) a.out_margin[2 * (size_t)b + 1] = nan;
+    }
+    if (ctl.bad) atomicOr(a.status, ctl.bad);
+  }
 };
 
 template <typename L, int NCW>
-__global__ void __launch_bounds__(NCW * 32 + 32, 16 / NCW) tv_tree_kernel(TravArgs args, int C,
-                                                                      int n_stages) {
-  constexpr int kConsumerWarps = NCW;
-  constexpr int kConsumers = NCW * 32;
-  constexpr int kThreads = kConsumers + 32;
-  constexpr int kStageBytes = stage_bytes(NCW);
-  constexpr int kSweep = kConsumers * kChunk;   // tokens one pass of all consumers covers
+__global__ void __launch_bounds__(TreeCta<L, NCW>::kThreads, 16 / NCW)
+    tv_tree_kernel(const __grid_constant__ TravArgs args, int C, int n_stages) {
+  using T = TreeCta<L, NCW>;
   extern __shared__ __align__(128) char smem_raw[];
-  __shared__ __align__(8) uint64_t full_bar[kMaxStages];
-  __shared__ __align__(8) uint64_t empty_bar[kMaxStages];
-  __shared__ __align__(8) uint64_t xbar;
-  __shared__ float2 xslots[2][kMaxCluster];
-  __shared__ Ctl ctl;
-  __shared__ float red_a[kConsumerWarps], red_b[kConsumerWarps];
-
-  using E = typename L::elem;
-  constexpr int kLB = L::kBytes;
-  constexpr int kPairElems = kStageBytes / (kLB + 4) / kTileElems * kTileElems;  // target + draft
-  constexpr int kRowElems = kStageBytes / kLB;               // target only per stage
+  __shared__ __align__(8) uint64_t full_bar[kTreeMaxStages];
+  __shared__ __align__(8) uint64_t empty_bar[kTreeMaxStages];
+  __shared__ __align__(8) uint64_t xbar[2];
+  __shared__ __align__(8) uint64_t job_bar, ack_bar, stat_bar, tile_bar;
+  __shared__ TreeShared sh;
 
   const int R = args.N + 1, V = args.V;
-  const uint32_t rank = (C > 1) ? cluster_rank() : 0u;
-  const int b = blockIdx.x / C;
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-  const bool producer = (wid == kConsumerWarps);
-  const float c_hi = args.c_hi, c_lo = args.c_lo;
+  T t(args, sh);
+  t.C = C;
+  t.n_stages = n_stages;
+  t.rank = (C > 1) ? cluster_rank() : 0u;
+  t.b = blockIdx.x / C;
   const int SL = slice_len(V, C);
-  const int v0 = min((int)rank * SL, V);
-  const int v1 = min(v0 + SL, V);
-  const int nt = n_tiles(V, C);
-
-  char* ring = smem_raw;
-  TreeSmem s = carve_tree(smem_raw + (size_t)n_stages * kStageBytes, R, V, C);
-  const E* logits = reinterpret_cast<const E*>(args.logits);
-  const size_t tree_row0 = (size_t)b * R;
-  const float* u = args.uniforms + (size_t)b * (R + 1);
+  t.v0 = min((int)t.rank * SL, V);
+  t.v1 = min(t.v0 + SL, V);
+  t.row0 = (size_t)t.b * R;
+  t.ring = smem_raw;
+  t.xs = reinterpret_cast<float2*>(smem_raw + (size_t)n_stages * T::kStageBytes);
+  char* tree_base = reinterpret_cast<char*>(t.xs + 2 * (size_t)kStatRows * C * NCW);
+  t.s = carve_tree_nt(tree_base, R, tree_tiles(V, C));
+  t.mtok_ahead = reinterpret_cast<int*>(
+      tree_base + ((tree_smem_bytes_nt(R, tree_tiles(V, C)) + 15) & ~(size_t)15));
+  t.full_bar = full_bar;
+  t.empty_bar = empty_bar;
+  t.xbar = xbar;
+  t.job_bar = &job_bar;
+  t.ack_bar = &ack_bar;
+  t.stat_bar = &stat_bar;
+  t.tile_bar = &tile_bar;
+  const TreeSmem& s = t.s;
+  Ctl& ctl = sh.ctl;
+  const typename L::elem* logits = reinterpret_cast<const typename L::elem*>(args.logits);
 
   // ---- set-up: barriers, tree structure, validation, gathers ----
   if (tid == 0) {
     for (int k = 0; k < n_stages; ++k) {
       mbar_init(&full_bar[k], 1);
-      mbar_init(&empty_bar[k], kConsumerWarps);
+      mbar_init(&empty_bar[k], NCW);
     }
-    mbar_init(&xbar, C);
+    mbar_init(&xbar[0], C > 1 ? 1 : NCW);
+    mbar_init(&xbar[1], C > 1 ? 1 : NCW);
+    mbar_init(&job_bar, 1);
+    mbar_init(&ack_bar, 1);
+    mbar_init(&stat_bar, NCW);
+    mbar_init(&tile_bar, NCW);
     fence_mbar_init();
     ctl.bad = 0u;
     ctl.accepted = -1;
@@ -107,14 +969,11 @@ __global__ void __launch_bounds__(NCW * 32 + 32, 16 / NCW) tv_tree_kernel(TravAr
     ctl.pending = -1;
     ctl.masked_sum = 0.0;
     ctl.n_tests = ctl.n_passes = 0;
-    ctl.xphase = 0u;
-    ctl.xbuf = 0;
     ctl.job.kind = 0;
-    ctl.bonus_y = -1;
   }
-  for (int i = tid; i < R; i += kThreads) {
-    s.par[i] = args.parents[tree_row0 + i];
-    s.tok[i] = args.tokens[tree_row0 + i];
+  for (int i = tid; i < R; i += T::kThreads) {
+    s.par[i] = args.parents[t.row0 + i];
+    s.tok[i] = args.tokens[t.row0 + i];
     s.first[i] = 0x7fffffff;
     s.npass[i] = 0;
     s.state[i] = kAlive;
@@ -130,15 +989,15 @@ __global__ void __launch_bounds__(NCW * 32 + 32, 16 / NCW) tv_tree_kernel(TravAr
   __syncthreads();
   {
     uint32_t bad = 0u;
-    for (int i = tid; i < R; i += kThreads) {
+    for (int i = tid; i < R; i += T::kThreads) {
       const int p = s.par[i];
       if (i == 0) {
         if (p != -1) bad |= 1u;
       } else {
         if (p < 0 || p >= i) bad |= 1u;
         else atomicMin(&s.first[p], i);
-        const int t = s.tok[i];
-        if (t < 0 || t >= V) bad |= 2u;
+        const int tk = s.tok[i];
+        if (tk < 0 || tk >= V) bad |= 2u;
       }
     }
     if (bad) atomicOr(&ctl.bad, bad);
@@ -146,21 +1005,23 @@ __global__ void __launch_bounds__(NCW * 32 + 32, 16 / NCW) tv_tree_kernel(TravAr
   __syncthreads();
   if (ctl.bad == 0u) {
     uint32_t bad = 0u;
-    for (int i = tid; i < R; i += kThreads) {
+    for (int i = tid; i < R; i += T::kThreads) {
       if (s.first[i] == 0x7fffffff) s.first[i] = -1;
       int nx = -1;
       if (i > 0) {
-        const int p = s.par[i], t = s.tok[i];
+        const int p = s.par[i], tk = s.tok[i];
+        const size_t prow = (t.row0 + p) * (size_t)V;
+        const float gl = L::at(logits + prow, tk);      // (in flight during the search)
+        const float gq = __ldg(args.draft_probs + prow + tk);
         for (int j = i + 1; j < R; ++j) {
           if (s.par[j] != p) continue;
           if (nx < 0) nx = j;
-          if (s.tok[j] == t) bad |= 4u;
+          if (s.tok[j] == tk) bad |= 4u;
         }
-        const size_t prow = (tree_row0 + p) * (size_t)V;
-        s.gl[i] = L::at(logits + prow, t);
-        s.gq[i] = __ldg(args.draft_probs + prow + t);
-        if (!(s.gq[i] > 0.f)) bad |= 8u;
-        s.invq[i] = 1.0 / (double)s.gq[i];
+        s.gl[i] = gl;
+        s.gq[i] = gq;
+        if (!(gq > 0.f)) bad |= 8u;
+        s.invq[i] = 1.0 / (double)gq;
       }
       s.next[i] = nx;
     }
@@ -171,514 +1032,18 @@ __global__ void __launch_bounds__(NCW * 32 + 32, 16 / NCW) tv_tree_kernel(TravAr
     if (ctl.bad == 0u) s.p[0] = 1.0;
     else ctl.job.kind = kJobDone;
   }
-  if (C > 1) cluster_sync_all();   // peers' barriers initialised before any remote arrive
+  if (C > 1) cluster_sync_all();   // peers' barriers initialised before any remote store
   else __syncthreads();
 
-  uint32_t timeout = 0u;
-
-  if (producer) {
-    // =================== producer warp: TMA bulk copies ===================
-    // One named barrier per job on every path (the consumers do the same).
-    int stage = 0, phase = 0;
-    for (;;) {
-      named_sync(1, kThreads);             // the next job is posted
-      const Job job = ctl.job;
-      if (job.kind == kJobDone) break;
-      if (timeout) continue;
-      const bool pair = (job.kind == kJobPass || job.kind == kJobBonusRes);
-      const int per = pair ? kPairElems : kRowElems;
-      const int nrows = (job.kind == kJobStats) ? job.n_rows : 1;
-      if (lane == 0) {
-        for (int r = 0; r < nrows && !timeout; ++r) {
-          const int node = (job.kind == kJobStats) ? s.job_rows[r] : job.node;
-          const size_t row = (tree_row0 + node) * (size_t)V;
-          for (int x = v0; x < v1; x += per) {
-            const int n = min(per, v1 - x);
-            if (!mbar_wait(&empty_bar[stage], phase ^ 1)) { timeout = 1u; break; }
-            char* dst = ring + (size_t)stage * kStageBytes;
-            const uint32_t lbytes = (uint32_t)n * kLB;
-            const uint32_t qbytes = pair ? (uint32_t)n * 4u : 0u;
-            mbar_arrive_expect_tx(&full_bar[stage], lbytes + qbytes);
-            tma_load_1d(dst, logits + row + x, lbytes, &full_bar[stage]);
-            if (pair)
-              tma_load_1d(dst + (size_t)kPairElems * kLB, args.draft_probs + row + x, qbytes,
-                          &full_bar[stage]);
-            if (++stage == n_stages) { stage = 0; phase ^= 1; }
-          }
-        }
-        if (timeout) atomicOr(&ctl.bad, 32u);
-      }
-      timeout = __shfl_sync(0xffffffffu, timeout, 0);
-      stage = __shfl_sync(0xffffffffu, stage, 0);
-      phase = __shfl_sync(0xffffffffu, phase, 0);
-    }
+  if (wid < NCW) {
+    t.consumer(wid, lane);
+  } else if (wid == NCW) {
+    if (lane == 0) t.producer((size_t)args.B * R * (size_t)V);
   } else {
-    // =================== consumer warps ===================
-    int stage = 0, phase = 0;
-    volatile uint32_t* vbad = &ctl.bad;
-    for (;;) {
-      if (tid == 0) {
-        if (*vbad & (32u | 64u)) ctl.job.kind = kJobDone;         // timeout / unusable row
-        else if (ctl.job.kind != kJobDone) advance(s, ctl, u, args.token_level != 0);
-      }
-      named_sync(1, kThreads);
-      const Job job = ctl.job;
-      if (job.kind == kJobDone) break;
-      const bool pair = (job.kind == kJobPass || job.kind == kJobBonusRes);
-      const int per = pair ? kPairElems : kRowElems;
-      const int nrows = (job.kind == kJobStats) ? job.n_rows : 1;
-      for (int r = 0; r < nrows; ++r) {
-        const int node = (job.kind == kJobStats) ? s.job_rows[r] : job.node;
-        float m_run = TV_NEG_INF;   // stats / leaf: running max
-        Comp acc;
-        int mp = 0;
-        for (int x = v0; x < v1; x += per) {
-          const int n = min(per, v1 - x);
-          if ((*vbad & 32u) || !mbar_wait(&full_bar[stage], phase)) {
-            atomicOr(&ctl.bad, 32u);
-            break;
-          }
-          const char* buf = ring + (size_t)stage * kStageBytes;
-          const E* lb = reinterpret_cast<const E*>(buf);
-          const float* qb = reinterpret_cast<const float*>(buf + (size_t)kPairElems * kLB);
-          // warp-uniform iteration over 256-element tiles (warp shuffles below)
-          for (int t0 = wid * kTileElems; t0 < n; t0 += kSweep) {
-            const int e0 = t0 + lane * kChunk;
-            const bool valid = e0 < n;
-            const int xg = x + e0;   // global token index of the lane's first element
-            if constexpr (kLB == 2) {
-              // ---------------- bf16 logits: packed-pair arithmetic ----------------
-              float2 vp[4];
-              if (valid) {
-                bf16x8_pairs(lds128(lb + e0), vp);
-              } else {
-#pragma unroll
-                for (int k2 = 0; k2 < 4; ++k2) vp[k2] = make_float2(-9984.f, -9984.f);
-              }
-              const float2 ch = make_float2(c_hi, c_hi), cl = make_float2(c_lo, c_lo);
-              if (job.kind == kJobStats) {
-                if (valid) {
-                  const float cm = fmaxf(fmaxf(fmaxf(vp[0].x, vp[0].y), fmaxf(vp[1].x, vp[1].y)),
-                                         fmaxf(fmaxf(vp[2].x, vp[2].y), fmaxf(vp[3].x, vp[3].y)));
-                  if (cm > m_run) {
-                    if (m_run != TV_NEG_INF) {
-                      const float sc = L::exp_rel(m_run, cm, c_hi, c_lo);
-                      acc.s *= sc;
-                      acc.c *= sc;
-                    }
-                    m_run = cm;
-                  }
-                  const float2 mm = make_float2(-m_run, -m_run);
-                  float2 e[4];
-#pragma unroll
-                  for (int k2 = 0; k2 < 4; ++k2) e[k2] = exp2_split_x2(__fadd2_rn(vp[k2], mm), ch, cl);
-                  const float2 s2 = __fadd2_rn(__fadd2_rn(e[0], e[1]), __fadd2_rn(e[2], e[3]));
-                  acc.add(s2.x + s2.y);
-                }
-              } else if (job.kind == kJobBonusLeaf) {
-                const float lm = fmaxf(fmaxf(fmaxf(vp[0].x, vp[0].y), fmaxf(vp[1].x, vp[1].y)),
-                                       fmaxf(fmaxf(vp[2].x, vp[2].y), fmaxf(vp[3].x, vp[3].y)));
-                const float tm = warp_max(lm);
-                const float2 mm = make_float2(-tm, -tm);
-                float2 e[4];
-#pragma unroll
-                for (int k2 = 0; k2 < 4; ++k2) e[k2] = exp2_corrected_x2(__fadd2_rn(vp[k2], mm), ch, cl);
-                const float2 s2 = __fadd2_rn(__fadd2_rn(e[0], e[1]), __fadd2_rn(e[2], e[3]));
-                const float ts = warp_sum(valid ? s2.x + s2.y : 0.f);
-                if (lane == 0) {
-                  const int tile = (x + t0 - v0) / kTileElems;
-                  s.tsum[tile] = ts;
-                  s.tmax[tile] = tm;
-                }
-              } else {
-                float2 qp[4];
-                if (valid) {
-                  const uint4 qa = lds128(qb + e0);
-                  const uint4 qc = lds128(qb + e0 + 4);
-                  qp[0] = make_float2(__uint_as_float(qa.x), __uint_as_float(qa.y));
-                  qp[1] = make_float2(__uint_as_float(qa.z), __uint_as_float(qa.w));
-                  qp[2] = make_float2(__uint_as_float(qc.x), __uint_as_float(qc.y));
-                  qp[3] = make_float2(__uint_as_float(qc.z), __uint_as_float(qc.w));
-                } else {
-#pragma unroll
-                  for (int k2 = 0; k2 < 4; ++k2) qp[k2] = make_float2(0.f, 0.f);
-                }
-                const float2 mm = make_float2(-job.rowmax, -job.rowmax);
-                const float2 al2 = make_float2(job.alpha1, job.alpha1);
-                const float2 nb2 = make_float2(-job.beta, -job.beta);
-                float t[8];
-#pragma unroll
-                for (int k2 = 0; k2 < 4; ++k2) {
-                  const float2 e = exp2_corrected_x2(__fadd2_rn(vp[k2], mm), ch, cl);
-                  const float2 xx = __ffma2_rn(al2, e, __fmul2_rn(nb2, qp[k2]));
-                  t[2 * k2] = fmaxf(xx.x, 0.f);
-                  t[2 * k2 + 1] = fmaxf(xx.y, 0.f);
-                }
-                while (mp < job.nmask && s.mask_tok[mp] < xg) ++mp;
-                for (int mq = mp; mq < job.nmask && s.mask_tok[mq] < xg + kChunk; ++mq) {
-                  const int off = s.mask_tok[mq] - xg;
-                  const float mv = (job.kind == kJobPass) ? 0.f : s.mask_val[mq];
-#pragma unroll
-                  for (int k2 = 0; k2 < 8; ++k2) if (k2 == off) t[k2] = mv;
-                }
-                if (job.kind == kJobPass) {
-                  if (valid) acc.add(sum8(t));
-                } else {
-                  const float ts = warp_sum(valid ? sum8(t) : 0.f);
-                  if (lane == 0) s.tsum[(x + t0 - v0) / kTileElems] = ts;
-                }
-              }
-            } else {
-            float v[8];
-            if (!valid) {
-#pragma unroll
-              for (int k2 = 0; k2 < 8; ++k2) v[k2] = TV_NEG_INF;
-            } else {
-              const uint4 a4 = lds128(lb + e0);
-              const uint4 b4 = lds128(lb + e0 + 4);
-              v[0] = __uint_as_float(a4.x); v[1] = __uint_as_float(a4.y);
-              v[2] = __uint_as_float(a4.z); v[3] = __uint_as_float(a4.w);
-              v[4] = __uint_as_float(b4.x); v[5] = __uint_as_float(b4.y);
-              v[6] = __uint_as_float(b4.z); v[7] = __uint_as_float(b4.w);
-            }
-            if (job.kind == kJobStats) {
-              float cm = fmaxf(fmaxf(fmaxf(v[0], v[1]), fmaxf(v[2], v[3])),
-                               fmaxf(fmaxf(v[4], v[5]), fmaxf(v[6], v[7])));
-              if (cm > m_run) {
-                if (m_run != TV_NEG_INF) {
-                  const float sc = L::exp_rel(m_run, cm, c_hi, c_lo);
-                  acc.s *= sc;
-                  acc.c *= sc;
-                }
-                m_run = cm;
-              }
-              float t[8];
-#pragma unroll
-              for (int k = 0; k < 8; ++k) t[k] = L::exp_rel(v[k], m_run, c_hi, c_lo);
-              acc.add(sum8(t));
-            } else if (job.kind == kJobBonusLeaf) {
-              float lm = fmaxf(fmaxf(fmaxf(v[0], v[1]), fmaxf(v[2], v[3])),
-                               fmaxf(fmaxf(v[4], v[5]), fmaxf(v[6], v[7])));
-              const float tm = warp_max(lm);
-              float t[8];
-#pragma unroll
-              for (int k = 0; k < 8; ++k) t[k] = L::exp_pass(v[k], tm, c_hi, c_lo);
-              const float ts = warp_sum(sum8(t));
-              if (lane == 0) {
-                const int tile = (x + t0 - v0) / kTileElems;
-                s.tsum[tile] = ts;
-                s.tmax[tile] = tm;
-              }
-            } else {
-              float q[8];
-              if (valid) {
-                const uint4 qa = lds128(qb + e0);
-                const uint4 qc = lds128(qb + e0 + 4);
-                q[0] = __uint_as_float(qa.x); q[1] = __uint_as_float(qa.y);
-                q[2] = __uint_as_float(qa.z); q[3] = __uint_as_float(qa.w);
-                q[4] = __uint_as_float(qc.x); q[5] = __uint_as_float(qc.y);
-                q[6] = __uint_as_float(qc.z); q[7] = __uint_as_float(qc.w);
-              } else {
-#pragma unroll
-                for (int k2 = 0; k2 < 8; ++k2) q[k2] = 0.f;
-              }
-              const float al = job.alpha1, be = job.beta, rm = job.rowmax;
-              float t[8];
-#pragma unroll
-              for (int k = 0; k < 8; ++k)
-                t[k] = fmaxf(fmaf(al, L::exp_pass(v[k], rm, c_hi, c_lo), -be * q[k]), 0.f);
-              while (mp < job.nmask && s.mask_tok[mp] < xg) ++mp;
-              for (int mq = mp; mq < job.nmask && s.mask_tok[mq] < xg + kChunk; ++mq) {
-                const int off = s.mask_tok[mq] - xg;
-                const float mv = (job.kind == kJobPass) ? 0.f : s.mask_val[mq];
-#pragma unroll
-                for (int k = 0; k < 8; ++k) if (k == off) t[k] = mv;
-              }
-              if (job.kind == kJobPass) {
-                acc.add(sum8(t));
-              } else {
-                const float ts = warp_sum(sum8(t));
-                if (lane == 0) s.tsum[(x + t0 - v0) / kTileElems] = ts;
-              }
-            }
-            }
-          }
-          __syncwarp();
-          if (lane == 0) mbar_arrive(&empty_bar[stage]);
-          if (++stage == n_stages) { stage = 0; phase ^= 1; }
-        }
-        // ---- per-row reduction over the consumers, then over the cluster ----
-        if (job.kind == kJobStats) {
-          const float wm = warp_max(m_run);
-          if (lane == 0) red_a[wid] = wm;
-          named_sync(2, kConsumers);
-          float M = red_a[0];
-#pragma unroll
-          for (int w = 1; w < kConsumerWarps; ++w) M = fmaxf(M, red_a[w]);
-          float part = (m_run == TV_NEG_INF) ? 0.f : acc.value() * L::exp_rel(m_run, M, c_hi, c_lo);
-          part = warp_sum(part);
-          named_sync(2, kConsumers);
-          if (lane == 0) red_b[wid] = part;
-          named_sync(2, kConsumers);
-          if (tid == 0) {
-            float S = 0.f;
-            for (int w = 0; w < kConsumerWarps; ++w) S += red_b[w];
-            if (C > 1) {
-              if (!exchange(xslots, &xbar, ctl, C, rank, M, S)) atomicOr(&ctl.bad, 32u);
-              const int bb = ctl.xbuf ^ 1;
-              float Mg = xslots[bb][0].x;
-              for (int rr = 1; rr < C; ++rr) Mg = fmaxf(Mg, xslots[bb][rr].x);
-              float Sg = 0.f;
-              for (int rr = 0; rr < C; ++rr) {
-                const float mr = xslots[bb][rr].x;
-                if (mr != TV_NEG_INF) Sg += xslots[bb][rr].y * L::exp_rel(mr, Mg, c_hi, c_lo);
-              }
-              M = Mg;
-              S = Sg;
-            }
-            s.rowm[node] = M;
-            s.rows[node] = S;
-            s.invs[node] = 1.0 / (double)S;
-            if (!(S > 0.f)) ctl.bad |= 64u;   // no finite logit in the row
-          }
-          __syncwarp();
-          if (wid == 0) {
-            children_mb0(s, node, args.c, lane);
-            __syncwarp();
-          }
-        } else if (job.kind == kJobPass) {
-          const float ws = warp_sum(acc.value());
-          if (lane == 0) red_a[wid] = ws;
-          named_sync(2, kConsumers);
-          if (tid == 0) {
-            float S = 0.f;
-            for (int w = 0; w < kConsumerWarps; ++w) S += red_a[w];
-            if (C > 1) {
-              if (!exchange(xslots, &xbar, ctl, C, rank, S, 0.f)) atomicOr(&ctl.bad, 32u);
-              const int bb = ctl.xbuf ^ 1;
-              float Sg = 0.f;
-              for (int rr = 0; rr < C; ++rr) Sg += xslots[bb][rr].x;
-              S = Sg;
-            }
-            ctl.S = S;
-          }
-        } else {
-          // ---- bonus draw: slice totals, crossing slice, crossing tile, token ----
-          named_sync(2, kConsumers);
-          if (wid == 0) {
-            const bool leaf = (job.kind == kJobBonusLeaf);
-            const int ntl = (v1 - v0 + kTileElems - 1) / kTileElems;
-            float Mc = 0.f;
-            if (leaf) {
-              float lm = TV_NEG_INF;
-              for (int k = lane; k < ntl; k += 32) lm = fmaxf(lm, s.tmax[k]);
-              Mc = warp_max(lm);
-              for (int k = lane; k < ntl; k += 32)
-                s.tsum[k] = (s.tmax[k] == TV_NEG_INF) ? 0.f : s.tsum[k] * L::exp_rel(s.tmax[k], Mc, c_hi, c_lo);
-              __syncwarp();
-            }
-            float Wc = 0.f;
-            for (int k0 = 0; k0 < ntl; k0 += 32) {
-              const float v = (k0 + lane < ntl) ? s.tsum[k0 + lane] : 0.f;
-              Wc += warp_sum(v);
-            }
-            // cluster: every CTA learns every slice's (max, total)
-            float scale = 1.f, target = 0.f, before = 0.f, Wtot = 0.f;
-            int owner = 0;
-            if (lane == 0) {
-              float Mg = Mc, W = Wc;
-              if (C > 1) {
-                if (!exchange(xslots, &xbar, ctl, C, rank, Mc, Wc)) atomicOr(&ctl.bad, 32u);
-                const int bb = ctl.xbuf ^ 1;
-                Mg = xslots[bb][0].x;
-                if (leaf) for (int rr = 1; rr < C; ++rr) Mg = fmaxf(Mg, xslots[bb][rr].x);
-                W = 0.f;
-                float sc[kMaxCluster];
-                for (int rr = 0; rr < C; ++rr) {
-                  sc[rr] = leaf ? ((xslots[bb][rr].x == TV_NEG_INF) ? 0.f
-                                       : L::exp_rel(xslots[bb][rr].x, Mg, c_hi, c_lo))
-                                : 1.f;
-                  W += xslots[bb][rr].y * sc[rr];
-                }
-                target = u[R] * W;
-                float acc0 = 0.f;
-                owner = -1;
-                for (int rr = 0; rr < C; ++rr) {
-                  const float wr = xslots[bb][rr].y * sc[rr];
-                  if (owner < 0 && target < acc0 + wr) { owner = rr; before = acc0; }
-                  acc0 += wr;
-                }
-                if (owner < 0) {   // rounding: the last slice with weight
-                  owner = C - 1;
-                  while (owner > 0 && !(xslots[bb][owner].y > 0.f)) --owner;
-                  before = 0.f;
-                  for (int rr = 0; rr < owner; ++rr) before += xslots[bb][rr].y * sc[rr];
-                }
-                scale = sc[rank];
-              } else {
-                target = u[R] * W;
-              }
-              (void)Mg;
-              Wtot = W;
-            }
-            owner = __shfl_sync(0xffffffffu, owner, 0);
-            if ((uint32_t)owner == rank) {
-              target = __shfl_sync(0xffffffffu, target, 0);
-              before = __shfl_sync(0xffffffffu, before, 0);
-              scale = __shfl_sync(0xffffffffu, scale, 0);
-              Wtot = __shfl_sync(0xffffffffu, Wtot, 0);
-              // local target in this slice's units
-              const float lt = (scale > 0.f) ? (target - before) / scale : 0.f;
-              int tile = -1;
-              float tbase = 0.f, base = 0.f;
-              for (int k0 = 0; k0 < ntl && tile < 0; k0 += 32) {
-                float v = (k0 + lane < ntl) ? s.tsum[k0 + lane] : 0.f;
-                const float own = v;
-#pragma unroll
-                for (int o = 1; o < 32; o <<= 1) {
-                  const float w2 = __shfl_up_sync(0xffffffffu, v, o);
-                  if (lane >= o) v += w2;
-                }
-                const unsigned hit = __ballot_sync(0xffffffffu, (k0 + lane < ntl) && (lt < base + v));
-                if (hit) {
-                  const int l = __ffs(hit) - 1;
-                  tile = k0 + l;
-                  tbase = base + __shfl_sync(0xffffffffu, v - own, l);
-                }
-                base += __shfl_sync(0xffffffffu, v, 31);
-              }
-              if (tile < 0) {
-                tile = ntl - 1;
-                while (tile > 0 && !(s.tsum[tile] > 0.f)) --tile;
-                float a0 = 0.f;
-                for (int k = 0; k < tile; ++k) a0 += s.tsum[k];
-                tbase = a0;
-              }
-              // element-level rescan of the crossing tile (global loads, L2-hot)
-              const int x0 = v0 + tile * kTileElems + lane * kChunk;
-              const size_t row = (tree_row0 + node) * (size_t)V;
-              float w[8];
-              if (leaf) {
-                float v[8];
-                if (x0 < v1) load_logits<L, true>(logits + row, x0, V, v);
-                else {
-#pragma unroll
-                  for (int e = 0; e < 8; ++e) v[e] = TV_NEG_INF;
-                }
-#pragma unroll
-                for (int e = 0; e < 8; ++e)
-                  w[e] = (v[e] == TV_NEG_INF) ? 0.f : L::exp_pass(v[e], Mc, c_hi, c_lo);
-              } else {
-                float v[8], q[8];
-                if (x0 < v1) {
-                  load_logits<L, true>(logits + row, x0, V, v);
-                  load_probs<true>(args.draft_probs + row, x0, V, q);
-                } else {
-#pragma unroll
-                  for (int e = 0; e < 8; ++e) { v[e] = TV_NEG_INF; q[e] = 0.f; }
-                }
-#pragma unroll
-                for (int e = 0; e < 8; ++e)
-                  w[e] = (v[e] == TV_NEG_INF) ? 0.f
-                         : fmaxf(fmaf(job.alpha1, L::exp_pass(v[e], job.rowmax, c_hi, c_lo), -job.beta * q[e]), 0.f);
-                for (int mq = 0; mq < job.nmask; ++mq) {
-                  const int off = s.mask_tok[mq] - x0;
-                  const float mv = s.mask_val[mq];
-#pragma unroll
-                  for (int e = 0; e < 8; ++e) if (e == off) w[e] = mv;
-                }
-              }
-              float pre[8];
-              float run = 0.f;
-#pragma unroll
-              for (int e = 0; e < 8; ++e) { run += w[e]; pre[e] = run; }
-              float v = run;
-#pragma unroll
-              for (int o = 1; o < 32; o <<= 1) {
-                const float w2 = __shfl_up_sync(0xffffffffu, v, o);
-                if (lane >= o) v += w2;
-              }
-              const float lbase = tbase + (v - run);
-              int found = 8;
-#pragma unroll
-              for (int e = 7; e >= 0; --e) if (lt < lbase + pre[e]) found = e;
-              const unsigned hit = __ballot_sync(0xffffffffu, found < 8);
-              // the draw's margin (kernel sums), in this slice's units, then
-              // relative to the total
-              float clo = lbase, chi = lbase;
-#pragma unroll
-              for (int e = 0; e < 8; ++e) {
-                if (e == found) chi = lbase + pre[e];
-                if (e + 1 == found) clo = lbase + pre[e];
-              }
-              const float my_margin = fminf(lt - clo, chi - lt) * scale / Wtot;
-              int yy;
-              float bm = 0.f;
-              if (hit) {
-                const int l = __ffs(hit) - 1;
-                yy = x0 - lane * kChunk + l * kChunk + __shfl_sync(0xffffffffu, found, l);
-                bm = __shfl_sync(0xffffffffu, my_margin, l);
-              } else {
-                int last = -1;
-#pragma unroll
-                for (int e = 0; e < 8; ++e) if (w[e] > 0.f) last = x0 + e;
-                const unsigned any = __ballot_sync(0xffffffffu, last >= 0);
-                yy = any ? __shfl_sync(0xffffffffu, last, 31 - __clz(any)) : v1 - 1;
-              }
-              if (lane == 0) {
-                args.out_bonus[b] = yy;
-                if (args.out_margin) args.out_margin[2 * (size_t)b + 1] = bm;
-              }
-            }
-          }
-          if (tid == 0) ctl.job.kind = kJobDone;   // the bonus ends the traversal
-        }
-      }
-    }
-    // ---- outputs (rank 0) ----
-    named_sync(2, kConsumers);
-    if (rank == 0) {
-      const bool ok = (ctl.bad & (15u | 32u | 64u)) == 0u;
-      const int N = args.N;
-      for (int k = tid; k < N; k += kConsumers) args.out_path[(size_t)b * N + k] = -1;
-      if (args.out_node_p)
-        for (int i = tid; i < R; i += kConsumers)
-          args.out_node_p[tree_row0 + i] = ok ? s.dbgp[i] : __int_as_float(0x7fc00000);
-      named_sync(2, kConsumers);
-      if (tid == 0) {
-        const int acc_node = ok ? ctl.accepted : -1;
-        if (acc_node >= 0) {
-          int depth = 0;
-          for (int j = acc_node; j != 0; j = s.par[j]) ++depth;
-          int k = depth - 1;
-          for (int j = acc_node; j != 0; j = s.par[j]) args.out_path[(size_t)b * N + (k--)] = j;
-          args.out_accept_len[b] = depth;
-        } else {
-          args.out_accept_len[b] = -1;
-          args.out_bonus[b] = -1;
-        }
-        if (args.out_stats) {
-          int distinct = 0;
-          for (int i = 0; i < R; ++i) distinct += (s.npass[i] > 0);
-          int normalised = 0;
-          for (int i = 0; i < R; ++i) normalised += (s.rows[i] > 0.f);
-          int32_t* o = args.out_stats + (size_t)b * 5;
-          o[0] = ok ? ctl.n_tests : 0;
-          o[1] = ok ? ctl.n_passes : 0;
-          o[2] = ok ? distinct : 0;
-          o[3] = (acc_node >= 0 && s.first[acc_node] < 0) ? 1 : 0;
-          o[4] = ok ? normalised : 0;
-        }
-        if (args.out_margin) {
-          // the bonus margin was written by the CTA that drew the bonus
-          const float nan = __int_as_float(0x7fc00000);
-          args.out_margin[2 * (size_t)b] = acc_node >= 0 ? test_margin_serial(s.dbgp, u, R) : nan;
-          if (acc_node < 0) args.out_margin[2 * (size_t)b + 1] = nan;
-        }
-        if (ctl.bad) atomicOr(args.status, ctl.bad);
-      }
-    }
+    t.control(lane);
   }
+  __syncthreads();                 // (a role that gave up has raised ctl.bad)
+  if (t.rank == 0 && wid == NCW + 1) t.outputs(lane);
   if (C > 1) cluster_sync_all();   // no CTA leaves while a peer may still write to it
 }
 
@@ -689,20 +1054,28 @@ __global__ void __launch_bounds__(NCW * 32 + 32, 16 / NCW) tv_tree_kernel(TravAr
 
 namespace {
 
-// Ring stages that fit when `per_sm` CTAs share an SM's shared memory.
-int stages_for(int ncw, int per_sm, size_t tree, int smem_per_sm, int smem_per_block) {
+size_t tree_cta_bytes(int ncw, int lb, int C, int stages, int R, int V) {
   using namespace tvk::fused;
-  const long reserve = 1024 + 512;   // per-CTA system reserve and static shared memory
+  return (size_t)stages * tree_stage_bytes(ncw, lb) + (size_t)2 * kStatRows * C * ncw * 8 +
+         ((tree_smem_bytes_nt(R, tree_tiles(V, C)) + 15) & ~(size_t)15) + (size_t)R * 8;
+}
+
+// Ring stages that fit when `per_sm` CTAs share an SM's shared memory.
+int stages_for(int ncw, int lb, int C, int per_sm, int R, int V, int smem_per_sm,
+               int smem_per_block) {
+  using namespace tvk::fused;
+  const long reserve = 1024 + 1536;   // per-CTA system reserve and static shared memory
   long per_cta = (long)smem_per_sm / per_sm - reserve;
-  if (per_cta > smem_per_block) per_cta = smem_per_block;
-  const long st = (per_cta - (long)tree) / stage_bytes(ncw);
-  return (int)(st > kMaxStages ? kMaxStages : st);
+  if (per_cta > smem_per_block - 1536) per_cta = smem_per_block - 1536;
+  const long st = (per_cta - (long)tree_cta_bytes(ncw, lb, C, 0, R, V)) /
+                  tree_stage_bytes(ncw, lb);
+  return (int)(st > kTreeMaxStages ? kTreeMaxStages : st);
 }
 
 }  // namespace
 
-FusedPlan tv_fused_plan(int B, int R, int V, int sm_count, int smem_per_sm, int smem_per_block,
-                        int force_ncw, int force_c, int force_stages) {
+FusedPlan tv_fused_plan(int B, int R, int V, int logit_bytes, int sm_count, int smem_per_sm,
+                        int smem_per_block, int force_ncw, int force_c, int force_stages) {
   using namespace tvk::fused;
   FusedPlan p;
   // Large batches fill the GPU with one CTA of 8 consumer warps per tree; smaller
@@ -710,25 +1083,23 @@ FusedPlan tv_fused_plan(int B, int R, int V, int sm_count, int smem_per_sm, int 
   // tree's vocabulary across up to 8 SMs, as many as fit in one wave, keeping
   // every CTA's slice at least 2048 tokens.
   int ncw = (B >= 2 * sm_count) ? 8 : 4;
-  if (force_ncw == 4 || force_ncw == 8) ncw = force_ncw;
+  if (force_ncw == 4 || force_ncw == 8 || force_ncw == 16) ncw = force_ncw;
   int per_sm = 16 / ncw;
   int C = 1;
-  while (C < kMaxCluster && (long)B * (2 * C) <= (long)sm_count * per_sm &&
-         V / (2 * C) >= 2048)
-    C *= 2;
-  if (force_c == 1 || force_c == 2 || force_c == 4 || force_c == 8) C = force_c;
-  const size_t tree = tree_smem_bytes(R, V, C);
-  int stages = stages_for(ncw, per_sm, tree, smem_per_sm, smem_per_block);
+  while (C < 8 && (long)B * (2 * C) <= (long)sm_count * per_sm && V / (2 * C) >= 2048) C *= 2;
+  if (force_c == 1 || force_c == 2 || force_c == 4 || force_c == 8 || force_c == 16) C = force_c;
+  int stages = stages_for(ncw, logit_bytes, C, per_sm, R, V, smem_per_sm, smem_per_block);
   while (stages < 3 && per_sm > 1) {
     --per_sm;
-    stages = stages_for(ncw, per_sm, tree, smem_per_sm, smem_per_block);
+    stages = stages_for(ncw, logit_bytes, C, per_sm, R, V, smem_per_sm, smem_per_block);
   }
-  if (force_stages >= 2 && force_stages <= kMaxStages && force_stages < stages) stages = force_stages;
+  if (force_stages >= 2 && force_stages <= kTreeMaxStages && force_stages < stages)
+    stages = force_stages;
   p.ncw = ncw;
   p.C = C;
   p.stages = stages;
-  p.smem = (size_t)stages * stage_bytes(ncw) + tree;
-  p.ok = stages >= 2 && p.smem <= (size_t)smem_per_block;
+  p.smem = stages >= 0 ? tree_cta_bytes(ncw, logit_bytes, C, stages, R, V) : 0;
+  p.ok = stages >= 2 && p.smem + 1536 <= (size_t)smem_per_block;
   return p;
 }
 
@@ -739,9 +1110,13 @@ cudaError_t launch_one(const TravArgs& a, const FusedPlan& plan, cudaStream_t st
   auto k = tvk::fused::tv_tree_kernel<L, NCW>;
   cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)plan.smem);
   if (e != cudaSuccess) return e;
+  if (plan.C > 8) {
+    e = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e != cudaSuccess) return e;
+  }
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)(a.B * plan.C), 1, 1);
-  cfg.blockDim = dim3(NCW * 32 + 32, 1, 1);
+  cfg.blockDim = dim3(tvk::fused::TreeCta<L, NCW>::kThreads, 1, 1);
   cfg.dynamicSmemBytes = plan.smem;
   cfg.stream = stream;
   cudaLaunchAttribute attr[1];
@@ -754,6 +1129,13 @@ cudaError_t launch_one(const TravArgs& a, const FusedPlan& plan, cudaStream_t st
   return cudaLaunchKernelEx(&cfg, k, a, plan.C, plan.stages);
 }
 
+template <typename L>
+cudaError_t launch_ncw(const TravArgs& a, const FusedPlan& plan, cudaStream_t stream) {
+  if (plan.ncw == 16) return launch_one<L, 16>(a, plan, stream);
+  if (plan.ncw == 8) return launch_one<L, 8>(a, plan, stream);
+  return launch_one<L, 4>(a, plan, stream);
+}
+
 }  // namespace
 
 int tv_launch_fused(const TravArgs& a, int logit_is_bf16, const FusedPlan& plan,
@@ -763,13 +1145,8 @@ int tv_launch_fused(const TravArgs& a, int logit_is_bf16, const FusedPlan& plan,
     for (int k = 0; k < 3; ++k)
       if (cudaEventRecord(ev[k], stream) != cudaSuccess) return -5;
   }
-  cudaError_t e;
-  if (logit_is_bf16)
-    e = plan.ncw == 8 ? launch_one<tvk::Bf16Logits, 8>(a, plan, stream)
-                      : launch_one<tvk::Bf16Logits, 4>(a, plan, stream);
-  else
-    e = plan.ncw == 8 ? launch_one<tvk::F32Logits, 8>(a, plan, stream)
-                      : launch_one<tvk::F32Logits, 4>(a, plan, stream);
+  const cudaError_t e = logit_is_bf16 ? launch_ncw<tvk::Bf16Logits>(a, plan, stream)
+                                      : launch_ncw<tvk::F32Logits>(a, plan, stream);
   if (e != cudaSuccess) {
     cudaGetLastError();
     return -5;
