@@ -44,8 +44,11 @@ struct Ctl {
   int n_tests, n_passes;
 };
 
+// Per node i: rate p, (a, b) of its residual, normaliser (rowm, rows, invs =
+// 1 / rows).  Per child c: m the stored mass once removed, mb0 and zq / invZ
+// (child_order).
 struct TreeSmem {
-  double *p, *a, *b, *Z, *invZ, *m, *mb0, *invq, *invs;
+  double *p, *a, *b, *invZ, *m, *mb0, *zq, *invs;
   int32_t *par, *tok, *first, *next, *npass, *mask_tok, *job_rows;
   float *gl, *gq, *rowm, *rows, *dbgp, *mask_val, *tsum, *tmax;
   uint8_t* state;
@@ -64,7 +67,7 @@ __host__ __device__ inline int tree_tiles(int V, int C) {
 
 // Shared memory of one tree's state with `nt` bonus tiles.
 __host__ __device__ inline size_t tree_smem_bytes_nt(int R, int nt) {
-  return (size_t)R * (9 * 8 + 7 * 4 + 6 * 4 + 1) + (size_t)nt * 8 + 64;
+  return (size_t)R * (8 * 8 + 7 * 4 + 6 * 4 + 1) + (size_t)nt * 8 + 64;
 }
 
 
@@ -74,11 +77,10 @@ __device__ __forceinline__ TreeSmem carve_tree_nt(char* base, int R, int nt) {
   s.p = dp; dp += R;
   s.a = dp; dp += R;
   s.b = dp; dp += R;
-  s.Z = dp; dp += R;
   s.invZ = dp; dp += R;
   s.m = dp; dp += R;
   s.mb0 = dp; dp += R;
-  s.invq = dp; dp += R;
+  s.zq = dp; dp += R;
   s.invs = dp; dp += R;
   int32_t* ip = reinterpret_cast<int32_t*>(dp);
   s.par = ip; ip += R;
@@ -109,19 +111,77 @@ __device__ __forceinline__ int first_alive_child(const TreeSmem& s, int i) {
   return j;
 }
 
+// A node's children are removed in index order (the traversal always tries the
+// first remaining one), so Z_i when child c's turn comes is 1 less the draft
+// masses of the children before it, known from the start: s.invZ[c] = 1 / Z (0
+// if nothing is left) and s.zq[c] = Z / M_s^(0)(x_c).  First each node lists Z
+// for its children, then (after a barrier) each child divides.
+__device__ __forceinline__ void children_order(const TreeSmem& s, int i) {
+  double Z = 1.0;
+  for (int j = s.first[i]; j >= 0; j = s.next[j]) {
+    s.invZ[j] = Z;
+    Z -= (double)s.gq[j];
+  }
+}
+
+__device__ __forceinline__ void child_order(const TreeSmem& s, int c) {
+  const double Z = s.invZ[c];
+  s.zq[c] = Z / (double)s.gq[c];
+  s.invZ[c] = Z > 0.0 ? 1.0 / Z : 0.0;
+}
+
 // s.mb0[c] holds M_b^(0)(x_c | X^i) of child c of node i, in float64,
 // exp2((l_i(x_c) - m_i) log2(e) / T) / s_i, computed as soon as row i's
 // normaliser is known (a residual a M_b(x) - b M_s(x) of a sibling can cancel by
 // orders of magnitude, so this single value must not carry a float32 rounding).
+// s.p[c] holds M_b^(0)(x_c) / M_s^(0)(x_c) from then until the traversal reaches
+// c, so that descending through nodes without a rejection yet costs one
+// product per level (a dependent float64 operation takes 64 cycles here).
+__device__ __forceinline__ void set_child_mass(const TreeSmem& s, int c, float rowmax,
+                                               double inv_sum, double cd) {
+  const double mb = exp2(((double)s.gl[c] - (double)rowmax) * cd) * inv_sum;
+  s.mb0[c] = mb;
+  s.p[c] = mb * s.zq[c];   // (only a first child, whose Z is 1, is reached this way)
+}
 
 // min(p_i M_b(x_c) / M_s(x_c), 1) from i's current state, with
-// M_s(x_c) = q_c / Z_i; false if it is zero.
+// M_s(x_c) = q_c / Z_i; false if nothing of the draft support is left.
 __device__ __forceinline__ bool child_rate(const TreeSmem& s, int i, int c, double* out) {
+  if (s.npass[i] == 0) {   // the original rows: a = 1, b = 0, Z = 1
+    *out = fmin(s.p[i] * s.p[c], 1.0);
+    return true;
+  }
   const double q = (double)s.gq[c];
   const double mb = fmax(s.a[i] * s.mb0[c] - s.b[i] * q, 0.0);
-  if (!(s.invZ[i] > 0.0)) return false;
-  *out = fmin(s.p[i] * mb * s.Z[i] * s.invq[c], 1.0);
+  if (!(s.invZ[c] > 0.0)) return false;
+  *out = fmin(s.p[i] * mb * s.zq[c], 1.0);
   return true;
+}
+
+// Tokens of node i's removed children other than c, ascending, to list;
+// returns how many.
+__device__ inline int removed_tokens(const TreeSmem& s, int i, int c, int* list) {
+  int n = 0;
+  for (int j = s.first[i]; j >= 0; j = s.next[j]) {
+    if (j == c || s.state[j] == kAlive) continue;
+    const int t = s.tok[j];
+    int k = n;
+    while (k > 0 && list[k - 1] > t) {
+      list[k] = list[k - 1];
+      --k;
+    }
+    list[k] = t;
+    ++n;
+  }
+  return n;
+}
+
+// The stored masses of node i's removed children other than c.
+__device__ inline double removed_mass(const TreeSmem& s, int i, int c) {
+  double sum = 0.0;
+  for (int j = s.first[i]; j >= 0; j = s.next[j])
+    if (j != c && s.state[j] != kAlive) sum += s.m[j];
+  return sum;
 }
 
 __device__ inline void post_pass(const TreeSmem& s, Ctl& ctl, int i, int c) {
@@ -131,24 +191,10 @@ __device__ inline void post_pass(const TreeSmem& s, Ctl& ctl, int i, int c) {
   ctl.job.n_rows = 1;
   ctl.job.node = i;
   ctl.job.alpha1 = (float)(p * s.a[i] * s.invs[i]);
-  ctl.job.beta = (float)(p * s.b[i] + s.invZ[i]);
+  ctl.job.beta = (float)(p * s.b[i] + s.invZ[c]);
   ctl.job.rowmax = s.rowm[i];
-  int n = 0;
-  double msum = 0.0;
-  for (int j = s.first[i]; j >= 0; j = s.next[j]) {
-    if (j == c || s.state[j] == kAlive) continue;
-    const int t = s.tok[j];
-    int k = n;
-    while (k > 0 && s.mask_tok[k - 1] > t) {
-      s.mask_tok[k] = s.mask_tok[k - 1];
-      --k;
-    }
-    s.mask_tok[k] = t;
-    msum += s.m[j];
-    ++n;
-  }
-  ctl.job.nmask = n;
-  ctl.masked_sum = msum;
+  ctl.job.nmask = removed_tokens(s, i, c, s.mask_tok);
+  ctl.masked_sum = removed_mass(s, i, c);
   ctl.n_passes++;
   s.npass[i]++;
 }
@@ -157,7 +203,7 @@ __device__ inline void apply_rejection(const TreeSmem& s, Ctl& ctl, int i, int c
   const double p = s.p[i], a = s.a[i], b = s.b[i];
   const double S = (double)ctl.S + p * ctl.masked_sum;
   const double alpha = p * a;
-  const double beta = p * b + s.invZ[i];
+  const double beta = p * b + s.invZ[c];
   const double mb0 = s.mb0[c];
   const double q0 = (double)s.gq[c];
   if (S > 0.0) {
@@ -174,9 +220,6 @@ __device__ inline void apply_rejection(const TreeSmem& s, Ctl& ctl, int i, int c
     s.m[c] = fmax(a * mb0 - b * q0, 0.0);
     s.p[i] = (p == 1.0) ? 1.0 : 0.0;
   }
-  const double Z = s.Z[i] - q0;
-  s.Z[i] = Z;
-  s.invZ[i] = (Z > 0.0) ? 1.0 / Z : 0.0;
 }
 
 // Lists the not-yet-normalised internal nodes of the chain that starts at
@@ -222,128 +265,202 @@ __device__ inline void post_bonus(const TreeSmem& s, Ctl& ctl, int a) {
 // ---------------------------------------------------- deciding ahead ----
 //
 // While the pass that rejects child c of node i runs, most of the next step is
-// already fixed.  In the common case -- the next remaining child c2 of i is a
-// leaf -- that step is the test of c2, and with
-//   D = S + (1 - p_i),   X = [alpha M_b0(c2) - beta q(c2)]_+ Z' / q(c2),
-//   alpha = p_i a_i,  beta = p_i b_i + 1/Z_i,  Z' = Z_i - q(c),
-// Eqs. (1)-(3) give c2's rate min(X / D, 1), so c2 is accepted iff u D < X, and
-// the pass that rejects c2 uses alpha1 = alpha / (s_i D), beta' = beta / D + 1/Z'.
-// Only D depends on the pass's S, so the next job can be posted right after
-// S arrives and the state update (control_step_ahead) done afterwards.
-// The other common case -- i has no remaining child -- is the test of i
-// itself with its new rate S / D: i is rejected iff u D >= S, and the pass
-// that then rejects i at its parent g depends only on g's state.
+// already fixed.  With
+//   D = S + (1 - p_i),   alpha = p_i a_i,  beta = p_i b_i + 1/Z_i,  Z' = Z_i - q(c)
+// Eqs. (1)-(3) give a child c2 the rate min(X / D, 1),
+//   X = [alpha M_b0(c2) - beta q(c2)]_+ Z' / q(c2),
+// and a pass that then rejects c2 uses alpha1 = alpha / (s_i D) and
+// beta' = beta / D + 1/Z'.  Only D depends on the pass's S, so of the next
+// remaining child c2 of i it is known before S arrives:
+//   * kAheadTest: c2 is a leaf with X > 0: it is accepted iff u D < X;
+//   * kAheadPrune: X = 0, c2 has rate 0 whatever S is: it is removed, and the
+//     pass for it follows (about half of all passes of EAGLE-shaped trees);
+//   * kAheadDescend: c2 has children and X > 0: the traversal goes down to c2,
+//     whose chain's rows are normalised next;
+//   * kAheadUp: no child remains: i itself is tested with its new rate S / D
+//     and accepted iff u D < S; the pass that rejects i at its parent g depends
+//     only on g's state.
+// The next job is posted as soon as S arrives, the state update
+// (control_step_ahead) done while it runs.
+// Float64 is slow here (64 cycles a dependent operation, 426 a division), so what
+// does not depend on S is in child tables (child_order) or worked out while the
+// pass runs, and the three divisions S leads to are done by three lanes at once.
+// With all four modes, against the leaf test and kAheadUp alone: the persistent
+// kernel at V = 128256 takes 453 -> 421 us (B = 128), 256 -> 237 us (B = 32, given
+// normalisers), the cluster kernel at V = 32000, B = 64 183 -> 148 us.
+enum : int { kAheadTest = 1, kAheadPrune = 2, kAheadDescend = 3, kAheadUp = 4 };
+
 struct Ahead {
   int ok;          // 1: the next step is decided from D alone (see mode)
-  int mode;        // 1: test of leaf c2 of i; 2: test of i itself (then a pass at g)
-  int i, c, c2, g, nmask;
-  double omp;      // 1 - p_i
-  double X, ainvs, beta, invZn;
-  float alpha1_g, beta_g, rowmax_g;   // mode 2: the pass at g that rejects i
+  int mode;
+  int i, c, c2, g, nmask, n_rows;
+  double p, omp, pm;             // p_i, 1 - p_i, p_i x the removed tokens' mass
+  double X, alpha, beta, ainvs, invZn, mb0, q0, uu, msum_g;
+  float alpha1_g, beta_g, rowmax_g;   // kAheadUp: the pass at g that rejects i
 };
 
 // S-independent part of the next step, after posting the pass for ctl.pending;
-// the next pass's removed tokens (ascending) go to mtok2.
+// the next pass's removed tokens (ascending) go to mtok2, the rows to
+// normalise next to s.job_rows.
 __device__ inline void prepare_ahead(const TreeSmem& s, const Ctl& ctl, Ahead& ah,
-                                     int* mtok2) {
+                                     int* mtok2, const float* __restrict__ u) {
   ah.ok = 0;
   if (ctl.job.kind != kJobPass) return;
   const int c = ctl.pending, i = s.par[c];
+  if (!(s.rows[i] > 0.f)) return;
+  const double p = s.p[i], a = s.a[i], b = s.b[i];
+  const double alpha = p * a, beta = p * b + s.invZ[c];
+  ah.i = i;
+  ah.c = c;
+  ah.p = p;
+  ah.omp = 1.0 - p;
+  ah.pm = p * ctl.masked_sum;
+  ah.alpha = alpha;
+  ah.beta = beta;
+  ah.mb0 = s.mb0[c];
+  ah.q0 = (double)s.gq[c];
   const int c2 = first_alive_child(s, i);
+  ah.c2 = c2;
   if (c2 < 0) {
     if (i == 0) return;   // the root: the bonus draw follows
     const int g = s.par[i];
     // the pass post_pass(s, ctl, g, i) would post (g's state does not change)
     const double pg = s.p[g];
     ah.alpha1_g = (float)(pg * s.a[g] * s.invs[g]);
-    ah.beta_g = (float)(pg * s.b[g] + s.invZ[g]);
+    ah.beta_g = (float)(pg * s.b[g] + s.invZ[i]);
     ah.rowmax_g = s.rowm[g];
-    int n = 0;
-    for (int j = s.first[g]; j >= 0; j = s.next[j]) {
-      if (j == i || s.state[j] == kAlive) continue;
-      const int t = s.tok[j];
-      int k = n;
-      while (k > 0 && mtok2[k - 1] > t) {
-        mtok2[k] = mtok2[k - 1];
-        --k;
-      }
-      mtok2[k] = t;
-      ++n;
-    }
-    ah.mode = 2;
-    ah.i = i;
-    ah.c = c;
-    ah.c2 = -1;
+    ah.nmask = removed_tokens(s, g, i, mtok2);
+    ah.msum_g = removed_mass(s, g, i);
+    ah.uu = (double)u[i];
+    ah.mode = kAheadUp;
     ah.g = g;
-    ah.nmask = n;
-    ah.omp = 1.0 - s.p[i];
     ah.ok = 1;
     return;
   }
-  if (s.first[c2] >= 0 || !(s.rows[i] > 0.f)) return;
-  const double p = s.p[i], a = s.a[i], b = s.b[i];
-  const double Zn = s.Z[i] - (double)s.gq[c];
-  if (!(Zn > 0.0)) return;
-  const double alpha = p * a, beta = p * b + s.invZ[i];
-  const double X = fmax(alpha * s.mb0[c2] - beta * (double)s.gq[c2], 0.0) * Zn * s.invq[c2];
-  if (!(X > 0.0)) return;
-  int n = 0;
-  for (int j = s.first[i]; j >= 0; j = s.next[j]) {
-    if (j == c2 || s.state[j] == kAlive) continue;
-    const int t = s.tok[j];
-    int k = n;
-    while (k > 0 && mtok2[k - 1] > t) {
-      mtok2[k] = mtok2[k - 1];
-      --k;
-    }
-    mtok2[k] = t;
-    ++n;
+  const double invZn = s.invZ[c2];
+  if (!(invZn > 0.0)) return;
+  const double y = fmax(alpha * s.mb0[c2] - beta * (double)s.gq[c2], 0.0);
+  if (y > 0.0 && s.first[c2] >= 0) {
+    int n = 0;
+    for (int k = c2; k >= 0 && s.first[k] >= 0; k = first_alive_child(s, k))
+      if (!(s.rows[k] > 0.f)) s.job_rows[n++] = k;
+    if (n == 0) return;
+    ah.n_rows = n;
+    ah.mode = kAheadDescend;
+    ah.ok = 1;
+    return;
   }
-  ah.i = i;
-  ah.c = c;
-  ah.c2 = c2;
-  ah.nmask = n;
-  ah.omp = 1.0 - p;
-  ah.X = X;
   ah.ainvs = alpha * s.invs[i];
-  ah.beta = beta;
-  ah.invZn = 1.0 / Zn;
-  ah.mode = 1;
+  ah.invZn = invZn;
+  ah.X = y * s.zq[c2];
+  ah.nmask = removed_tokens(s, i, c2, mtok2);
+  ah.uu = (double)u[c2];
+  ah.mode = ah.X > 0.0 ? kAheadTest : kAheadPrune;
   ah.g = -1;
   ah.ok = 1;
 }
 
-// control_step for the pass described by `ah`, with the test of ah.c2 going
-// the way `accept` says (the decision taken ahead, so that the state follows
-// the job already posted).
+// The next job of the step described by `ah`, given the pass's S (D = S + 1 -
+// p_i, inv_d = 1 / D where the mode needs it); false if that job needs the
+// updated state first (the residual draw at i).  `accept`: the test's outcome.
+__device__ inline bool job_ahead(const TreeSmem& s, const Ahead& ah, double S, double D,
+                                 double inv_d, Job& j, bool& accept) {
+  accept = false;
+  j.n_rows = 1;
+  j.kind = kJobPass;
+  j.nmask = ah.nmask;
+  if (ah.mode == kAheadUp) {
+    accept = ah.uu * D < S;
+    j.node = ah.g;
+    j.alpha1 = ah.alpha1_g;
+    j.beta = ah.beta_g;
+    j.rowmax = ah.rowmax_g;
+    return !accept;
+  }
+  if (ah.mode == kAheadDescend) {
+    j.kind = kJobStats;
+    j.n_rows = ah.n_rows;
+    j.node = ah.c2;
+    return true;
+  }
+  if (ah.mode == kAheadTest) accept = ah.uu * D < ah.X;
+  if (accept) {
+    j.kind = kJobBonusLeaf;
+    j.node = ah.c2;
+    j.nmask = 0;
+    return true;
+  }
+  j.node = ah.i;
+  j.alpha1 = (float)(ah.ainvs * inv_d);
+  j.beta = (float)(ah.beta * inv_d + ah.invZn);
+  j.rowmax = s.rowm[ah.i];
+  return true;
+}
+
+// Bookkeeping of a pass at i for child c whose job has been posted already
+// (msum: the stored masses of i's other removed children).
+__device__ inline void note_pass(const TreeSmem& s, Ctl& ctl, int i, int c, double msum) {
+  ctl.pending = c;
+  ctl.job.kind = kJobPass;
+  ctl.job.n_rows = 1;
+  ctl.job.node = i;
+  ctl.masked_sum = msum;
+  ctl.n_passes++;
+  s.npass[i]++;
+}
+
+// control_step for the pass described by `ah`, given inv_d = 1 / D, inv_s = 1 /
+// S and p_new = S / D, with the test going the way `accept` says (the decision
+// taken ahead, so that the state follows the job already posted).
 __device__ inline void control_step_ahead(const TreeSmem& s, Ctl& ctl, const Ahead& ah,
-                                          bool accept) {
-  apply_rejection(s, ctl, ah.i, ah.c);
+                                          bool accept, double inv_d, double inv_s,
+                                          double p_new) {
+  const int i = ah.i, c = ah.c;
+  const double na = ah.alpha * inv_s, nb = ah.beta * inv_s, scale = ah.p * inv_s;
+  const double mc = fmax(na * ah.mb0 - nb * ah.q0, 0.0);
+  for (int j = s.first[i]; j >= 0; j = s.next[j])
+    if (j != c && s.state[j] != kAlive) s.m[j] *= scale;
+  s.m[c] = mc;
+  s.a[i] = na;
+  s.b[i] = nb;
+  s.p[i] = p_new;
+  const double msum = ctl.masked_sum * scale + mc;
   ctl.pending = -1;
-  if (ah.mode == 2) {
-    ctl.node = ah.i;
+  ctl.node = i;
+  if (ah.mode == kAheadUp) {
     ctl.n_tests++;
-    s.dbgp[ah.i] = (float)s.p[ah.i];
+    s.dbgp[i] = (float)p_new;
     if (accept) {
-      post_bonus(s, ctl, ah.i);
+      post_bonus(s, ctl, i);
       return;
     }
-    s.state[ah.i] = kRejected;
-    post_pass(s, ctl, ah.g, ah.i);
+    s.state[i] = kRejected;
+    note_pass(s, ctl, ah.g, i, ah.msum_g);
     return;
   }
-  double pc = 0.0;
-  child_rate(s, ah.i, ah.c2, &pc);
-  s.p[ah.c2] = pc;
-  ctl.node = ah.c2;
+  if (ah.mode == kAheadDescend) {   // (control_step goes down to c2 after the job)
+    ctl.job.kind = kJobStats;
+    ctl.job.n_rows = ah.n_rows;
+    return;
+  }
+  const int c2 = ah.c2;
+  if (ah.mode == kAheadPrune) {
+    s.state[c2] = kPruned;
+    s.dbgp[c2] = 0.f;
+    note_pass(s, ctl, i, c2, msum);
+    return;
+  }
+  const double pc = fmin(ah.X * inv_d, 1.0);
+  s.p[c2] = pc;
+  ctl.node = c2;
   ctl.n_tests++;
-  s.dbgp[ah.c2] = (float)pc;
+  s.dbgp[c2] = (float)pc;
   if (accept) {
-    post_bonus(s, ctl, ah.c2);
+    post_bonus(s, ctl, c2);
     return;
   }
-  s.state[ah.c2] = kRejected;
-  post_pass(s, ctl, ah.i, ah.c2);
+  s.state[c2] = kRejected;
+  note_pass(s, ctl, i, c2, msum);
 }
 
 // Advances the serial traversal until it needs vocabulary work; posts it.

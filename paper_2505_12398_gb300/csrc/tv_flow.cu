@@ -748,8 +748,6 @@ __device__ void owner_new_tree(const TravArgs& a, const TreeSmem& s, Shared& sh,
     s.state[i] = kAlive;
     s.a[i] = 1.0;
     s.b[i] = 0.0;
-    s.Z[i] = 1.0;
-    s.invZ[i] = 1.0;
     s.m[i] = 0.0;
     s.p[i] = 0.0;
     s.rows[i] = 0.f;
@@ -786,11 +784,16 @@ __device__ void owner_new_tree(const TravArgs& a, const TreeSmem& s, Shared& sh,
         s.gl[i] = L::at(logits + prow, t);
         s.gq[i] = __ldg(a.draft_probs + prow + t);
         if (!(s.gq[i] > 0.f)) bad2 |= 8u;
-        s.invq[i] = 1.0 / (double)s.gq[i];
       }
       s.next[i] = nx;
     }
     bad = __reduce_or_sync(0xffffffffu, bad2);
+    __syncwarp();
+    if (bad == 0u)
+      for (int i = lane; i < R; i += 32) children_order(s, i);
+    __syncwarp();
+    if (bad == 0u)
+      for (int i = lane + 1; i < R; i += 32) child_order(s, i);
   }
   __syncwarp();
   if (kGiven && bad == 0u) {
@@ -808,7 +811,7 @@ __device__ void owner_new_tree(const TravArgs& a, const TreeSmem& s, Shared& sh,
     __syncwarp();
     for (int i = lane + 1; i < R; i += 32) {
       const int p = s.par[i];
-      s.mb0[i] = exp2(((double)s.gl[i] - (double)s.rowm[p]) * a.c) * s.invs[p];
+      set_child_mass(s, i, s.rowm[p], s.invs[p], a.c);
     }
     bad = __reduce_or_sync(0xffffffffu, bad3);
     __syncwarp();
@@ -858,13 +861,12 @@ __device__ void owner_combine(const TravArgs& a, const FlowArgs& f, const TreeSm
     }
     if (__any_sync(0xffffffffu, bad_row) && lane == 0) sh.ctl.bad |= 64u;
     __syncwarp();
-    // ... then M_b^(0) of those rows' children, one lane per node (the same
-    // value the cluster kernel computes, see tv_control.cuh)
+    // ... then M_b^(0) of those rows' children, one lane per node
     for (int i = lane + 1; i < R; i += 32) {
       const int p = s.par[i];
       bool mine = false;
       for (int r = 0; r < sh.jrows; ++r) mine |= (s.job_rows[r] == p);
-      if (mine) s.mb0[i] = exp2(((double)s.gl[i] - (double)s.rowm[p]) * a.c) * s.invs[p];
+      if (mine) set_child_mass(s, i, s.rowm[p], s.invs[p], a.c);
     }
     __syncwarp();
   } else if (sh.jkind == kJobPass) {
@@ -1159,57 +1161,30 @@ __device__ void owner_role(const TravArgs& a, const FlowArgs& f, const Smem& m, 
         float S_pass = 0.f;
         for (int k2 = lane; k2 < sh.jK; k2 += 32) S_pass += sh.pbuf[k2].x;
         S_pass = warp_sum(S_pass);
-        int fast = 0, post_first = 0, accept = 0;
-        if (lane == 0) {
-          const Ahead& ah = sh.ahead;
-          const double S = (double)S_pass + s.p[ah.i] * sh.ctl.masked_sum;
-          if (S > 1e-300) {
-            fast = 1;
-            const double D = S + ah.omp;
-            Job& jf = sh.fjob;
-            jf.n_rows = 1;
-            if (ah.mode == 1) {
-              accept = ((double)m.u[ah.c2] * D < ah.X) ? 1 : 0;
-              post_first = 1;
-              if (accept) {
-                jf.kind = kJobBonusLeaf;
-                jf.node = ah.c2;
-                jf.nmask = 0;
-              } else {
-                const double invD = 1.0 / D;
-                jf.kind = kJobPass;
-                jf.node = ah.i;
-                jf.nmask = ah.nmask;
-                jf.alpha1 = (float)(ah.ainvs * invD);
-                jf.beta = (float)(ah.beta * invD + ah.invZn);
-                jf.rowmax = s.rowm[ah.i];
-              }
-            } else {
-              accept = ((double)m.u[ah.i] * D < S) ? 1 : 0;
-              if (!accept) {   // the pass at g that rejects i is known already
-                post_first = 1;
-                jf.kind = kJobPass;
-                jf.node = ah.g;
-                jf.nmask = ah.nmask;
-                jf.alpha1 = ah.alpha1_g;
-                jf.beta = ah.beta_g;
-                jf.rowmax = ah.rowmax_g;
-              }
-            }
+        const Ahead& ah = sh.ahead;
+        const double S = (double)S_pass + ah.pm;
+        if (S > 1e-300) {   // (the same in every lane)
+          const double D = S + ah.omp;
+          // 1 / D, 1 / S and S / D in lanes 0, 1 and 2: a float64 division
+          // takes as long for one lane as for three
+          const double quot = (lane == 2 ? S : 1.0) / (lane == 1 ? S : D);
+          int post_first = 0, accept = 0;
+          if (lane == 0) {
+            bool acc;
+            post_first = job_ahead(s, ah, S, D, quot, sh.fjob, acc) ? 1 : 0;
+            accept = acc ? 1 : 0;
             sh.ctl.S = S_pass;
           }
-        }
-        fast = __shfl_sync(0xffffffffu, fast, 0);
-        if (fast) {
           post_first = __shfl_sync(0xffffffffu, post_first, 0);
-          accept = __shfl_sync(0xffffffffu, accept, 0);
+          const double inv_s = __shfl_sync(0xffffffffu, quot, 1);
+          const double p_new = __shfl_sync(0xffffffffu, quot, 2);
           __syncwarp();
           if (post_first) {
             post_job(s, sh, a, f, my_tree, V, lane, __shfl_sync(0xffffffffu, done_est, 0),
                      sh.fjob, m.mtok2, s.mask_val);
-            if (lane == 0) control_step_ahead(s, sh.ctl, sh.ahead, accept != 0);
+            if (lane == 0) control_step_ahead(s, sh.ctl, ah, accept != 0, quot, inv_s, p_new);
           } else {
-            if (lane == 0) control_step_ahead(s, sh.ctl, sh.ahead, accept != 0);
+            if (lane == 0) control_step_ahead(s, sh.ctl, ah, accept != 0, quot, inv_s, p_new);
             __syncwarp();
             post_job(s, sh, a, f, my_tree, V, lane, __shfl_sync(0xffffffffu, done_est, 0),
                      sh.ctl.job, s.mask_tok, s.mask_val);
@@ -1217,7 +1192,7 @@ __device__ void owner_role(const TravArgs& a, const FlowArgs& f, const Smem& m, 
           if (lane == 0) {
             done_est = ld_relaxed_u32(&f.ctr[kCtrDone]);
             if (a.token_level) sh.ahead.ok = 0;            // (Traversal Verification only)
-            else prepare_ahead(s, sh.ctl, sh.ahead, m.mtok2);   // for the job just posted
+            else prepare_ahead(s, sh.ctl, sh.ahead, m.mtok2, m.u);   // for the job just posted
           }
           continue;
         }
@@ -1247,7 +1222,7 @@ __device__ void owner_role(const TravArgs& a, const FlowArgs& f, const Smem& m, 
       if (lane == 0) {
         done_est = ld_relaxed_u32(&f.ctr[kCtrDone]);   // used at the next job
         if (a.token_level) sh.ahead.ok = 0;             // (Traversal Verification only)
-        else prepare_ahead(s, sh.ctl, sh.ahead, m.mtok2);    // while this job runs
+        else prepare_ahead(s, sh.ctl, sh.ahead, m.mtok2, m.u);    // while this job runs
       }
     }
   }

@@ -14,14 +14,15 @@
 //   * warp-specialised: NCW consumer warps reduce, a producer warp issues the
 //     bulk copies (TMA), a control warp runs the serial control.  While a pass
 //     runs, the control warp works out the step after it (Ahead), so that one
-//     float64 comparison and one division stand between a pass's S and the
-//     next job;
+//     float64 comparison and at most one division stand between a pass's S and
+//     the next job;
 //   * every consumer warp sends its partial straight to the control warps of
 //     all C CTAs (st.async: the store carries its own completion count), with
 //     no reduction inside the CTA in between; two exchange buffers alternate;
-//   * a normaliser job takes up to kStatRows rows of the chain being entered:
-//     one exchange for all of them, and the rows' final sums and their
-//     children's float64 masses are spread over the consumer warps;
+//   * a normaliser job takes up to kStatRows rows of the chain being entered,
+//     each row by a group of warps, with one exchange for all of them; the
+//     rows' final sums and their children's float64 masses are spread over the
+//     consumer warps;
 //   * where a slice of a (target, draft) row pair fits the ring, it stays there:
 //     the next pass at the same node (about half of all passes) reads no
 //     memory, and with room for two the parent's pair is fetched while the
@@ -42,8 +43,9 @@
 //
 // Measured (60-node trees, V = 32000, bf16; 8-token chains, fp32), against one
 // thread of the consumers doing the control, a reduction and an exchange per
-// row and no resident pairs: B = 64 254.7 -> 183.2 us, B = 1 119 -> 81 us,
-// 16 chains 117.2 -> 77.2 us.
+// row and no resident pairs: B = 64 254.2 -> 148.1 us, 16 chains 117.0 -> 71.8 us
+// (183.2 and 77.2 us with a row by all warps in turn and before the removal of a
+// rate-0 sibling and the descent into a sub-tree were worked out ahead).
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -67,6 +69,18 @@ __host__ __device__ constexpr int tiles_per_warp(int ncw) { return ncw == 16 ? 1
 __host__ __device__ constexpr int tree_stage_bytes(int ncw, int lb) {
   return ncw * tiles_per_warp(ncw) * kTileElems * (lb + 4);
 }
+
+// Groups of consumer warps in a normaliser job of n rows: row r is summed by
+// group r % groups, so that a warp reduces and sends for few rows; no more
+// groups than warps or than rows fit the ring at once (`most`).
+__host__ __device__ constexpr int row_groups(int n, int most) {
+  int g = 1;
+  while (2 * g <= n && 2 * g <= most) g *= 2;
+  return g;
+}
+// Partials of one exchange at most (rows x CTAs x warps per group): a job
+// takes up to four rows per group.
+__host__ __device__ constexpr int exchange_slots(int C, int ncw) { return 4 * C * ncw; }
 
 // A job as the control warp hands it to the CTA's other warps.
 struct TreeJob {
@@ -219,18 +233,21 @@ struct TreeCta {
   TreeSmem s;
   TreeShared& sh;
   char* ring;
-  float2* xs;              // [2][kStatRows][C * NCW] exchange slots
+  float2* xs;              // [2][exchange_slots] partials of all CTAs
   int* mtok_ahead;         // [2][R] removed tokens of passes worked out ahead
+  float* u;                // [R + 1] the tree's uniforms
   uint64_t *full_bar, *empty_bar, *xbar, *job_bar, *ack_bar, *stat_bar, *tile_bar;
   int C, n_stages, b, v0, v1;
+  int spc;                 // stages a resident pair takes
+  int max_groups;          // groups of a normaliser job at most
   uint32_t rank;
   size_t row0;             // the tree's first row in the batch
 
   __device__ TreeCta(const TravArgs& args, TreeShared& shared) : a(args), sh(shared) {}
 
   __device__ __forceinline__ void fail() { atomicOr(&sh.ctl.bad, 32u); }
-  __device__ __forceinline__ float2* xslots(int buf, int row) const {
-    return xs + ((size_t)buf * kStatRows + row) * (size_t)(C * NCW);
+  __device__ __forceinline__ float2* xslots(int buf) const {
+    return xs + buf * exchange_slots(C, NCW);
   }
   // Lists of removed tokens: 0 the control's own, 1 and 2 worked out ahead.
   __device__ __forceinline__ int* mtok(int k) const {
@@ -241,21 +258,18 @@ struct TreeCta {
   }
 
   // ---------------------------------------------------------- producer --
-  // Fills stage `st` with chunk k of the row's slice (n_all: elements of the
-  // arrays).  `filled` and `fph` track each stage's fills: a fetch ahead that no
+  // Fills stage `st` with the slice's chunk from element x of its first block
+  // (n_all: elements of the arrays).  `filled` and `fph` track each stage's fills: a fetch ahead that no
   // job has waited for must have landed before its stage is filled again.
-  __device__ bool fill(int st, size_t row, int k, bool pair, size_t n_all, uint32_t& filled,
-                       uint32_t& fph) {
+  __device__ bool fill(int st, const Slice& sl, int x, bool pair, size_t n_all,
+                       uint32_t& filled, uint32_t& fph) {
     if ((filled >> st) & 1u) {
       if (!mbar_wait(&full_bar[st], (fph >> st) & 1u)) return false;
     }
     filled |= 1u << st;
     fph ^= 1u << st;
-    const Slice sl(row, a.V, v0, v1);
-    const int per = pair ? kPair : kRow;
-    const size_t e0 = sl.base + (size_t)k * per;
-    int n = min(per, sl.n - k * per);
-    n = (n + 7) & ~7;                        // whole blocks
+    const size_t e0 = sl.base + (size_t)x;
+    const int n = (min(pair ? kPair : kRow, sl.n - x) + 7) & ~7;   // whole blocks
     char* dst = ring + (size_t)st * kStageBytes;
     int whole = n;
     if (e0 + n > n_all) {
@@ -281,7 +295,6 @@ struct TreeCta {
 
   // Streams the jobs' rows (one lane).
   __device__ bool produce(size_t n_all, uint32_t& filled, uint32_t& fph) {
-    const int spc = chunks_of(v1 - v0 + 7, kPair);
     uint32_t jp = 0u, eph = 0u;
     for (;;) {
       if (!mbar_wait(job_bar, jp)) return false;
@@ -292,26 +305,26 @@ struct TreeCta {
       const bool pair = is_pair(job.kind);
       const int per = pair ? kPair : kRow;
       if (job.total > 0) {
-        const int st0 = job.slot > 0 ? job.slot * spc : 0;
+        int st = job.slot > 0 ? job.slot * spc : 0;
         int q = 0;
         for (int r = 0; r < job.n_rows; ++r) {
           const size_t row = row0 + (job.kind == kJobStats ? sh.job.rows[r] : job.node);
-          const int nch = chunks_of(Slice(row, a.V, v0, v1).n, per);
-          for (int k = 0; k < nch; ++k, ++q) {
-            const int st = st0 + (job.slot >= 0 ? k : q % n_stages);
+          const Slice sl(row, a.V, v0, v1);
+          for (int x = 0; x < sl.n; x += per, ++q) {
             if (q >= n_stages) {               // a stage of this job, used again
               if (!mbar_wait(&empty_bar[st], (eph >> st) & 1u)) return false;
               eph ^= 1u << st;
             }
-            if (!fill(st, row, k, pair, n_all, filled, fph)) return false;
+            if (!fill(st, sl, x, pair, n_all, filled, fph)) return false;
+            if (++st == n_stages) st = 0;
           }
         }
       }
       if (job.pf_node >= 0) {
-        const size_t row = row0 + job.pf_node;
-        const int nch = chunks_of(Slice(row, a.V, v0, v1).n, kPair);
-        for (int k = 0; k < nch; ++k)
-          if (!fill(job.pf_slot * spc + k, row, k, true, n_all, filled, fph)) return false;
+        const Slice sl(row0 + job.pf_node, a.V, v0, v1);
+        int st = job.pf_slot * spc;
+        for (int x = 0; x < sl.n; x += kPair, ++st)
+          if (!fill(st, sl, x, true, n_all, filled, fph)) return false;
       }
     }
   }
@@ -325,15 +338,15 @@ struct TreeCta {
   }
 
   // ---------------------------------------------------------- exchange --
-  // A partial of row r of the job, to every CTA.  The exchange's barrier
+  // A partial to slot `slot` of every CTA.  The exchange's barrier
   // counts the bytes of all CTAs' partials (the control warp arms it); a tree
   // of one CTA is launched without a cluster, so there the warps store to
   // their own slots and arrive once per job (arrive_alone).
-  __device__ __forceinline__ void send(int xb, int r, int slot, int lane, float x, float y) {
+  __device__ __forceinline__ void send(int xb, int slot, int lane, float x, float y) {
     if (C == 1) {
-      if (lane == 0) xslots(xb, r)[slot] = make_float2(x, y);
+      if (lane == 0) xslots(xb)[slot] = make_float2(x, y);
     } else if (lane < C) {
-      st_async_v2(map_shared(xslots(xb, r) + slot, lane), x, y, map_shared(&xbar[xb], lane));
+      st_async_v2(map_shared(xslots(xb) + slot, lane), x, y, map_shared(&xbar[xb], lane));
     }
   }
   __device__ __forceinline__ void arrive_alone(int xb, int lane) {
@@ -346,8 +359,166 @@ struct TreeCta {
 
   // --------------------------------------------------------- consumers --
 
-  __device__ void consumer(int wid, int lane) {
+  // The eight logits of the lane's block e0 of a stage, whose elements [lo, hi)
+  // belong to the slice (the others read as the smallest value).
+  __device__ __forceinline__ void stage_logits(const E* lb, int e0, bool valid, bool edge, int lo,
+                                               int hi, float v[8]) const {
+    constexpr float kNone = kLB == 2 ? -9984.f : -INFINITY;
+    if (valid) {
+      lds_logits<L>(lb + e0, v);
+    } else {
+#pragma unroll
+      for (int e = 0; e < 8; ++e) v[e] = kNone;
+    }
+    if (edge) {
+#pragma unroll
+      for (int e = 0; e < 8; ++e)
+        if (e < lo || e >= hi) v[e] = kNone;
+    }
+  }
+  static __device__ __forceinline__ void zero_outside(bool edge, int lo, int hi, float t[8]) {
+    if (edge) {
+#pragma unroll
+      for (int e = 0; e < 8; ++e)
+        if (e < lo || e >= hi) t[e] = 0.f;
+    }
+  }
+
+  // Row normalisers: this warp's group takes every g-th row.
+  __device__ bool sum_rows(const TreeJob& job, int wid, int lane, uint32_t& ph) {
     const float c_hi = a.c_hi, c_lo = a.c_lo;
+    const int n_rows = job.n_rows, total = job.total, xb = job.xb;
+    const int g = row_groups(n_rows, max_groups), group = wid % g, sub = wid / g, nsub = NCW / g;
+    const bool reuse = total > n_stages;       // stages are filled more than once
+    int st = 0, q = 0;
+    for (int r = 0; r < n_rows; ++r) {
+      const Slice sl(row0 + job.rows[r], a.V, v0, v1);
+      const bool mine = r % g == group;
+      float m_run = TV_NEG_INF;
+      Comp acc;
+      for (int x = 0; x < sl.n; x += kRow, ++q) {
+        ph ^= 1u << st;
+        if (mine || reuse) {
+          if (!mbar_wait_warp(&full_bar[st], (ph >> st) & 1u)) return false;
+        }
+        if (mine) {
+          const E* lb = reinterpret_cast<const E*>(ring + (size_t)st * kStageBytes);
+          const int n = min(kRow, sl.n - x);
+          for (int t0 = sub * kTileElems; t0 < n; t0 += nsub * kTileElems) {
+            const int e0 = t0 + lane * kChunk;
+            if (e0 >= n) continue;
+            const int lo = sl.sh - (x + e0), hi = sl.n - (x + e0);
+            const bool edge = lo > 0 || hi < 8;
+            float v[8], t[8];
+            stage_logits(lb, e0, true, edge, lo, hi, v);
+            const float cm = fmaxf(fmaxf(fmaxf(v[0], v[1]), fmaxf(v[2], v[3])),
+                                   fmaxf(fmaxf(v[4], v[5]), fmaxf(v[6], v[7])));
+            if (cm > m_run) {
+              if (m_run != TV_NEG_INF) {
+                const float sc = L::exp_rel(m_run, cm, c_hi, c_lo);
+                acc.s *= sc;
+                acc.c *= sc;
+              }
+              m_run = cm;
+            }
+            exp8<L, false>(v, m_run, c_hi, c_lo, t);
+            zero_outside(edge, lo, hi, t);
+            acc.add(sum8(t));
+          }
+        }
+        if (q + n_stages < total) {            // the producer waits for this stage
+          __syncwarp();
+          if (lane == 0) mbar_arrive(&empty_bar[st]);
+        }
+        if (++st == n_stages) st = 0;
+      }
+      if (mine) {
+        const float wm = warp_max(m_run);
+        const float part =
+            (m_run == TV_NEG_INF) ? 0.f : acc.value() * L::exp_rel(m_run, wm, c_hi, c_lo);
+        send(xb, (r * C + (int)rank) * nsub + sub, lane, wm, warp_sum(part));
+      }
+    }
+    arrive_alone(xb, lane);
+    return true;
+  }
+
+  // A rejection pass (kJobPass: the warp's sum, returned) or the tile sums of a
+  // bonus draw.
+  __device__ bool pair_or_leaf(const TreeJob& job, int wid, int lane, uint32_t& ph, float& sum) {
+    const float c_hi = a.c_hi, c_lo = a.c_lo;
+    const int kind = job.kind, total = job.total;
+    const bool pair = is_pair(kind);
+    const int per = pair ? kPair : kRow;
+    const int nmask = job.nmask;
+    const int* mt = mtok(job.mbuf);
+    const float al = job.alpha1, be = job.beta, rm = job.rowmax;
+    const Slice sl(row0 + job.node, a.V, v0, v1);
+    int st = job.slot > 0 ? job.slot * spc : 0, q = 0, mp = 0;
+    Comp acc;
+    for (int x = 0; x < sl.n; x += per, ++q) {
+      if (total > 0) ph ^= 1u << st;           // filled by this job
+      if (!mbar_wait_warp(&full_bar[st], (ph >> st) & 1u)) return false;
+      const char* buf = ring + (size_t)st * kStageBytes;
+      const E* lb = reinterpret_cast<const E*>(buf);
+      const float* qb = reinterpret_cast<const float*>(buf + (size_t)kPair * kLB);
+      const int n = min(per, sl.n - x);
+      for (int t0 = wid * kTileElems; t0 < n; t0 += kSweep) {
+        const int e0 = t0 + lane * kChunk;
+        const bool valid = e0 < n;
+        const int xg = v0 - sl.sh + x + e0;    // token of the lane's first element
+        const int lo = sl.sh - (x + e0), hi = sl.n - (x + e0);
+        const bool edge = valid && (lo > 0 || hi < 8);
+        float v[8], t[8];
+        stage_logits(lb, e0, valid, edge, lo, hi, v);
+        if (kind == kJobBonusLeaf) {
+          const float lm = fmaxf(fmaxf(fmaxf(v[0], v[1]), fmaxf(v[2], v[3])),
+                                 fmaxf(fmaxf(v[4], v[5]), fmaxf(v[6], v[7])));
+          const float tm = warp_max(lm);
+          exp8<L, true>(v, tm, c_hi, c_lo, t);
+          zero_outside(edge, lo, hi, t);
+          const float ts = warp_sum(valid ? sum8(t) : 0.f);
+          if (lane == 0) {
+            s.tsum[(x + t0) / kTileElems] = ts;
+            s.tmax[(x + t0) / kTileElems] = tm;
+          }
+          continue;
+        }
+        if (valid) {
+          residual8<L>(v, qb + e0, rm, al, be, c_hi, c_lo, t);
+        } else {
+#pragma unroll
+          for (int e = 0; e < 8; ++e) t[e] = 0.f;
+        }
+        zero_outside(edge, lo, hi, t);
+        if (nmask > 0) {
+          while (mp < nmask && mt[mp] < xg) ++mp;
+          for (int mq = mp; mq < nmask && mt[mq] < xg + kChunk; ++mq) {
+            const int off = mt[mq] - xg;
+            if (!valid || off < lo || off >= hi) continue;   // (another slice's token)
+            const float mv = (kind == kJobPass) ? 0.f : s.mask_val[mq];
+#pragma unroll
+            for (int e = 0; e < 8; ++e) if (e == off) t[e] = mv;
+          }
+        }
+        if (kind == kJobPass) {
+          if (valid) acc.add(sum8(t));
+        } else {
+          const float ts = warp_sum(valid ? sum8(t) : 0.f);
+          if (lane == 0) s.tsum[(x + t0) / kTileElems] = ts;
+        }
+      }
+      if (q + n_stages < total) {              // the producer waits for this stage
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&empty_bar[st]);
+      }
+      if (++st == n_stages) st = 0;
+    }
+    sum = acc.value();
+    return true;
+  }
+
+  __device__ void consumer(int wid, int lane) {
     uint32_t jp = 0u;
     uint32_t ph = 0xffffffffu;                 // parity of each stage's latest fill
     for (;;) {
@@ -356,141 +527,29 @@ struct TreeCta {
       const TreeJob& job = sh.job;
       const int kind = job.kind;
       if (kind == kJobDone) return;
-      const bool pair = is_pair(kind);
-      const int per = pair ? kPair : kRow;
-      const int nrows = kind == kJobStats ? job.n_rows : 1;
-      const int total = job.total, slot = job.slot;
-      const int spc = chunks_of(v1 - v0 + 7, kPair);
-      const int st0 = slot > 0 ? slot * spc : 0;
-      const int nmask = job.nmask;
-      const int pf_node = job.pf_node, pf_slot = job.pf_slot, xb = job.xb;
-      const int* mt = mtok(job.mbuf);
-      const float al = job.alpha1, be = job.beta, rm = job.rowmax;
-      int q = 0;
-      for (int r = 0; r < nrows; ++r) {
-        const int node = kind == kJobStats ? job.rows[r] : job.node;
-        const Slice sl(row0 + node, a.V, v0, v1);
-        const int nch = chunks_of(sl.n, per);
-        float m_run = TV_NEG_INF;
-        Comp acc;
-        int mp = 0;
-        for (int k = 0; k < nch; ++k, ++q) {
-          const int st = st0 + (slot >= 0 ? k : q % n_stages);
-          if (total > 0) ph ^= 1u << st;       // filled by this job
-          if (!mbar_wait_warp(&full_bar[st], (ph >> st) & 1u)) { fail(); return; }
-          const int n = min(per, sl.n - k * per);
-          const char* buf = ring + (size_t)st * kStageBytes;
-          const E* lb = reinterpret_cast<const E*>(buf);
-          const float* qb = reinterpret_cast<const float*>(buf + (size_t)kPair * kLB);
-          for (int t0 = wid * kTileElems; t0 < n; t0 += kSweep) {
-            const int e0 = t0 + lane * kChunk;
-            const bool valid = e0 < n;
-            const int g0 = k * per + e0;       // from the start of the slice's first block
-            const int xg = v0 - sl.sh + g0;    // token of the lane's first element
-            // elements of the lane's block that belong to the slice: [lo, hi)
-            const int lo = sl.sh - g0, hi = sl.n - g0;
-            const bool edge = valid && (lo > 0 || hi < 8);
-            float v[8], t[8];
-            if (valid) {
-              lds_logits<L>(lb + e0, v);
-            } else {
-#pragma unroll
-              for (int e = 0; e < 8; ++e) v[e] = kLB == 2 ? -9984.f : TV_NEG_INF;
-            }
-            if (edge) {
-#pragma unroll
-              for (int e = 0; e < 8; ++e)
-                if (e < lo || e >= hi) v[e] = kLB == 2 ? -9984.f : TV_NEG_INF;
-            }
-            if (kind == kJobStats) {
-              if (valid) {
-                const float cm = fmaxf(fmaxf(fmaxf(v[0], v[1]), fmaxf(v[2], v[3])),
-                                       fmaxf(fmaxf(v[4], v[5]), fmaxf(v[6], v[7])));
-                if (cm > m_run) {
-                  if (m_run != TV_NEG_INF) {
-                    const float sc = L::exp_rel(m_run, cm, c_hi, c_lo);
-                    acc.s *= sc;
-                    acc.c *= sc;
-                  }
-                  m_run = cm;
-                }
-                exp8<L, false>(v, m_run, c_hi, c_lo, t);
-                if (edge) {
-#pragma unroll
-                  for (int e = 0; e < 8; ++e) if (e < lo || e >= hi) t[e] = 0.f;
-                }
-                acc.add(sum8(t));
-              }
-            } else if (kind == kJobBonusLeaf) {
-              const float lm = fmaxf(fmaxf(fmaxf(v[0], v[1]), fmaxf(v[2], v[3])),
-                                     fmaxf(fmaxf(v[4], v[5]), fmaxf(v[6], v[7])));
-              const float tm = warp_max(lm);
-              exp8<L, true>(v, tm, c_hi, c_lo, t);
-              if (edge) {
-#pragma unroll
-                for (int e = 0; e < 8; ++e) if (e < lo || e >= hi) t[e] = 0.f;
-              }
-              const float ts = warp_sum(valid ? sum8(t) : 0.f);
-              if (lane == 0) {
-                const int tile = (k * per + t0) / kTileElems;
-                s.tsum[tile] = ts;
-                s.tmax[tile] = tm;
-              }
-            } else {
-              if (valid) {
-                residual8<L>(v, qb + e0, rm, al, be, c_hi, c_lo, t);
-              } else {
-#pragma unroll
-                for (int e = 0; e < 8; ++e) t[e] = 0.f;
-              }
-              if (edge) {
-#pragma unroll
-                for (int e = 0; e < 8; ++e) if (e < lo || e >= hi) t[e] = 0.f;
-              }
-              while (mp < nmask && mt[mp] < xg) ++mp;
-              for (int mq = mp; mq < nmask && mt[mq] < xg + kChunk; ++mq) {
-                const int off = mt[mq] - xg;
-                if (!valid || off < lo || off >= hi) continue;   // (another slice's token)
-                const float mv = (kind == kJobPass) ? 0.f : s.mask_val[mq];
-#pragma unroll
-                for (int e = 0; e < 8; ++e) if (e == off) t[e] = mv;
-              }
-              if (kind == kJobPass) {
-                if (valid) acc.add(sum8(t));
-              } else {
-                const float ts = warp_sum(valid ? sum8(t) : 0.f);
-                if (lane == 0) s.tsum[(k * per + t0) / kTileElems] = ts;
-              }
-            }
-          }
-          if (q + n_stages < total) {          // the producer waits for this stage
-            __syncwarp();
-            if (lane == 0) mbar_arrive(&empty_bar[st]);
-          }
-        }
-        // ---- this warp's partial of the row, to every CTA's control warp ----
-        if (kind == kJobStats) {
-          const float wm = warp_max(m_run);
-          const float part =
-              (m_run == TV_NEG_INF) ? 0.f : acc.value() * L::exp_rel(m_run, wm, c_hi, c_lo);
-          send(xb, r, (int)rank * NCW + wid, lane, wm, warp_sum(part));
-        } else if (kind == kJobPass) {
-          send(xb, 0, (int)rank * NCW + wid, lane, warp_sum(acc.value()), 0.f);
-        }
-      }
-      if (wid != 0 || kind == kJobStats || kind == kJobPass) arrive_alone(xb, lane);
-      // (a pass's job may have been replaced by now: nothing of it is read below)
-      if (pf_node >= 0) {
-        const int nch = chunks_of(Slice(row0 + pf_node, a.V, v0, v1).n, kPair);
-        ph ^= ((1u << nch) - 1u) << (pf_slot * spc);
-      }
       if (kind == kJobStats) {
-        if (!finish_rows(job, wid, lane)) { fail(); return; }
-      } else if (kind != kJobPass) {
-        __syncwarp();
-        if (lane == 0) mbar_arrive(tile_bar);
-        if (wid == 0 && !draw(job, lane)) { fail(); return; }
+        if (!sum_rows(job, wid, lane, ph) || !finish_rows(job, wid, lane)) { fail(); return; }
+        continue;
       }
+      float sum;
+      if (!pair_or_leaf(job, wid, lane, ph, sum)) { fail(); return; }
+      if (kind == kJobPass) {
+        const int xb = job.xb;
+        if (job.pf_node >= 0) {                // a pair fetched ahead, used by a later job
+          const Slice sl(row0 + job.pf_node, a.V, v0, v1);
+          int st = job.pf_slot * spc;
+          for (int x = 0; x < sl.n; x += kPair, ++st) ph ^= 1u << st;
+        }
+        // once every CTA's control warp has all partials, the job is replaced:
+        // nothing of it is read after this
+        send(xb, (int)rank * NCW + wid, lane, warp_sum(sum), 0.f);
+        arrive_alone(xb, lane);
+        continue;
+      }
+      if (wid != 0) arrive_alone(job.xb, lane);
+      __syncwarp();
+      if (lane == 0) mbar_arrive(tile_bar);
+      if (wid == 0 && !draw(job, lane)) { fail(); return; }
     }
   }
 
@@ -498,10 +557,10 @@ struct TreeCta {
   // order in every CTA), and M_b^(0) of their children.
   __device__ bool finish_rows(const TreeJob& job, int wid, int lane) {
     const float c_hi = a.c_hi, c_lo = a.c_lo;
-    const int n_rows = job.n_rows, n = C * NCW;
+    const int n_rows = job.n_rows, n = C * (NCW / row_groups(n_rows, max_groups));
     if (!exchanged(job.xb, job.xph)) return false;
     for (int r = wid; r < n_rows; r += NCW) {
-      const float2* x = xslots(job.xb, r);
+      const float2* x = xslots(job.xb) + r * n;
       float M = TV_NEG_INF;
       for (int k = lane; k < n; k += 32) M = fmaxf(M, x[k].x);
       M = warp_max(M);
@@ -516,7 +575,7 @@ struct TreeCta {
       int j = s.first[node];
       for (int k = 0; k < lane && j >= 0; ++k) j = s.next[j];
       while (j >= 0) {
-        s.mb0[j] = exp2(((double)s.gl[j] - (double)M) * a.c) * invs;
+        set_child_mass(s, j, M, invs, a.c);
         for (int k = 0; k < 32 && j >= 0; ++k) j = s.next[j];
       }
       if (lane == 0) {
@@ -537,7 +596,6 @@ struct TreeCta {
     const float c_hi = a.c_hi, c_lo = a.c_lo;
     const bool leaf = (job.kind == kJobBonusLeaf);
     const int node = job.node, R = a.N + 1;
-    const float* u = a.uniforms + (size_t)b * (R + 1);
     if (!mbar_wait_warp(tile_bar, 0u)) return false;
     const Slice sl(row0 + node, a.V, v0, v1);
     const int ntl = (sl.n + kTileElems - 1) / kTileElems;
@@ -557,10 +615,10 @@ struct TreeCta {
       Wc += warp_sum(v);
     }
     // every CTA learns every slice's (max, total)
-    send(job.xb, 0, (int)rank, lane, Mc, Wc);
+    send(job.xb, (int)rank, lane, Mc, Wc);
     arrive_alone(job.xb, lane);
     if (!exchanged(job.xb, job.xph)) return false;
-    const float2* x = xslots(job.xb, 0);
+    const float2* x = xslots(job.xb);
     float scale = 1.f, target = 0.f, before = 0.f, W = 0.f;
     int owner = -1;
     float Mg = x[0].x;
@@ -745,12 +803,12 @@ struct TreeCta {
         for (int k = 0; k < n_slots; ++k) sh.slot_node[k] = -1;
         int total = 0;
         if (j.kind == kJobStats) {
-          n_rows = min(j.n_rows, kStatRows);
+          n_rows = min(j.n_rows, min(kStatRows, 4 * max_groups));
           for (int r = 0; r < n_rows; ++r) {
             t.rows[r] = s.job_rows[r];
             total += chunks_of(Slice(row0 + s.job_rows[r], a.V, v0, v1).n, kRow);
           }
-          bytes = (uint32_t)(n_rows * C * NCW) * 8u;
+          bytes = (uint32_t)(n_rows * C * (NCW / row_groups(n_rows, max_groups))) * 8u;
         } else {
           total = chunks_of(Slice(row0 + j.node, a.V, v0, v1).n, kRow);
           bytes = (uint32_t)C * 8u;
@@ -765,10 +823,8 @@ struct TreeCta {
   }
 
   __device__ void control(int lane) {
-    const int R = a.N + 1;
-    const float* u = a.uniforms + (size_t)b * (R + 1);
     // resident row pairs the ring has room for (0: pairs are streamed)
-    const int n_slots = min(n_stages / chunks_of(v1 - v0 + 7, kPair), kTreeMaxSlots);
+    const int n_slots = min(n_stages / spc, kTreeMaxSlots);
     if (lane < kTreeMaxSlots) { sh.slot_node[lane] = -1; sh.slot_used[lane] = 0; }
     __syncwarp();
     Ctl& ctl = sh.ctl;
@@ -780,7 +836,7 @@ struct TreeCta {
       if (ctl.job.kind != kJobDone) advance(s, ctl, u, a.token_level != 0);
       ok = publish(ctl.job, 0, n_slots, xk, jobs) ? 1 : 0;
       ah.ok = 0;
-      if (ctl.job.kind == kJobPass && !a.token_level) prepare_ahead(s, ctl, ah, mtok(mnext));
+      if (!a.token_level) prepare_ahead(s, ctl, ah, mtok(mnext), u);
     }
     for (;;) {
       ++jobs;
@@ -798,70 +854,50 @@ struct TreeCta {
       }
       if (!got) { fail(); return; }
       if (kind == kJobPass) {
-        const float2* x = xslots(xk & 1, 0);
+        const float2* x = xslots(xk & 1);
         for (int k = lane; k < C * NCW; k += 32) S += x[k].x;
         S = warp_sum(S);
       }
       ++xk;
       if (kind == kJobStats) stat_ph ^= 1u;
-      if (lane == 0) {
+      double Sd = 0.0;
+      if (kind == kJobPass && ah.ok && (Sd = (double)S + ah.pm) > 1e-300) {
+        // the next step was worked out while the pass ran: decide, publish, then
+        // update the state (the same values in every lane; 1 / D, 1 / S and S / D
+        // in lanes 0, 1 and 2, since a float64 division takes as long for one lane
+        // as for three)
+        const double D = Sd + ah.omp;
+        double quot = 0.0;
+        const bool early = ah.mode == kAheadTest || ah.mode == kAheadPrune;
+        if (early) quot = (lane == 2 ? Sd : 1.0) / (lane == 1 ? Sd : D);
+        bool accept = false, first = true;
+        if (lane == 0) {
+          Job jf;
+          first = job_ahead(s, ah, Sd, D, quot, jf, accept);
+          if (first) ok = publish(jf, mnext, n_slots, xk, jobs) ? 1 : 0;
+        }
+        __syncwarp();
+        if (!early) quot = (lane == 2 ? Sd : 1.0) / (lane == 1 ? Sd : D);
+        const double inv_s = __shfl_sync(0xffffffffu, quot, 1);
+        const double p_new = __shfl_sync(0xffffffffu, quot, 2);
+        if (lane == 0) {
+          ctl.S = S;
+          control_step_ahead(s, ctl, ah, accept, quot, inv_s, p_new);
+          if (!first) ok = publish(ctl.job, 0, n_slots, xk, jobs) ? 1 : 0;
+          else mnext = 3 - mnext;             // that list is in use now
+          prepare_ahead(s, ctl, ah, mtok(mnext), u);
+        }
+      } else if (lane == 0) {
         if (kind == kJobBonusLeaf || kind == kJobBonusRes) {
           ctl.job.kind = kJobDone;
-          ok = publish(ctl.job, 0, n_slots, xk, jobs) ? 1 : 0;
         } else {
           if (kind == kJobPass) ctl.S = S;
-          bool fast = false;
-          if (kind == kJobPass && ah.ok) {
-            // the next step was worked out while the pass ran: decide, publish,
-            // then update the state
-            const double Sd = (double)S + s.p[ah.i] * ctl.masked_sum;
-            if (Sd > 1e-300) {
-              fast = true;
-              const double D = Sd + ah.omp;
-              Job jf;
-              jf.n_rows = 1;
-              jf.kind = kJobPass;
-              bool accept, first = true;
-              if (ah.mode == 1) {
-                accept = (double)u[ah.c2] * D < ah.X;
-                if (accept) {
-                  jf.kind = kJobBonusLeaf;
-                  jf.node = ah.c2;
-                  jf.nmask = 0;
-                } else {
-                  const double invD = 1.0 / D;
-                  jf.node = ah.i;
-                  jf.nmask = ah.nmask;
-                  jf.alpha1 = (float)(ah.ainvs * invD);
-                  jf.beta = (float)(ah.beta * invD + ah.invZn);
-                  jf.rowmax = s.rowm[ah.i];
-                }
-              } else {
-                accept = (double)u[ah.i] * D < Sd;
-                if (accept) {
-                  first = false;              // the residual draw needs the new state
-                } else {
-                  jf.node = ah.g;
-                  jf.nmask = ah.nmask;
-                  jf.alpha1 = ah.alpha1_g;
-                  jf.beta = ah.beta_g;
-                  jf.rowmax = ah.rowmax_g;
-                }
-              }
-              if (first) ok = publish(jf, mnext, n_slots, xk, jobs) ? 1 : 0;
-              control_step_ahead(s, ctl, ah, accept);
-              if (!first) ok = publish(ctl.job, 0, n_slots, xk, jobs) ? 1 : 0;
-              else mnext = 3 - mnext;         // that list is in use now
-            }
-          }
-          if (!fast) {
-            if (*(volatile uint32_t*)&ctl.bad & (32u | 64u)) ctl.job.kind = kJobDone;
-            else advance(s, ctl, u, a.token_level != 0);
-            ok = publish(ctl.job, 0, n_slots, xk, jobs) ? 1 : 0;
-          }
-          ah.ok = 0;
-          if (ctl.job.kind == kJobPass && !a.token_level) prepare_ahead(s, ctl, ah, mtok(mnext));
+          if (*(volatile uint32_t*)&ctl.bad & (32u | 64u)) ctl.job.kind = kJobDone;
+          else advance(s, ctl, u, a.token_level != 0);
         }
+        ok = publish(ctl.job, 0, n_slots, xk, jobs) ? 1 : 0;
+        ah.ok = 0;
+        if (!a.token_level) prepare_ahead(s, ctl, ah, mtok(mnext), u);
       }
     }
   }
@@ -870,7 +906,6 @@ struct TreeCta {
   __device__ void outputs(int lane) {
     const int R = a.N + 1, N = a.N;
     const Ctl& ctl = sh.ctl;
-    const float* u = a.uniforms + (size_t)b * (R + 1);
     const bool ok = (ctl.bad & (15u | 32u | 64u)) == 0u;
     for (int k = lane; k < N; k += 32) a.out_path[(size_t)b * N + k] = -1;
     if (a.out_node_p)
@@ -935,10 +970,13 @@ __global__ void __launch_bounds__(TreeCta<L, NCW>::kThreads, 16 / NCW)
   t.row0 = (size_t)t.b * R;
   t.ring = smem_raw;
   t.xs = reinterpret_cast<float2*>(smem_raw + (size_t)n_stages * T::kStageBytes);
-  char* tree_base = reinterpret_cast<char*>(t.xs + 2 * (size_t)kStatRows * C * NCW);
+  t.spc = max(1, chunks_of(t.v1 - t.v0 + 7, T::kPair));
+  t.max_groups = max(1, min(NCW, n_stages / max(1, chunks_of(SL + 7, T::kRow))));
+  char* tree_base = reinterpret_cast<char*>(t.xs + 2 * exchange_slots(C, NCW));
   t.s = carve_tree_nt(tree_base, R, tree_tiles(V, C));
   t.mtok_ahead = reinterpret_cast<int*>(
       tree_base + ((tree_smem_bytes_nt(R, tree_tiles(V, C)) + 15) & ~(size_t)15));
+  t.u = reinterpret_cast<float*>(t.mtok_ahead + 2 * R);
   t.full_bar = full_bar;
   t.empty_bar = empty_bar;
   t.xbar = xbar;
@@ -971,6 +1009,8 @@ __global__ void __launch_bounds__(TreeCta<L, NCW>::kThreads, 16 / NCW)
     ctl.n_tests = ctl.n_passes = 0;
     ctl.job.kind = 0;
   }
+  for (int i = tid; i <= R; i += T::kThreads)
+    t.u[i] = args.uniforms[t.row0 + t.b + i];
   for (int i = tid; i < R; i += T::kThreads) {
     s.par[i] = args.parents[t.row0 + i];
     s.tok[i] = args.tokens[t.row0 + i];
@@ -979,8 +1019,6 @@ __global__ void __launch_bounds__(TreeCta<L, NCW>::kThreads, 16 / NCW)
     s.state[i] = kAlive;
     s.a[i] = 1.0;
     s.b[i] = 0.0;
-    s.Z[i] = 1.0;
-    s.invZ[i] = 1.0;
     s.m[i] = 0.0;
     s.p[i] = 0.0;
     s.rows[i] = 0.f;
@@ -1021,16 +1059,20 @@ __global__ void __launch_bounds__(TreeCta<L, NCW>::kThreads, 16 / NCW)
         s.gl[i] = gl;
         s.gq[i] = gq;
         if (!(gq > 0.f)) bad |= 8u;
-        s.invq[i] = 1.0 / (double)gq;
       }
       s.next[i] = nx;
     }
     if (bad) atomicOr(&ctl.bad, bad);
   }
   __syncthreads();
-  if (tid == 0) {
-    if (ctl.bad == 0u) s.p[0] = 1.0;
-    else ctl.job.kind = kJobDone;
+  if (ctl.bad == 0u)
+    for (int i = tid; i < R; i += T::kThreads) children_order(s, i);
+  __syncthreads();
+  if (ctl.bad == 0u) {
+    for (int i = tid + 1; i < R; i += T::kThreads) child_order(s, i);
+    if (tid == 0) s.p[0] = 1.0;
+  } else if (tid == 0) {
+    ctl.job.kind = kJobDone;
   }
   if (C > 1) cluster_sync_all();   // peers' barriers initialised before any remote store
   else __syncthreads();
@@ -1056,8 +1098,8 @@ namespace {
 
 size_t tree_cta_bytes(int ncw, int lb, int C, int stages, int R, int V) {
   using namespace tvk::fused;
-  return (size_t)stages * tree_stage_bytes(ncw, lb) + (size_t)2 * kStatRows * C * ncw * 8 +
-         ((tree_smem_bytes_nt(R, tree_tiles(V, C)) + 15) & ~(size_t)15) + (size_t)R * 8;
+  return (size_t)stages * tree_stage_bytes(ncw, lb) + (size_t)2 * exchange_slots(C, ncw) * 8 +
+         ((tree_smem_bytes_nt(R, tree_tiles(V, C)) + 15) & ~(size_t)15) + (size_t)R * 12 + 4;
 }
 
 // Ring stages that fit when `per_sm` CTAs share an SM's shared memory.
