@@ -73,11 +73,12 @@ enum {
 };
 
 /* Flags for tv_create.  At most one path flag may be given; with none the
-   library picks the path: when V % 8 == 0, the cluster-per-tree kernel for
-   V <= 49152 and N + 1 <= 128 (short rows, where one cluster per tree is
-   faster than publishing every job through the persistent kernel's queue;
-   calls with given row normalisers still run the persistent kernel), else the
-   persistent kernel; the three-kernel path otherwise.  All paths compute the
+   library picks the path for each call: when V % 8 == 0, the cluster-per-tree
+   kernel where trees are few or rows short (a job costs less to exchange
+   inside a cluster than through the persistent kernel's queue: N + 1 <= 128
+   and V <= 28672, or V <= 49152 and B V <= 10.3 million, or B V <= 4.9 million
+   and B < 64, B < 33 above V = 98304), else the persistent kernel; the
+   three-kernel path otherwise.  All paths compute the
    same results; the two single-kernel paths read rows with bulk copies and
    need V % 8 == 0, other vocabularies always take the three-kernel path. */
 enum {
@@ -298,8 +299,8 @@ int tv_draft_children(tv_handle* h, int B, int N, const int32_t* parents,
  * temperature), so no row is streamed to normalise it.  out_node_p and
  * out_stats are optional (NULL) and have the layouts of tv_verify_batch_debug
  * (out_stats[b][4], rows normalised by this call, is then 0).  Runs on the
- * persistent kernel only (a handle that picks its path itself uses it here
- * for every V): handles created for the other paths, and calls on a
+ * persistent kernel, or the cluster kernel where a handle that picks its path
+ * itself takes it: handles created for the other paths, and calls on a
  * capturing stream, return TV_ERR_INVALID_ARG.
  * Errors: those of tv_verify_batch.
  */

@@ -80,26 +80,37 @@ int flow_min_slice(const tv_handle* h) {
   return p.slice_min;
 }
 
-// Largest vocabulary and tree for which a handle that chose its path itself
-// takes the cluster path rather than the persistent kernel.
-constexpr int kClusterMaxVocab = 49152;
+// Whether a handle that chooses its path itself takes the cluster kernel
+// rather than the persistent one.  A job of the persistent kernel costs about
+// 8 us to publish, spread over the grid and combine, one of the cluster kernel
+// 3 to 5 us, while the persistent kernel balances trees over the whole GPU and
+// so streams more bytes a second once there are enough of them.  Measured (us;
+// 60-node trees, bf16; cluster against persistent):
+//   V = 16384: B = 300 232 / 283, B = 1024 500 / 604
+//   V = 32000: B = 1 63 / 108, B = 64 149 / 252, B = 300 313 / 347, B = 400 417 / 391,
+//   B = 1024 756 / 749; V = 49152: B = 256 429 / 373
+//   V = 65536: B = 16 114 / 186, B = 32 134 / 221, B = 64 190 / 236
+//   V = 128256: B = 1 112 / 221, B = 16 144 / 258, B = 32 211 / 283, B = 64 295 / 289
+//   V = 262144: B = 8 134 / 181, B = 24 286 / 281
+//   V = 8000, B = 300 (26 nodes): 117 / 187
 constexpr int kClusterMaxRows = 128;
+
+bool prefer_cluster(int V, int B, int R) {
+  if (R > kClusterMaxRows) return false;
+  if (V <= 49152) return V <= 28672 || (long long)B * V <= 10300000;
+  return (long long)B * V <= 4900000 && B < (V <= 98304 ? 64 : 33);
+}
 
 Path choose_path(const tv_handle* h, int B, int R, FusedPlan* plan) {
   if ((h->vocab % 8) != 0 || (h->flags & TV_FLAG_UNFUSED)) return kPathThree;
   if (h->flags & TV_FLAG_CLUSTER) {
-    *plan = tv_fused_plan(B, R, h->vocab, (int)logit_bytes(h), h->sm_count, h->smem_per_sm, h->smem_per_block,
+    *plan = tv_fused_plan(B, R, h->vocab, (int)logit_bytes(h), h->smem_per_sm, h->smem_per_block,
                           h->force_ncw, h->force_c, h->force_stages);
     return plan->ok ? kPathCluster : kPathThree;
   }
   if (!h->flow_ws || !flow_plan(h, R, B).ok) return kPathThree;
-  if (!(h->flags & TV_FLAG_PERSISTENT) && h->vocab <= kClusterMaxVocab && R <= kClusterMaxRows) {
-    // short rows: a job of the persistent kernel costs more to publish and
-    // combine through its global queue than to stream, and one cluster per
-    // tree, exchanging partials through distributed shared memory, is faster
-    // (V = 32000, EAGLE-shaped trees: 13-22 % less time at 16 to 2048 trees;
-    // the persistent kernel is faster from V = 128256 and on deep trees)
-    *plan = tv_fused_plan(B, R, h->vocab, (int)logit_bytes(h), h->sm_count, h->smem_per_sm, h->smem_per_block,
+  if (!(h->flags & TV_FLAG_PERSISTENT) && prefer_cluster(h->vocab, B, R)) {
+    *plan = tv_fused_plan(B, R, h->vocab, (int)logit_bytes(h), h->smem_per_sm, h->smem_per_block,
                           h->force_ncw, h->force_c, h->force_stages);
     if (plan->ok) return kPathCluster;
   }
@@ -272,19 +283,17 @@ int verify_impl(tv_handle* h, int B, int N, const int32_t* parents, const int32_
     // graph must not replay it: under capture, a handle that chose the path
     // itself uses the cluster path (else the three-kernel one)
     if ((h->flags & TV_FLAG_PERSISTENT) || row_stats) return TV_ERR_INVALID_ARG;
-    plan = tv_fused_plan(B, N + 1, h->vocab, (int)logit_bytes(h), h->sm_count, h->smem_per_sm, h->smem_per_block,
+    plan = tv_fused_plan(B, N + 1, h->vocab, (int)logit_bytes(h), h->smem_per_sm, h->smem_per_block,
                          h->force_ncw, h->force_c, h->force_stages);
     path = plan.ok ? kPathCluster : kPathThree;
   }
-  // given row normalisers are read by the persistent kernel only: a handle
-  // that chose the cluster path itself runs them there
-  if (row_stats && path == kPathCluster && !(h->flags & TV_FLAG_CLUSTER) && h->flow_ws &&
-      flow_plan(h, N + 1, B).ok)
-    path = kPathPersistent;
   // the three-kernel path implements Traversal Verification only
   if (path == kPathThree && a.token_level) return TV_ERR_INVALID_ARG;
-  // given row normalisers are read by the persistent kernel only
-  if (row_stats && path != kPathPersistent) return TV_ERR_INVALID_ARG;
+  // given row normalisers: the persistent kernel, or the cluster kernel where
+  // the handle chose it itself (and neither under capture)
+  if (row_stats && (path == kPathThree || (h->flags & TV_FLAG_CLUSTER) ||
+                    (path == kPathCluster && capturing(st))))
+    return TV_ERR_INVALID_ARG;
   const int bf16 = h->dtype == TV_BF16 ? 1 : 0;
   cudaEvent_t* ev = h->timing ? h->ev : nullptr;
   if (path == kPathCluster) {

@@ -45,7 +45,7 @@ struct FusedPlan {
   bool ok = false;
 };
 
-FusedPlan tv_fused_plan(int B, int R, int V, int logit_bytes, int sm_count, int smem_per_sm,
+FusedPlan tv_fused_plan(int B, int R, int V, int logit_bytes, int smem_per_sm,
                         int smem_per_block, int force_ncw, int force_c, int force_stages);
 
 // Queues the fused kernel (one cluster of plan.C CTAs per tree).  Requires

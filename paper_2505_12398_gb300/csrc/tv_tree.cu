@@ -2,7 +2,7 @@
 // Traversal Verification (sm_103a).
 //
 // One kernel does all of Algorithm 3 (§3.1) for a batch of trees.  Each tree
-// is owned by a cluster of C CTAs: CTA r streams the vocabulary slice
+// is owned by a cluster of C CTAs (1 to 16): CTA r streams the vocabulary slice
 // [v0_r, v1_r) of every row the tree needs, and every CTA runs the same serial
 // control on identical data, so their decisions agree without being broadcast;
 // only partial results cross the cluster.
@@ -934,7 +934,7 @@ struct TreeCta {
       o[1] = ok ? ctl.n_passes : 0;
       o[2] = ok ? distinct : 0;
       o[3] = (acc_node >= 0 && s.first[acc_node] < 0) ? 1 : 0;
-      o[4] = ok ? normalised : 0;
+      o[4] = (ok && !a.row_stats) ? normalised : 0;   // rows this call streamed
     }
     if (a.out_margin) {
       // the bonus margin was written by the CTA that drew the bonus
@@ -1070,12 +1070,38 @@ __global__ void __launch_bounds__(TreeCta<L, NCW>::kThreads, 16 / NCW)
   __syncthreads();
   if (ctl.bad == 0u) {
     for (int i = tid + 1; i < R; i += T::kThreads) child_order(s, i);
+    if (args.row_stats) {
+      // given normalisers (from the LM head's epilogue): every internal row is
+      // normalised up front and no normaliser job is ever posted
+      uint32_t bad = 0u;
+      for (int i = tid; i < R; i += T::kThreads) {
+        if (s.first[i] < 0) continue;
+        const float2 st = args.row_stats[t.row0 + i];
+        const double invs = 1.0 / (double)st.y;
+        s.rowm[i] = st.x;
+        s.rows[i] = st.y;
+        s.invs[i] = invs;
+        if (!(st.y > 0.f)) bad |= 64u;
+      }
+      if (bad) atomicOr(&ctl.bad, bad);
+    }
     if (tid == 0) s.p[0] = 1.0;
   } else if (tid == 0) {
     ctl.job.kind = kJobDone;
   }
   if (C > 1) cluster_sync_all();   // peers' barriers initialised before any remote store
   else __syncthreads();
+  if (args.row_stats) {
+    const uint32_t bad = ctl.bad;
+    __syncthreads();
+    if (bad == 0u) {
+      for (int i = tid + 1; i < R; i += T::kThreads)
+        set_child_mass(s, i, s.rowm[s.par[i]], s.invs[s.par[i]], args.c);
+    } else if (tid == 0) {
+      ctl.job.kind = kJobDone;
+    }
+    __syncthreads();
+  }
 
   if (wid < NCW) {
     t.consumer(wid, lane);
@@ -1116,19 +1142,32 @@ int stages_for(int ncw, int lb, int C, int per_sm, int R, int V, int smem_per_sm
 
 }  // namespace
 
-FusedPlan tv_fused_plan(int B, int R, int V, int logit_bytes, int sm_count, int smem_per_sm,
+FusedPlan tv_fused_plan(int B, int R, int V, int logit_bytes, int smem_per_sm,
                         int smem_per_block, int force_ncw, int force_c, int force_stages) {
   using namespace tvk::fused;
   FusedPlan p;
-  // Large batches fill the GPU with one CTA of 8 consumer warps per tree; smaller
-  // ones use CTAs of 4 consumer warps (four per SM) and clusters that split a
-  // tree's vocabulary across up to 8 SMs, as many as fit in one wave, keeping
-  // every CTA's slice at least 2048 tokens.
-  int ncw = (B >= 2 * sm_count) ? 8 : 4;
+  // Few trees: as many SMs per tree as keep all trees in one wave (152 SMs, two
+  // CTAs of 8 consumer warps or one of 16 on each; clusters do not cross a GPC,
+  // so about 8 clusters of 16 whole SMs fit), down to slices of 1000 tokens, below
+  // which a job is all latency.  Measured (us; 60-node trees; ncw x C):
+  //   V = 128256, B = 1: 16x16 112, 8x16 118, 16x8 132, 8x8 151, 4x8 212
+  //   V = 128256, B = 16: 8x16 144, 16x8 160, 8x8 188, 16x16 218, 4x8 267
+  //   V = 128256, B = 32: 8x8 211, 16x4 236, 8x16 288, 4x8 288
+  //   V = 32000, B = 1: 8x16 63, 8x8 65, 4x8 71; B = 16: 8x8 120, 4x8 124, 8x16 143
+  //   V = 32000, B = 64: 8x4 149, 4x8 154, 8x8 160; B = 128: 8x4 212, 4x4 218, 8x2 225
+  //   V = 32000, B = 256: 8x2 298, 4x2 300, 8x1 320, 8x4 344; B = 300: 8x2 313, 8x1 356
+  //   V = 16384, B = 300: 4x2 227, 8x1 232, 8x2 244; B = 1024: 8x1 500, 4x2 532, 8x2 607
+  //   V = 1000, B = 1024 (26 nodes): 4x1 213, 8x1 280
+  int ncw = 8, C = 1;
+  if (V > 98304 && B <= 4) ncw = 16, C = 16;
+  else if (B <= 8 || (V > 98304 && B <= 16)) C = 16;
+  else if (B <= 32) C = 8;
+  else if (B <= 128) C = 4;
+  else if (B <= 256 || (B <= 320 && V > 20000)) C = 2;
+  else if (V <= 4096) ncw = 4;
+  while (C > 1 && V / C < 1000) C /= 2;
   if (force_ncw == 4 || force_ncw == 8 || force_ncw == 16) ncw = force_ncw;
   int per_sm = 16 / ncw;
-  int C = 1;
-  while (C < 8 && (long)B * (2 * C) <= (long)sm_count * per_sm && V / (2 * C) >= 2048) C *= 2;
   if (force_c == 1 || force_c == 2 || force_c == 4 || force_c == 8 || force_c == 16) C = force_c;
   int stages = stages_for(ncw, logit_bytes, C, per_sm, R, V, smem_per_sm, smem_per_block);
   while (stages < 3 && per_sm > 1) {
