@@ -254,7 +254,7 @@ int tv_last_host_copy_bytes(tv_handle* h, uint64_t* h2d, uint64_t* d2h);
  *   out_logits     [M][V] bf16, 16-byte aligned.
  *   out_row_stats  [M][2] fp32 (max, sum), 8-byte aligned.
  * The handle must have been created for bf16 logits with V % 8 == 0.  The
- * first call allocates the handle's per-(row, 256-column tile) scratch for
+ * first call allocates the handle's per-(row, column tile) scratch for
  * max_batch * (max_nodes + 1) rows (a later call with a larger vocabulary
  * cannot happen: V is the handle's).
  * Errors: TV_ERR_INVALID_ARG, TV_ERR_CAPACITY, TV_ERR_TEMPERATURE, TV_ERR_CUDA.

@@ -620,7 +620,7 @@ int tv_lm_head(tv_handle* h, int M, int K, const void* hidden, const void* weigh
   DeviceGuard guard(h->device);
   if (!guard.ok()) return TV_ERR_CUDA;
   const size_t need = (size_t)h->max_batch * (h->max_nodes + 1) *
-                      (size_t)tv_lm_head_tiles(h->vocab) * sizeof(float2);
+                      (size_t)tv_lm_head_parts(h->vocab) * sizeof(float2);
   if (h->lmh_part_bytes < need) {
     if (h->lmh_part) cudaFree(h->lmh_part);
     h->lmh_part = nullptr;

@@ -125,11 +125,11 @@ int tv_launch_flow(const TravArgs& a, FlowArgs f, int logit_is_bf16, const FlowP
 
 // ---- LM head fused with the row normalisers (tv_gemm.cu) ----
 
-// Tiles of 256 logits per row (the per-row workspace of tv_launch_lm_head).
-int tv_lm_head_tiles(int V);
+// Partial normalisers per row at most (the per-row workspace of tv_launch_lm_head).
+int tv_lm_head_parts(int V);
 // logits[M][V] (bf16) = hidden[M][K] x weight[V][K]^T (bf16) on the tensor
 // cores, and row_stats[M] = (max, sum of 2^((l - max) (c_hi + c_lo))) of the
-// stored logits.  part is [M][tv_lm_head_tiles(V)] scratch.  Requires K % 64
+// stored logits.  part is [M][tv_lm_head_parts(V)] scratch.  Requires K % 64
 // == 0, V % 8 == 0 and 16-byte aligned arrays.  0 on success, -5 on a CUDA
 // or tensor-map error.
 int tv_launch_lm_head(const void* hidden, const void* weight, int M, int K, int V, float c_hi,

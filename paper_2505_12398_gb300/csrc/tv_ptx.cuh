@@ -1,5 +1,5 @@
-// tv_ptx.cuh -- inline-PTX wrappers: mbarriers, 1-D TMA bulk copies, named
-// barriers and distributed shared memory inside a thread-block cluster.
+// tv_ptx.cuh -- inline-PTX wrappers: mbarriers, 1-D TMA bulk copies and
+// distributed shared memory inside a thread-block cluster.
 //
 // Every wait is bounded: try_wait is polled at most kSpinLimit times, each
 // try suspending at most kTrySuspendNs, and the caller turns a timeout into an
@@ -88,11 +88,6 @@ __device__ __forceinline__ void tma_load_1d(void* dst, const void* src, uint32_t
       : "memory");
 }
 
-// Named barrier among `count` threads (a multiple of 32).
-__device__ __forceinline__ void named_sync(uint32_t id, uint32_t count) {
-  asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(count) : "memory");
-}
-
 __device__ __forceinline__ uint32_t cluster_rank() {
   uint32_t r;
   asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
@@ -106,13 +101,8 @@ __device__ __forceinline__ uint32_t map_shared(const void* p, uint32_t rank) {
   return r;
 }
 
-__device__ __forceinline__ void st_cluster_v2(uint32_t addr, float a, float b) {
-  asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(addr), "f"(a), "f"(b)
-               : "memory");
-}
-
-__device__ __forceinline__ void st_cluster_s32(uint32_t addr, int v) {
-  asm volatile("st.shared::cluster.s32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
+__device__ __forceinline__ void st_cluster_f32(uint32_t addr, float v) {
+  asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(addr), "f"(v) : "memory");
 }
 
 // Arrive on an mbarrier of a peer CTA (address from map_shared), releasing
