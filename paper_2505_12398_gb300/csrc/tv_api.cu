@@ -646,7 +646,7 @@ int tv_draft_children(tv_handle* h, int B, int N, const int32_t* parents,
   NvtxRange range("tv_draft_children");
   if (!h || B < 0 || N < 0) return TV_ERR_INVALID_ARG;
   if (B > h->max_batch || N > h->max_nodes) return TV_ERR_CAPACITY;
-  if (tv_draft_smem_bytes(N, h->vocab) > 48u * 1024u) return TV_ERR_VOCAB;
+  if (!tv_draft_fits(N, h->vocab)) return TV_ERR_VOCAB;
   if (B == 0) return TV_OK;
   if (!parents || !draft_probs || !uniforms || !out_tokens ||
       (reinterpret_cast<uintptr_t>(draft_probs) & 3u))
@@ -654,7 +654,8 @@ int tv_draft_children(tv_handle* h, int B, int N, const int32_t* parents,
   DeviceGuard guard(h->device);
   if (!guard.ok()) return TV_ERR_CUDA;
   const int rc = tv_launch_draft(parents, draft_probs, uniforms, out_tokens, B, N, h->vocab,
-                                 h->status, static_cast<cudaStream_t>(cuda_stream));
+                                 h->sm_count, h->status,
+                                 static_cast<cudaStream_t>(cuda_stream));
   return rc == 0 ? TV_OK : TV_ERR_CUDA;
 }
 
