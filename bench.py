@@ -471,7 +471,7 @@ def main():
     peak, peak_kind = measured_peaks()
     ph = [sum(p[i] for p in phase) / len(phase) for i in range(3)]
     if path_code == 0:
-        names = ["tv_prep_kernel", "tv_row_stats_kernel", "tv_traverse_kernel"]
+        names = ["tv_prep_kernel", "tv_row_stats_kernel", "tv_tree_kernel"]
         kbytes = [0, row_bytes, trav_bytes]
         launches_per_step = 3
     else:

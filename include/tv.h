@@ -83,8 +83,8 @@ enum {
    need V % 8 == 0, other vocabularies always take the three-kernel path. */
 enum {
   TV_FLAG_NONE = 0u,
-  /* Three kernels: row normalisers of every internal row, then one CTA per
-     tree. */
+  /* Three kernels: internal rows listed, row normalisers of every one, then
+     the traversal by one thread-block cluster per tree. */
   TV_FLAG_UNFUSED = 1u,
   /* One kernel, one thread-block cluster per tree (rows read lazily, the
      vocabulary split across the cluster's CTAs). */

@@ -101,19 +101,16 @@ bool prefer_cluster(int V, int B, int R) {
   return (long long)B * V <= 4900000 && B < (V <= 98304 ? 64 : 33);
 }
 
+// The path of a call, and the cluster kernel's plan (also for the three-kernel
+// path, whose last kernel it is).
 Path choose_path(const tv_handle* h, int B, int R, FusedPlan* plan) {
+  *plan = tv_fused_plan(B, R, h->vocab, (int)logit_bytes(h), h->smem_per_sm, h->smem_per_block,
+                        h->force_ncw, h->force_c, h->force_stages);
   if ((h->vocab % 8) != 0 || (h->flags & TV_FLAG_UNFUSED)) return kPathThree;
-  if (h->flags & TV_FLAG_CLUSTER) {
-    *plan = tv_fused_plan(B, R, h->vocab, (int)logit_bytes(h), h->smem_per_sm, h->smem_per_block,
-                          h->force_ncw, h->force_c, h->force_stages);
-    return plan->ok ? kPathCluster : kPathThree;
-  }
+  if (h->flags & TV_FLAG_CLUSTER) return plan->ok ? kPathCluster : kPathThree;
   if (!h->flow_ws || !flow_plan(h, R, B).ok) return kPathThree;
-  if (!(h->flags & TV_FLAG_PERSISTENT) && prefer_cluster(h->vocab, B, R)) {
-    *plan = tv_fused_plan(B, R, h->vocab, (int)logit_bytes(h), h->smem_per_sm, h->smem_per_block,
-                          h->force_ncw, h->force_c, h->force_stages);
-    if (plan->ok) return kPathCluster;
-  }
+  if (!(h->flags & TV_FLAG_PERSISTENT) && plan->ok && prefer_cluster(h->vocab, B, R))
+    return kPathCluster;
   return kPathPersistent;
 }
 
@@ -271,6 +268,8 @@ int verify_impl(tv_handle* h, int B, int N, const int32_t* parents, const int32_
   a.status = h->status;
   a.token_level = (h->flags & TV_FLAG_TOKEN_LEVEL) ? 1 : 0;
   a.row_stats = row_stats;
+  a.stats_given = row_stats ? 1 : 0;
+  a.exact_exp = 0;
   const int rows = B * (N + 1);
   int grid = h->sm_count * 4;
   if (grid > rows) grid = rows;
@@ -283,8 +282,6 @@ int verify_impl(tv_handle* h, int B, int N, const int32_t* parents, const int32_
     // graph must not replay it: under capture, a handle that chose the path
     // itself uses the cluster path (else the three-kernel one)
     if ((h->flags & TV_FLAG_PERSISTENT) || row_stats) return TV_ERR_INVALID_ARG;
-    plan = tv_fused_plan(B, N + 1, h->vocab, (int)logit_bytes(h), h->smem_per_sm, h->smem_per_block,
-                         h->force_ncw, h->force_c, h->force_stages);
     path = plan.ok ? kPathCluster : kPathThree;
   }
   // the three-kernel path implements Traversal Verification only
@@ -308,7 +305,7 @@ int verify_impl(tv_handle* h, int B, int N, const int32_t* parents, const int32_
     h->withhold_tree = -1;
     rc = tv_launch_flow(a, f, bf16, fp, h->sm_count, st, ev);
   } else {
-    rc = tv_launch_all(a, bf16, h->row_list, h->n_rows, grid, st, ev);
+    rc = tv_launch_all(a, bf16, h->row_list, h->n_rows, grid, plan, st, ev);
   }
   if (rc == TV_OK && h->timing) h->timed_call = true;
   return rc;
@@ -339,8 +336,7 @@ int tv_create(tv_handle** out, int device, int vocab, int max_nodes, int max_bat
   cudaDeviceProp prop;
   if (cudaGetDeviceProperties(&prop, device) != cudaSuccess) return TV_ERR_CUDA;
   if (prop.major < 10) return TV_ERR_DEVICE;
-  const size_t smem = tv_traverse_smem_bytes(max_nodes + 1, vocab);
-  if (smem > static_cast<size_t>(prop.sharedMemPerBlockOptin)) return TV_ERR_VOCAB;
+  if (!tv_tree_fits(max_nodes + 1, vocab, prop.sharedMemPerBlockOptin)) return TV_ERR_VOCAB;
 
   tv_handle* h = new (std::nothrow) tv_handle;
   if (!h) return TV_ERR_CUDA;

@@ -23,8 +23,10 @@ struct TravArgs {
   float* out_margin;           // [B][2] decision margins (test, bonus) or nullptr
   uint32_t* status;            // status word (OR of TV_STATUS_* bits)
   int token_level;             // 1: token-level (top-down) verification instead (fused paths)
-  const float2* row_stats;     // [B][N+1] given row normalisers (max, sum), or nullptr
-                               // (persistent path)
+  const float2* row_stats;     // [B][N+1] row normalisers (max, sum) computed before the
+                               // traversal, or nullptr (it normalises rows as it reaches them)
+  int stats_given;             // 1: row_stats come from the caller (no row counted as normalised)
+  int exact_exp;               // 1: cluster kernel: passes and draws with exp_rel, not exp_pass
 };
 
 // The bonus draws at accepted original leaves, one CTA per entry of pending
@@ -48,20 +50,26 @@ struct FusedPlan {
 FusedPlan tv_fused_plan(int B, int R, int V, int logit_bytes, int smem_per_sm,
                         int smem_per_block, int force_ncw, int force_c, int force_stages);
 
-// Queues the fused kernel (one cluster of plan.C CTAs per tree).  Requires
-// V % 8 == 0 (16-byte aligned rows for the bulk copies).  With `events`,
-// events[0..2] are recorded before and events[3] after it.
+// Queues the fused kernel (one cluster of plan.C CTAs per tree; any V).  With
+// `events`, events[0..2] are recorded before and events[3] after it.
 int tv_launch_fused(const TravArgs& a, int logit_is_bf16, const FusedPlan& plan,
                     cudaStream_t stream, cudaEvent_t* events);
 
-// Dynamic shared memory the traversal kernel needs for R = N+1 rows.
-size_t tv_traverse_smem_bytes(int R, int V);
+// Queues the cluster kernel alone.  0 or -5 (launch failed).
+int tv_launch_tree(const TravArgs& a, int logit_is_bf16, const FusedPlan& plan,
+                   cudaStream_t stream);
 
-// Queues the three kernels on `stream`; 0 on success, TV_ERR_CUDA otherwise.
-// With `events` non-null, events[0..3] are recorded before the first kernel,
-// between the kernels and after the last one.
+// Whether trees of R = N+1 rows of V tokens are small enough for a device whose
+// blocks may use smem_per_block bytes of shared memory.
+bool tv_tree_fits(int R, int V, size_t smem_per_block);
+
+// Queues the three kernels on `stream` (the traversal with the cluster kernel's
+// `plan`); 0 on success, TV_ERR_CUDA otherwise.  With `events` non-null,
+// events[0..3] are recorded before the first kernel, between the kernels and
+// after the last one.
 int tv_launch_all(const TravArgs& a, int logit_is_bf16, int* row_list, int* n_rows,
-                  int stats_grid, cudaStream_t stream, cudaEvent_t* events);
+                  int stats_grid, const FusedPlan& plan, cudaStream_t stream,
+                  cudaEvent_t* events);
 
 // ---- persistent load-balanced kernel (tv_flow.cu) ----
 

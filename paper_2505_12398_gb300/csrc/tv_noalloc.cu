@@ -48,6 +48,7 @@ std::mutex g_setup_mutex;
 void* g_scratch_addr[kMaxDevices] = {};
 int g_sm_count[kMaxDevices] = {};
 int g_smem_optin[kMaxDevices] = {};
+int g_smem_sm[kMaxDevices] = {};
 
 // Once per device, with that device current: the array's device address and
 // the two device properties the launch needs.
@@ -59,9 +60,11 @@ int setup_device(int device) {
     cudaGetLastError();
     return TV_ERR_CUDA;
   }
-  int sms = 0, smem = 0, major = 0;
+  int sms = 0, smem = 0, smem_sm = 0, major = 0;
   if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess ||
       cudaDeviceGetAttribute(&smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, device) !=
+          cudaSuccess ||
+      cudaDeviceGetAttribute(&smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, device) !=
           cudaSuccess ||
       cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, device) != cudaSuccess) {
     cudaGetLastError();
@@ -70,6 +73,7 @@ int setup_device(int device) {
   if (major < 10) return TV_ERR_DEVICE;
   g_sm_count[device] = sms;
   g_smem_optin[device] = smem;
+  g_smem_sm[device] = smem_sm;
   g_scratch_addr[device] = ptr;
   return TV_OK;
 }
@@ -106,7 +110,7 @@ extern "C" int tv_verify_batch_noalloc(int device, int B, int N, int vocab, tv_d
     return TV_ERR_CUDA;
   }
   int rc = setup_device(device);
-  if (rc == TV_OK && tv_traverse_smem_bytes(N + 1, vocab) > (size_t)g_smem_optin[device])
+  if (rc == TV_OK && !tv_tree_fits(N + 1, vocab, (size_t)g_smem_optin[device]))
     rc = TV_ERR_VOCAB;
   if (rc == TV_OK) {
     unsigned char* base = static_cast<unsigned char*>(g_scratch_addr[device]);
@@ -142,11 +146,16 @@ extern "C" int tv_verify_batch_noalloc(int device, int B, int N, int vocab, tv_d
       a.status = status;
       a.token_level = 0;
       a.row_stats = nullptr;
+      a.stats_given = 0;
+      a.exact_exp = 0;
       const int rows = B * (N + 1);
       int grid = g_sm_count[device] * 4;
       if (grid > rows) grid = rows;
       if (grid < 1) grid = 1;
-      rc = tv_launch_all(a, logit_dtype == TV_BF16 ? 1 : 0, row_list, n_rows, grid, st, nullptr);
+      const FusedPlan plan = tv_fused_plan(B, N + 1, vocab, logit_dtype == TV_BF16 ? 2 : 4,
+                                           g_smem_sm[device], g_smem_optin[device], 0, 0, 0);
+      rc = tv_launch_all(a, logit_dtype == TV_BF16 ? 1 : 0, row_list, n_rows, grid, plan, st,
+                         nullptr);
     }
   }
   if (prev != device) cudaSetDevice(prev);

@@ -36,7 +36,8 @@
 //
 // Rows need no alignment: slices are copied as whole 8-element blocks of the
 // flat [B][N+1][V] arrays and the elements of the neighbouring rows in the
-// first and last block are masked.  (Handles use this kernel for V % 8 == 0.)
+// first and last block are masked.  (With V % 8 != 0 the kernel runs as the last
+// of the three-kernel path, with the row normalisers that path computes first.)
 //
 // Every wait is bounded; one that gives up raises TV_STATUS_TIMEOUT, and all
 // roles still reach the cluster barrier at the end.
@@ -172,17 +173,30 @@ __device__ __forceinline__ void exp8(const float v[8], float m, float c_hi, floa
   }
 }
 
+// e(x) in passes and draws: the cheaper form, or (the three-kernel path, whose
+// normalisers come from exp_rel) the other one.
+template <typename L>
+__device__ __forceinline__ void exp8_pass(const float v[8], float m, bool exact, float c_hi,
+                                          float c_lo, float e[8]) {
+  if (L::kBytes == 2 && exact) exp8<L, false>(v, m, c_hi, c_lo, e);
+  else exp8<L, true>(v, m, c_hi, c_lo, e);
+}
+template <typename L>
+__device__ __forceinline__ float exp1_pass(float v, float m, bool exact, float c_hi, float c_lo) {
+  return exact ? L::exp_rel(v, m, c_hi, c_lo) : L::exp_pass(v, m, c_hi, c_lo);
+}
+
 // [alpha e(x) - beta q(x)]_+ of eight tokens.
 template <typename L>
 __device__ __forceinline__ void residual8(const float v[8], const float* qp, float rowmax,
-                                          float alpha, float beta, float c_hi, float c_lo,
-                                          float t[8]) {
+                                          float alpha, float beta, bool exact, float c_hi,
+                                          float c_lo, float t[8]) {
   const uint4 qa = lds128(qp), qc = lds128(qp + 4);
   const float q[8] = {__uint_as_float(qa.x), __uint_as_float(qa.y), __uint_as_float(qa.z),
                       __uint_as_float(qa.w), __uint_as_float(qc.x), __uint_as_float(qc.y),
                       __uint_as_float(qc.z), __uint_as_float(qc.w)};
   float e[8];
-  exp8<L, true>(v, rowmax, c_hi, c_lo, e);
+  exp8_pass<L>(v, rowmax, exact, c_hi, c_lo, e);
   if constexpr (L::kBytes == 2) {
     const float2 al2 = make_float2(alpha, alpha), nb2 = make_float2(-beta, -beta);
 #pragma unroll
@@ -448,7 +462,7 @@ struct TreeCta {
   __device__ bool pair_or_leaf(const TreeJob& job, int wid, int lane, uint32_t& ph, float& sum) {
     const float c_hi = a.c_hi, c_lo = a.c_lo;
     const int kind = job.kind, total = job.total;
-    const bool pair = is_pair(kind);
+    const bool pair = is_pair(kind), exact = a.exact_exp != 0;
     const int per = pair ? kPair : kRow;
     const int nmask = job.nmask;
     const int* mt = mtok(job.mbuf);
@@ -475,7 +489,7 @@ struct TreeCta {
           const float lm = fmaxf(fmaxf(fmaxf(v[0], v[1]), fmaxf(v[2], v[3])),
                                  fmaxf(fmaxf(v[4], v[5]), fmaxf(v[6], v[7])));
           const float tm = warp_max(lm);
-          exp8<L, true>(v, tm, c_hi, c_lo, t);
+          exp8_pass<L>(v, tm, exact, c_hi, c_lo, t);
           zero_outside(edge, lo, hi, t);
           const float ts = warp_sum(valid ? sum8(t) : 0.f);
           if (lane == 0) {
@@ -485,7 +499,7 @@ struct TreeCta {
           continue;
         }
         if (valid) {
-          residual8<L>(v, qb + e0, rm, al, be, c_hi, c_lo, t);
+          residual8<L>(v, qb + e0, rm, al, be, exact, c_hi, c_lo, t);
         } else {
 #pragma unroll
           for (int e = 0; e < 8; ++e) t[e] = 0.f;
@@ -682,7 +696,8 @@ struct TreeCta {
       if (leaf) {
 #pragma unroll
         for (int e = 0; e < 8; ++e)
-          w[e] = (v[e] == TV_NEG_INF) ? 0.f : L::exp_pass(v[e], Mc, c_hi, c_lo);
+          w[e] = (v[e] == TV_NEG_INF) ? 0.f
+                                      : exp1_pass<L>(v[e], Mc, a.exact_exp != 0, c_hi, c_lo);
       } else {
         float qv[8];
         block_probs(a.draft_probs + at, lo, hi, qv);
@@ -690,7 +705,8 @@ struct TreeCta {
         for (int e = 0; e < 8; ++e)
           w[e] = (v[e] == TV_NEG_INF)
                      ? 0.f
-                     : fmaxf(fmaf(job.alpha1, L::exp_pass(v[e], job.rowmax, c_hi, c_lo),
+                     : fmaxf(fmaf(job.alpha1,
+                                  exp1_pass<L>(v[e], job.rowmax, a.exact_exp != 0, c_hi, c_lo),
                                   -job.beta * qv[e]), 0.f);
         const int* mt = mtok(job.mbuf);
         for (int mq = 0; mq < job.nmask; ++mq) {
@@ -934,7 +950,7 @@ struct TreeCta {
       o[1] = ok ? ctl.n_passes : 0;
       o[2] = ok ? distinct : 0;
       o[3] = (acc_node >= 0 && s.first[acc_node] < 0) ? 1 : 0;
-      o[4] = (ok && !a.row_stats) ? normalised : 0;   // rows this call streamed
+      o[4] = (ok && !a.stats_given) ? normalised : 0;   // rows this call streamed
     }
     if (a.out_margin) {
       // the bonus margin was written by the CTA that drew the bonus
@@ -1071,8 +1087,9 @@ __global__ void __launch_bounds__(TreeCta<L, NCW>::kThreads, 16 / NCW)
   if (ctl.bad == 0u) {
     for (int i = tid + 1; i < R; i += T::kThreads) child_order(s, i);
     if (args.row_stats) {
-      // given normalisers (from the LM head's epilogue): every internal row is
-      // normalised up front and no normaliser job is ever posted
+      // given normalisers (from the LM head's epilogue, or the three-kernel
+      // path's): every internal row is normalised up front and no normaliser
+      // job is ever posted
       uint32_t bad = 0u;
       for (int i = tid; i < R; i += T::kThreads) {
         if (s.first[i] < 0) continue;
@@ -1166,6 +1183,7 @@ FusedPlan tv_fused_plan(int B, int R, int V, int logit_bytes, int smem_per_sm,
   else if (B <= 256 || (B <= 320 && V > 20000)) C = 2;
   else if (V <= 4096) ncw = 4;
   while (C > 1 && V / C < 1000) C /= 2;
+  while (C < 8 && tree_tiles(V, C) * 8 > 32768) C *= 2;   // bonus tiles' shared memory
   if (force_ncw == 4 || force_ncw == 8 || force_ncw == 16) ncw = force_ncw;
   int per_sm = 16 / ncw;
   if (force_c == 1 || force_c == 2 || force_c == 4 || force_c == 8 || force_c == 16) C = force_c;
@@ -1219,6 +1237,15 @@ cudaError_t launch_ncw(const TravArgs& a, const FusedPlan& plan, cudaStream_t st
 
 }  // namespace
 
+int tv_launch_tree(const TravArgs& a, int logit_is_bf16, const FusedPlan& plan,
+                   cudaStream_t stream) {
+  const cudaError_t e = logit_is_bf16 ? launch_ncw<tvk::Bf16Logits>(a, plan, stream)
+                                      : launch_ncw<tvk::F32Logits>(a, plan, stream);
+  if (e == cudaSuccess) return 0;
+  cudaGetLastError();
+  return -5;
+}
+
 int tv_launch_fused(const TravArgs& a, int logit_is_bf16, const FusedPlan& plan,
                     cudaStream_t stream, cudaEvent_t* ev) {
   if (!plan.ok) return -3;
@@ -1226,12 +1253,7 @@ int tv_launch_fused(const TravArgs& a, int logit_is_bf16, const FusedPlan& plan,
     for (int k = 0; k < 3; ++k)
       if (cudaEventRecord(ev[k], stream) != cudaSuccess) return -5;
   }
-  const cudaError_t e = logit_is_bf16 ? launch_ncw<tvk::Bf16Logits>(a, plan, stream)
-                                      : launch_ncw<tvk::F32Logits>(a, plan, stream);
-  if (e != cudaSuccess) {
-    cudaGetLastError();
-    return -5;
-  }
+  if (tv_launch_tree(a, logit_is_bf16, plan, stream) != 0) return -5;
   if (ev && cudaEventRecord(ev[3], stream) != cudaSuccess) return -5;
   return 0;
 }
