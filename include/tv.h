@@ -76,9 +76,8 @@ enum {
    library picks the path for each call: when V % 8 == 0, the cluster-per-tree
    kernel where trees are few or rows short (a job costs less to exchange
    inside a cluster than through the persistent kernel's queue: N + 1 <= 128
-   and V <= 28672, or V <= 49152 and B V <= 10.3 million, or B V <= 4.9 million
-   and B < 64, B < 33 above V = 98304), else the persistent kernel; the
-   three-kernel path otherwise.  All paths compute the
+   and V <= 32768, or V <= 49152 and B V <= 14 million, or B < 64 and B V <= 8.4
+   million), else the persistent kernel; the three-kernel path otherwise.  All paths compute the
    same results; the two single-kernel paths read rows with bulk copies and
    need V % 8 == 0, other vocabularies always take the three-kernel path. */
 enum {

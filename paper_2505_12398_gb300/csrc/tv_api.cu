@@ -83,22 +83,23 @@ int flow_min_slice(const tv_handle* h) {
 // Whether a handle that chooses its path itself takes the cluster kernel
 // rather than the persistent one.  A job of the persistent kernel costs about
 // 8 us to publish, spread over the grid and combine, one of the cluster kernel
-// 3 to 5 us, while the persistent kernel balances trees over the whole GPU and
+// 3 to 4 us, while the persistent kernel balances trees over the whole GPU and
 // so streams more bytes a second once there are enough of them.  Measured (us;
 // 60-node trees, bf16; cluster against persistent):
-//   V = 16384: B = 300 232 / 283, B = 1024 500 / 604
-//   V = 32000: B = 1 63 / 108, B = 64 149 / 252, B = 300 313 / 347, B = 400 417 / 391,
-//   B = 1024 756 / 749; V = 49152: B = 256 429 / 373
-//   V = 65536: B = 16 114 / 186, B = 32 134 / 221, B = 64 190 / 236
-//   V = 128256: B = 1 112 / 221, B = 16 144 / 258, B = 32 211 / 283, B = 64 295 / 289
-//   V = 262144: B = 8 134 / 181, B = 24 286 / 281
-//   V = 8000, B = 300 (26 nodes): 117 / 187
+//   V = 32000: B = 1 63 / 106, B = 64 143 / 250, B = 128 192 / 281, B = 400 377 / 387,
+//   B = 1024 651 / 725; V = 49152, B = 256: 365 / 376
+//   V = 65536: B = 16 100 / 186, B = 32 133 / 221
+//   V = 128256: B = 1 81 / 163, B = 16 140 / 215, B = 32 142 / 228, B = 48 218 / 263,
+//   B = 128 419 / 376
+//   V = 151936: B = 128 395 / 355, B = 1024 2155 / 1796
+//   V = 262144: B = 32 255 / 342
 constexpr int kClusterMaxRows = 128;
 
 bool prefer_cluster(int V, int B, int R) {
   if (R > kClusterMaxRows) return false;
-  if (V <= 49152) return V <= 28672 || (long long)B * V <= 10300000;
-  return (long long)B * V <= 4900000 && B < (V <= 98304 ? 64 : 33);
+  if (V <= 32768) return true;
+  if (V <= 49152) return (long long)B * V <= 14000000;
+  return B < 64 && (long long)B * V <= 8400000;
 }
 
 // The path of a call, and the cluster kernel's plan (also for the three-kernel

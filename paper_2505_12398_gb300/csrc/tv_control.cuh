@@ -158,12 +158,11 @@ __device__ __forceinline__ bool child_rate(const TreeSmem& s, int i, int c, doub
   return true;
 }
 
-// Tokens of node i's removed children other than c, ascending, to list;
-// returns how many.
+// Tokens of the children of node i removed before c (those in front of it),
+// ascending, to list; returns how many.
 __device__ inline int removed_tokens(const TreeSmem& s, int i, int c, int* list) {
   int n = 0;
-  for (int j = s.first[i]; j >= 0; j = s.next[j]) {
-    if (j == c || s.state[j] == kAlive) continue;
+  for (int j = s.first[i]; j != c; j = s.next[j]) {
     const int t = s.tok[j];
     int k = n;
     while (k > 0 && list[k - 1] > t) {
@@ -176,11 +175,10 @@ __device__ inline int removed_tokens(const TreeSmem& s, int i, int c, int* list)
   return n;
 }
 
-// The stored masses of node i's removed children other than c.
+// The stored masses of the children of node i removed before c.
 __device__ inline double removed_mass(const TreeSmem& s, int i, int c) {
   double sum = 0.0;
-  for (int j = s.first[i]; j >= 0; j = s.next[j])
-    if (j != c && s.state[j] != kAlive) sum += s.m[j];
+  for (int j = s.first[i]; j != c; j = s.next[j]) sum += s.m[j];
   return sum;
 }
 
@@ -209,8 +207,7 @@ __device__ inline void apply_rejection(const TreeSmem& s, Ctl& ctl, int i, int c
   if (S > 0.0) {
     const double invS = 1.0 / S;
     const double na = alpha * invS, nb = beta * invS, scale = p * invS;
-    for (int j = s.first[i]; j >= 0; j = s.next[j])
-      if (j != c && s.state[j] != kAlive) s.m[j] *= scale;
+    for (int j = s.first[i]; j != c; j = s.next[j]) s.m[j] *= scale;
     s.m[c] = fmax(na * mb0 - nb * q0, 0.0);
     s.a[i] = na;
     s.b[i] = nb;
@@ -319,7 +316,7 @@ __device__ inline void prepare_ahead(const TreeSmem& s, const Ctl& ctl, Ahead& a
   ah.beta = beta;
   ah.mb0 = s.mb0[c];
   ah.q0 = (double)s.gq[c];
-  const int c2 = first_alive_child(s, i);
+  const int c2 = s.next[c];   // (the children after c all remain)
   ah.c2 = c2;
   if (c2 < 0) {
     if (i == 0) return;   // the root: the bonus draw follows
@@ -418,8 +415,7 @@ __device__ inline void control_step_ahead(const TreeSmem& s, Ctl& ctl, const Ahe
   const int i = ah.i, c = ah.c;
   const double na = ah.alpha * inv_s, nb = ah.beta * inv_s, scale = ah.p * inv_s;
   const double mc = fmax(na * ah.mb0 - nb * ah.q0, 0.0);
-  for (int j = s.first[i]; j >= 0; j = s.next[j])
-    if (j != c && s.state[j] != kAlive) s.m[j] *= scale;
+  for (int j = s.first[i]; j != c; j = s.next[j]) s.m[j] *= scale;
   s.m[c] = mc;
   s.a[i] = na;
   s.b[i] = nb;

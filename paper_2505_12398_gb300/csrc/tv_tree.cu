@@ -23,6 +23,10 @@
 //     each row by a group of warps, with one exchange for all of them; the
 //     rows' final sums and their children's float64 masses are spread over the
 //     consumer warps;
+//   * the consumers take all their tiles of a chunk in one straight line (no
+//     test per tile for removed tokens, edges or lengths where a look at the
+//     whole chunk rules them out), so that the tiles' chains of dependent
+//     operations overlap: one tile at a time a warp took 1160 cycles a tile.
 //   * where a slice of a (target, draft) row pair fits the ring, it stays there:
 //     the next pass at the same node (about half of all passes) reads no
 //     memory, and with room for two the parent's pair is fetched while the
@@ -42,11 +46,12 @@
 // Every wait is bounded; one that gives up raises TV_STATUS_TIMEOUT, and all
 // roles still reach the cluster barrier at the end.
 //
-// Measured (60-node trees, V = 32000, bf16; 8-token chains, fp32), against one
-// thread of the consumers doing the control, a reduction and an exchange per
-// row and no resident pairs: B = 64 254.2 -> 148.1 us, 16 chains 117.0 -> 71.8 us
-// (183.2 and 77.2 us with a row by all warps in turn and before the removal of a
-// rate-0 sibling and the descent into a sub-tree were worked out ahead).
+// Measured (60-node trees, bf16; 8-token chains, fp32), against one thread of the
+// consumers doing the control, a reduction and an exchange per row and no
+// resident pairs: V = 32000, B = 64 254 -> 143 us (183 with a row by all warps in turn
+// and before the removal of a rate-0 sibling and the descent into a sub-tree were
+// worked out ahead, 149 one tile at a time); 16 chains 117 -> 64 us; V = 128256, B =
+// 32 368 -> 184 us (213 one tile at a time).
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -89,7 +94,7 @@ struct TreeJob {
   float alpha1, beta, rowmax;
   int total;               // ring chunks the job loads (0: its pair is resident)
   int slot;                // resident slot of a pair (-1: streamed through the ring)
-  int pf_node, pf_slot;    // pair to fetch ahead into another slot (-1: none)
+  uint32_t ph;             // parities of the stages' latest fills before the job
   int mbuf;                // which list of removed tokens
   int xb, xph;             // exchange buffer and the parity of its barrier
   int rows[kStatRows];
@@ -151,6 +156,11 @@ __device__ __forceinline__ void lds_logits(const typename L::elem* p, float v[8]
   }
 }
 
+__device__ __forceinline__ float max8(const float v[8]) {
+  return fmaxf(fmaxf(fmaxf(v[0], v[1]), fmaxf(v[2], v[3])),
+               fmaxf(fmaxf(v[4], v[5]), fmaxf(v[6], v[7])));
+}
+
 // e(x) of eight logits relative to m (kPass: the cheaper form of passes and
 // draws; see tv_device.cuh).
 template <typename L, bool kPass>
@@ -173,30 +183,17 @@ __device__ __forceinline__ void exp8(const float v[8], float m, float c_hi, floa
   }
 }
 
-// e(x) in passes and draws: the cheaper form, or (the three-kernel path, whose
-// normalisers come from exp_rel) the other one.
-template <typename L>
-__device__ __forceinline__ void exp8_pass(const float v[8], float m, bool exact, float c_hi,
-                                          float c_lo, float e[8]) {
-  if (L::kBytes == 2 && exact) exp8<L, false>(v, m, c_hi, c_lo, e);
-  else exp8<L, true>(v, m, c_hi, c_lo, e);
-}
-template <typename L>
-__device__ __forceinline__ float exp1_pass(float v, float m, bool exact, float c_hi, float c_lo) {
-  return exact ? L::exp_rel(v, m, c_hi, c_lo) : L::exp_pass(v, m, c_hi, c_lo);
-}
-
 // [alpha e(x) - beta q(x)]_+ of eight tokens.
-template <typename L>
+template <typename L, bool kExact>
 __device__ __forceinline__ void residual8(const float v[8], const float* qp, float rowmax,
-                                          float alpha, float beta, bool exact, float c_hi,
-                                          float c_lo, float t[8]) {
+                                          float alpha, float beta, float c_hi, float c_lo,
+                                          float t[8]) {
   const uint4 qa = lds128(qp), qc = lds128(qp + 4);
   const float q[8] = {__uint_as_float(qa.x), __uint_as_float(qa.y), __uint_as_float(qa.z),
                       __uint_as_float(qa.w), __uint_as_float(qc.x), __uint_as_float(qc.y),
                       __uint_as_float(qc.z), __uint_as_float(qc.w)};
   float e[8];
-  exp8_pass<L>(v, rowmax, exact, c_hi, c_lo, e);
+  exp8<L, !kExact>(v, rowmax, c_hi, c_lo, e);
   if constexpr (L::kBytes == 2) {
     const float2 al2 = make_float2(alpha, alpha), nb2 = make_float2(-beta, -beta);
 #pragma unroll
@@ -232,7 +229,7 @@ __device__ __forceinline__ void block_probs(const float* p, int lo, int hi, floa
 
 // ------------------------------------------------------------- kernel -----
 
-template <typename L, int NCW>
+template <typename L, int NCW, bool kExact>
 struct TreeCta {
   using E = typename L::elem;
   static constexpr int kLB = L::kBytes;
@@ -240,6 +237,7 @@ struct TreeCta {
   static constexpr int kPair = kStageBytes / (kLB + 4);   // tokens of a pair chunk
   static constexpr int kRow = kStageBytes / kLB;          // tokens of a target-only chunk
   static constexpr int kSweep = NCW * kTileElems;
+  static constexpr int kTiles = tiles_per_warp(NCW);      // per warp in a pair chunk
   static constexpr int kThreads = NCW * 32 + 64;          // + producer, control warps
   static_assert(kPair % kTileElems == 0, "whole tiles per stage");
 
@@ -271,17 +269,16 @@ struct TreeCta {
     return kind == kJobPass || kind == kJobBonusRes;
   }
 
+  // e(x) in draws and passes: the cheaper form, or (kExact: the three-kernel path,
+  // whose normalisers come from exp_rel) that one.
+  __device__ __forceinline__ float exp1(float v, float m) const {
+    return kExact ? L::exp_rel(v, m, a.c_hi, a.c_lo) : L::exp_pass(v, m, a.c_hi, a.c_lo);
+  }
+
   // ---------------------------------------------------------- producer --
   // Fills stage `st` with the slice's chunk from element x of its first block
-  // (n_all: elements of the arrays).  `filled` and `fph` track each stage's fills: a fetch ahead that no
-  // job has waited for must have landed before its stage is filled again.
-  __device__ bool fill(int st, const Slice& sl, int x, bool pair, size_t n_all,
-                       uint32_t& filled, uint32_t& fph) {
-    if ((filled >> st) & 1u) {
-      if (!mbar_wait(&full_bar[st], (fph >> st) & 1u)) return false;
-    }
-    filled |= 1u << st;
-    fph ^= 1u << st;
+  // (n_all: elements of the arrays).
+  __device__ void fill(int st, const Slice& sl, int x, bool pair, size_t n_all) {
     const size_t e0 = sl.base + (size_t)x;
     const int n = (min(pair ? kPair : kRow, sl.n - x) + 7) & ~7;   // whole blocks
     char* dst = ring + (size_t)st * kStageBytes;
@@ -304,51 +301,47 @@ struct TreeCta {
       if (pair)
         tma_load_1d(dst + (size_t)kPair * kLB, a.draft_probs + e0, qbytes, &full_bar[st]);
     }
-    return true;
   }
+  __device__ size_t elements() const { return (size_t)a.B * (a.N + 1) * (size_t)a.V; }
 
   // Streams the jobs' rows (one lane).
-  __device__ bool produce(size_t n_all, uint32_t& filled, uint32_t& fph) {
+  __device__ bool produce() {
+    const size_t n_all = elements();
     uint32_t jp = 0u, eph = 0u;
     for (;;) {
       if (!mbar_wait(job_bar, jp)) return false;
       jp ^= 1u;
-      const TreeJob job = sh.job;
-      mbar_arrive(ack_bar);                    // the job may be replaced from here on
-      if (job.kind == kJobDone) return true;
-      const bool pair = is_pair(job.kind);
+      const TreeJob& t = sh.job;
+      const int kind = t.kind, total = t.total, slot = t.slot, n_rows = t.n_rows, node = t.node;
+      mbar_arrive(ack_bar);   // (a job that loads is replaced only once its rows are reduced)
+      if (kind == kJobDone) return true;
+      if (total == 0) continue;
+      const bool pair = is_pair(kind);
       const int per = pair ? kPair : kRow;
-      if (job.total > 0) {
-        int st = job.slot > 0 ? job.slot * spc : 0;
-        int q = 0;
-        for (int r = 0; r < job.n_rows; ++r) {
-          const size_t row = row0 + (job.kind == kJobStats ? sh.job.rows[r] : job.node);
-          const Slice sl(row, a.V, v0, v1);
-          for (int x = 0; x < sl.n; x += per, ++q) {
-            if (q >= n_stages) {               // a stage of this job, used again
-              if (!mbar_wait(&empty_bar[st], (eph >> st) & 1u)) return false;
-              eph ^= 1u << st;
+      int st = slot > 0 ? slot * spc : 0;
+      int q = 0;
+      uint32_t ph = t.ph, mine = 0u;
+      for (int r = 0; r < n_rows; ++r) {
+        const Slice sl(row0 + (kind == kJobStats ? sh.job.rows[r] : node), a.V, v0, v1);
+        for (int x = 0; x < sl.n; x += per, ++q) {
+          if (q >= n_stages) {               // a stage of this job, used again
+            if (!mbar_wait(&empty_bar[st], (eph >> st) & 1u)) {
+              // (the consumers gave up: the copies under way land first)
+              for (; mine != 0u; mine &= mine - 1u) {
+                const int k = __ffs(mine) - 1;
+                mbar_wait(&full_bar[k], (ph >> k) & 1u);
+              }
+              return false;
             }
-            if (!fill(st, sl, x, pair, n_all, filled, fph)) return false;
-            if (++st == n_stages) st = 0;
+            eph ^= 1u << st;
           }
+          fill(st, sl, x, pair, n_all);
+          mine |= 1u << st;
+          ph ^= 1u << st;
+          if (++st == n_stages) st = 0;
         }
       }
-      if (job.pf_node >= 0) {
-        const Slice sl(row0 + job.pf_node, a.V, v0, v1);
-        int st = job.pf_slot * spc;
-        for (int x = 0; x < sl.n; x += kPair, ++st)
-          if (!fill(st, sl, x, true, n_all, filled, fph)) return false;
-      }
     }
-  }
-
-  __device__ void producer(size_t n_all) {
-    uint32_t filled = 0u, fph = 0xffffffffu;
-    if (!produce(n_all, filled, fph)) fail();
-    // copies in flight land before the CTA may exit
-    for (int st = 0; st < n_stages; ++st)
-      if (((filled >> st) & 1u) && !mbar_wait(&full_bar[st], (fph >> st) & 1u)) fail();
   }
 
   // ---------------------------------------------------------- exchange --
@@ -398,12 +391,38 @@ struct TreeCta {
     }
   }
 
+  // After chunk q of `total` in stage st: releases the stage where the producer
+  // waits for it, and moves to the next.
+  __device__ __forceinline__ void end_chunk(int q, int total, int& st, int lane) {
+    if (q + n_stages < total) {
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&empty_bar[st]);
+    }
+    if (++st == n_stages) st = 0;
+  }
+
+  // Whether all of this warp's tiles of a pair chunk (n tokens from element x of
+  // the slice's first block, which starts sh elements before the slice) are
+  // whole and hold no removed token (the same in the whole warp).
+  __device__ __forceinline__ bool plain_tiles(int n, int x, int sh, bool ragged, const int* mt,
+                                              int nmask, int wid) const {
+    if (ragged || n < (wid + (kTiles - 1) * NCW + 1) * kTileElems) return false;
+    const int xs = v0 - sh + x;
+    for (int k = 0; k < nmask; ++k) {
+      const int off = mt[k] - xs;
+      if ((unsigned)off < (unsigned)n && (off / kTileElems) % NCW == wid) return false;
+    }
+    return true;
+  }
+
   // Row normalisers: this warp's group takes every g-th row.
-  __device__ bool sum_rows(const TreeJob& job, int wid, int lane, uint32_t& ph) {
+  __device__ bool sum_rows(const TreeJob& job, int wid, int lane) {
     const float c_hi = a.c_hi, c_lo = a.c_lo;
     const int n_rows = job.n_rows, total = job.total, xb = job.xb;
+    uint32_t ph = job.ph;
     const int g = row_groups(n_rows, max_groups), group = wid % g, sub = wid / g, nsub = NCW / g;
     const bool reuse = total > n_stages;       // stages are filled more than once
+    const bool ragged = (a.V & 7) != 0;
     int st = 0, q = 0;
     for (int r = 0; r < n_rows; ++r) {
       const Slice sl(row0 + job.rows[r], a.V, v0, v1);
@@ -418,15 +437,37 @@ struct TreeCta {
         if (mine) {
           const E* lb = reinterpret_cast<const E*>(ring + (size_t)st * kStageBytes);
           const int n = min(kRow, sl.n - x);
-          for (int t0 = sub * kTileElems; t0 < n; t0 += nsub * kTileElems) {
+          const int hop = nsub * kTileElems;
+          int t0 = sub * kTileElems;
+          // two whole tiles at a time: their chains of dependent operations overlap
+          if (!ragged) {
+            for (; t0 + hop + kTileElems <= n; t0 += 2 * hop) {
+              float v[2][8], t[2][8];
+              lds_logits<L>(lb + t0 + lane * kChunk, v[0]);
+              lds_logits<L>(lb + t0 + hop + lane * kChunk, v[1]);
+              const float cm = fmaxf(max8(v[0]), max8(v[1]));
+              if (cm > m_run) {
+                if (m_run != TV_NEG_INF) {
+                  const float sc = L::exp_rel(m_run, cm, c_hi, c_lo);
+                  acc.s *= sc;
+                  acc.c *= sc;
+                }
+                m_run = cm;
+              }
+              exp8<L, false>(v[0], m_run, c_hi, c_lo, t[0]);
+              exp8<L, false>(v[1], m_run, c_hi, c_lo, t[1]);
+              acc.add(sum8(t[0]));
+              acc.add(sum8(t[1]));
+            }
+          }
+          for (; t0 < n; t0 += hop) {
             const int e0 = t0 + lane * kChunk;
             if (e0 >= n) continue;
             const int lo = sl.sh - (x + e0), hi = sl.n - (x + e0);
-            const bool edge = lo > 0 || hi < 8;
+            const bool edge = ragged && (lo > 0 || hi < 8);
             float v[8], t[8];
             stage_logits(lb, e0, true, edge, lo, hi, v);
-            const float cm = fmaxf(fmaxf(fmaxf(v[0], v[1]), fmaxf(v[2], v[3])),
-                                   fmaxf(fmaxf(v[4], v[5]), fmaxf(v[6], v[7])));
+            const float cm = max8(v);
             if (cm > m_run) {
               if (m_run != TV_NEG_INF) {
                 const float sc = L::exp_rel(m_run, cm, c_hi, c_lo);
@@ -440,11 +481,7 @@ struct TreeCta {
             acc.add(sum8(t));
           }
         }
-        if (q + n_stages < total) {            // the producer waits for this stage
-          __syncwarp();
-          if (lane == 0) mbar_arrive(&empty_bar[st]);
-        }
-        if (++st == n_stages) st = 0;
+        end_chunk(q, total, st, lane);
       }
       if (mine) {
         const float wm = warp_max(m_run);
@@ -459,15 +496,17 @@ struct TreeCta {
 
   // A rejection pass (kJobPass: the warp's sum, returned) or the tile sums of a
   // bonus draw.
-  __device__ bool pair_or_leaf(const TreeJob& job, int wid, int lane, uint32_t& ph, float& sum) {
+  __device__ bool pair_or_leaf(const TreeJob& job, int wid, int lane, float& sum) {
     const float c_hi = a.c_hi, c_lo = a.c_lo;
     const int kind = job.kind, total = job.total;
-    const bool pair = is_pair(kind), exact = a.exact_exp != 0;
+    uint32_t ph = job.ph;
+    const bool pair = is_pair(kind);
     const int per = pair ? kPair : kRow;
     const int nmask = job.nmask;
     const int* mt = mtok(job.mbuf);
     const float al = job.alpha1, be = job.beta, rm = job.rowmax;
     const Slice sl(row0 + job.node, a.V, v0, v1);
+    const bool ragged = (a.V & 7) != 0;
     int st = job.slot > 0 ? job.slot * spc : 0, q = 0, mp = 0;
     Comp acc;
     for (int x = 0; x < sl.n; x += per, ++q) {
@@ -477,19 +516,31 @@ struct TreeCta {
       const E* lb = reinterpret_cast<const E*>(buf);
       const float* qb = reinterpret_cast<const float*>(buf + (size_t)kPair * kLB);
       const int n = min(per, sl.n - x);
+      if (kind == kJobPass && plain_tiles(n, x, sl.sh, ragged, mt, nmask, wid)) {
+        float v[kTiles][8], t[kTiles][8];
+#pragma unroll
+        for (int k = 0; k < kTiles; ++k)
+          lds_logits<L>(lb + (wid + k * NCW) * kTileElems + lane * kChunk, v[k]);
+#pragma unroll
+        for (int k = 0; k < kTiles; ++k)
+          residual8<L, kExact>(v[k], qb + (wid + k * NCW) * kTileElems + lane * kChunk, rm, al,
+                               be, c_hi, c_lo, t[k]);
+#pragma unroll
+        for (int k = 0; k < kTiles; ++k) acc.add(sum8(t[k]));
+        end_chunk(q, total, st, lane);
+        continue;
+      }
       for (int t0 = wid * kTileElems; t0 < n; t0 += kSweep) {
         const int e0 = t0 + lane * kChunk;
         const bool valid = e0 < n;
         const int xg = v0 - sl.sh + x + e0;    // token of the lane's first element
         const int lo = sl.sh - (x + e0), hi = sl.n - (x + e0);
-        const bool edge = valid && (lo > 0 || hi < 8);
+        const bool edge = ragged && valid && (lo > 0 || hi < 8);
         float v[8], t[8];
         stage_logits(lb, e0, valid, edge, lo, hi, v);
         if (kind == kJobBonusLeaf) {
-          const float lm = fmaxf(fmaxf(fmaxf(v[0], v[1]), fmaxf(v[2], v[3])),
-                                 fmaxf(fmaxf(v[4], v[5]), fmaxf(v[6], v[7])));
-          const float tm = warp_max(lm);
-          exp8_pass<L>(v, tm, exact, c_hi, c_lo, t);
+          const float tm = warp_max(max8(v));
+          exp8<L, !kExact>(v, tm, c_hi, c_lo, t);
           zero_outside(edge, lo, hi, t);
           const float ts = warp_sum(valid ? sum8(t) : 0.f);
           if (lane == 0) {
@@ -499,7 +550,7 @@ struct TreeCta {
           continue;
         }
         if (valid) {
-          residual8<L>(v, qb + e0, rm, al, be, exact, c_hi, c_lo, t);
+          residual8<L, kExact>(v, qb + e0, rm, al, be, c_hi, c_lo, t);
         } else {
 #pragma unroll
           for (int e = 0; e < 8; ++e) t[e] = 0.f;
@@ -522,11 +573,7 @@ struct TreeCta {
           if (lane == 0) s.tsum[(x + t0) / kTileElems] = ts;
         }
       }
-      if (q + n_stages < total) {              // the producer waits for this stage
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&empty_bar[st]);
-      }
-      if (++st == n_stages) st = 0;
+      end_chunk(q, total, st, lane);
     }
     sum = acc.value();
     return true;
@@ -534,7 +581,6 @@ struct TreeCta {
 
   __device__ void consumer(int wid, int lane) {
     uint32_t jp = 0u;
-    uint32_t ph = 0xffffffffu;                 // parity of each stage's latest fill
     for (;;) {
       if (!mbar_wait_warp(job_bar, jp)) { fail(); return; }
       jp ^= 1u;
@@ -542,18 +588,13 @@ struct TreeCta {
       const int kind = job.kind;
       if (kind == kJobDone) return;
       if (kind == kJobStats) {
-        if (!sum_rows(job, wid, lane, ph) || !finish_rows(job, wid, lane)) { fail(); return; }
+        if (!sum_rows(job, wid, lane) || !finish_rows(job, wid, lane)) { fail(); return; }
         continue;
       }
       float sum;
-      if (!pair_or_leaf(job, wid, lane, ph, sum)) { fail(); return; }
+      if (!pair_or_leaf(job, wid, lane, sum)) { fail(); return; }
       if (kind == kJobPass) {
         const int xb = job.xb;
-        if (job.pf_node >= 0) {                // a pair fetched ahead, used by a later job
-          const Slice sl(row0 + job.pf_node, a.V, v0, v1);
-          int st = job.pf_slot * spc;
-          for (int x = 0; x < sl.n; x += kPair, ++st) ph ^= 1u << st;
-        }
         // once every CTA's control warp has all partials, the job is replaced:
         // nothing of it is read after this
         send(xb, (int)rank * NCW + wid, lane, warp_sum(sum), 0.f);
@@ -697,7 +738,7 @@ struct TreeCta {
 #pragma unroll
         for (int e = 0; e < 8; ++e)
           w[e] = (v[e] == TV_NEG_INF) ? 0.f
-                                      : exp1_pass<L>(v[e], Mc, a.exact_exp != 0, c_hi, c_lo);
+                                      : exp1(v[e], Mc);
       } else {
         float qv[8];
         block_probs(a.draft_probs + at, lo, hi, qv);
@@ -706,7 +747,7 @@ struct TreeCta {
           w[e] = (v[e] == TV_NEG_INF)
                      ? 0.f
                      : fmaxf(fmaf(job.alpha1,
-                                  exp1_pass<L>(v[e], job.rowmax, a.exact_exp != 0, c_hi, c_lo),
+                                  exp1(v[e], job.rowmax),
                                   -job.beta * qv[e]), 0.f);
         const int* mt = mtok(job.mbuf);
         for (int mq = 0; mq < job.nmask; ++mq) {
@@ -763,61 +804,89 @@ struct TreeCta {
   }
 
   // ----------------------------------------------------------- control --
+  // What lane 0 of the control warp keeps of the ring: the parities of the
+  // stages' latest fills, the stages whose latest fill was a fetch ahead that may
+  // still be on its way, the resident slots, the node and slot of the latest
+  // pair, jobs and exchanges so far.
+  struct Ring {
+    uint32_t ph = 0xffffffffu, coming = 0u;
+    int n_slots = 0, node = -1, slot = 0, jobs = 0, xk = 0;
+    __device__ __forceinline__ void took(uint32_t stages) { ph ^= stages; }
+    // `total` chunks through a ring of n stages, from stage 0
+    __device__ __forceinline__ void streamed(int total, int n) {
+      for (; total >= n; total -= n) took((1u << n) - 1u);
+      took((1u << total) - 1u);
+    }
+  };
+
+  // Waits until every fetch ahead has landed: before a stage is filled again,
+  // since a wait on a barrier's parity cannot tell the fill before the latest one
+  // from it.
+  __device__ bool settle(Ring& ring) const {
+    for (; ring.coming != 0u; ring.coming &= ring.coming - 1u) {
+      const int st = __ffs(ring.coming) - 1;
+      if (!mbar_wait(&full_bar[st], (ring.ph >> st) & 1u)) return false;
+    }
+    return true;
+  }
+
+  // The slot of a pair: the one that holds it, or the one used longest ago
+  // (other than `keep`).
+  __device__ int find_slot(const Ring& ring, int node, int keep, bool& held) const {
+    int old = -1;
+    for (int k = 0; k < ring.n_slots; ++k) {
+      if (sh.slot_node[k] == node) { held = true; return k; }
+      if (k != keep && (old < 0 || sh.slot_used[k] < sh.slot_used[old])) old = k;
+    }
+    held = false;
+    return old;
+  }
+
   // Lane 0: completes the job's ring, slot and exchange fields and publishes it.
-  __device__ bool publish(const Job& j, int mbuf, int n_slots, int xk, int jobs) {
+  // This stands between a pass's result and the next job's start, so the usual
+  // case, a pass at the node of the latest one, looks nothing up.
+  __device__ bool publish(const Job& j, int mbuf, Ring& ring) {
     TreeJob& t = sh.job;
     // the producer has copied the job before (the consumers have finished it)
-    if (jobs > 0 && !mbar_wait(ack_bar, (uint32_t)(jobs - 1) & 1u)) return false;
+    if (ring.jobs > 0 && !mbar_wait(ack_bar, (uint32_t)(ring.jobs - 1) & 1u)) return false;
     t.kind = j.kind;
-    t.pf_node = -1;
     if (j.kind != kJobDone) {
+      uint32_t bytes;
+      int n_rows = 1, total = 0, slot = -1;
+      t.ph = ring.ph;
       t.node = j.node;
       t.nmask = j.nmask;
       t.alpha1 = j.alpha1;
       t.beta = j.beta;
       t.rowmax = j.rowmax;
       t.mbuf = mbuf;
-      t.xb = xk & 1;
-      t.xph = (xk >> 1) & 1;
-      t.slot = -1;
-      int n_rows = 1;
-      uint32_t bytes;
+      t.xb = ring.xk & 1;
+      t.xph = (ring.xk >> 1) & 1;
       if (is_pair(j.kind)) {
-        const int nch = chunks_of(Slice(row0 + j.node, a.V, v0, v1).n, kPair);
-        t.total = nch;
-        if (n_slots > 0) {
-          int at = -1, old = 0;
-          for (int k = 0; k < n_slots; ++k) {
-            if (sh.slot_node[k] == j.node) at = k;
-            if (sh.slot_used[k] < sh.slot_used[old]) old = k;
+        bytes = (j.kind == kJobPass) ? (uint32_t)(C * NCW) * 8u : (uint32_t)C * 8u;
+        if (ring.n_slots > 0 && ring.node == j.node) {
+          slot = ring.slot;
+        } else {
+          bool held = false;
+          if (ring.n_slots > 0) {
+            slot = find_slot(ring, j.node, -1, held);
+            sh.slot_node[slot] = j.node;
+            sh.slot_used[slot] = ring.jobs + 1;
+            ring.node = j.node;
+            ring.slot = slot;
           }
-          if (at >= 0) t.total = 0;
-          else at = old;
-          t.slot = at;
-          sh.slot_node[at] = j.node;
-          sh.slot_used[at] = jobs + 1;
-          // the parent's pair, for the pass there that a rejection of this node
-          // leads to (unless the traversal goes down into another child first)
-          if (j.kind == kJobPass && n_slots > 1 && j.node != 0 && !a.token_level) {
-            const int g = s.par[j.node];
-            bool have = false;
-            for (int k = 0; k < n_slots; ++k) have |= sh.slot_node[k] == g;
-            if (!have) {
-              int o2 = at == 0 ? 1 : 0;
-              for (int k = 0; k < n_slots; ++k)
-                if (k != at && sh.slot_used[k] < sh.slot_used[o2]) o2 = k;
-              t.pf_node = g;
-              t.pf_slot = o2;
-              sh.slot_node[o2] = g;
-              sh.slot_used[o2] = jobs + 1;
-            }
+          if (!held) {
+            if (!settle(ring)) return false;
+            total = chunks_of(Slice(row0 + j.node, a.V, v0, v1).n, kPair);
+            if (slot >= 0) ring.took(((1u << total) - 1u) << (slot * spc));
+            else ring.streamed(total, n_stages);
           }
         }
-        bytes = (j.kind == kJobPass) ? (uint32_t)(C * NCW) * 8u : (uint32_t)C * 8u;
       } else {
         // target rows only: through the whole ring
-        for (int k = 0; k < n_slots; ++k) sh.slot_node[k] = -1;
-        int total = 0;
+        if (!settle(ring)) return false;
+        for (int k = 0; k < ring.n_slots; ++k) sh.slot_node[k] = -1;
+        ring.node = -1;
         if (j.kind == kJobStats) {
           n_rows = min(j.n_rows, min(kStatRows, 4 * max_groups));
           for (int r = 0; r < n_rows; ++r) {
@@ -829,60 +898,75 @@ struct TreeCta {
           total = chunks_of(Slice(row0 + j.node, a.V, v0, v1).n, kRow);
           bytes = (uint32_t)C * 8u;
         }
-        t.total = total;
+        ring.streamed(total, n_stages);
       }
+      t.total = total;
+      t.slot = slot;
       t.n_rows = n_rows;
-      if (C > 1) mbar_arrive_expect_tx(&xbar[xk & 1], bytes);
+      if (C > 1) mbar_arrive_expect_tx(&xbar[ring.xk & 1], bytes);
     }
     mbar_arrive(job_bar);
+    ++ring.jobs;
     return true;
   }
 
-  __device__ void control(int lane) {
-    // resident row pairs the ring has room for (0: pairs are streamed)
-    const int n_slots = min(n_stages / spc, kTreeMaxSlots);
-    if (lane < kTreeMaxSlots) { sh.slot_node[lane] = -1; sh.slot_used[lane] = 0; }
-    __syncwarp();
+  // Lane 0, while a pass at node i runs: fetches the pair of i's parent into
+  // another slot, for the pass there that a rejection of i leads to.
+  __device__ bool fetch_parent(Ring& ring) {
+    const int i = ring.node;
+    if (ring.n_slots < 2 || i <= 0 || a.token_level) return true;
+    const int g = s.par[i];
+    bool held;
+    const int slot = find_slot(ring, g, ring.slot, held);
+    if (held) return true;
+    if (!settle(ring)) return false;
+    const Slice sl(row0 + g, a.V, v0, v1);
+    const int n = chunks_of(sl.n, kPair);
+    for (int k = 0; k < n; ++k) fill(slot * spc + k, sl, k * kPair, true, elements());
+    ring.coming = ((1u << n) - 1u) << (slot * spc);
+    ring.took(ring.coming);
+    sh.slot_node[slot] = g;
+    sh.slot_used[slot] = ring.jobs + 1;
+    return true;
+  }
+
+  __device__ void run_tree(int lane, Ring& ring) {
     Ctl& ctl = sh.ctl;
     Ahead& ah = sh.ahead;
-    int xk = 0, jobs = 0, mnext = 1;     // exchanges, jobs, next list of removed tokens
+    const bool ahead = a.token_level == 0;
+    int mnext = 1;                       // next list of removed tokens
     uint32_t stat_ph = 0u;               // parity of stat_bar
     int ok = 1;
     if (lane == 0) {
       if (ctl.job.kind != kJobDone) advance(s, ctl, u, a.token_level != 0);
-      ok = publish(ctl.job, 0, n_slots, xk, jobs) ? 1 : 0;
+      ok = publish(ctl.job, 0, ring) ? 1 : 0;
       ah.ok = 0;
-      if (!a.token_level) prepare_ahead(s, ctl, ah, mtok(mnext), u);
+      if (ahead) prepare_ahead(s, ctl, ah, mtok(mnext), u);
     }
     for (;;) {
-      ++jobs;
       __syncwarp();
       ok = __shfl_sync(0xffffffffu, ok, 0);
       if (!ok) { fail(); return; }
       const int kind = ctl.job.kind;
       if (kind == kJobDone) return;
-      float S = 0.f;
-      bool got;
-      if (kind == kJobStats) {
-        got = mbar_wait_warp(stat_bar, stat_ph);
-      } else {
-        got = exchanged(xk & 1, (uint32_t)(xk >> 1) & 1u);
-      }
+      const int xk = ring.xk;            // (the same in every lane)
+      const bool got = kind == kJobStats ? mbar_wait_warp(stat_bar, stat_ph)
+                                         : exchanged(xk & 1, (uint32_t)(xk >> 1) & 1u);
       if (!got) { fail(); return; }
+      float S = 0.f;
       if (kind == kJobPass) {
         const float2* x = xslots(xk & 1);
         for (int k = lane; k < C * NCW; k += 32) S += x[k].x;
         S = warp_sum(S);
       }
-      ++xk;
+      ++ring.xk;
       if (kind == kJobStats) stat_ph ^= 1u;
-      double Sd = 0.0;
-      if (kind == kJobPass && ah.ok && (Sd = (double)S + ah.pm) > 1e-300) {
+      if (kind == kJobPass && ah.ok && S > 0.f) {
         // the next step was worked out while the pass ran: decide, publish, then
         // update the state (the same values in every lane; 1 / D, 1 / S and S / D
         // in lanes 0, 1 and 2, since a float64 division takes as long for one lane
         // as for three)
-        const double D = Sd + ah.omp;
+        const double Sd = (double)S + ah.pm, D = Sd + ah.omp;
         double quot = 0.0;
         const bool early = ah.mode == kAheadTest || ah.mode == kAheadPrune;
         if (early) quot = (lane == 2 ? Sd : 1.0) / (lane == 1 ? Sd : D);
@@ -890,7 +974,7 @@ struct TreeCta {
         if (lane == 0) {
           Job jf;
           first = job_ahead(s, ah, Sd, D, quot, jf, accept);
-          if (first) ok = publish(jf, mnext, n_slots, xk, jobs) ? 1 : 0;
+          if (first) ok = publish(jf, mnext, ring) ? 1 : 0;
         }
         __syncwarp();
         if (!early) quot = (lane == 2 ? Sd : 1.0) / (lane == 1 ? Sd : D);
@@ -899,9 +983,10 @@ struct TreeCta {
         if (lane == 0) {
           ctl.S = S;
           control_step_ahead(s, ctl, ah, accept, quot, inv_s, p_new);
-          if (!first) ok = publish(ctl.job, 0, n_slots, xk, jobs) ? 1 : 0;
+          if (!first) ok = publish(ctl.job, 0, ring) ? 1 : 0;
           else mnext = 3 - mnext;             // that list is in use now
           prepare_ahead(s, ctl, ah, mtok(mnext), u);
+          if (ctl.job.kind == kJobPass && !fetch_parent(ring)) ok = 0;
         }
       } else if (lane == 0) {
         if (kind == kJobBonusLeaf || kind == kJobBonusRes) {
@@ -911,11 +996,25 @@ struct TreeCta {
           if (*(volatile uint32_t*)&ctl.bad & (32u | 64u)) ctl.job.kind = kJobDone;
           else advance(s, ctl, u, a.token_level != 0);
         }
-        ok = publish(ctl.job, 0, n_slots, xk, jobs) ? 1 : 0;
+        ok = publish(ctl.job, 0, ring) ? 1 : 0;
         ah.ok = 0;
-        if (!a.token_level) prepare_ahead(s, ctl, ah, mtok(mnext), u);
+        if (ahead) prepare_ahead(s, ctl, ah, mtok(mnext), u);
+        if (ctl.job.kind == kJobPass && !fetch_parent(ring)) ok = 0;
       }
     }
+  }
+
+  __device__ void control(int lane) {
+    if (lane < kTreeMaxSlots) { sh.slot_node[lane] = -1; sh.slot_used[lane] = 0; }
+    __syncwarp();
+    Ring ring;
+    // resident row pairs the ring has room for (0: pairs are streamed)
+    ring.n_slots = min(n_stages / spc, kTreeMaxSlots);
+    run_tree(lane, ring);
+    // copies in flight land before the CTA may exit: fetches ahead here, those of
+    // a job the consumers gave up on in produce()
+    if (lane == 0 && !settle(ring)) fail();
+    __syncwarp();
   }
 
   // Writes the tree's outputs (control warp of rank 0).
@@ -962,10 +1061,10 @@ struct TreeCta {
   }
 };
 
-template <typename L, int NCW>
-__global__ void __launch_bounds__(TreeCta<L, NCW>::kThreads, 16 / NCW)
+template <typename L, int NCW, bool kExact>
+__global__ void __launch_bounds__(TreeCta<L, NCW, kExact>::kThreads, 16 / NCW)
     tv_tree_kernel(const __grid_constant__ TravArgs args, int C, int n_stages) {
-  using T = TreeCta<L, NCW>;
+  using T = TreeCta<L, NCW, kExact>;
   extern __shared__ __align__(128) char smem_raw[];
   __shared__ __align__(8) uint64_t full_bar[kTreeMaxStages];
   __shared__ __align__(8) uint64_t empty_bar[kTreeMaxStages];
@@ -1123,7 +1222,7 @@ __global__ void __launch_bounds__(TreeCta<L, NCW>::kThreads, 16 / NCW)
   if (wid < NCW) {
     t.consumer(wid, lane);
   } else if (wid == NCW) {
-    if (lane == 0) t.producer((size_t)args.B * R * (size_t)V);
+    if (lane == 0 && !t.produce()) t.fail();
   } else {
     t.control(lane);
   }
@@ -1169,18 +1268,21 @@ FusedPlan tv_fused_plan(int B, int R, int V, int logit_bytes, int smem_per_sm,
   // which a job is all latency.  Measured (us; 60-node trees; ncw x C):
   //   V = 128256, B = 1: 16x16 112, 8x16 118, 16x8 132, 8x8 151, 4x8 212
   //   V = 128256, B = 16: 8x16 144, 16x8 160, 8x8 188, 16x16 218, 4x8 267
-  //   V = 128256, B = 32: 8x8 211, 16x4 236, 8x16 288, 4x8 288
+  //   V = 128256, B = 48: 4x8 215, 8x4 218, 16x4 220, 8x8 221; B = 64: 8x4 239, 4x8
+  //   240, 8x8 287; B = 128: 8x2 419, 8x4 424, 4x4 429
+  //   V = 262144, B = 32: 8x8 255, 4x8 341, 16x4 346, 8x4 364
   //   V = 32000, B = 1: 8x16 63, 8x8 65, 4x8 71; B = 16: 8x8 120, 4x8 124, 8x16 143
-  //   V = 32000, B = 64: 8x4 149, 4x8 154, 8x8 160; B = 128: 8x4 212, 4x4 218, 8x2 225
-  //   V = 32000, B = 256: 8x2 298, 4x2 300, 8x1 320, 8x4 344; B = 300: 8x2 313, 8x1 356
-  //   V = 16384, B = 300: 4x2 227, 8x1 232, 8x2 244; B = 1024: 8x1 500, 4x2 532, 8x2 607
+  //   V = 32000, B = 64: 8x4 149, 4x8 154, 8x8 160; B = 128: 4x4 191, 8x2 192, 8x4 212
+  //   V = 32000, B = 400: 8x2 377, 8x1 385, 4x4 431; B = 1024: 8x1 651, 8x2 731
+  //   V = 16384, B = 300: 8x1 232, 8x2 244; V = 8000 (26 nodes): 8x1 117, 8x2 158
   //   V = 1000, B = 1024 (26 nodes): 4x1 213, 8x1 280
+  // (B = 1, 16 and V <= 16384 before the consumers took a chunk's tiles together)
   int ncw = 8, C = 1;
   if (V > 98304 && B <= 4) ncw = 16, C = 16;
   else if (B <= 8 || (V > 98304 && B <= 16)) C = 16;
   else if (B <= 32) C = 8;
-  else if (B <= 128) C = 4;
-  else if (B <= 256 || (B <= 320 && V > 20000)) C = 2;
+  else if (B <= 76) C = 4;
+  else if (B <= 152 || (B <= 400 && V > 20000)) C = 2;
   else if (V <= 4096) ncw = 4;
   while (C > 1 && V / C < 1000) C /= 2;
   while (C < 8 && tree_tiles(V, C) * 8 > 32768) C *= 2;   // bonus tiles' shared memory
@@ -1204,9 +1306,9 @@ FusedPlan tv_fused_plan(int B, int R, int V, int logit_bytes, int smem_per_sm,
 
 namespace {
 
-template <typename L, int NCW>
+template <typename L, int NCW, bool kExact>
 cudaError_t launch_one(const TravArgs& a, const FusedPlan& plan, cudaStream_t stream) {
-  auto k = tvk::fused::tv_tree_kernel<L, NCW>;
+  auto k = tvk::fused::tv_tree_kernel<L, NCW, kExact>;
   cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)plan.smem);
   if (e != cudaSuccess) return e;
   if (plan.C > 8) {
@@ -1215,7 +1317,7 @@ cudaError_t launch_one(const TravArgs& a, const FusedPlan& plan, cudaStream_t st
   }
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)(a.B * plan.C), 1, 1);
-  cfg.blockDim = dim3(tvk::fused::TreeCta<L, NCW>::kThreads, 1, 1);
+  cfg.blockDim = dim3(tvk::fused::TreeCta<L, NCW, kExact>::kThreads, 1, 1);
   cfg.dynamicSmemBytes = plan.smem;
   cfg.stream = stream;
   cudaLaunchAttribute attr[1];
@@ -1228,19 +1330,22 @@ cudaError_t launch_one(const TravArgs& a, const FusedPlan& plan, cudaStream_t st
   return cudaLaunchKernelEx(&cfg, k, a, plan.C, plan.stages);
 }
 
-template <typename L>
+template <typename L, bool kExact>
 cudaError_t launch_ncw(const TravArgs& a, const FusedPlan& plan, cudaStream_t stream) {
-  if (plan.ncw == 16) return launch_one<L, 16>(a, plan, stream);
-  if (plan.ncw == 8) return launch_one<L, 8>(a, plan, stream);
-  return launch_one<L, 4>(a, plan, stream);
+  if (plan.ncw == 16) return launch_one<L, 16, kExact>(a, plan, stream);
+  if (plan.ncw == 8) return launch_one<L, 8, kExact>(a, plan, stream);
+  return launch_one<L, 4, kExact>(a, plan, stream);
 }
 
 }  // namespace
 
 int tv_launch_tree(const TravArgs& a, int logit_is_bf16, const FusedPlan& plan,
                    cudaStream_t stream) {
-  const cudaError_t e = logit_is_bf16 ? launch_ncw<tvk::Bf16Logits>(a, plan, stream)
-                                      : launch_ncw<tvk::F32Logits>(a, plan, stream);
+  // (fp32 logits have one exponential: the two forms are the same kernel)
+  const cudaError_t e =
+      !logit_is_bf16 ? launch_ncw<tvk::F32Logits, false>(a, plan, stream)
+                     : (a.exact_exp ? launch_ncw<tvk::Bf16Logits, true>(a, plan, stream)
+                                    : launch_ncw<tvk::Bf16Logits, false>(a, plan, stream));
   if (e == cudaSuccess) return 0;
   cudaGetLastError();
   return -5;
