@@ -41,7 +41,6 @@ struct tv_handle {
   int withhold_tree = -1;        // test hook for the next persistent call (-1: none)
   // per-(row, tile) scratch of tv_lm_head (allocated on first use)
   float2* lmh_part = nullptr;
-  size_t lmh_part_bytes = 0;
   // staging for tv_verify_batch_host (allocated on first use), and the bytes
   // its last call copied each way
   char* stage = nullptr;
@@ -616,17 +615,14 @@ int tv_lm_head(tv_handle* h, int M, int K, const void* hidden, const void* weigh
     return TV_ERR_INVALID_ARG;
   DeviceGuard guard(h->device);
   if (!guard.ok()) return TV_ERR_CUDA;
-  const size_t need = (size_t)h->max_batch * (h->max_nodes + 1) *
-                      (size_t)tv_lm_head_parts(h->vocab) * sizeof(float2);
-  if (h->lmh_part_bytes < need) {
-    if (h->lmh_part) cudaFree(h->lmh_part);
-    h->lmh_part = nullptr;
-    h->lmh_part_bytes = 0;
-    if (cudaMalloc(&h->lmh_part, need) != cudaSuccess) {
+  if (!h->lmh_part) {   // sized for the handle's limits, once
+    const size_t need =
+        tv_lm_head_scratch(h->max_batch * (h->max_nodes + 1), h->vocab) * sizeof(float2);
+    if (need == 0 || cudaMalloc(&h->lmh_part, need) != cudaSuccess) {
       cudaGetLastError();
+      h->lmh_part = nullptr;
       return TV_ERR_CUDA;
     }
-    h->lmh_part_bytes = need;
   }
   const double c = 1.4426950408889634 / static_cast<double>(temperature);
   const float c_hi = static_cast<float>(c);

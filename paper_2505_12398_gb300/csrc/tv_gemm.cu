@@ -29,8 +29,9 @@
 // The tile width bn is chosen for the waves it makes (tile_width): at 61 rows and
 // V = 128256, 4 waves of 224 columns on 152 SMs instead of 4 of 256 (3.3 full).
 // With 30 to 55 KB more in flight per SM (the H box of the rows that exist) and
-// a block per row in the merge, 185.0 -> 164.3 us there (157 us of bytes at 6.8
-// TB/s), one row 225 -> 158 us.
+// a block per row in the merge, already waiting when this kernel ends (a
+// programmatic dependent launch), 188.9 -> 163 us there (157 us of bytes at 6.8
+// TB/s; 165 us without that launch), one row 225 -> 156 us.
 // In both:
 //   * warp 0 (one lane) streams 64-element K slices of H and W into a ring of
 //     shared memory with 2-D TMA copies (128-byte swizzle, the layout the
@@ -364,6 +365,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   if constexpr (kPair) cluster_sync_all();   // the peer's barriers and tensor memory are ready
   tc_fence_after();
   const uint32_t tmem = tmem_slot;
+  asm volatile("griddepcontrol.launch_dependents;");   // (the merge waits for the whole grid)
 
   if (warp == 0) {
     // ---- TMA producer: one ring across all of this CTA's tiles ----
@@ -508,12 +510,14 @@ __global__ void __launch_bounds__(kThreads, 1)
 // Merges the partial (max, sum) of each row into the row's normaliser: one
 // block per row, so that a few rows with a thousand partials each do not wait
 // on one warp's loads (partials in order within each thread, then across
-// lanes and warps).
+// lanes and warps).  Launched as a programmatic dependent of lm_head_kernel: its
+// blocks are already waiting when that kernel ends.
 constexpr int kMergeThreads = 128;
 __global__ void __launch_bounds__(kMergeThreads)
     lm_head_merge_kernel(const float2* __restrict__ part, int n_parts, float c_hi, float c_lo,
                          float2* __restrict__ out) {
   __shared__ float red[2][kMergeThreads / 32];
+  asm volatile("griddepcontrol.wait;" ::: "memory");   // the partials are there
   const int row = blockIdx.x, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   const float2* p = part + (size_t)row * n_parts;
   constexpr int kKeep = 8;          // partials kept in registers (1024 a row)
@@ -686,8 +690,37 @@ bool gemm_device(int device, GemmDevice* out) {
 
 }  // namespace
 
-int tv_lm_head_parts(int V) {
-  return tvk::gemm::kParts * ((V + 127) / 128);   // the narrowest tile is 128 columns
+namespace {
+
+// One row tile: single SMs, bound by W's bytes; more: SM pairs.
+bool pairs_for(int M) { return M > tvk::gemm::kBM; }
+
+int width_for(int M, int V, const GemmDevice& g) {
+  const bool pair = pairs_for(M);
+  const int tile_rows = pair ? 2 * tvk::gemm::kBM : tvk::gemm::kBM;
+  return tile_width((M + tile_rows - 1) / tile_rows, V, pair ? g.pairs : g.sms, pair,
+                    pair ? 256 : 64);
+}
+
+}  // namespace
+
+size_t tv_lm_head_scratch(int rows, int V) {
+  using namespace tvk::gemm;
+  int device = 0;
+  GemmDevice g;
+  if (cudaGetDevice(&device) != cudaSuccess || device < 0 || device >= kGemmDevices ||
+      !gemm_device(device, &g)) {
+    cudaGetLastError();
+    return 0;
+  }
+  // the most any call of up to `rows` rows takes (the width depends on its row
+  // tiles only)
+  size_t most = 0;
+  for (int M = std::min(rows, kBM);; M = std::min(rows, (M / (2 * kBM) + 1) * 2 * kBM)) {
+    const int bn = width_for(M, V, g);
+    most = std::max(most, (size_t)M * kParts * ((V + bn - 1) / bn));
+    if (M >= rows) return most;
+  }
 }
 
 int tv_launch_lm_head(const void* hidden, const void* weight, int M, int K, int V, float c_hi,
@@ -702,14 +735,13 @@ int tv_launch_lm_head(const void* hidden, const void* weight, int M, int K, int 
     cudaGetLastError();
     return -5;
   }
-  // one row tile: single SMs, bound by W's bytes; more: SM pairs
-  const bool pair = M > kBM;
+  const bool pair = pairs_for(M);
   const int tile_rows = pair ? 2 * kBM : kBM;
   const int units = pair ? g.pairs : g.sms;
   const int m_tiles = (M + tile_rows - 1) / tile_rows;
   Shape shape;
   shape.a_box = std::min(kBM, (M + 7) / 8 * 8);
-  shape.bn = tile_width(m_tiles, V, units, pair, pair ? 256 : 64);
+  shape.bn = width_for(M, V, g);
   shape.stages = (int)std::min<size_t>(
       kMaxStages, kRingBytes / (shape.a_bytes() + shape.b_bytes(pair)));
   CUtensorMap map_h, map_w;
@@ -727,8 +759,19 @@ int tv_launch_lm_head(const void* hidden, const void* weight, int M, int K, int 
     cudaGetLastError();
     return -5;
   }
-  lm_head_merge_kernel<<<M, kMergeThreads, 0, stream>>>(part, n_tiles * kParts, c_hi, c_lo,
-                                                        row_stats);
-  if (cudaGetLastError() != cudaSuccess) return -5;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)M, 1, 1);
+  cfg.blockDim = dim3(kMergeThreads, 1, 1);
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  if (cudaLaunchKernelEx(&cfg, lm_head_merge_kernel, (const float2*)part, n_tiles * kParts, c_hi,
+                         c_lo, row_stats) != cudaSuccess) {
+    cudaGetLastError();
+    return -5;
+  }
   return 0;
 }

@@ -133,11 +133,12 @@ int tv_launch_flow(const TravArgs& a, FlowArgs f, int logit_is_bf16, const FlowP
 
 // ---- LM head fused with the row normalisers (tv_gemm.cu) ----
 
-// Partial normalisers per row at most (the per-row workspace of tv_launch_lm_head).
-int tv_lm_head_parts(int V);
+// Partial normalisers (float2) that calls of up to `rows` rows need on the current
+// device; 0 on a CUDA error.
+size_t tv_lm_head_scratch(int rows, int V);
 // logits[M][V] (bf16) = hidden[M][K] x weight[V][K]^T (bf16) on the tensor
 // cores, and row_stats[M] = (max, sum of 2^((l - max) (c_hi + c_lo))) of the
-// stored logits.  part is [M][tv_lm_head_parts(V)] scratch.  Requires K % 64
+// stored logits.  part holds tv_lm_head_scratch(M, V) entries.  Requires K % 64
 // == 0, V % 8 == 0 and 16-byte aligned arrays.  0 on success, -5 on a CUDA
 // or tensor-map error.
 int tv_launch_lm_head(const void* hidden, const void* weight, int M, int K, int V, float c_hi,
