@@ -378,7 +378,7 @@ int tv_create(tv_handle** out, int device, int vocab, int max_nodes, int max_bat
     const FlowPlan fp = flow_plan(h, max_nodes + 1, 1);
     int min_slice = fp.slice_min;
     while (tv_flow_workspace_bytes(max_batch, max_nodes + 1, vocab, min_slice) > (1ull << 30) &&
-           min_slice < fp.slice_pass)
+           min_slice * 2 <= fp.slice_pass)
       min_slice *= 2;
     h->flow_force[4] = min_slice;
     h->flow_ws_bytes = tv_flow_workspace_bytes(max_batch, max_nodes + 1, vocab,

@@ -1375,8 +1375,13 @@ FlowPlan tv_flow_plan(int R, int B, int V, int smem_per_sm, int smem_per_block, 
   // the largest slices grow with the batch: while many trees stream at once
   // every CTA is busy anyway, and larger slices mean fewer queue items,
   // partials and combines per byte (at 1024 trees of 128256 tokens, 32768-
-  // token slices stream 14 % faster than 8192; at 128 trees, where a job's
-  // latency sets the time, 8192 is best).  From 1024 trees a pass takes a
+  // token slices stream 14 % faster than 8192).  Below 1024 trees they are whole
+  // ring stages of bf16 rows (3072 tokens of a pass, 9216 of a normaliser):
+  // 9216 / 18432 up to 159 trees, where a job's latency sets the time, 18432 /
+  // 36864 up to 383 and 27648 / 55296 above, against 8192 / 16384 and, from 256
+  // trees, 16384 / 32768 (60 nodes; us): V = 128256, B = 128 379 -> 377; V = 151936,
+  // B = 200 582 -> 563, B = 256 682 -> 675, B = 512 1268 -> 1230 (120 nodes 1771 ->
+  // 1680).  From 1024 trees a pass takes a
   // quarter row per slice and a normaliser half a row when that is larger
   // (V = 151936: 4 % faster than 32768 for both; V = 128256: 64512-token
   // normaliser slices, 4 % faster), rounded up to whole ring stages of bf16
@@ -1388,9 +1393,9 @@ FlowPlan tv_flow_plan(int R, int B, int V, int smem_per_sm, int smem_per_block, 
   const long long row_unit = tvk::flow::flow_stage_bytes(p.ncw) / 2;
   auto up_to = [](long long x, long long unit) { return (int)((x + unit - 1) / unit * unit); };
   p.slice_pass = B >= 1024 ? std::max(32768, up_to((V + 3LL) / 4, pass_unit))
-                           : (B >= 256 ? 16384 : 8192);
+                           : (B >= 384 ? 27648 : (B >= 160 ? 18432 : 9216));
   p.slice_stats = B >= 1024 ? std::max(32768, up_to((V + 1LL) / 2, row_unit))
-                            : (B >= 256 ? 32768 : 16384);
+                            : 2 * p.slice_pass;
   if (force_slice_pass >= 256 && force_slice_pass % 256 == 0) p.slice_pass = force_slice_pass;
   if (force_slice_stats >= 256 && force_slice_stats % 256 == 0) p.slice_stats = force_slice_stats;
   if (force_slice_min >= 256 && force_slice_min % 256 == 0) p.slice_min = force_slice_min;

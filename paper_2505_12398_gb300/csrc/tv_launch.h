@@ -109,8 +109,8 @@ struct FlowArgs {
 struct FlowPlan {
   int ncw = 4;                   // consumer warps per CTA (4 or 8)
   int stages = 3;                // ring stages of 3 KB per consumer warp
-  int slice_pass = 8192;         // largest slice of a pass / bonus draw (tokens; by batch)
-  int slice_stats = 16384;       // largest slice of a row normaliser (tokens; by batch)
+  int slice_pass = 9216;         // largest slice of a pass / bonus draw (tokens; by batch)
+  int slice_stats = 18432;       // largest slice of a row normaliser (tokens; by batch)
   int slice_min = 2048;          // slices shrink to this as fewer trees remain
   size_t smem = 0;
   bool ok = false;

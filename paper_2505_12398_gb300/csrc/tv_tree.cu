@@ -401,18 +401,16 @@ struct TreeCta {
     if (++st == n_stages) st = 0;
   }
 
-  // Whether all of this warp's tiles of a pair chunk (n tokens from element x of
-  // the slice's first block, which starts sh elements before the slice) are
-  // whole and hold no removed token (the same in the whole warp).
-  __device__ __forceinline__ bool plain_tiles(int n, int x, int sh, bool ragged, const int* mt,
-                                              int nmask, int wid) const {
-    if (ragged || n < (wid + (kTiles - 1) * NCW + 1) * kTileElems) return false;
-    const int xs = v0 - sh + x;
+  // Whether a removed token lies in this warp's tiles of a pair chunk (n tokens
+  // from element x of the slice; the same in the whole warp).
+  __device__ __forceinline__ bool removed_here(int n, int x, const int* mt, int nmask,
+                                               int wid) const {
+    const int xs = v0 + x;
     for (int k = 0; k < nmask; ++k) {
       const int off = mt[k] - xs;
-      if ((unsigned)off < (unsigned)n && (off / kTileElems) % NCW == wid) return false;
+      if ((unsigned)off < (unsigned)n && (off / kTileElems) % NCW == wid) return true;
     }
-    return true;
+    return false;
   }
 
   // Row normalisers: this warp's group takes every g-th row.
@@ -516,17 +514,30 @@ struct TreeCta {
       const E* lb = reinterpret_cast<const E*>(buf);
       const float* qb = reinterpret_cast<const float*>(buf + (size_t)kPair * kLB);
       const int n = min(per, sl.n - x);
-      if (kind == kJobPass && plain_tiles(n, x, sl.sh, ragged, mt, nmask, wid)) {
-        float v[kTiles][8], t[kTiles][8];
+      if (kind == kJobPass && !ragged && !removed_here(n, x, mt, nmask, wid)) {
+        int t0 = wid * kTileElems;
+        if (n >= t0 + (kTiles - 1) * kSweep + kTileElems) {   // all of the warp's tiles, whole
+          float v[kTiles][8], t[kTiles][8];
 #pragma unroll
-        for (int k = 0; k < kTiles; ++k)
-          lds_logits<L>(lb + (wid + k * NCW) * kTileElems + lane * kChunk, v[k]);
+          for (int k = 0; k < kTiles; ++k)
+            lds_logits<L>(lb + t0 + k * kSweep + lane * kChunk, v[k]);
 #pragma unroll
-        for (int k = 0; k < kTiles; ++k)
-          residual8<L, kExact>(v[k], qb + (wid + k * NCW) * kTileElems + lane * kChunk, rm, al,
-                               be, c_hi, c_lo, t[k]);
+          for (int k = 0; k < kTiles; ++k)
+            residual8<L, kExact>(v[k], qb + t0 + k * kSweep + lane * kChunk, rm, al, be, c_hi,
+                                 c_lo, t[k]);
 #pragma unroll
-        for (int k = 0; k < kTiles; ++k) acc.add(sum8(t[k]));
+          for (int k = 0; k < kTiles; ++k) acc.add(sum8(t[k]));
+        } else {
+          for (; t0 < n; t0 += kSweep) {
+            const int e0 = t0 + lane * kChunk;
+            if (e0 < n) {
+              float v[8], t[8];
+              lds_logits<L>(lb + e0, v);
+              residual8<L, kExact>(v, qb + e0, rm, al, be, c_hi, c_lo, t);
+              acc.add(sum8(t));
+            }
+          }
+        }
         end_chunk(q, total, st, lane);
         continue;
       }
@@ -1273,17 +1284,19 @@ FusedPlan tv_fused_plan(int B, int R, int V, int logit_bytes, int smem_per_sm,
   //   V = 262144, B = 32: 8x8 255, 4x8 341, 16x4 346, 8x4 364
   //   V = 32000, B = 1: 8x16 63, 8x8 65, 4x8 71; B = 16: 8x8 120, 4x8 124, 8x16 143
   //   V = 32000, B = 64: 8x4 149, 4x8 154, 8x8 160; B = 128: 4x4 191, 8x2 192, 8x4 212
-  //   V = 32000, B = 400: 8x2 377, 8x1 385, 4x4 431; B = 1024: 8x1 651, 8x2 731
-  //   V = 16384, B = 300: 8x1 232, 8x2 244; V = 8000 (26 nodes): 8x1 117, 8x2 158
-  //   V = 1000, B = 1024 (26 nodes): 4x1 213, 8x1 280
-  // (B = 1, 16 and V <= 16384 before the consumers took a chunk's tiles together)
+  //   V = 32000, B = 200: 8x2 230, 4x4 255, 4x2 280; B = 256: 4x2 250, 8x1 260, 8x2 261;
+  //   B = 512: 4x2 386, 8x1 388, 8x2 399; B = 1024: 4x2 661, 8x1 662, 4x1 727, 8x2 731
+  //   V = 16384, B = 300: 4x2 195, 8x1 200, 8x2 232; B = 1024: 8x1 470, 4x1 479
+  //   V = 4000, B = 512: 4x1 183, 8x1 235; V = 8000, B = 1024 (26 nodes): 4x1 258, 8x1 308
+  // (B = 1 and 16 before the consumers took a chunk's tiles together)
   int ncw = 8, C = 1;
   if (V > 98304 && B <= 4) ncw = 16, C = 16;
   else if (B <= 8 || (V > 98304 && B <= 16)) C = 16;
   else if (B <= 32) C = 8;
   else if (B <= 76) C = 4;
-  else if (B <= 152 || (B <= 400 && V > 20000)) C = 2;
-  else if (V <= 4096) ncw = 4;
+  else if (B <= 224) C = 2;
+  else if (B <= 320 || (B <= 512 && V > 20000)) ncw = 4, C = 2;
+  else if (V <= 12288) ncw = 4;
   while (C > 1 && V / C < 1000) C /= 2;
   while (C < 8 && tree_tiles(V, C) * 8 > 32768) C *= 2;   // bonus tiles' shared memory
   if (force_ncw == 4 || force_ncw == 8 || force_ncw == 16) ncw = force_ncw;
