@@ -19,10 +19,10 @@
 //     tile's W rows in its shared memory; the leader issues the MMAs of both.
 //     Each SM then loads 32 KB for a stage's 128 x 256 x 64 multiply-adds
 //     instead of the 48 KB that a tile of its own takes.  Bound by the tensor
-//     cores (86 % of their cycles busy at 3904 x 4096 x 32000, the clock at 1.8
-//     GHz under the power cap; 27 waves for 26.3, 4096 rows for 3904):
-//     645 -> 618 us there, 976 x 4096 x 128256 702 -> 585 us, 7808 x 4096 x 128256
-//     4929 -> 4898 us, against single SMs with 4 epilogue warps.
+//     cores and the clock that the power cap leaves them (27 waves for 26.3 and 4096
+//     rows for 3904 at 3904 x 4096 x 32000): 645 -> 618 us there, 976 x 4096 x
+//     128256 702 -> 585 us, 7808 x 4096 x 128256 4929 -> 4898 us, against single
+//     SMs with 4 epilogue warps.
 //   * single SMs (up to 128 rows): 128 x bn tiles, W's bytes from HBM bound
 //     it.  Only the box of H rows that exist is loaded (the MMA's other rows
 //     read whatever is next in shared memory; their results are not used).
@@ -33,13 +33,17 @@
 // programmatic dependent launch), 188.9 -> 163 us there (157 us of bytes at 6.8
 // TB/s; 165 us without that launch), one row 225 -> 156 us.
 // In both:
-//   * warp 0 (one lane) streams 64-element K slices of H and W into a ring of
-//     shared memory with 2-D TMA copies (128-byte swizzle, the layout the
-//     tensor cores read), across tile boundaries;
+//   * warp 0 streams 64-element K slices of H and W into a ring of shared
+//     memory with 2-D TMA copies (128-byte swizzle, the layout the tensor cores
+//     read), across tile boundaries;
 //   * warp 1 allocates all 512 columns of tensor memory, two fp32
-//     accumulators of up to 256 columns, and one lane (of the leader) issues
-//     tcgen05.mma (K=16 per instruction) into them in turn, releasing each stage
-//     with tcgen05.commit;
+//     accumulators of up to 256 columns, and (of the leader) issues tcgen05.mma
+//     (K=16 per instruction) into them in turn, releasing each stage with
+//     tcgen05.commit.  Both loops run in the whole warp and one elected lane
+//     issues (elect_one): with loops of one lane the tensor cores waited for the
+//     issue, 618 -> 590 us at 3904 x 4096 x 32000, 4929 -> 4608 us at 7808 x 4096 x
+//     128256, 750 -> 695 us at 1952 x 2048 x 151936 (and 536 -> 469, 4000 -> 3477
+//     us for the first two on operands of zeros, where no power cap bounds it);
 //   * warps 2-9 (two per TMEM lane quarter, each taking every other 32
 //     columns, one row per thread) read the finished accumulator with
 //     tcgen05.ld, round to bf16, store the logits and keep the row's running
@@ -142,6 +146,19 @@ __device__ __forceinline__ void tile_coords(int t, int m_tiles, int n_tiles, int
     mt = (m_tiles / g) * g + r % gt;
     nt = r / gt;
   }
+}
+
+// True in one lane of a converged warp.  The loops around the tensor-core and TMA
+// instructions run in the whole warp with those instructions alone in the chosen
+// lane: their operands (descriptors, addresses, coordinates) then stay in the
+// warp's uniform registers, which the instructions read, instead of being moved
+// there one by one from a divergent lane's.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(p));
+  return p != 0;
 }
 
 template <bool kPair>
@@ -248,6 +265,10 @@ __device__ __forceinline__ void st_global_32b(void* p, const uint32_t* w) {   //
                : "memory");
 }
 
+__device__ __forceinline__ bool wait_warp(uint64_t* bar, uint32_t parity) {
+  return __all_sync(0xffffffffu, mbar_wait(bar, parity) ? 1 : 0) != 0;
+}
+
 // Launch shape: tile width, H rows a TMA box takes per CTA, ring stages.
 struct Shape {
   int bn, a_box, stages;
@@ -336,7 +357,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   const uint32_t raw = smem_u32(smem_raw);
   uint8_t* smem = smem_raw + (((raw + 1023u) & ~1023u) - raw);
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
   const uint32_t rank = kPair ? cluster_rank() : 0u;
   const int first = kPair ? (int)blockIdx.x >> 1 : (int)blockIdx.x;
   const int step = kPair ? (int)gridDim.x >> 1 : (int)gridDim.x;
@@ -369,40 +390,41 @@ __global__ void __launch_bounds__(kThreads, 1)
 
   if (warp == 0) {
     // ---- TMA producer: one ring across all of this CTA's tiles ----
-    if (lane == 0) {
-      uint32_t it = 0, s = 0, ph = 0;
-      bool ok = true;
-      for (int t = first; t < n_total && ok; t += step) {
-        int mt, nt;
-        tile_coords(t, m_tiles, n_tiles, group, mt, nt);
-        const int m0 = mt * tile_rows + (int)rank * kBM, n0 = nt * bn + (int)rank * bn_own;
-        for (int kb = 0; kb < nkb; ++kb, ++it) {
-          if (it >= n_stages && !mbar_wait(&empty_bar[s], ph ^ 1u)) {
-            ok = false;
-            break;
-          }
-          uint8_t* a = smem + (size_t)s * stage_bytes;
-          uint32_t bar = smem_u32(&full_bar[s]);
-          if constexpr (kPair) bar = map_shared(&full_bar[s], 0);
+    uint32_t it = 0, s = 0, ph = 0;
+    bool ok = true;
+    for (int t = first; t < n_total && ok; t += step) {
+      int mt, nt;
+      tile_coords(t, m_tiles, n_tiles, group, mt, nt);
+      const int m0 = mt * tile_rows + (int)rank * kBM, n0 = nt * bn + (int)rank * bn_own;
+      for (int kb = 0; kb < nkb; ++kb, ++it) {
+        if (it >= n_stages && !wait_warp(&empty_bar[s], ph ^ 1u)) {
+          ok = false;
+          break;
+        }
+        uint8_t* a = smem + s * stage_bytes;
+        uint32_t bar = smem_u32(&full_bar[s]);
+        if constexpr (kPair) bar = map_shared(&full_bar[s], 0);
+        if (elect_one()) {
           // (kPair: the leader's barrier counts both CTAs' bytes)
           if (rank == 0) mbar_arrive_expect_tx(&full_bar[s], kPair ? 2 * stage_bytes : stage_bytes);
           tma_load_2d<kPair>(a, &map_h, kb * kBK, m0, bar);
           tma_load_2d<kPair>(a + a_bytes, &map_w, kb * kBK, n0, bar);
-          if (++s == n_stages) { s = 0; ph ^= 1u; }
         }
+        __syncwarp();
+        if (++s == n_stages) { s = 0; ph ^= 1u; }
       }
-      if (!ok) failed = 1;
-      // the copies issued last have landed before the CTA may exit (kPair: the
-      // leader waits for both CTAs' copies, the peer for the leader at the end)
-      if (rank == 0)
-        for (uint32_t j = it > n_stages ? it - n_stages : 0u; j < it; ++j)
-          if (!mbar_wait(&full_bar[j % n_stages], (j / n_stages) & 1)) failed = 1;
     }
-    __syncwarp();
+    if (!ok) failed = 1;
+    // the copies issued last have landed before the CTA may exit (kPair: the
+    // leader waits for both CTAs' copies, the peer for the leader at the end)
+    if (rank == 0)
+      for (uint32_t j = it > n_stages ? it - n_stages : 0u; j < it; ++j)
+        if (!wait_warp(&full_bar[j % n_stages], (j / n_stages) & 1)) failed = 1;
   } else if (warp == 1) {
-    // ---- tensor-core issue (one lane), the two accumulators in turn ----
-    if (lane == 0 && rank == 0) {
+    // ---- tensor-core issue, the two accumulators in turn ----
+    if (rank == 0) {
       const uint32_t idesc = instr_desc(tile_rows, bn);
+      const uint64_t desc0 = smem_desc(smem);
       uint32_t s = 0, ph = 0;
       bool ok = true;
       int j = 0;
@@ -410,7 +432,9 @@ __global__ void __launch_bounds__(kThreads, 1)
         const uint32_t acc = (uint32_t)j & 1u;
         if (j >= kAccBufs) {
           const uint32_t par = ((j >> 1) - 1) & 1;
-          if (!(kPair ? mbar_wait_cluster(&acc_empty[acc], par) : mbar_wait(&acc_empty[acc], par))) {
+          const bool got = kPair ? mbar_wait_cluster(&acc_empty[acc], par)
+                                 : mbar_wait(&acc_empty[acc], par);
+          if (!__all_sync(0xffffffffu, got)) {
             ok = false;
             break;
           }
@@ -418,32 +442,35 @@ __global__ void __launch_bounds__(kThreads, 1)
         tc_fence_after();
         const uint32_t d = tmem + acc * (uint32_t)kBN;
         for (int kb = 0; kb < nkb; ++kb) {
-          if (!mbar_wait(&full_bar[s], ph)) {
+          if (!wait_warp(&full_bar[s], ph)) {
             ok = false;
             break;
           }
           tc_fence_after();
-          const uint8_t* a = smem + (size_t)s * stage_bytes;
-          const uint64_t da = smem_desc(a), db = smem_desc(a + a_bytes);
+          // (the start address field counts 16 bytes)
+          const uint64_t da = desc0 + (uint64_t)((s * stage_bytes) >> 4);
+          const uint64_t db = da + (uint64_t)(a_bytes >> 4);
+          if (elect_one()) {
 #pragma unroll
-          for (int k = 0; k < kBK / kUmmaK; ++k) {
-            const uint64_t off = (uint64_t)((k * kUmmaK * 2) >> 4);   // 32 bytes of K
-            umma_bf16<kPair>(d, da + off, db + off, idesc, (kb > 0 || k > 0) ? 1u : 0u);
+            for (int k = 0; k < kBK / kUmmaK; ++k) {
+              const uint64_t off = (uint64_t)((k * kUmmaK * 2) >> 4);   // 32 bytes of K
+              umma_bf16<kPair>(d, da + off, db + off, idesc, (kb > 0 || k > 0) ? 1u : 0u);
+            }
+            umma_commit<kPair>(&empty_bar[s]);   // the stage is free once these MMAs are done
+            if (kb == nkb - 1) umma_commit<kPair>(&acc_full[acc]);   // the accumulator is complete
           }
-          umma_commit<kPair>(&empty_bar[s]);   // the stage is free once these MMAs are done
+          __syncwarp();
           if (++s == n_stages) { s = 0; ph ^= 1u; }
         }
-        if (ok) umma_commit<kPair>(&acc_full[acc]);   // the accumulator is complete
       }
       if (!ok) failed = 1;
       // every MMA issued has finished before tensor memory is freed
-      umma_commit<kPair>(&drain_bar);
-      if (!mbar_wait(&drain_bar, 0)) failed = 1;
-    } else if (kPair && lane == 0) {
-      // the leader's last signal: none is on its way to this CTA after it
-      if (!mbar_wait(&drain_bar, 0)) failed = 1;
+      if (elect_one()) umma_commit<kPair>(&drain_bar);
+      __syncwarp();
     }
-    __syncwarp();
+    // (kPair, the peer: the leader's last signal; none is on its way to this CTA
+    // after it)
+    if (!wait_warp(&drain_bar, 0)) failed = 1;
   } else {
     // ---- epilogue: one row per thread, every other 32-column chunk ----
     const int q = warp & 3;                       // the TMEM lane quarter of this warp
