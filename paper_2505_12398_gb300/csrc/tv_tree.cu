@@ -48,9 +48,9 @@
 //
 // Measured (60-node trees, bf16; 8-token chains, fp32), against one thread of the
 // consumers doing the control, a reduction and an exchange per row and no
-// resident pairs: V = 32000, B = 64 254 -> 143 us (183 with a row by all warps in turn
+// resident pairs: V = 32000, B = 64 254 -> 141 us (183 with a row by all warps in turn
 // and before the removal of a rate-0 sibling and the descent into a sub-tree were
-// worked out ahead, 149 one tile at a time); 16 chains 117 -> 64 us; V = 128256, B =
+// worked out ahead, 149 one tile at a time); 16 chains 117 -> 63 us; V = 128256, B =
 // 32 368 -> 184 us (213 one tile at a time).
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -248,7 +248,8 @@ struct TreeCta {
   float2* xs;              // [2][exchange_slots] partials of all CTAs
   int* mtok_ahead;         // [2][R] removed tokens of passes worked out ahead
   float* u;                // [R + 1] the tree's uniforms
-  uint64_t *full_bar, *empty_bar, *xbar, *job_bar, *ack_bar, *stat_bar, *tile_bar;
+  uint64_t *full_bar, *empty_bar, *xbar, *job_bar, *ack_bar, *stat_bar, *tile_bar,
+      *order_bar;
   int C, n_stages, b, v0, v1;
   int spc;                 // stages a resident pair takes
   int max_groups;          // groups of a normaliser job at most
@@ -624,7 +625,7 @@ struct TreeCta {
   __device__ bool finish_rows(const TreeJob& job, int wid, int lane) {
     const float c_hi = a.c_hi, c_lo = a.c_lo;
     const int n_rows = job.n_rows, n = C * (NCW / row_groups(n_rows, max_groups));
-    if (!exchanged(job.xb, job.xph)) return false;
+    if (!exchanged(job.xb, job.xph) || !mbar_wait_warp(order_bar, 0u)) return false;
     for (int r = wid; r < n_rows; r += NCW) {
       const float2* x = xslots(job.xb) + r * n;
       float M = TV_NEG_INF;
@@ -954,6 +955,21 @@ struct TreeCta {
       ah.ok = 0;
       if (ahead) prepare_ahead(s, ctl, ah, mtok(mnext), u);
     }
+    if (!a.row_stats) {
+      // the first job is a normaliser's (or a leaf's draw): the children's order
+      // is needed only once it is done (before the first job: 64.4 -> 62.5 us at 16
+      // chains of 8, 113.6 -> 111.8 us at 16 and 142.3 -> 141.2 us at 64 trees of 60
+      // nodes, V = 32000)
+      __syncwarp();
+      if (sh.ctl.job.kind == kJobStats) {
+        const int R = a.N + 1;
+        for (int i = lane; i < R; i += 32) children_order(s, i);
+        __syncwarp();
+        for (int i = lane + 1; i < R; i += 32) child_order(s, i);
+        __syncwarp();
+      }
+      if (lane == 0) mbar_arrive(order_bar);
+    }
     for (;;) {
       __syncwarp();
       ok = __shfl_sync(0xffffffffu, ok, 0);
@@ -1080,7 +1096,7 @@ __global__ void __launch_bounds__(TreeCta<L, NCW, kExact>::kThreads, 16 / NCW)
   __shared__ __align__(8) uint64_t full_bar[kTreeMaxStages];
   __shared__ __align__(8) uint64_t empty_bar[kTreeMaxStages];
   __shared__ __align__(8) uint64_t xbar[2];
-  __shared__ __align__(8) uint64_t job_bar, ack_bar, stat_bar, tile_bar;
+  __shared__ __align__(8) uint64_t job_bar, ack_bar, stat_bar, tile_bar, order_bar;
   __shared__ TreeShared sh;
 
   const int R = args.N + 1, V = args.V;
@@ -1110,6 +1126,7 @@ __global__ void __launch_bounds__(TreeCta<L, NCW, kExact>::kThreads, 16 / NCW)
   t.ack_bar = &ack_bar;
   t.stat_bar = &stat_bar;
   t.tile_bar = &tile_bar;
+  t.order_bar = &order_bar;
   const TreeSmem& s = t.s;
   Ctl& ctl = sh.ctl;
   const typename L::elem* logits = reinterpret_cast<const typename L::elem*>(args.logits);
@@ -1126,6 +1143,7 @@ __global__ void __launch_bounds__(TreeCta<L, NCW, kExact>::kThreads, 16 / NCW)
     mbar_init(&ack_bar, 1);
     mbar_init(&stat_bar, NCW);
     mbar_init(&tile_bar, NCW);
+    mbar_init(&order_bar, 1);
     fence_mbar_init();
     ctl.bad = 0u;
     ctl.accepted = -1;
@@ -1191,45 +1209,38 @@ __global__ void __launch_bounds__(TreeCta<L, NCW, kExact>::kThreads, 16 / NCW)
     if (bad) atomicOr(&ctl.bad, bad);
   }
   __syncthreads();
-  if (ctl.bad == 0u)
-    for (int i = tid; i < R; i += T::kThreads) children_order(s, i);
-  __syncthreads();
-  if (ctl.bad == 0u) {
-    for (int i = tid + 1; i < R; i += T::kThreads) child_order(s, i);
-    if (args.row_stats) {
-      // given normalisers (from the LM head's epilogue, or the three-kernel
-      // path's): every internal row is normalised up front and no normaliser
-      // job is ever posted
+  if (args.row_stats) {
+    // given normalisers (from the LM head's epilogue, or the three-kernel
+    // path's): every internal row is normalised up front and no normaliser job
+    // is ever posted.  (Otherwise the control warp works out the children's order
+    // while the first normaliser job runs.)
+    if (ctl.bad == 0u) {
       uint32_t bad = 0u;
       for (int i = tid; i < R; i += T::kThreads) {
         if (s.first[i] < 0) continue;
+        children_order(s, i);
         const float2 st = args.row_stats[t.row0 + i];
-        const double invs = 1.0 / (double)st.y;
         s.rowm[i] = st.x;
         s.rows[i] = st.y;
-        s.invs[i] = invs;
+        s.invs[i] = 1.0 / (double)st.y;
         if (!(st.y > 0.f)) bad |= 64u;
       }
       if (bad) atomicOr(&ctl.bad, bad);
     }
-    if (tid == 0) s.p[0] = 1.0;
-  } else if (tid == 0) {
-    ctl.job.kind = kJobDone;
+    __syncthreads();
+    if (ctl.bad == 0u)
+      for (int i = tid + 1; i < R; i += T::kThreads) {
+        child_order(s, i);
+        set_child_mass(s, i, s.rowm[s.par[i]], s.invs[s.par[i]], args.c);
+      }
+    __syncthreads();
+  }
+  if (tid == 0) {
+    if (ctl.bad == 0u) s.p[0] = 1.0;
+    else ctl.job.kind = kJobDone;
   }
   if (C > 1) cluster_sync_all();   // peers' barriers initialised before any remote store
   else __syncthreads();
-  if (args.row_stats) {
-    const uint32_t bad = ctl.bad;
-    __syncthreads();
-    if (bad == 0u) {
-      for (int i = tid + 1; i < R; i += T::kThreads)
-        set_child_mass(s, i, s.rowm[s.par[i]], s.invs[s.par[i]], args.c);
-    } else if (tid == 0) {
-      ctl.job.kind = kJobDone;
-    }
-    __syncthreads();
-  }
-
   if (wid < NCW) {
     t.consumer(wid, lane);
   } else if (wid == NCW) {
