@@ -89,7 +89,6 @@ constexpr uint32_t kRowBytes = kBK * 2;         // one row of a stage's operand 
 constexpr int kAccBufs = 2;                     // accumulators in tensor memory
 constexpr uint32_t kTmemCols = kAccBufs * kBN;  // fp32: one column per output column
 constexpr size_t kSmemBytes = kRingBytes + 1024;   // + alignment slack
-constexpr int kParts = 2;         // partial normalisers per row and tile (column chunks by parity)
 
 // Instruction descriptor of tcgen05.mma kind::f16: fp32 accumulator (bits
 // 4-5 = 1), bf16 A and B (bits 7-9, 10-12 = 1), both K-major (bits 15, 16 =
@@ -335,8 +334,8 @@ __device__ __forceinline__ void store_and_sum(const uint32_t (&r)[32], __nv_bflo
 
 // The tiles t = first, first + step, ... of l = H W^T (in the order of
 // tile_coords), stored as bf16, and each row's (max, sum of 2^((l - max) c))
-// over the even and the odd 32-column chunks of a tile in part[row][2 tile +
-// parity].  kPair: launched as clusters of two CTAs.
+// over a tile's columns in part[row][tile].  kPair: launched as clusters of two
+// CTAs.
 template <bool kPair>
 __global__ void __launch_bounds__(kThreads, 1)
     lm_head_kernel(const __grid_constant__ CUtensorMap map_h,
@@ -351,6 +350,10 @@ __global__ void __launch_bounds__(kThreads, 1)
   __shared__ __align__(8) uint64_t acc_empty[kAccBufs];   // accumulator read (epilogue warps;
                                                           // kPair: the leader's is used)
   __shared__ __align__(8) uint64_t drain_bar;
+  // the odd chunks' (max, sum) of a row, from one warp of a lane quarter to the other
+  __shared__ __align__(8) uint64_t half_full[4];
+  __shared__ __align__(8) uint64_t half_empty[4];
+  __shared__ float2 half_ms[kBM];
   __shared__ uint32_t tmem_slot;
   __shared__ int failed;
   // the TMA tiles need 1024-byte alignment (128-byte swizzle atoms)
@@ -377,6 +380,10 @@ __global__ void __launch_bounds__(kThreads, 1)
       mbar_init(&acc_empty[k], kPair ? 2 * kEpiWarps : kEpiWarps);
     }
     mbar_init(&drain_bar, 1);
+    for (int k = 0; k < 4; ++k) {
+      mbar_init(&half_full[k], 1);
+      mbar_init(&half_empty[k], 1);
+    }
     failed = 0;
     fence_mbar_init();
   }
@@ -519,8 +526,31 @@ __global__ void __launch_bounds__(kThreads, 1)
         if (row < M && n > 0)
           store_and_sum(r, logits + (size_t)row * V + col0, n, wide, ch, cl, m_run, s_run);
       }
-      if (row < M)
-        part[((size_t)row * n_tiles + n_tile) * kParts + half] = make_float2(m_run, s_run);
+      // the quarter's two warps: one partial per row and tile (one from each doubles
+      // the scratch that a new handle allocates: its first pass over 183 rows of 2304,
+      // V = 151936, took 284 us for 193; repeated passes 136 for 132)
+      if (half == 1) {
+        if (j > 0 && !wait_warp(&half_empty[q], (j - 1) & 1)) {
+          if (lane == 0) failed = 1;
+          break;
+        }
+        half_ms[q * 32 + lane] = make_float2(m_run, s_run);
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&half_full[q]);
+      } else {
+        if (!wait_warp(&half_full[q], j & 1)) {
+          if (lane == 0) failed = 1;
+          break;
+        }
+        const float2 o = half_ms[q * 32 + lane];
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&half_empty[q]);
+        const float mx = fmaxf(m_run, o.x);
+        float sum = 0.f;
+        if (m_run != TV_NEG_INF) sum = s_run * exp2_split(m_run - mx, 0.f, c_hi, c_lo);
+        if (o.x != TV_NEG_INF) sum += o.y * exp2_split(o.x - mx, 0.f, c_hi, c_lo);
+        if (row < M) part[(size_t)row * n_tiles + n_tile] = make_float2(mx, sum);
+      }
     }
   }
   tc_fence_before();
@@ -745,7 +775,7 @@ size_t tv_lm_head_scratch(int rows, int V) {
   size_t most = 0;
   for (int M = std::min(rows, kBM);; M = std::min(rows, (M / (2 * kBM) + 1) * 2 * kBM)) {
     const int bn = width_for(M, V, g);
-    most = std::max(most, (size_t)M * kParts * ((V + bn - 1) / bn));
+    most = std::max(most, (size_t)M * ((V + bn - 1) / bn));
     if (M >= rows) return most;
   }
 }
@@ -795,7 +825,7 @@ int tv_launch_lm_head(const void* hidden, const void* weight, int M, int K, int 
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  if (cudaLaunchKernelEx(&cfg, lm_head_merge_kernel, (const float2*)part, n_tiles * kParts, c_hi,
+  if (cudaLaunchKernelEx(&cfg, lm_head_merge_kernel, (const float2*)part, n_tiles, c_hi,
                          c_lo, row_stats) != cudaSuccess) {
     cudaGetLastError();
     return -5;
