@@ -35,7 +35,8 @@ struct Ctl {
   Job job;
   uint32_t bad;        // TV_STATUS_* bits
   int accepted;        // accepted node (-1: invalid tree)
-  float S;             // result of the last pass
+  float S;             // result of the last pass, in the units of its job:
+  double s_unit;       // x s_unit is the sum of Eqs. (1)/(3) (job_ahead)
   float bmargin;       // margin of the bonus draw (out_margin[b][1])
   // serial control state (thread 0)
   int node;
@@ -184,6 +185,7 @@ __device__ inline double removed_mass(const TreeSmem& s, int i, int c) {
 
 __device__ inline void post_pass(const TreeSmem& s, Ctl& ctl, int i, int c) {
   ctl.pending = c;
+  ctl.s_unit = 1.0;
   const double p = s.p[i];
   ctl.job.kind = kJobPass;
   ctl.job.n_rows = 1;
@@ -199,7 +201,7 @@ __device__ inline void post_pass(const TreeSmem& s, Ctl& ctl, int i, int c) {
 
 __device__ inline void apply_rejection(const TreeSmem& s, Ctl& ctl, int i, int c) {
   const double p = s.p[i], a = s.a[i], b = s.b[i];
-  const double S = (double)ctl.S + p * ctl.masked_sum;
+  const double S = (double)ctl.S * ctl.s_unit + p * ctl.masked_sum;
   const double alpha = p * a;
   const double beta = p * b + s.invZ[c];
   const double mb0 = s.mb0[c];
@@ -267,7 +269,9 @@ __device__ inline void post_bonus(const TreeSmem& s, Ctl& ctl, int a) {
 // Eqs. (1)-(3) give a child c2 the rate min(X / D, 1),
 //   X = [alpha M_b0(c2) - beta q(c2)]_+ Z' / q(c2),
 // and a pass that then rejects c2 uses alpha1 = alpha / (s_i D) and
-// beta' = beta / D + 1/Z'.  Only D depends on the pass's S, so of the next
+// beta' = beta / D + 1/Z', posted as 2^-e alpha / s_i and 2^-e (beta + D / Z')
+// with 2^e <= D < 2^(e+1): its sum then comes in units of D / 2^e (Ctl::s_unit) and
+// no division stands before it.  Only D depends on the pass's S, so of the next
 // remaining child c2 of i it is known before S arrives:
 //   * kAheadTest: c2 is a leaf with X > 0: it is accepted iff u D < X;
 //   * kAheadPrune: X = 0, c2 has rate 0 whatever S is: it is removed, and the
@@ -285,6 +289,10 @@ __device__ inline void post_bonus(const TreeSmem& s, Ctl& ctl, int a) {
 // With all four modes, against the leaf test and kAheadUp alone: the persistent
 // kernel at V = 128256 takes 453 -> 421 us (B = 128), 256 -> 237 us (B = 32, given
 // normalisers), the cluster kernel at V = 32000, B = 64 183 -> 148 us.
+// The passes in units of D / 2^e, with 1 / D worked out after they are posted
+// instead of before: persistent kernel, V = 128256, B = 128 408 -> 399 us; cluster
+// kernel, V = 128256, B = 32, given normalisers 117 -> 112 us, V = 32000, B = 64
+// 134 -> 132 us.
 enum : int { kAheadTest = 1, kAheadPrune = 2, kAheadDescend = 3, kAheadUp = 4 };
 
 struct Ahead {
@@ -292,7 +300,8 @@ struct Ahead {
   int mode;
   int i, c, c2, g, nmask, n_rows;
   double p, omp, pm;             // p_i, 1 - p_i, p_i x the removed tokens' mass
-  double X, alpha, beta, ainvs, invZn, mb0, q0, uu, msum_g;
+  double X, alpha, beta, invZn, mb0, q0, uu, msum_g;
+  float ainvs;                        // the next pass at i: alpha / s_i
   float alpha1_g, beta_g, rowmax_g;   // kAheadUp: the pass at g that rejects i
 };
 
@@ -347,7 +356,7 @@ __device__ inline void prepare_ahead(const TreeSmem& s, const Ctl& ctl, Ahead& a
     ah.ok = 1;
     return;
   }
-  ah.ainvs = alpha * s.invs[i];
+  ah.ainvs = (float)(alpha * s.invs[i]);
   ah.invZn = invZn;
   ah.X = y * s.zq[c2];
   ah.nmask = removed_tokens(s, i, c2, mtok2);
@@ -357,11 +366,16 @@ __device__ inline void prepare_ahead(const TreeSmem& s, const Ctl& ctl, Ahead& a
   ah.ok = 1;
 }
 
+// e with 2^e <= D < 2^(e+1), within what a float32 scale can undo.
+__device__ __forceinline__ int unit_exponent(double D) {
+  return min(max((__double2hiint(D) >> 20) - 1023, -100), 100);
+}
+
 // The next job of the step described by `ah`, given the pass's S (D = S + 1 -
-// p_i, inv_d = 1 / D where the mode needs it); false if that job needs the
-// updated state first (the residual draw at i).  `accept`: the test's outcome.
+// p_i); false if that job needs the updated state first (the residual draw at i).
+// `accept`: the test's outcome.
 __device__ inline bool job_ahead(const TreeSmem& s, const Ahead& ah, double S, double D,
-                                 double inv_d, Job& j, bool& accept) {
+                                 Job& j, bool& accept) {
   accept = false;
   j.n_rows = 1;
   j.kind = kJobPass;
@@ -388,16 +402,19 @@ __device__ inline bool job_ahead(const TreeSmem& s, const Ahead& ah, double S, d
     return true;
   }
   j.node = ah.i;
-  j.alpha1 = (float)(ah.ainvs * inv_d);
-  j.beta = (float)(ah.beta * inv_d + ah.invZn);
+  const float unit = __int_as_float((127 - unit_exponent(D)) << 23);
+  j.alpha1 = ah.ainvs * unit;
+  j.beta = (float)(ah.beta + ah.invZn * D) * unit;
   j.rowmax = s.rowm[ah.i];
   return true;
 }
 
 // Bookkeeping of a pass at i for child c whose job has been posted already
 // (msum: the stored masses of i's other removed children).
-__device__ inline void note_pass(const TreeSmem& s, Ctl& ctl, int i, int c, double msum) {
+__device__ inline void note_pass(const TreeSmem& s, Ctl& ctl, int i, int c, double msum,
+                                 double s_unit) {
   ctl.pending = c;
+  ctl.s_unit = s_unit;
   ctl.job.kind = kJobPass;
   ctl.job.n_rows = 1;
   ctl.job.node = i;
@@ -406,12 +423,12 @@ __device__ inline void note_pass(const TreeSmem& s, Ctl& ctl, int i, int c, doub
   s.npass[i]++;
 }
 
-// control_step for the pass described by `ah`, given inv_d = 1 / D, inv_s = 1 /
+// control_step for the pass described by `ah`, given D, inv_d = 1 / D, inv_s = 1 /
 // S and p_new = S / D, with the test going the way `accept` says (the decision
 // taken ahead, so that the state follows the job already posted).
 __device__ inline void control_step_ahead(const TreeSmem& s, Ctl& ctl, const Ahead& ah,
-                                          bool accept, double inv_d, double inv_s,
-                                          double p_new) {
+                                          bool accept, double D, double inv_d,
+                                          double inv_s, double p_new) {
   const int i = ah.i, c = ah.c;
   const double na = ah.alpha * inv_s, nb = ah.beta * inv_s, scale = ah.p * inv_s;
   const double mc = fmax(na * ah.mb0 - nb * ah.q0, 0.0);
@@ -431,7 +448,7 @@ __device__ inline void control_step_ahead(const TreeSmem& s, Ctl& ctl, const Ahe
       return;
     }
     s.state[i] = kRejected;
-    note_pass(s, ctl, ah.g, i, ah.msum_g);
+    note_pass(s, ctl, ah.g, i, ah.msum_g, 1.0);
     return;
   }
   if (ah.mode == kAheadDescend) {   // (control_step goes down to c2 after the job)
@@ -440,10 +457,11 @@ __device__ inline void control_step_ahead(const TreeSmem& s, Ctl& ctl, const Ahe
     return;
   }
   const int c2 = ah.c2;
+  const double s_unit = inv_d * __hiloint2double((unit_exponent(D) + 1023) << 20, 0);
   if (ah.mode == kAheadPrune) {
     s.state[c2] = kPruned;
     s.dbgp[c2] = 0.f;
-    note_pass(s, ctl, i, c2, msum);
+    note_pass(s, ctl, i, c2, msum, s_unit);
     return;
   }
   const double pc = fmin(ah.X * inv_d, 1.0);
@@ -456,7 +474,7 @@ __device__ inline void control_step_ahead(const TreeSmem& s, Ctl& ctl, const Ahe
     return;
   }
   s.state[c2] = kRejected;
-  note_pass(s, ctl, i, c2, msum);
+  note_pass(s, ctl, i, c2, msum, s_unit);
 }
 
 // Advances the serial traversal until it needs vocabulary work; posts it.

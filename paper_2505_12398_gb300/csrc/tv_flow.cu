@@ -736,6 +736,7 @@ __device__ void owner_new_tree(const TravArgs& a, const TreeSmem& s, Shared& sh,
     c.node = 0;
     c.pending = -1;
     c.masked_sum = 0.0;
+    c.s_unit = 1.0;
     c.n_tests = c.n_passes = 0;
     c.job.kind = 0;
   }
@@ -1162,29 +1163,28 @@ __device__ void owner_role(const TravArgs& a, const FlowArgs& f, const Smem& m, 
         for (int k2 = lane; k2 < sh.jK; k2 += 32) S_pass += sh.pbuf[k2].x;
         S_pass = warp_sum(S_pass);
         const Ahead& ah = sh.ahead;
-        const double S = (double)S_pass + ah.pm;
+        const double S = (double)S_pass * sh.ctl.s_unit + ah.pm;
         if (S > 1e-300) {   // (the same in every lane)
           const double D = S + ah.omp;
-          // 1 / D, 1 / S and S / D in lanes 0, 1 and 2: a float64 division
-          // takes as long for one lane as for three
-          const double quot = (lane == 2 ? S : 1.0) / (lane == 1 ? S : D);
           int post_first = 0, accept = 0;
           if (lane == 0) {
             bool acc;
-            post_first = job_ahead(s, ah, S, D, quot, sh.fjob, acc) ? 1 : 0;
+            post_first = job_ahead(s, ah, S, D, sh.fjob, acc) ? 1 : 0;
             accept = acc ? 1 : 0;
             sh.ctl.S = S_pass;
           }
           post_first = __shfl_sync(0xffffffffu, post_first, 0);
-          const double inv_s = __shfl_sync(0xffffffffu, quot, 1);
-          const double p_new = __shfl_sync(0xffffffffu, quot, 2);
           __syncwarp();
-          if (post_first) {
+          if (post_first)
             post_job(s, sh, a, f, my_tree, V, lane, __shfl_sync(0xffffffffu, done_est, 0),
                      sh.fjob, m.mtok2, s.mask_val);
-            if (lane == 0) control_step_ahead(s, sh.ctl, ah, accept != 0, quot, inv_s, p_new);
-          } else {
-            if (lane == 0) control_step_ahead(s, sh.ctl, ah, accept != 0, quot, inv_s, p_new);
+          // 1 / D, 1 / S and S / D in lanes 0, 1 and 2: a float64 division
+          // takes as long for one lane as for three
+          const double quot = (lane == 2 ? S : 1.0) / (lane == 1 ? S : D);
+          const double inv_s = __shfl_sync(0xffffffffu, quot, 1);
+          const double p_new = __shfl_sync(0xffffffffu, quot, 2);
+          if (lane == 0) control_step_ahead(s, sh.ctl, ah, accept != 0, D, quot, inv_s, p_new);
+          if (!post_first) {
             __syncwarp();
             post_job(s, sh, a, f, my_tree, V, lane, __shfl_sync(0xffffffffu, done_est, 0),
                      sh.ctl.job, s.mask_tok, s.mask_val);

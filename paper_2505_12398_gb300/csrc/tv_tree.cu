@@ -48,7 +48,7 @@
 //
 // Measured (60-node trees, bf16; 8-token chains, fp32), against one thread of the
 // consumers doing the control, a reduction and an exchange per row and no
-// resident pairs: V = 32000, B = 64 254 -> 141 us (183 with a row by all warps in turn
+// resident pairs: V = 32000, B = 64 254 -> 139 us (183 with a row by all warps in turn
 // and before the removal of a rate-0 sibling and the descent into a sub-tree were
 // worked out ahead, 149 one tile at a time); 16 chains 117 -> 63 us; V = 128256, B =
 // 32 368 -> 184 us (213 one tile at a time).
@@ -990,26 +990,23 @@ struct TreeCta {
       if (kind == kJobStats) stat_ph ^= 1u;
       if (kind == kJobPass && ah.ok && S > 0.f) {
         // the next step was worked out while the pass ran: decide, publish, then
-        // update the state (the same values in every lane; 1 / D, 1 / S and S / D
-        // in lanes 0, 1 and 2, since a float64 division takes as long for one lane
-        // as for three)
-        const double Sd = (double)S + ah.pm, D = Sd + ah.omp;
-        double quot = 0.0;
-        const bool early = ah.mode == kAheadTest || ah.mode == kAheadPrune;
-        if (early) quot = (lane == 2 ? Sd : 1.0) / (lane == 1 ? Sd : D);
+        // update the state (the same values in every lane)
+        const double Sd = (double)S * ctl.s_unit + ah.pm, D = Sd + ah.omp;
         bool accept = false, first = true;
         if (lane == 0) {
           Job jf;
-          first = job_ahead(s, ah, Sd, D, quot, jf, accept);
+          first = job_ahead(s, ah, Sd, D, jf, accept);
           if (first) ok = publish(jf, mnext, ring) ? 1 : 0;
         }
         __syncwarp();
-        if (!early) quot = (lane == 2 ? Sd : 1.0) / (lane == 1 ? Sd : D);
+        // 1 / D, 1 / S and S / D in lanes 0, 1 and 2: a float64 division takes as
+        // long for one lane as for three
+        const double quot = (lane == 2 ? Sd : 1.0) / (lane == 1 ? Sd : D);
         const double inv_s = __shfl_sync(0xffffffffu, quot, 1);
         const double p_new = __shfl_sync(0xffffffffu, quot, 2);
         if (lane == 0) {
           ctl.S = S;
-          control_step_ahead(s, ctl, ah, accept, quot, inv_s, p_new);
+          control_step_ahead(s, ctl, ah, accept, D, quot, inv_s, p_new);
           if (!first) ok = publish(ctl.job, 0, ring) ? 1 : 0;
           else mnext = 3 - mnext;             // that list is in use now
           prepare_ahead(s, ctl, ah, mtok(mnext), u);
@@ -1150,6 +1147,7 @@ __global__ void __launch_bounds__(TreeCta<L, NCW, kExact>::kThreads, 16 / NCW)
     ctl.node = 0;
     ctl.pending = -1;
     ctl.masked_sum = 0.0;
+    ctl.s_unit = 1.0;
     ctl.n_tests = ctl.n_passes = 0;
     ctl.job.kind = 0;
   }

@@ -97,3 +97,14 @@ def test_given_normalisers(tv, V, B):
     keep = [b for b in range(B) if b != 1]
     for x, y in zip(bad[:3], out[:3]):
         assert torch.equal(x[keep], y[keep])
+
+
+@pytest.mark.parametrize("path", ["cluster", "persistent"])
+@pytest.mark.parametrize("sigma", [0.05, 0.5, 3.0])
+def test_runs_of_siblings(tv, path, sigma):
+    """Passes that follow a sibling's rejection or removal at the same node, whose
+    sums come in units of D / 2^e: leaves of one root, drafts close to the target (D
+    near 0, wherever the rate is near 1) and far from it (rate 0, many removals)."""
+    w = Workload("siblings", 24, 8008, levels=(12, 3), branching=(12, 3), sigma=sigma)
+    inp = make_inputs(w, seed=int(100 * sigma), device="cuda")
+    _check(inp, _verify(tv, inp, path))
