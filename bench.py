@@ -471,9 +471,9 @@ def main():
     peak, peak_kind = measured_peaks()
     ph = [sum(p[i] for p in phase) / len(phase) for i in range(3)]
     if path_code == 0:
-        names = ["tv_prep_kernel", "tv_row_stats_kernel", "tv_tree_kernel"]
+        names = ["-", "tv_row_stats_kernel", "tv_tree_kernel"]
         kbytes = [0, row_bytes, trav_bytes]
-        launches_per_step = 3
+        launches_per_step = 2
     else:
         # one kernel reads every row the traversal needs; the first two
         # phases are empty (their events are recorded back to back)
@@ -523,7 +523,7 @@ def main():
                    "temperature": w.temperature, "sigma": w.sigma, "seed": args.seed,
                    "l2": "flushed by a 256 MiB write before every timed step (untimed)",
                    "parallelism": f"dp{world} (independent trees per GPU)",
-                   "kernel_path": ["three-kernel", "cluster-per-tree",
+                   "kernel_path": ["two-kernel", "cluster-per-tree",
                                    "persistent"][path_code],
                    "ctas_per_tree": cluster, "consumer_warps": warps, "ring_stages": stages},
         "verified_logit_gbps": round(step_gbs, 2),

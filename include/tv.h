@@ -77,13 +77,13 @@ enum {
    kernel where trees are few or rows short (a job costs less to exchange
    inside a cluster than through the persistent kernel's queue: N + 1 <= 128
    and V <= 32768, or V <= 49152 and B V <= 14 million, or B < 64 and B V <= 8.4
-   million), else the persistent kernel; the three-kernel path otherwise.  All paths compute the
+   million), else the persistent kernel; the two-kernel path otherwise.  All paths compute the
    same results; the two single-kernel paths read rows with bulk copies and
-   need V % 8 == 0, other vocabularies always take the three-kernel path. */
+   need V % 8 == 0, other vocabularies always take the two-kernel path. */
 enum {
   TV_FLAG_NONE = 0u,
-  /* Three kernels: internal rows listed, row normalisers of every one, then
-     the traversal by one thread-block cluster per tree. */
+  /* Two kernels: row normalisers of every internal row, then the traversal by
+     one thread-block cluster per tree. */
   TV_FLAG_UNFUSED = 1u,
   /* One kernel, one thread-block cluster per tree (rows read lazily, the
      vocabulary split across the cluster's CTAs). */
@@ -102,7 +102,7 @@ enum {
      node is rejected.  Same arguments, outputs and uniforms convention.
      Needs a single-kernel path: tv_create returns TV_ERR_INVALID_ARG with
      TV_FLAG_UNFUSED or when V % 8 != 0, and a call that could only run the
-     three-kernel path returns TV_ERR_INVALID_ARG. */
+     two-kernel path returns TV_ERR_INVALID_ARG. */
   TV_FLAG_TOKEN_LEVEL = 8u
 };
 
@@ -158,7 +158,7 @@ int tv_create(tv_handle** out, int device, int vocab, int max_nodes, int max_bat
  * CUDA graphs: the call may be captured.  A launch of the persistent kernel
  * carries the call's queue epoch and must not be replayed, so while
  * cuda_stream is capturing, a handle that picks its path itself verifies with
- * the cluster path (else the three-kernel path), and a handle created with
+ * the cluster path (else the two-kernel path), and a handle created with
  * TV_FLAG_PERSISTENT returns TV_ERR_INVALID_ARG.  Make one call outside the
  * capture first: first calls set kernel attributes and allocate scratch.
  * Errors (host-side, nothing launched): TV_ERR_INVALID_ARG, TV_ERR_TEMPERATURE,
@@ -182,7 +182,7 @@ int tv_verify_batch(tv_handle* h, int B, int N, const int32_t* parents,
  *               bonus token came from an original leaf's row else 0, number of
  *               target rows whose normaliser (softmax denominator) the call
  *               computed }.  The first four follow from Algorithm 3; the last
- *               depends on the kernel path (the three-kernel path normalises
+ *               depends on the kernel path (the two-kernel path normalises
  *               every internal row, the single-kernel paths only the rows the
  *               traversal reaches).
  *   out_margin  [B][2] fp32 (device): the tree's decision margins, computed
@@ -334,26 +334,26 @@ int tv_get_status(tv_handle* h, uint32_t* status);
 
 /*
  * tv_set_phase_timing -- when enable != 0, later verify calls on this handle
- * record CUDA events on their stream around each of the three kernels
- * (row preparation, row normalisers, traversal).  Costs three event records
+ * record CUDA events on their stream around each of the kernels (row
+ * normalisers, traversal).  Costs three event records
  * per call; off by default.  Errors: TV_ERR_INVALID_ARG, TV_ERR_CUDA.
  */
 int tv_set_phase_timing(tv_handle* h, int enable);
 
 /*
  * tv_last_phase_ms -- waits for the events of the most recent timed call and
- * writes the device time of its three kernels, in milliseconds, to ms[0..2]
- * (preparation, row normalisers, traversal).  Errors: TV_ERR_INVALID_ARG
+ * writes the device time of its phases, in milliseconds, to ms[0..2] (before
+ * the row normalisers, where no kernel runs; row normalisers; traversal).  Errors: TV_ERR_INVALID_ARG
  * (timing off or no timed call yet), TV_ERR_CUDA.
  */
 int tv_last_phase_ms(tv_handle* h, float* ms);
 
 /*
  * tv_launch_shape -- how a call with these B and N would run on this handle:
- * *path = 0 for the three-kernel path, 1 for the cluster-per-tree kernel, 2
+ * *path = 0 for the two-kernel path, 1 for the cluster-per-tree kernel, 2
  * for the persistent kernel; *cluster = CTAs per tree (cluster path; 1
  * otherwise), *warps = consumer warps per CTA, *stages = ring stages (0 for
- * the three-kernel path).  Any output pointer may be NULL.
+ * the two-kernel path).  Any output pointer may be NULL.
  * Errors: TV_ERR_INVALID_ARG, TV_ERR_CAPACITY.
  */
 int tv_launch_shape(tv_handle* h, int B, int N, int* path, int* cluster, int* warps,
@@ -367,10 +367,10 @@ int tv_launch_shape(tv_handle* h, int B, int N, int* path, int* cluster, int* wa
  * tv_create allocates a handle's workspace, so such callers cannot use it.
  * The paper has no counterpart: this is a deployment entry point.
  *
- * Needs no handle and allocates nothing: its scratch (internal-row list, row
- * statistics, status word) is one fixed array of static device memory in the
- * library image (about 0.8 MB, held by every GPU that loads the library until
- * the process exits), used through the three-kernel path.  Limit:
+ * Needs no handle and allocates nothing: its scratch (row statistics, status
+ * word) is one fixed array of static device memory in the library image (about
+ * 0.5 MB, held by every GPU that loads the library until
+ * the process exits), used through the two-kernel path.  Limit:
  * B * (N + 1) <= 65536 rows; larger calls return TV_ERR_CAPACITY and launch
  * nothing.  The first call on a device makes that device current and looks up
  * the array's device address (cudaGetSymbolAddress) once; issue that first

@@ -323,7 +323,7 @@ class Verifier:
 
     def launch_shape(self, B, N):
         """(path code, CTAs per tree, consumer warps per CTA, ring stages);
-        path code 0 = three kernels, 1 = cluster per tree, 2 = persistent."""
+        path code 0 = two kernels, 1 = cluster per tree, 2 = persistent."""
         out = [ctypes.c_int() for _ in range(4)]
         rc = self.lib.tv_launch_shape(self.handle, B, N, *[ctypes.byref(o) for o in out])
         if rc != 0:

@@ -31,8 +31,6 @@ struct tv_handle {
   int force_ncw = 0, force_c = 0, force_stages = 0;   // tuning override (TV_FUSED_PLAN)
   int flow_force[5] = {0, 0, 0, 0, 0};                 // tuning override (TV_FLOW_PLAN)
   // device workspace
-  int32_t* row_list = nullptr;   // [max_batch * (max_nodes + 1)]
-  int32_t* n_rows = nullptr;     // [1]
   float2* stats = nullptr;       // [max_batch * (max_nodes + 1)]
   uint32_t* status = nullptr;    // [1]
   void* flow_ws = nullptr;       // persistent kernel's queue and partials
@@ -63,7 +61,7 @@ constexpr int kMaxRows = 1024;   // N + 1
 constexpr int kMaxVocab = 1 << 28;
 constexpr unsigned kPathFlags = TV_FLAG_UNFUSED | TV_FLAG_CLUSTER | TV_FLAG_PERSISTENT;
 
-enum Path { kPathThree = 0, kPathCluster = 1, kPathPersistent = 2 };
+enum Path { kPathTwo = 0, kPathCluster = 1, kPathPersistent = 2 };
 
 size_t logit_bytes(const tv_handle* h) { return h->dtype == TV_BF16 ? 2 : 4; }
 
@@ -101,14 +99,14 @@ bool prefer_cluster(int V, int B, int R) {
   return B < 64 && (long long)B * V <= 8400000;
 }
 
-// The path of a call, and the cluster kernel's plan (also for the three-kernel
+// The path of a call, and the cluster kernel's plan (also for the two-kernel
 // path, whose last kernel it is).
 Path choose_path(const tv_handle* h, int B, int R, FusedPlan* plan) {
   *plan = tv_fused_plan(B, R, h->vocab, (int)logit_bytes(h), h->smem_per_sm, h->smem_per_block,
                         h->force_ncw, h->force_c, h->force_stages);
-  if ((h->vocab % 8) != 0 || (h->flags & TV_FLAG_UNFUSED)) return kPathThree;
-  if (h->flags & TV_FLAG_CLUSTER) return plan->ok ? kPathCluster : kPathThree;
-  if (!h->flow_ws || !flow_plan(h, R, B).ok) return kPathThree;
+  if ((h->vocab % 8) != 0 || (h->flags & TV_FLAG_UNFUSED)) return kPathTwo;
+  if (h->flags & TV_FLAG_CLUSTER) return plan->ok ? kPathCluster : kPathTwo;
+  if (!h->flow_ws || !flow_plan(h, R, B).ok) return kPathTwo;
   if (!(h->flags & TV_FLAG_PERSISTENT) && plan->ok && prefer_cluster(h->vocab, B, R))
     return kPathCluster;
   return kPathPersistent;
@@ -270,25 +268,21 @@ int verify_impl(tv_handle* h, int B, int N, const int32_t* parents, const int32_
   a.row_stats = row_stats;
   a.stats_given = row_stats ? 1 : 0;
   a.exact_exp = 0;
-  const int rows = B * (N + 1);
-  int grid = h->sm_count * 4;
-  if (grid > rows) grid = rows;
-  if (grid < 1) grid = 1;
   FusedPlan plan;
   Path path = choose_path(h, B, N + 1, &plan);
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   if (path == kPathPersistent && capturing(st)) {
     // a launch of the persistent kernel carries the call's queue epoch, so a
     // graph must not replay it: under capture, a handle that chose the path
-    // itself uses the cluster path (else the three-kernel one)
+    // itself uses the cluster path (else the two-kernel one)
     if ((h->flags & TV_FLAG_PERSISTENT) || row_stats) return TV_ERR_INVALID_ARG;
-    path = plan.ok ? kPathCluster : kPathThree;
+    path = plan.ok ? kPathCluster : kPathTwo;
   }
-  // the three-kernel path implements Traversal Verification only
-  if (path == kPathThree && a.token_level) return TV_ERR_INVALID_ARG;
+  // the two-kernel path implements Traversal Verification only
+  if (path == kPathTwo && a.token_level) return TV_ERR_INVALID_ARG;
   // given row normalisers: the persistent kernel, or the cluster kernel where
   // the handle chose it itself (and neither under capture)
-  if (row_stats && (path == kPathThree || (h->flags & TV_FLAG_CLUSTER) ||
+  if (row_stats && (path == kPathTwo || (h->flags & TV_FLAG_CLUSTER) ||
                     (path == kPathCluster && capturing(st))))
     return TV_ERR_INVALID_ARG;
   const int bf16 = h->dtype == TV_BF16 ? 1 : 0;
@@ -305,7 +299,7 @@ int verify_impl(tv_handle* h, int B, int N, const int32_t* parents, const int32_
     h->withhold_tree = -1;
     rc = tv_launch_flow(a, f, bf16, fp, h->sm_count, st, ev);
   } else {
-    rc = tv_launch_all(a, bf16, h->row_list, h->n_rows, grid, plan, st, ev);
+    rc = tv_launch_all(a, bf16, plan, st, ev);
   }
   if (rc == TV_OK && h->timing) h->timed_call = true;
   return rc;
@@ -364,9 +358,7 @@ int tv_create(tv_handle** out, int device, int vocab, int max_nodes, int max_bat
     return TV_ERR_CUDA;
   }
   const size_t rows = static_cast<size_t>(max_batch) * (max_nodes + 1);
-  bool ok = cudaMalloc(&h->row_list, rows * sizeof(int32_t)) == cudaSuccess &&
-            cudaMalloc(&h->n_rows, sizeof(int32_t)) == cudaSuccess &&
-            cudaMalloc(&h->stats, rows * sizeof(float2)) == cudaSuccess &&
+  bool ok = cudaMalloc(&h->stats, rows * sizeof(float2)) == cudaSuccess &&
             cudaMalloc(&h->status, sizeof(uint32_t)) == cudaSuccess &&
             cudaMemset(h->status, 0, sizeof(uint32_t)) == cudaSuccess;
   if (ok && (vocab % 8) == 0 && !(flags & (TV_FLAG_UNFUSED | TV_FLAG_CLUSTER))) {
@@ -555,7 +547,7 @@ int tv_verify_batch_host(tv_handle* h, int B, int N, const int32_t* parents,
         leaf_bytes += lrow;
       }
       // the (tree, row) list is staged in the row-statistics buffer of the
-      // three-kernel path ([max_batch (max_nodes + 1)] float2 >= B int2),
+      // two-kernel path ([max_batch (max_nodes + 1)] float2 >= B int2),
       // which no kernel reads once the verification above has finished
       int2* d_pend = reinterpret_cast<int2*>(h->stats);
       pend_bytes = pend.size() * sizeof(int2);
@@ -730,8 +722,6 @@ int tv_destroy(tv_handle* h) {
       if (h->copy_st[k]) cudaStreamDestroy(h->copy_st[k]);
     for (int k = 0; k < 3; ++k)
       if (h->copy_ev[k]) cudaEventDestroy(h->copy_ev[k]);
-    cudaFree(h->row_list);
-    cudaFree(h->n_rows);
     cudaFree(h->stats);
     cudaFree(h->status);
     if (h->flow_ws) cudaFree(h->flow_ws);

@@ -95,10 +95,14 @@ __device__ __forceinline__ float2 exp2_corrected_x2(float2 d, float2 c_hi, float
 
 // exp2_split on a pair (d already clamped below).  Results below 2^-125 are
 // returned as a value under 2^-124 instead of the exact tiny number.
-__device__ __forceinline__ float2 exp2_split_x2(float2 d, float2 c_hi, float2 c_lo) {
+// kLow: d + d_lo.
+template <bool kLow = false>
+__device__ __forceinline__ float2 exp2_split_x2(float2 d, float2 c_hi, float2 c_lo,
+                                                float2 d_lo = make_float2(0.f, 0.f)) {
   const float2 e_hi = __fmul2_rn(d, c_hi);
   float2 e_lo = __ffma2_rn(d, c_hi, make_float2(-e_hi.x, -e_hi.y));
   e_lo = __ffma2_rn(d, c_lo, e_lo);
+  if constexpr (kLow) e_lo = __ffma2_rn(d_lo, c_hi, e_lo);
   const float2 t = __fadd2_rn(e_hi, make_float2(12582912.f, 12582912.f));
   const float2 nf = __fadd2_rn(t, make_float2(-12582912.f, -12582912.f));
   const float2 f = __fadd2_rn(__fadd2_rn(e_hi, make_float2(-nf.x, -nf.y)), e_lo);
@@ -132,6 +136,39 @@ struct Bf16Logits {
   __device__ static __forceinline__ float exp_rel(float v, float m, float c_hi, float c_lo) {
     return exp2_split(v - m, 0.f, c_hi, c_lo);
   }
+  // Eight logits as a block, and exp_rel of them relative to m, v - m clamped below
+  // at d_min (weights there are under 2^-124 instead of 0).
+  using block = uint4;
+  __device__ static __forceinline__ block load_block(const elem* p) { return ld_nc16(p); }
+  __device__ static __forceinline__ block make_block(const elem* p, int lo, int hi) {
+    uint32_t w[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const uint32_t a = 2 * k >= lo && 2 * k < hi ? p[2 * k] : 0xFF80u;
+      const uint32_t b = 2 * k + 1 >= lo && 2 * k + 1 < hi ? p[2 * k + 1] : 0xFF80u;
+      w[k] = a | (b << 16);
+    }
+    return make_uint4(w[0], w[1], w[2], w[3]);
+  }
+  __device__ static __forceinline__ float block_max(const block& b) {
+    const uint32_t w[4] = {b.x, b.y, b.z, b.w};
+    __nv_bfloat162 h[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) h[k] = *reinterpret_cast<const __nv_bfloat162*>(&w[k]);
+    const __nv_bfloat162 m = __hmax2(__hmax2(h[0], h[1]), __hmax2(h[2], h[3]));
+    const uint32_t u = *reinterpret_cast<const uint32_t*>(&m);
+    return fmaxf(bf16_lo(u), bf16_hi(u));
+  }
+  __device__ static __forceinline__ void block_exp(const block& b, float m, float d_min,
+                                                   float2 c_hi, float2 c_lo, float2 t[4]) {
+    const uint32_t w[4] = {b.x, b.y, b.z, b.w};
+    const float2 nm = make_float2(-m, -m);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const float2 d = __fadd2_rn(make_float2(bf16_lo(w[k]), bf16_hi(w[k])), nm);
+      t[k] = exp2_split_x2(make_float2(fmaxf(d.x, d_min), fmaxf(d.y, d_min)), c_hi, c_lo);
+    }
+  }
   // cheaper form for the per-element work of rejection passes and bonus draws
   __device__ static __forceinline__ float exp_pass(float v, float m, float c_hi, float c_lo) {
     return exp2_corrected(v - m, c_hi, c_lo);
@@ -159,6 +196,36 @@ struct F32Logits {
     const float bb = d - v;
     const float d_lo = (v - (d - bb)) + (-m - bb);
     return exp2_split(d, d_lo, c_hi, c_lo);
+  }
+  struct block { float v[8]; };
+  __device__ static __forceinline__ block load_block(const elem* p) {
+    block b;
+    chunk_vec(p, 0, b.v);
+    return b;
+  }
+  __device__ static __forceinline__ block make_block(const elem* p, int lo, int hi) {
+    block b;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) b.v[k] = k >= lo && k < hi ? p[k] : TV_NEG_INF;
+    return b;
+  }
+  __device__ static __forceinline__ float block_max(const block& b) {
+    return fmaxf(fmaxf(fmaxf(b.v[0], b.v[1]), fmaxf(b.v[2], b.v[3])),
+                 fmaxf(fmaxf(b.v[4], b.v[5]), fmaxf(b.v[6], b.v[7])));
+  }
+  __device__ static __forceinline__ void block_exp(const block& b, float m, float d_min,
+                                                   float2 c_hi, float2 c_lo, float2 t[4]) {
+    const float least = m + d_min;
+    const float2 nm = make_float2(-m, -m);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const float2 v = make_float2(fmaxf(b.v[2 * k], least), fmaxf(b.v[2 * k + 1], least));
+      const float2 d = __fadd2_rn(v, nm);
+      const float2 bb = __fadd2_rn(d, make_float2(-v.x, -v.y));
+      const float2 nbb = make_float2(-bb.x, -bb.y), x = __fadd2_rn(d, nbb);
+      const float2 d_lo = __fadd2_rn(__fadd2_rn(v, make_float2(-x.x, -x.y)), __fadd2_rn(nm, nbb));
+      t[k] = exp2_split_x2<true>(d, c_hi, c_lo, d_lo);
+    }
   }
   __device__ static __forceinline__ float exp_pass(float v, float m, float c_hi, float c_lo) {
     return exp_rel(v, m, c_hi, c_lo);

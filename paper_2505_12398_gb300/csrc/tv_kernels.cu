@@ -1,15 +1,14 @@
 // tv_kernels.cu -- CUDA kernels of batched Traversal Verification (sm_103a).
 //
-// One call verifies B independent trees in three kernels on one stream:
+// The path with separate row normalisers: one call verifies B independent trees in
+// two kernels on one stream:
 //
-//   tv_prep_kernel       one warp per tree: structural checks of the parent
-//                        array and the token range, then appends the tree's
-//                        internal rows (rows with >= 1 child) to a work list.
-//   tv_row_stats_kernel  the row normaliser of every internal row, fully
-//                        parallel over B x |I| rows: one streaming pass with an
-//                        online max / sum of exp2((l - m) log2(e) / T).  These
-//                        are the target distributions M_b(.|X^i) Algorithm 3
-//                        initialises its acceptance rates from (§3.1).
+//   tv_row_stats_kernel  the row normaliser of every internal row (a row with at
+//                        least one child; the others' blocks leave at once), one
+//                        block per row: one streaming pass with an online max /
+//                        sum of exp2((l - m) log2(e) / T).  These are the target
+//                        distributions M_b(.|X^i) Algorithm 3 initialises its
+//                        acceptance rates from (§3.1).
 //   tv_tree_kernel       (tv_tree.cu) the traversal of Algorithm 3 (Appendix E
 //                        order), one cluster per tree, with those normalisers.
 //
@@ -17,7 +16,18 @@
 // anywhere, so they are read as whole 8-element blocks of the flat
 // [B][N+1][V] arrays (16- or 32-byte loads), the neighbouring rows' elements in
 // the first and last block masked.  Measured (32 trees of 60 nodes, V = 32003,
-// bf16), against element loads and one CTA per tree: 330.6 -> 149.8 us.
+// bf16), against element loads and one CTA per tree: 330.6 -> 149.8 us; then the
+// list of internal rows that a first kernel made (with a cleared counter) left to
+// the normalisers' blocks, and their arithmetic as below: -> 119 us.
+//
+// The normaliser kernel is bound by its arithmetic, a third of the HBM rate: 16
+// instructions per logit at 69 % of the issue slots before the maximum of a pair
+// of bf16 took one instruction, the weights below 2^-125 one clamp instead of a
+// comparison and a selection, and the logits stayed packed until they are used (48
+// registers, five blocks per SM).  With four blocks of logits per thread at a time,
+// also at a row's end, and two weights per instruction, against one block at a time
+// and scalar arithmetic: 256 trees, V = 32003 270 -> 159 us, 32 trees 45 -> 30 us
+// (the bytes alone 92 and 11 us).
 //
 // The mutable distributions of Algorithm 3 are never materialised.  After k
 // rejections at node i (children tokens t_0..t_{k-1} removed) they are, for
@@ -38,164 +48,103 @@
 
 namespace tvk {
 
-// ------------------------------------------------------------------ prep --
-
-__global__ void __launch_bounds__(256) tv_prep_kernel(const int32_t* __restrict__ parents,
-                                                      const int32_t* __restrict__ tokens,
-                                                      int B, int R, int V,
-                                                      int32_t* __restrict__ row_list,
-                                                      int32_t* __restrict__ n_rows) {
-  __shared__ uint32_t s_has[8][32];   // one bit per row (R <= 1024), per warp
-  const int wl = threadIdx.x >> 5;
-  const int lane = threadIdx.x & 31;
-  const int tree = blockIdx.x * 8 + wl;
-  s_has[wl][lane] = 0u;
-  __syncwarp();
-  if (tree >= B) return;
-  const int32_t* par = parents + (size_t)tree * R;
-  const int32_t* tok = tokens + (size_t)tree * R;
-  bool bad = false;
-  for (int i = lane; i < R; i += 32) {
-    int p = par[i];
-    if (i == 0) {
-      bad |= (p != -1);
-    } else {
-      int t = tok[i];
-      bad |= (t < 0 || t >= V);
-      if (p < 0 || p >= i) bad = true;
-      else atomicOr(&s_has[wl][p >> 5], 1u << (p & 31));
-    }
-  }
-  bad = __any_sync(0xffffffffu, bad);
-  __syncwarp();
-  if (bad) return;   // the traversal kernel reports it; no row work queued
-  uint32_t word = s_has[wl][lane];
-  int cnt = __popc(word);
-  int incl = cnt;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    int v = __shfl_up_sync(0xffffffffu, incl, o);
-    if (lane >= o) incl += v;
-  }
-  int total = __shfl_sync(0xffffffffu, incl, 31);
-  int base = 0;
-  if (lane == 31) base = atomicAdd(n_rows, total);
-  base = __shfl_sync(0xffffffffu, base, 31);
-  int pos = base + incl - cnt;
-  while (word) {
-    int bit = __ffs(word) - 1;
-    word &= word - 1;
-    row_list[pos++] = tree * R + lane * 32 + bit;
-  }
-}
-
 // ------------------------------------------------------------- row stats --
 
-constexpr int kStatsThreads = 256;
 constexpr int kStatsUnroll = 4;
 
-// One block's eight logits added to a thread's running (max, sum): `n_all`
-// elements in the arrays, [lo, hi) of the block's belong to the row.
-template <typename L>
-__device__ __forceinline__ void stats_block(const typename L::elem* logits, size_t at,
-                                            size_t n_all, int lo, int hi, float v[8]) {
-  if (at + 8 <= n_all) {
-    L::chunk_vec(logits + at, 0, v);
-  } else {                       // the arrays' last, partial block
-#pragma unroll
-    for (int k = 0; k < 8; ++k) v[k] = k < hi ? L::at(logits + at, k) : TV_NEG_INF;
-  }
-  if (lo > 0 || hi < 8) {
-#pragma unroll
-    for (int k = 0; k < 8; ++k)
-      if (k < lo || k >= hi) v[k] = TV_NEG_INF;
-  }
-}
-
-template <typename L>
-__device__ __forceinline__ void stats_add(const float v[8], int lo, int hi, float c_hi, float c_lo,
-                                          float& m, Comp& acc) {
-  const float cm = fmaxf(fmaxf(fmaxf(v[0], v[1]), fmaxf(v[2], v[3])),
-                         fmaxf(fmaxf(v[4], v[5]), fmaxf(v[6], v[7])));
-  if (cm > m) {
-    if (m != TV_NEG_INF) {
-      const float sc = L::exp_rel(m, cm, c_hi, c_lo);
-      acc.s *= sc;
-      acc.c *= sc;
-    }
-    m = cm;
-  }
-  if (m != TV_NEG_INF) {
-    float t[8];
-#pragma unroll
-    for (int e = 0; e < 8; ++e) t[e] = L::exp_rel(v[e], m, c_hi, c_lo);
-    if (lo > 0 || hi < 8) {
-#pragma unroll
-      for (int e = 0; e < 8; ++e)
-        if (e < lo || e >= hi) t[e] = 0.f;
-    }
-    acc.add(sum8(t));
-  }
-}
-
-template <typename L>
-__global__ void __launch_bounds__(kStatsThreads) tv_row_stats_kernel(
-    const typename L::elem* __restrict__ logits, int V, size_t n_all, float c_hi, float c_lo,
-    const int32_t* __restrict__ row_list, const int32_t* __restrict__ n_rows,
-    float2* __restrict__ stats) {
+template <typename L, int kStatsThreads>
+__global__ void __launch_bounds__(kStatsThreads, kStatsThreads == 256 ? 6 - L::kBytes / 2 : 1)
+    tv_row_stats_kernel(const typename L::elem* __restrict__ logits,
+                        const int32_t* __restrict__ parents, int R, int V, float c_hi, float c_lo,
+                        float2* __restrict__ stats) {
   __shared__ float s_red[kStatsThreads / 32];
   __shared__ float s_max;
-  const int n = *n_rows;
+  asm volatile("griddepcontrol.launch_dependents;");   // (the traversal waits for this grid)
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  for (int r = blockIdx.x; r < n; r += gridDim.x) {
-    const int g = row_list[r];
-    // the row's first 8-element block and its elements of the row before
-    const size_t first = (size_t)g * V;
-    const int sh = (int)(first & 7u);
-    const size_t base = first - (size_t)sh;
-    const int end = V + sh;              // the row is [sh, end) from base
-    // phase 1: per-thread online max / sum relative to that max
-    float m = TV_NEG_INF;
-    Comp acc;
-    const int step = kStatsThreads * kChunk;
-    int x0 = threadIdx.x * kChunk;
-    for (; x0 + (kStatsUnroll - 1) * step < end; x0 += kStatsUnroll * step) {
-      float v[kStatsUnroll][8];
+  const int g = blockIdx.x, node = g % R;
+  {
+    const int32_t* par = parents + (g - node);
+    int child = 0;
+    for (int i = threadIdx.x; i < R; i += kStatsThreads) child |= i > 0 && par[i] == node;
+    if (!__syncthreads_or(child)) return;
+  }
+  // the row's first 8-element block and its elements of the row before
+  const size_t first = (size_t)g * V;
+  const int sh = (int)(first & 7u);
+  const size_t base = first - (size_t)sh;
+  const int end = V + sh;              // the row is [sh, end) from base
+  // phase 1: per-thread online max / sum relative to that max
+  float m = TV_NEG_INF;
+  Comp acc;
+  const int step = kStatsThreads * kChunk;
+  const float2 ch = make_float2(c_hi, c_hi), cl = make_float2(c_lo, c_lo);
+  const float d_min = fmaxf(-150.f / c_hi, -1.0e4f);
+  for (int x0 = threadIdx.x * kChunk; x0 < end; x0 += kStatsUnroll * step) {
+    typename L::block v[kStatsUnroll];
+    const bool edge = x0 < sh || x0 + (kStatsUnroll - 1) * step + kChunk > end;
+    if (!edge) {
 #pragma unroll
       for (int u = 0; u < kStatsUnroll; ++u)
-        stats_block<L>(logits, base + x0 + u * step, n_all, sh - (x0 + u * step),
-                       end - (x0 + u * step), v[u]);
+        v[u] = L::load_block(logits + base + x0 + u * step);
+    } else {
 #pragma unroll
-      for (int u = 0; u < kStatsUnroll; ++u)
-        stats_add<L>(v[u], sh - (x0 + u * step), end - (x0 + u * step), c_hi, c_lo, m, acc);
+      for (int u = 0; u < kStatsUnroll; ++u) {
+        const int x = x0 + u * step;
+        if (x >= sh && x + kChunk <= end) v[u] = L::load_block(logits + base + x);
+        else v[u] = L::make_block(logits + base + x, sh - x, end - x);
+      }
     }
-    for (; x0 < end; x0 += step) {
-      float v[8];
-      stats_block<L>(logits, base + x0, n_all, sh - x0, end - x0, v);
-      stats_add<L>(v, sh - x0, end - x0, c_hi, c_lo, m, acc);
+    float cm = L::block_max(v[0]);
+#pragma unroll
+    for (int u = 1; u < kStatsUnroll; ++u) cm = fmaxf(cm, L::block_max(v[u]));
+    if (cm > m) {
+      if (m != TV_NEG_INF) {
+        const float sc = L::exp_rel(m, cm, c_hi, c_lo);
+        acc.s *= sc;
+        acc.c *= sc;
+      }
+      m = cm;
     }
-    // phase 2: the row max, then every partial rescaled once to it and summed
-    float bm = warp_max(m);
-    if (lane == 0) s_red[wid] = bm;
-    __syncthreads();
-    if (wid == 0) {
-      float x = (lane < kStatsThreads / 32) ? s_red[lane] : TV_NEG_INF;
-      x = warp_max(x);
-      if (lane == 0) s_max = x;
+    if (m == TV_NEG_INF) continue;
+#pragma unroll
+    for (int u = 0; u < kStatsUnroll; ++u) {
+      const int x = x0 + u * step;
+      if (x >= end) break;
+      float2 t[4];
+      L::block_exp(v[u], m, d_min, ch, cl, t);
+      if (edge) {              // (-inf has a weight at a high temperature)
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          if (x + 2 * k < sh || x + 2 * k >= end) t[k].x = 0.f;
+          if (x + 2 * k + 1 < sh || x + 2 * k + 1 >= end) t[k].y = 0.f;
+        }
+      }
+      const float2 p = __fadd2_rn(__fadd2_rn(t[0], t[1]), __fadd2_rn(t[2], t[3]));
+      acc.add(p.x + p.y);
     }
-    __syncthreads();
-    const float M = s_max;
-    float part = (m == TV_NEG_INF) ? 0.f : acc.value() * L::exp_rel(m, M, c_hi, c_lo);
-    part = warp_sum(part);
-    __syncthreads();
-    if (lane == 0) s_red[wid] = part;
-    __syncthreads();
-    if (wid == 0) {
-      float x = (lane < kStatsThreads / 32) ? s_red[lane] : 0.f;
-      x = warp_sum(x);
-      if (lane == 0) stats[g] = make_float2(M, x);
-    }
-    __syncthreads();
+  }
+  // phase 2: the row max, then every partial rescaled once to it and summed
+  float bm = warp_max(m);
+  if (lane == 0) s_red[wid] = bm;
+  __syncthreads();
+  if (wid == 0) {
+    float x = (lane < kStatsThreads / 32) ? s_red[lane] : TV_NEG_INF;
+    x = warp_max(x);
+    if (lane == 0) s_max = x;
+  }
+  __syncthreads();
+  const float M = s_max;
+  float part = (m == TV_NEG_INF) ? 0.f : acc.value() * L::exp_rel(m, M, c_hi, c_lo);
+  part = warp_sum(part);
+  __syncthreads();
+  if (lane == 0) s_red[wid] = part;
+  __syncthreads();
+  if (wid == 0) {
+    float x = (lane < kStatsThreads / 32) ? s_red[lane] : 0.f;
+    x = warp_sum(x);
+    // a finite max has weight 1: no normaliser where there is none
+    if (!(x >= 1e-30f) || (L::kBytes == 4 && M == -TV_NEG_INF)) x = 0.f;
+    if (lane == 0) stats[g] = make_float2(M, x);
   }
 }
 
@@ -217,37 +166,51 @@ bool tv_tree_fits(int R, int V, size_t smem_per_block) {
 
 namespace {
 
-template <typename L>
-int launch_typed(const TravArgs& a, int logit_is_bf16, int* row_list, int* n_rows, int stats_grid,
-                 const FusedPlan& plan, cudaStream_t stream, cudaEvent_t* ev) {
+template <typename L, int kThreads>
+void launch_stats(const TravArgs& a, cudaStream_t stream) {
   const int R = a.N + 1;
-  const auto* lg = reinterpret_cast<const typename L::elem*>(a.logits);
+  tvk::tv_row_stats_kernel<L, kThreads><<<a.B * R, kThreads, 0, stream>>>(
+      reinterpret_cast<const typename L::elem*>(a.logits), a.parents, R, a.V, a.c_hi, a.c_lo,
+      a.stats);
+}
+
+template <typename L>
+int launch_typed(const TravArgs& a, int logit_is_bf16, const FusedPlan& plan, cudaStream_t stream,
+                 cudaEvent_t* ev) {
   if (ev && cudaEventRecord(ev[0], stream) != cudaSuccess) return -5;
-  if (cudaMemsetAsync(n_rows, 0, sizeof(int), stream) != cudaSuccess) return -5;
-  tvk::tv_prep_kernel<<<(a.B + 7) / 8, 256, 0, stream>>>(a.parents, a.tokens, a.B, R, a.V,
-                                                          row_list, n_rows);
-  if (launch_error()) return -5;
   if (ev && cudaEventRecord(ev[1], stream) != cudaSuccess) return -5;
-  tvk::tv_row_stats_kernel<L><<<stats_grid, tvk::kStatsThreads, 0, stream>>>(
-      lg, a.V, (size_t)a.B * R * (size_t)a.V, a.c_hi, a.c_lo, row_list, n_rows, a.stats);
+  // Few rows: more threads on each, as long as every thread has a block or more.
+  // Measured (us; the call with 256 / 512 / 1024 threads; 60-node trees, half of
+  // their rows internal): V = 128251 bf16, 61 rows 48 / 41 / 38; V = 151933 fp32, 244
+  // rows 136 / 124 / 120; V = 32003, 61 rows 94 / 93 / 93, 488 rows 99 / 97 / 99, 1952
+  // rows 119 / 124 / 141; V = 1003, 1952 rows 105 / 109 / 117.
+  const long rows = (long)a.B * (a.N + 1);
+  if (rows <= 304 && a.V > 32768) launch_stats<L, 1024>(a, stream);
+  else if (rows <= 608 && a.V > 8192) launch_stats<L, 512>(a, stream);
+  else launch_stats<L, 256>(a, stream);
   if (launch_error()) return -5;
   if (ev && cudaEventRecord(ev[2], stream) != cudaSuccess) return -5;
   TravArgs t = a;
   t.row_stats = a.stats;
   t.stats_given = 0;
   t.exact_exp = 1;
-  if (tv_launch_tree(t, logit_is_bf16, plan, stream) != 0) return -5;
+  // The traversal starts while the normalisers' last blocks run (a programmatic
+  // dependent launch): 54 -> 48 us at B = 1, V = 128251, 104 -> 99 us at B = 8, V =
+  // 32003.  Not where its clusters share SMs: they would then crowd on the SMs that
+  // are free first (119 -> 126 us at B = 32, V = 32003, 449 -> 463 us at B = 256);
+  // single CTAs do not: 170 -> 165 us at B = 512, V = 4001, 774 -> 767 us at B = 600, V
+  // = 32003.
+  const bool dependent = ev == nullptr && (plan.C == 1 || a.B * plan.C <= 152);
+  if (tv_launch_tree(t, logit_is_bf16, plan, stream, dependent) != 0) return -5;
   if (ev && cudaEventRecord(ev[3], stream) != cudaSuccess) return -5;
   return 0;
 }
 
 }  // namespace
 
-int tv_launch_all(const TravArgs& a, int logit_is_bf16, int* row_list, int* n_rows,
-                  int stats_grid, const FusedPlan& plan, cudaStream_t stream,
-                  cudaEvent_t* events) {
+int tv_launch_all(const TravArgs& a, int logit_is_bf16, const FusedPlan& plan,
+                  cudaStream_t stream, cudaEvent_t* events) {
   if (!plan.ok) return -5;
-  return logit_is_bf16
-             ? launch_typed<tvk::Bf16Logits>(a, 1, row_list, n_rows, stats_grid, plan, stream, events)
-             : launch_typed<tvk::F32Logits>(a, 0, row_list, n_rows, stats_grid, plan, stream, events);
+  return logit_is_bf16 ? launch_typed<tvk::Bf16Logits>(a, 1, plan, stream, events)
+                       : launch_typed<tvk::F32Logits>(a, 0, plan, stream, events);
 }

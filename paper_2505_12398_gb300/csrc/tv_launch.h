@@ -55,21 +55,21 @@ FusedPlan tv_fused_plan(int B, int R, int V, int logit_bytes, int smem_per_sm,
 int tv_launch_fused(const TravArgs& a, int logit_is_bf16, const FusedPlan& plan,
                     cudaStream_t stream, cudaEvent_t* events);
 
-// Queues the cluster kernel alone.  0 or -5 (launch failed).
+// Queues the cluster kernel alone.  0 or -5 (launch failed).  `dependent`: it may
+// start while the kernel before it on the stream, which works out a.row_stats, ends.
 int tv_launch_tree(const TravArgs& a, int logit_is_bf16, const FusedPlan& plan,
-                   cudaStream_t stream);
+                   cudaStream_t stream, bool dependent);
 
 // Whether trees of R = N+1 rows of V tokens are small enough for a device whose
 // blocks may use smem_per_block bytes of shared memory.
 bool tv_tree_fits(int R, int V, size_t smem_per_block);
 
-// Queues the three kernels on `stream` (the traversal with the cluster kernel's
+// Queues the two kernels on `stream` (the traversal with the cluster kernel's
 // `plan`); 0 on success, TV_ERR_CUDA otherwise.  With `events` non-null,
 // events[0..3] are recorded before the first kernel, between the kernels and
 // after the last one.
-int tv_launch_all(const TravArgs& a, int logit_is_bf16, int* row_list, int* n_rows,
-                  int stats_grid, const FusedPlan& plan, cudaStream_t stream,
-                  cudaEvent_t* events);
+int tv_launch_all(const TravArgs& a, int logit_is_bf16, const FusedPlan& plan,
+                  cudaStream_t stream, cudaEvent_t* events);
 
 // ---- persistent load-balanced kernel (tv_flow.cu) ----
 

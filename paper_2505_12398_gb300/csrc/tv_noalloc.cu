@@ -5,17 +5,15 @@
 // memory pool reserved the device up front and forbids new allocations once
 // it has warmed up, or an embedding whose allocator owns every byte of the
 // device.  tv_create allocates a handle's workspace, so those callers cannot
-// use it.  This entry point runs the three-kernel path (internal-row list,
-// row normalisers, per-tree traversal) with its scratch -- the internal-row
-// list, the row statistics and the status word -- in one fixed-size array of
-// static device memory that is part of the library image: every GPU that
-// loads the library holds those kScratchBytes (about 0.75 MiB) until the
-// process exits.
+// use it.  This entry point runs the two-kernel path (row normalisers,
+// per-tree traversal) with its scratch -- the row statistics and the status
+// word -- in one fixed-size array of static device memory that is part of the
+// library image: every GPU that loads the library holds those kScratchBytes
+// (about 0.5 MiB) until the process exits.
 //
 // The caller still owns and passes every input and output.  All calls share
 // the one array and it keeps whatever the last call left there; each call
-// clears what must start at zero (the row counter, the status word) before
-// its kernels run.  Calls whose work overlaps on the GPU (different streams,
+// clears what must start at zero (the status word) before its kernels run.  Calls whose work overlaps on the GPU (different streams,
 // different host threads without ordering) race on the array and must not be
 // issued.  The status word is written by the kernels but never returned:
 // through this entry point an invalid tree shows only as -1 outputs.
@@ -33,9 +31,7 @@ namespace {
 constexpr int kMaxScratchRows = 1 << 16;   // B * (N + 1) rows at most
 constexpr size_t kAlign = 256;
 constexpr size_t kOffStatus = 0;
-constexpr size_t kOffCount = kAlign;
-constexpr size_t kOffRows = 2 * kAlign;
-constexpr size_t kOffStats = kOffRows + (size_t)kMaxScratchRows * sizeof(int32_t);
+constexpr size_t kOffStats = kAlign;
 constexpr size_t kScratchBytes = kOffStats + (size_t)kMaxScratchRows * sizeof(float2);
 constexpr int kMaxDevices = 64;
 
@@ -115,8 +111,6 @@ extern "C" int tv_verify_batch_noalloc(int device, int B, int N, int vocab, tv_d
   if (rc == TV_OK) {
     unsigned char* base = static_cast<unsigned char*>(g_scratch_addr[device]);
     uint32_t* status = reinterpret_cast<uint32_t*>(base + kOffStatus);
-    int32_t* n_rows = reinterpret_cast<int32_t*>(base + kOffCount);
-    int32_t* row_list = reinterpret_cast<int32_t*>(base + kOffRows);
     float2* stats = reinterpret_cast<float2*>(base + kOffStats);
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
     if (cudaMemsetAsync(status, 0, sizeof(uint32_t), st) != cudaSuccess) {
@@ -148,14 +142,9 @@ extern "C" int tv_verify_batch_noalloc(int device, int B, int N, int vocab, tv_d
       a.row_stats = nullptr;
       a.stats_given = 0;
       a.exact_exp = 0;
-      const int rows = B * (N + 1);
-      int grid = g_sm_count[device] * 4;
-      if (grid > rows) grid = rows;
-      if (grid < 1) grid = 1;
       const FusedPlan plan = tv_fused_plan(B, N + 1, vocab, logit_dtype == TV_BF16 ? 2 : 4,
                                            g_smem_sm[device], g_smem_optin[device], 0, 0, 0);
-      rc = tv_launch_all(a, logit_dtype == TV_BF16 ? 1 : 0, row_list, n_rows, grid, plan, st,
-                         nullptr);
+      rc = tv_launch_all(a, logit_dtype == TV_BF16 ? 1 : 0, plan, st, nullptr);
     }
   }
   if (prev != device) cudaSetDevice(prev);

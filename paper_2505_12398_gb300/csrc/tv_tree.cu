@@ -41,7 +41,7 @@
 // Rows need no alignment: slices are copied as whole 8-element blocks of the
 // flat [B][N+1][V] arrays and the elements of the neighbouring rows in the
 // first and last block are masked.  (With V % 8 != 0 the kernel runs as the last
-// of the three-kernel path, with the row normalisers that path computes first.)
+// of the two-kernel path, with the row normalisers that path computes first.)
 //
 // Every wait is bounded; one that gives up raises TV_STATUS_TIMEOUT, and all
 // roles still reach the cluster barrier at the end.
@@ -270,7 +270,7 @@ struct TreeCta {
     return kind == kJobPass || kind == kJobBonusRes;
   }
 
-  // e(x) in draws and passes: the cheaper form, or (kExact: the three-kernel path,
+  // e(x) in draws and passes: the cheaper form, or (kExact: the two-kernel path,
   // whose normalisers come from exp_rel) that one.
   __device__ __forceinline__ float exp1(float v, float m) const {
     return kExact ? L::exp_rel(v, m, a.c_hi, a.c_lo) : L::exp_pass(v, m, a.c_hi, a.c_lo);
@@ -1208,7 +1208,9 @@ __global__ void __launch_bounds__(TreeCta<L, NCW, kExact>::kThreads, 16 / NCW)
   }
   __syncthreads();
   if (args.row_stats) {
-    // given normalisers (from the LM head's epilogue, or the three-kernel
+    // launched as a dependent of the kernel that works them out: it has ended
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    // given normalisers (from the LM head's epilogue, or the two-kernel
     // path's): every internal row is normalised up front and no normaliser job
     // is ever posted.  (Otherwise the control warp works out the children's order
     // while the first normaliser job runs.)
@@ -1329,7 +1331,8 @@ FusedPlan tv_fused_plan(int B, int R, int V, int logit_bytes, int smem_per_sm,
 namespace {
 
 template <typename L, int NCW, bool kExact>
-cudaError_t launch_one(const TravArgs& a, const FusedPlan& plan, cudaStream_t stream) {
+cudaError_t launch_one(const TravArgs& a, const FusedPlan& plan, cudaStream_t stream,
+                       bool dependent) {
   auto k = tvk::fused::tv_tree_kernel<L, NCW, kExact>;
   cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)plan.smem);
   if (e != cudaSuccess) return e;
@@ -1342,32 +1345,41 @@ cudaError_t launch_one(const TravArgs& a, const FusedPlan& plan, cudaStream_t st
   cfg.blockDim = dim3(tvk::fused::TreeCta<L, NCW, kExact>::kThreads, 1, 1);
   cfg.dynamicSmemBytes = plan.smem;
   cfg.stream = stream;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = (unsigned)plan.C;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
+  cudaLaunchAttribute attr[2];
+  unsigned n = 0;
+  if (plan.C > 1) {
+    attr[n].id = cudaLaunchAttributeClusterDimension;
+    attr[n].val.clusterDim.x = (unsigned)plan.C;
+    attr[n].val.clusterDim.y = 1;
+    attr[n++].val.clusterDim.z = 1;
+  }
+  if (dependent) {
+    attr[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[n++].val.programmaticStreamSerializationAllowed = 1;
+  }
   cfg.attrs = attr;
-  cfg.numAttrs = (plan.C > 1) ? 1 : 0;
+  cfg.numAttrs = n;
   return cudaLaunchKernelEx(&cfg, k, a, plan.C, plan.stages);
 }
 
 template <typename L, bool kExact>
-cudaError_t launch_ncw(const TravArgs& a, const FusedPlan& plan, cudaStream_t stream) {
-  if (plan.ncw == 16) return launch_one<L, 16, kExact>(a, plan, stream);
-  if (plan.ncw == 8) return launch_one<L, 8, kExact>(a, plan, stream);
-  return launch_one<L, 4, kExact>(a, plan, stream);
+cudaError_t launch_ncw(const TravArgs& a, const FusedPlan& plan, cudaStream_t stream,
+                       bool dependent) {
+  if (plan.ncw == 16) return launch_one<L, 16, kExact>(a, plan, stream, dependent);
+  if (plan.ncw == 8) return launch_one<L, 8, kExact>(a, plan, stream, dependent);
+  return launch_one<L, 4, kExact>(a, plan, stream, dependent);
 }
 
 }  // namespace
 
 int tv_launch_tree(const TravArgs& a, int logit_is_bf16, const FusedPlan& plan,
-                   cudaStream_t stream) {
+                   cudaStream_t stream, bool dependent) {
   // (fp32 logits have one exponential: the two forms are the same kernel)
   const cudaError_t e =
-      !logit_is_bf16 ? launch_ncw<tvk::F32Logits, false>(a, plan, stream)
-                     : (a.exact_exp ? launch_ncw<tvk::Bf16Logits, true>(a, plan, stream)
-                                    : launch_ncw<tvk::Bf16Logits, false>(a, plan, stream));
+      !logit_is_bf16
+          ? launch_ncw<tvk::F32Logits, false>(a, plan, stream, dependent)
+          : (a.exact_exp ? launch_ncw<tvk::Bf16Logits, true>(a, plan, stream, dependent)
+                         : launch_ncw<tvk::Bf16Logits, false>(a, plan, stream, dependent));
   if (e == cudaSuccess) return 0;
   cudaGetLastError();
   return -5;
@@ -1380,7 +1392,7 @@ int tv_launch_fused(const TravArgs& a, int logit_is_bf16, const FusedPlan& plan,
     for (int k = 0; k < 3; ++k)
       if (cudaEventRecord(ev[k], stream) != cudaSuccess) return -5;
   }
-  if (tv_launch_tree(a, logit_is_bf16, plan, stream) != 0) return -5;
+  if (tv_launch_tree(a, logit_is_bf16, plan, stream, false) != 0) return -5;
   if (ev && cudaEventRecord(ev[3], stream) != cudaSuccess) return -5;
   return 0;
 }
