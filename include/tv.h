@@ -77,9 +77,9 @@ enum {
    kernel where trees are few or rows short (a job costs less to exchange
    inside a cluster than through the persistent kernel's queue: N + 1 <= 128
    and V <= 32768, or V <= 49152 and B V <= 14 million, or B < 64 and B V <= 8.4
-   million), else the persistent kernel; the two-kernel path otherwise.  All paths compute the
-   same results; the two single-kernel paths read rows with bulk copies and
-   need V % 8 == 0, other vocabularies always take the two-kernel path. */
+   million), else the persistent kernel; the two-kernel path otherwise.  All
+   paths compute the same results; the two single-kernel paths need V % 8 == 0,
+   other vocabularies always take the two-kernel path. */
 enum {
   TV_FLAG_NONE = 0u,
   /* Two kernels: row normalisers of every internal row, then the traversal by
