@@ -115,6 +115,29 @@ __device__ __forceinline__ float2 exp2_split_x2(float2 d, float2 c_hi, float2 c_
                      __int_as_float(__float_as_int(r1) + (tb1 << 23) + k));
 }
 
+// exp2_split on a pair, with the same results (0 below the normal range), for d of
+// -1.0e4 or more (NaN: 0).
+// The hot loops of fp32 logits are bound by their arithmetic: in pairs, with the
+// clamp of d left to the caller's of v, persistent kernel: 60-node trees, V = 151936, B =
+// 256 966 -> 886 us, V = 128256, B = 64 472 -> 439 us, 26-node trees, V = 151936, B = 512
+// 1239 -> 1125 us; cluster kernel: V = 32000, B = 64 177 -> 167 us, 1024 chains of 8 730
+// -> 642 us.
+__device__ __forceinline__ float2 exp2_split_zero_x2(float2 d, float2 d_lo, float2 c_hi,
+                                                     float2 c_lo) {
+  const float2 e_hi = __fmul2_rn(d, c_hi);
+  float2 e_lo = __ffma2_rn(d, c_hi, make_float2(-e_hi.x, -e_hi.y));
+  e_lo = __ffma2_rn(d, c_lo, e_lo);
+  e_lo = __ffma2_rn(d_lo, c_hi, e_lo);
+  const float2 t = __fadd2_rn(e_hi, make_float2(12582912.f, 12582912.f));
+  const float2 nf = __fadd2_rn(t, make_float2(-12582912.f, -12582912.f));
+  const float2 f = __fadd2_rn(__fadd2_rn(e_hi, make_float2(-nf.x, -nf.y)), e_lo);
+  const uint32_t k = 0u - (0x4B400000u << 23);   // (as in exp2_split_x2)
+  const float r0 = __uint_as_float(__float_as_uint(ex2(f.x)) + (__float_as_uint(t.x) << 23) + k);
+  const float r1 = __uint_as_float(__float_as_uint(ex2(f.y)) + (__float_as_uint(t.y) << 23) + k);
+  const float least = 12582912.f - 125.f;
+  return make_float2(t.x >= least ? r0 : 0.f, t.y >= least ? r1 : 0.f);
+}
+
 // Two bf16 values packed in one 32-bit word -> float (bf16 is the upper half
 // of an IEEE float32, so widening is a shift or a mask).
 __device__ __forceinline__ float bf16_lo(uint32_t w) { return __uint_as_float(w << 16); }
@@ -196,6 +219,18 @@ struct F32Logits {
     const float bb = d - v;
     const float d_lo = (v - (d - bb)) + (-m - bb);
     return exp2_split(d, d_lo, c_hi, c_lo);
+  }
+  // exp_rel of two logits, the same results
+  __device__ static __forceinline__ float2 exp_rel_x2(float2 v, float m, float2 c_hi,
+                                                      float2 c_lo) {
+    const float least = m - 1.0e4f;
+    v = make_float2(fmaxf(v.x, least), fmaxf(v.y, least));
+    const float2 nm = make_float2(-m, -m);
+    const float2 d = __fadd2_rn(v, nm);
+    const float2 bb = __fadd2_rn(d, make_float2(-v.x, -v.y));
+    const float2 nbb = make_float2(-bb.x, -bb.y), x = __fadd2_rn(d, nbb);
+    const float2 d_lo = __fadd2_rn(__fadd2_rn(v, make_float2(-x.x, -x.y)), __fadd2_rn(nm, nbb));
+    return exp2_split_zero_x2(d, d_lo, c_hi, c_lo);
   }
   struct block { float v[8]; };
   __device__ static __forceinline__ block load_block(const elem* p) {

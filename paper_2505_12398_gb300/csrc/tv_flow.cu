@@ -487,10 +487,12 @@ __device__ void consumer_role(const TravArgs& a, const FlowArgs& f, const Smem& 
             const float2 s2 = __fadd2_rn(__fadd2_rn(e[0], e[1]), __fadd2_rn(e[2], e[3]));
             sum = s2.x + s2.y;
           } else {
-            float t[8];
+            float2 e[4];
 #pragma unroll
-            for (int k2 = 0; k2 < 8; ++k2) t[k2] = L::exp_rel(v[k2], m_run, c_hi, c_lo);
-            sum = sum8(t);
+            for (int k2 = 0; k2 < 4; ++k2)
+              e[k2] = L::exp_rel_x2(make_float2(v[2 * k2], v[2 * k2 + 1]), m_run, ch, cl);
+            const float2 s2 = __fadd2_rn(__fadd2_rn(e[0], e[1]), __fadd2_rn(e[2], e[3]));
+            sum = s2.x + s2.y;
           }
           acc.add(sum);
         }
@@ -519,23 +521,20 @@ __device__ void consumer_role(const TravArgs& a, const FlowArgs& f, const Smem& 
           for (int k2 = 0; k2 < 8; ++k2) q[k2] = 0.f;
         }
         float t[8];
-        if constexpr (S::kLB == 2) {
-          const float2 mm = make_float2(-rowmax, -rowmax);
-          const float2 al2 = make_float2(alpha1, alpha1);
-          const float2 nb2 = make_float2(-beta, -beta);
+        const float2 mm = make_float2(-rowmax, -rowmax);
+        const float2 al2 = make_float2(alpha1, alpha1);
+        const float2 nb2 = make_float2(-beta, -beta);
 #pragma unroll
-          for (int k2 = 0; k2 < 4; ++k2) {
-            const float2 e = exp2_corrected_x2(__fadd2_rn(vp[k2], mm), ch, cl);
-            const float2 xx =
-                __ffma2_rn(al2, e, __fmul2_rn(nb2, make_float2(q[2 * k2], q[2 * k2 + 1])));
-            t[2 * k2] = fmaxf(xx.x, 0.f);
-            t[2 * k2 + 1] = fmaxf(xx.y, 0.f);
-          }
-        } else {
-#pragma unroll
-          for (int k2 = 0; k2 < 8; ++k2)
-            t[k2] = fmaxf(fmaf(alpha1, L::exp_pass(v[k2], rowmax, c_hi, c_lo), -beta * q[k2]),
-                          0.f);
+        for (int k2 = 0; k2 < 4; ++k2) {
+          float2 e;
+          if constexpr (S::kLB == 2)
+            e = exp2_corrected_x2(__fadd2_rn(vp[k2], mm), ch, cl);
+          else
+            e = L::exp_rel_x2(make_float2(v[2 * k2], v[2 * k2 + 1]), rowmax, ch, cl);
+          const float2 xx =
+              __ffma2_rn(al2, e, __fmul2_rn(nb2, make_float2(q[2 * k2], q[2 * k2 + 1])));
+          t[2 * k2] = fmaxf(xx.x, 0.f);
+          t[2 * k2 + 1] = fmaxf(xx.y, 0.f);
         }
         while (mp < nmask && mtok[mp] < xg) ++mp;
         for (int mq = mp; mq < nmask && mtok[mq] < xg + kChunk; ++mq) {

@@ -50,7 +50,7 @@
 // consumers doing the control, a reduction and an exchange per row and no
 // resident pairs: V = 32000, B = 64 254 -> 139 us (183 with a row by all warps in turn
 // and before the removal of a rate-0 sibling and the descent into a sub-tree were
-// worked out ahead, 149 one tile at a time); 16 chains 117 -> 63 us; V = 128256, B =
+// worked out ahead, 149 one tile at a time); 16 chains 117 -> 61 us; V = 128256, B =
 // 32 368 -> 184 us (213 one tile at a time).
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -177,9 +177,13 @@ __device__ __forceinline__ void exp8(const float v[8], float m, float c_hi, floa
       e[2 * k + 1] = r.y;
     }
   } else {
+    const float2 ch = make_float2(c_hi, c_hi), cl = make_float2(c_lo, c_lo);
 #pragma unroll
-    for (int k = 0; k < 8; ++k)
-      e[k] = kPass ? L::exp_pass(v[k], m, c_hi, c_lo) : L::exp_rel(v[k], m, c_hi, c_lo);
+    for (int k = 0; k < 4; ++k) {
+      const float2 r = L::exp_rel_x2(make_float2(v[2 * k], v[2 * k + 1]), m, ch, cl);
+      e[2 * k] = r.x;
+      e[2 * k + 1] = r.y;
+    }
   }
 }
 
@@ -194,18 +198,13 @@ __device__ __forceinline__ void residual8(const float v[8], const float* qp, flo
                       __uint_as_float(qc.z), __uint_as_float(qc.w)};
   float e[8];
   exp8<L, !kExact>(v, rowmax, c_hi, c_lo, e);
-  if constexpr (L::kBytes == 2) {
-    const float2 al2 = make_float2(alpha, alpha), nb2 = make_float2(-beta, -beta);
+  const float2 al2 = make_float2(alpha, alpha), nb2 = make_float2(-beta, -beta);
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      const float2 x = __ffma2_rn(al2, make_float2(e[2 * k], e[2 * k + 1]),
-                                  __fmul2_rn(nb2, make_float2(q[2 * k], q[2 * k + 1])));
-      t[2 * k] = fmaxf(x.x, 0.f);
-      t[2 * k + 1] = fmaxf(x.y, 0.f);
-    }
-  } else {
-#pragma unroll
-    for (int k = 0; k < 8; ++k) t[k] = fmaxf(fmaf(alpha, e[k], -beta * q[k]), 0.f);
+  for (int k = 0; k < 4; ++k) {
+    const float2 x = __ffma2_rn(al2, make_float2(e[2 * k], e[2 * k + 1]),
+                                __fmul2_rn(nb2, make_float2(q[2 * k], q[2 * k + 1])));
+    t[2 * k] = fmaxf(x.x, 0.f);
+    t[2 * k + 1] = fmaxf(x.y, 0.f);
   }
 }
 

@@ -108,3 +108,29 @@ def test_runs_of_siblings(tv, path, sigma):
     w = Workload("siblings", 24, 8008, levels=(12, 3), branching=(12, 3), sigma=sigma)
     inp = make_inputs(w, seed=int(100 * sigma), device="cuda")
     _check(inp, _verify(tv, inp, path))
+
+
+@pytest.mark.parametrize("path", ["cluster", "persistent"])
+@pytest.mark.parametrize("value", [float("inf"), float("-inf")])
+def test_fp32_rows_without_a_normaliser(tv, path, value):
+    """The packed exponentials of fp32 logits give such rows the weights of the scalar
+    ones: 0, so the tree is invalid and the others are what they were."""
+    w = Workload("nonfinite", 5, 8008, levels=(2, 3), branching=(2, 2),
+                 logit_dtype=torch.float32, sigma=1.0)
+    inp = make_inputs(w, seed=8, device="cuda")
+    clean = [x.clone() for x in _verify(tv, inp, path)[:3]]
+    if value > 0:
+        inp.logits[3, 0, 4001] = value
+    else:
+        inp.logits[3, 0] = value
+    R = inp.parents.shape[1]
+    v = tv.Verifier(8008, R - 1, 5, "fp32", path=path)
+    out = v.verify(inp.parents, inp.tokens, inp.logits, inp.draft_probs, inp.temperature,
+                   inp.uniforms)
+    torch.cuda.synchronize()
+    assert v.status() & ~16 == 64
+    v.close()
+    assert int(out[1][3]) == -1 and int(out[2][3]) == -1
+    keep = [0, 1, 2, 4]
+    for x, y in zip(out[:3], clean):
+        assert torch.equal(x[keep], y[keep])
