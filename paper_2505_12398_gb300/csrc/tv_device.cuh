@@ -115,19 +115,22 @@ __device__ __forceinline__ float2 exp2_split_x2(float2 d, float2 c_hi, float2 c_
                      __int_as_float(__float_as_int(r1) + (tb1 << 23) + k));
 }
 
-// exp2_split on a pair, with the same results (0 below the normal range), for d of
-// -1.0e4 or more (NaN: 0).
+// exp2_split on a pair, with the same results (0 below the normal range), for any d <= 0:
+// the comparison takes out whatever the bits below it hold, also where |E| is so
+// large that e_lo alone passes 2 (a masked logit at a temperature under 2e-4), for d
+// = -inf and for NaN.  kLow: d + d_lo.
 // The hot loops of fp32 logits are bound by their arithmetic: in pairs, with the
 // clamp of d left to the caller's of v, persistent kernel: 60-node trees, V = 151936, B =
 // 256 966 -> 886 us, V = 128256, B = 64 472 -> 439 us, 26-node trees, V = 151936, B = 512
 // 1239 -> 1125 us; cluster kernel: V = 32000, B = 64 177 -> 167 us, 1024 chains of 8 730
 // -> 642 us.
-__device__ __forceinline__ float2 exp2_split_zero_x2(float2 d, float2 d_lo, float2 c_hi,
-                                                     float2 c_lo) {
+template <bool kLow = false>
+__device__ __forceinline__ float2 exp2_split_zero_x2(float2 d, float2 c_hi, float2 c_lo,
+                                                     float2 d_lo = make_float2(0.f, 0.f)) {
   const float2 e_hi = __fmul2_rn(d, c_hi);
   float2 e_lo = __ffma2_rn(d, c_hi, make_float2(-e_hi.x, -e_hi.y));
   e_lo = __ffma2_rn(d, c_lo, e_lo);
-  e_lo = __ffma2_rn(d_lo, c_hi, e_lo);
+  if constexpr (kLow) e_lo = __ffma2_rn(d_lo, c_hi, e_lo);
   const float2 t = __fadd2_rn(e_hi, make_float2(12582912.f, 12582912.f));
   const float2 nf = __fadd2_rn(t, make_float2(-12582912.f, -12582912.f));
   const float2 f = __fadd2_rn(__fadd2_rn(e_hi, make_float2(-nf.x, -nf.y)), e_lo);
@@ -230,7 +233,7 @@ struct F32Logits {
     const float2 bb = __fadd2_rn(d, make_float2(-v.x, -v.y));
     const float2 nbb = make_float2(-bb.x, -bb.y), x = __fadd2_rn(d, nbb);
     const float2 d_lo = __fadd2_rn(__fadd2_rn(v, make_float2(-x.x, -x.y)), __fadd2_rn(nm, nbb));
-    return exp2_split_zero_x2(d, d_lo, c_hi, c_lo);
+    return exp2_split_zero_x2<true>(d, c_hi, c_lo, d_lo);
   }
   struct block { float v[8]; };
   __device__ static __forceinline__ block load_block(const elem* p) {

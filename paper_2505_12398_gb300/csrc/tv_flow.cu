@@ -466,35 +466,26 @@ __device__ void consumer_role(const TravArgs& a, const FlowArgs& f, const Smem& 
         }
       }
       if (kind == kJobStats) {
-        if (valid) {
-          float cm = v[0];
+        if constexpr (S::kLB == 4) {   // (bf16: above)
+          if (valid) {
+            float cm = v[0];
 #pragma unroll
-          for (int k2 = 1; k2 < 8; ++k2) cm = fmaxf(cm, v[k2]);
-          if (cm > m_run) {
-            if (m_run != TV_NEG_INF) {
-              const float sc = L::exp_rel(m_run, cm, c_hi, c_lo);
-              acc.s *= sc;
-              acc.c *= sc;
+            for (int k2 = 1; k2 < 8; ++k2) cm = fmaxf(cm, v[k2]);
+            if (cm > m_run) {
+              if (m_run != TV_NEG_INF) {
+                const float sc = L::exp_rel(m_run, cm, c_hi, c_lo);
+                acc.s *= sc;
+                acc.c *= sc;
+              }
+              m_run = cm;
             }
-            m_run = cm;
-          }
-          float sum;
-          if constexpr (S::kLB == 2) {
-            const float2 mm = make_float2(-m_run, -m_run);
-            float2 e[4];
-#pragma unroll
-            for (int k2 = 0; k2 < 4; ++k2) e[k2] = exp2_split_x2(__fadd2_rn(vp[k2], mm), ch, cl);
-            const float2 s2 = __fadd2_rn(__fadd2_rn(e[0], e[1]), __fadd2_rn(e[2], e[3]));
-            sum = s2.x + s2.y;
-          } else {
             float2 e[4];
 #pragma unroll
             for (int k2 = 0; k2 < 4; ++k2)
               e[k2] = L::exp_rel_x2(make_float2(v[2 * k2], v[2 * k2 + 1]), m_run, ch, cl);
             const float2 s2 = __fadd2_rn(__fadd2_rn(e[0], e[1]), __fadd2_rn(e[2], e[3]));
-            sum = s2.x + s2.y;
+            acc.add(s2.x + s2.y);
           }
-          acc.add(sum);
         }
       } else if (kind == kJobBonusLeaf) {
         float lm = v[0];

@@ -172,7 +172,7 @@ __device__ __forceinline__ void exp8(const float v[8], float m, float c_hi, floa
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
       const float2 d = __fadd2_rn(make_float2(v[2 * k], v[2 * k + 1]), mm);
-      const float2 r = kPass ? exp2_corrected_x2(d, ch, cl) : exp2_split_x2(d, ch, cl);
+      const float2 r = kPass ? exp2_corrected_x2(d, ch, cl) : exp2_split_zero_x2(d, ch, cl);
       e[2 * k] = r.x;
       e[2 * k + 1] = r.y;
     }
