@@ -93,28 +93,6 @@ __device__ __forceinline__ float2 exp2_corrected_x2(float2 d, float2 c_hi, float
   return __ffma2_rn(r, t, r);
 }
 
-// exp2_split on a pair (d already clamped below).  Results below 2^-125 are
-// returned as a value under 2^-124 instead of the exact tiny number.
-// kLow: d + d_lo.
-template <bool kLow = false>
-__device__ __forceinline__ float2 exp2_split_x2(float2 d, float2 c_hi, float2 c_lo,
-                                                float2 d_lo = make_float2(0.f, 0.f)) {
-  const float2 e_hi = __fmul2_rn(d, c_hi);
-  float2 e_lo = __ffma2_rn(d, c_hi, make_float2(-e_hi.x, -e_hi.y));
-  e_lo = __ffma2_rn(d, c_lo, e_lo);
-  if constexpr (kLow) e_lo = __ffma2_rn(d_lo, c_hi, e_lo);
-  const float2 t = __fadd2_rn(e_hi, make_float2(12582912.f, 12582912.f));
-  const float2 nf = __fadd2_rn(t, make_float2(-12582912.f, -12582912.f));
-  const float2 f = __fadd2_rn(__fadd2_rn(e_hi, make_float2(-nf.x, -nf.y)), e_lo);
-  const int tb0 = max(__float_as_int(t.x), 0x4B400000 - 125);
-  const int tb1 = max(__float_as_int(t.y), 0x4B400000 - 125);
-  const float r0 = ex2(f.x), r1 = ex2(f.y);
-  // bits(r) + n * 2^23, n = bits(t) - bits(1.5 * 2^23), in modular arithmetic
-  const int k = (int)(0u - (0x4B400000u << 23));
-  return make_float2(__int_as_float(__float_as_int(r0) + (tb0 << 23) + k),
-                     __int_as_float(__float_as_int(r1) + (tb1 << 23) + k));
-}
-
 // exp2_split on a pair, with the same results (0 below the normal range), for any d <= 0:
 // the comparison takes out whatever the bits below it hold, also where |E| is so
 // large that e_lo alone passes 2 (a masked logit at a temperature under 2e-4), for d
@@ -134,7 +112,8 @@ __device__ __forceinline__ float2 exp2_split_zero_x2(float2 d, float2 c_hi, floa
   const float2 t = __fadd2_rn(e_hi, make_float2(12582912.f, 12582912.f));
   const float2 nf = __fadd2_rn(t, make_float2(-12582912.f, -12582912.f));
   const float2 f = __fadd2_rn(__fadd2_rn(e_hi, make_float2(-nf.x, -nf.y)), e_lo);
-  const uint32_t k = 0u - (0x4B400000u << 23);   // (as in exp2_split_x2)
+  // bits(2^f) + n * 2^23, n = bits(t) - bits(1.5 * 2^23), in modular arithmetic
+  const uint32_t k = 0u - (0x4B400000u << 23);
   const float r0 = __uint_as_float(__float_as_uint(ex2(f.x)) + (__float_as_uint(t.x) << 23) + k);
   const float r1 = __uint_as_float(__float_as_uint(ex2(f.y)) + (__float_as_uint(t.y) << 23) + k);
   const float least = 12582912.f - 125.f;
@@ -162,8 +141,7 @@ struct Bf16Logits {
   __device__ static __forceinline__ float exp_rel(float v, float m, float c_hi, float c_lo) {
     return exp2_split(v - m, 0.f, c_hi, c_lo);
   }
-  // Eight logits as a block, and exp_rel of them relative to m, v - m clamped below
-  // at d_min (weights there are under 2^-124 instead of 0).
+  // Eight logits as a block, and exp_rel of them relative to m.
   using block = uint4;
   __device__ static __forceinline__ block load_block(const elem* p) { return ld_nc16(p); }
   __device__ static __forceinline__ block make_block(const elem* p, int lo, int hi) {
@@ -185,15 +163,14 @@ struct Bf16Logits {
     const uint32_t u = *reinterpret_cast<const uint32_t*>(&m);
     return fmaxf(bf16_lo(u), bf16_hi(u));
   }
-  __device__ static __forceinline__ void block_exp(const block& b, float m, float d_min,
-                                                   float2 c_hi, float2 c_lo, float2 t[4]) {
+  __device__ static __forceinline__ void block_exp(const block& b, float m, float2 c_hi,
+                                                   float2 c_lo, float2 t[4]) {
     const uint32_t w[4] = {b.x, b.y, b.z, b.w};
     const float2 nm = make_float2(-m, -m);
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      const float2 d = __fadd2_rn(make_float2(bf16_lo(w[k]), bf16_hi(w[k])), nm);
-      t[k] = exp2_split_x2(make_float2(fmaxf(d.x, d_min), fmaxf(d.y, d_min)), c_hi, c_lo);
-    }
+    for (int k = 0; k < 4; ++k)
+      t[k] = exp2_split_zero_x2(__fadd2_rn(make_float2(bf16_lo(w[k]), bf16_hi(w[k])), nm), c_hi,
+                                c_lo);
   }
   // cheaper form for the per-element work of rejection passes and bonus draws
   __device__ static __forceinline__ float exp_pass(float v, float m, float c_hi, float c_lo) {
@@ -251,19 +228,11 @@ struct F32Logits {
     return fmaxf(fmaxf(fmaxf(b.v[0], b.v[1]), fmaxf(b.v[2], b.v[3])),
                  fmaxf(fmaxf(b.v[4], b.v[5]), fmaxf(b.v[6], b.v[7])));
   }
-  __device__ static __forceinline__ void block_exp(const block& b, float m, float d_min,
-                                                   float2 c_hi, float2 c_lo, float2 t[4]) {
-    const float least = m + d_min;
-    const float2 nm = make_float2(-m, -m);
+  __device__ static __forceinline__ void block_exp(const block& b, float m, float2 c_hi,
+                                                   float2 c_lo, float2 t[4]) {
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      const float2 v = make_float2(fmaxf(b.v[2 * k], least), fmaxf(b.v[2 * k + 1], least));
-      const float2 d = __fadd2_rn(v, nm);
-      const float2 bb = __fadd2_rn(d, make_float2(-v.x, -v.y));
-      const float2 nbb = make_float2(-bb.x, -bb.y), x = __fadd2_rn(d, nbb);
-      const float2 d_lo = __fadd2_rn(__fadd2_rn(v, make_float2(-x.x, -x.y)), __fadd2_rn(nm, nbb));
-      t[k] = exp2_split_x2<true>(d, c_hi, c_lo, d_lo);
-    }
+    for (int k = 0; k < 4; ++k)
+      t[k] = exp_rel_x2(make_float2(b.v[2 * k], b.v[2 * k + 1]), m, c_hi, c_lo);
   }
   __device__ static __forceinline__ float exp_pass(float v, float m, float c_hi, float c_lo) {
     return exp_rel(v, m, c_hi, c_lo);

@@ -22,11 +22,10 @@
 //
 // The normaliser kernel is bound by its arithmetic, a third of the HBM rate: 16
 // instructions per logit at 69 % of the issue slots before the maximum of a pair
-// of bf16 took one instruction, the weights below 2^-125 one clamp instead of a
-// comparison and a selection, and the logits stayed packed until they are used (48
+// of bf16 took one instruction and the logits stayed packed until they are used (48
 // registers, five blocks per SM).  With four blocks of logits per thread at a time,
 // also at a row's end, and two weights per instruction, against one block at a time
-// and scalar arithmetic: 256 trees, V = 32003 270 -> 159 us, 32 trees 45 -> 30 us
+// and scalar arithmetic: 256 trees, V = 32003 270 -> 155 us, 32 trees 45 -> 30 us
 // (the bytes alone 92 and 11 us).
 //
 // The mutable distributions of Algorithm 3 are never materialised.  After k
@@ -78,7 +77,6 @@ __global__ void __launch_bounds__(kStatsThreads, kStatsThreads == 256 ? 6 - L::k
   Comp acc;
   const int step = kStatsThreads * kChunk;
   const float2 ch = make_float2(c_hi, c_hi), cl = make_float2(c_lo, c_lo);
-  const float d_min = fmaxf(-150.f / c_hi, -1.0e4f);
   for (int x0 = threadIdx.x * kChunk; x0 < end; x0 += kStatsUnroll * step) {
     typename L::block v[kStatsUnroll];
     const bool edge = x0 < sh || x0 + (kStatsUnroll - 1) * step + kChunk > end;
@@ -111,7 +109,7 @@ __global__ void __launch_bounds__(kStatsThreads, kStatsThreads == 256 ? 6 - L::k
       const int x = x0 + u * step;
       if (x >= end) break;
       float2 t[4];
-      L::block_exp(v[u], m, d_min, ch, cl, t);
+      L::block_exp(v[u], m, ch, cl, t);
       if (edge) {              // (-inf has a weight at a high temperature)
 #pragma unroll
         for (int k = 0; k < 4; ++k) {

@@ -67,3 +67,30 @@ def test_masked_logits_at_low_temperatures(path, V, dtype, T):
     """The weight of a masked token is 0 however large the exponent."""
     inp = _inputs(8, V, dtype, T, seed=V % 1000)
     _check(inp, _run(inp, path))
+
+
+@pytest.mark.parametrize("path,V,dtype", [
+    ("two", 8005, torch.float32), ("two", 40003, torch.float32), ("two", 8005, torch.bfloat16),
+    ("cluster", 8008, torch.float32), ("cluster", 8008, torch.bfloat16),
+    ("persistent", 8008, torch.float32), ("persistent", 8008, torch.bfloat16)])
+@pytest.mark.parametrize("T", [1e-6, 1e-9, 1e-20])
+def test_one_token_holds_the_mass(path, V, dtype, T):
+    """Ordinary logits at a temperature that leaves each row's largest all of the mass,
+    down to where the least exponent times T is lost beside the logit; even trees drafted
+    it, so that leaves are accepted."""
+    inp = _inputs(6, V, dtype, 1.0, masked=0.1, seed=V % 1000)
+    inp.temperature = T
+    par = inp.parents[0].tolist()
+    for i in range(len(par)):
+        kids = [c for c in range(1, len(par)) if par[c] == i]
+        if not kids:
+            continue
+        # (bf16 rows have ties at the top)
+        top = inp.logits[:, i].float().argmax(dim=-1).to(torch.int32)
+        inp.logits[torch.arange(6), i, top.long()] += 1.0
+        for b in range(0, 6, 2):
+            for c in kids[1:]:
+                if inp.tokens[b, c] == top[b]:
+                    inp.tokens[b, c] = inp.tokens[b, kids[0]]
+            inp.tokens[b, kids[0]] = top[b]
+    _check(inp, _run(inp, path))
