@@ -68,22 +68,19 @@ __device__ __forceinline__ float exp2_corrected(float d, float c_hi, float c_lo)
 
 // ---- packed-pair (float2) forms for the bf16 hot loops (sm_100+ f32x2) ----
 
-// Eight bf16 logits from one 16-byte word, clamped below at -9984 (so -inf and
-// NaN become a finite number whose weight is 0 or below 2^-125) and widened
-// to four (even, odd) float pairs.
+// Eight bf16 logits from one 16-byte word, widened to four (even, odd) float pairs
+// (bf16 is the upper half of an IEEE float32).
 __device__ __forceinline__ void bf16x8_pairs(uint4 w, float2 out[4]) {
-  const uint32_t lo_clamp = 0xC61CC61Cu;   // two bf16 -9984
-  uint32_t ws[4] = {w.x, w.y, w.z, w.w};
+  const uint32_t ws[4] = {w.x, w.y, w.z, w.w};
 #pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    __nv_bfloat162 h = *reinterpret_cast<__nv_bfloat162*>(&ws[k]);
-    h = __hmax2(h, *reinterpret_cast<const __nv_bfloat162*>(&lo_clamp));
-    const uint32_t c = *reinterpret_cast<uint32_t*>(&h);
-    out[k] = make_float2(__uint_as_float(c << 16), __uint_as_float(c & 0xffff0000u));
-  }
+  for (int k = 0; k < 4; ++k)
+    out[k] = make_float2(__uint_as_float(ws[k] << 16), __uint_as_float(ws[k] & 0xffff0000u));
 }
 
-// exp2_corrected on a pair (d already clamped below).
+// exp2_corrected on a pair, for finite d <= 0.  d = -inf and NaN, and a finite d whose
+// exponent overflows, give NaN (or 0): the caller's maximum with 0 (kept from a residual,
+// added to a sum of weights) makes that a weight of 0.  A bound on the logits in its
+// place would have to be relative to the row's maximum, which may be anywhere.
 __device__ __forceinline__ float2 exp2_corrected_x2(float2 d, float2 c_hi, float2 c_lo) {
   const float2 e_hi = __fmul2_rn(d, c_hi);
   float2 e_lo = __ffma2_rn(d, c_hi, make_float2(-e_hi.x, -e_hi.y));

@@ -394,12 +394,11 @@ __device__ void consumer_role(const TravArgs& a, const FlowArgs& f, const Smem& 
     if constexpr (S::kLB == 2) {
       if (kind == kJobStats) {
         // Row normaliser, bf16: this warp's maximum over its part of the stage
-        // first (exact on bf16 pairs, after the same clamp as the sums), so
-        // that the running sum is rescaled at most once per stage, then the
-        // sum of e(x) relative to it.  exp2_corrected is used here as in the
+        // first (exact on bf16 pairs), so that the running sum is rescaled at
+        // most once per stage, then the sum of e(x) relative to it.  exp2_corrected is used here as in the
         // passes: its small uniform bias then cancels in alpha1 e(x) = p a e(x)/s.
-        const uint32_t lo_clamp = 0xC61CC61Cu;   // two bf16 -9984
-        __nv_bfloat162 hm = *reinterpret_cast<const __nv_bfloat162*>(&lo_clamp);
+        const uint32_t none = 0xFF80FF80u;   // two bf16 -inf
+        __nv_bfloat162 hm = *reinterpret_cast<const __nv_bfloat162*>(&none);
         for (int t0 = wid * kTileElems; t0 < n; t0 += S::kSweep) {
           const int e0 = t0 + lane * kChunk;
           if (e0 < n) {
@@ -429,8 +428,10 @@ __device__ void consumer_role(const TravArgs& a, const FlowArgs& f, const Smem& 
             bf16x8_pairs(lds128(lb + e0), vp);
             float2 e[4];
 #pragma unroll
-            for (int k2 = 0; k2 < 4; ++k2)
+            for (int k2 = 0; k2 < 4; ++k2) {
               e[k2] = exp2_corrected_x2(__fadd2_rn(vp[k2], mm), ch, cl);
+              e[k2] = make_float2(fmaxf(e[k2].x, 0.f), fmaxf(e[k2].y, 0.f));
+            }
             const float2 s2 = __fadd2_rn(__fadd2_rn(e[0], e[1]), __fadd2_rn(e[2], e[3]));
             acc.add(s2.x + s2.y);
           }
@@ -448,7 +449,7 @@ __device__ void consumer_role(const TravArgs& a, const FlowArgs& f, const Smem& 
         if (valid) bf16x8_pairs(lds128(lb + e0), vp);
         else {
 #pragma unroll
-          for (int k2 = 0; k2 < 4; ++k2) vp[k2] = make_float2(-9984.f, -9984.f);
+          for (int k2 = 0; k2 < 4; ++k2) vp[k2] = make_float2(TV_NEG_INF, TV_NEG_INF);
         }
 #pragma unroll
         for (int k2 = 0; k2 < 4; ++k2) { v[2 * k2] = vp[k2].x; v[2 * k2 + 1] = vp[k2].y; }
@@ -493,8 +494,17 @@ __device__ void consumer_role(const TravArgs& a, const FlowArgs& f, const Smem& 
         for (int k2 = 1; k2 < 8; ++k2) lm = fmaxf(lm, v[k2]);
         const float tm = warp_max(lm);
         float t[8];
+        const float2 mm = make_float2(-tm, -tm);
 #pragma unroll
-        for (int k2 = 0; k2 < 8; ++k2) t[k2] = L::exp_pass(v[k2], tm, c_hi, c_lo);
+        for (int k2 = 0; k2 < 4; ++k2) {
+          float2 e;
+          if constexpr (S::kLB == 2)
+            e = exp2_corrected_x2(__fadd2_rn(vp[k2], mm), ch, cl);
+          else
+            e = L::exp_rel_x2(make_float2(v[2 * k2], v[2 * k2 + 1]), tm, ch, cl);
+          t[2 * k2] = fmaxf(e.x, 0.f);
+          t[2 * k2 + 1] = fmaxf(e.y, 0.f);
+        }
         const float ts = warp_sum(valid ? sum8(t) : 0.f);
         if (lane == 0)
           __stcg(f.tiles + (size_t)b * f.ntiles + (x + t0) / kTileElems, make_float2(ts, tm));

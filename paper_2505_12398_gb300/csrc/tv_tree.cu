@@ -139,7 +139,7 @@ struct Slice {
 
 __device__ __forceinline__ int chunks_of(int n, int per) { return (n + per - 1) / per; }
 
-// Eight logits of one lane: bf16 clamped and widened, or fp32.
+// Eight logits of one lane: bf16 widened, or fp32.
 template <typename L>
 __device__ __forceinline__ void lds_logits(const typename L::elem* p, float v[8]) {
   if constexpr (L::kBytes == 2) {
@@ -162,7 +162,7 @@ __device__ __forceinline__ float max8(const float v[8]) {
 }
 
 // e(x) of eight logits relative to m (kPass: the cheaper form of passes and
-// draws; see tv_device.cuh).
+// draws, which leaves NaN for a weight of 0; see tv_device.cuh).
 template <typename L, bool kPass>
 __device__ __forceinline__ void exp8(const float v[8], float m, float c_hi, float c_lo,
                                      float e[8]) {
@@ -367,20 +367,19 @@ struct TreeCta {
   // --------------------------------------------------------- consumers --
 
   // The eight logits of the lane's block e0 of a stage, whose elements [lo, hi)
-  // belong to the slice (the others read as the smallest value).
+  // belong to the slice (the others read as -inf).
   __device__ __forceinline__ void stage_logits(const E* lb, int e0, bool valid, bool edge, int lo,
                                                int hi, float v[8]) const {
-    constexpr float kNone = kLB == 2 ? -9984.f : -INFINITY;
     if (valid) {
       lds_logits<L>(lb + e0, v);
     } else {
 #pragma unroll
-      for (int e = 0; e < 8; ++e) v[e] = kNone;
+      for (int e = 0; e < 8; ++e) v[e] = TV_NEG_INF;
     }
     if (edge) {
 #pragma unroll
       for (int e = 0; e < 8; ++e)
-        if (e < lo || e >= hi) v[e] = kNone;
+        if (e < lo || e >= hi) v[e] = TV_NEG_INF;
     }
   }
   static __device__ __forceinline__ void zero_outside(bool edge, int lo, int hi, float t[8]) {
@@ -552,6 +551,8 @@ struct TreeCta {
         if (kind == kJobBonusLeaf) {
           const float tm = warp_max(max8(v));
           exp8<L, !kExact>(v, tm, c_hi, c_lo, t);
+#pragma unroll
+          for (int e = 0; e < 8; ++e) t[e] = fmaxf(t[e], 0.f);
           zero_outside(edge, lo, hi, t);
           const float ts = warp_sum(valid ? sum8(t) : 0.f);
           if (lane == 0) {

@@ -94,3 +94,63 @@ def test_one_token_holds_the_mass(path, V, dtype, T):
                     inp.tokens[b, c] = inp.tokens[b, kids[0]]
             inp.tokens[b, kids[0]] = top[b]
     _check(inp, _run(inp, path))
+
+
+def _given(inp):
+    """(max, sum of 2^((l - max) log2(e) / T)) of every row, in float64."""
+    lf = inp.logits.double()
+    m = lf.max(dim=-1).values
+    s = torch.exp((lf - m[..., None]) / inp.temperature).sum(dim=-1)
+    return torch.stack([m, s], dim=-1).float().contiguous()
+
+
+@pytest.mark.parametrize("path,V,dtype", [
+    ("cluster", 8008, torch.bfloat16), ("cluster", 65544, torch.bfloat16),
+    ("persistent", 8008, torch.bfloat16), ("two", 8005, torch.bfloat16),
+    ("cluster", 8008, torch.float32), ("persistent", 8008, torch.float32),
+    ("two", 8005, torch.float32)])
+@pytest.mark.parametrize("shift", [-30000.0, 30000.0])
+def test_rows_far_from_zero(path, V, dtype, shift):
+    """Weights depend on the distance to the row's maximum alone: rows wholly below (or
+    above) what a masked logit might be taken for, with normalisers of the call's own
+    and given ones."""
+    inp = _inputs(8, V, dtype, 300.0, shift=shift, seed=V % 1000)
+    _check(inp, _run(inp, path))
+    if path == "two":
+        return
+    import paper_2505_12398_gb300 as tv
+    B, R = inp.parents.shape
+    # (a handle of the cluster path does not take normalisers; one that chooses does)
+    v = tv.Verifier(V, R - 1, B, "bf16" if dtype == torch.bfloat16 else "fp32",
+                    path="auto" if path == "cluster" else path)
+    assert v.launch_shape(B, R - 1)[0] == PATH_CODE[path]
+    out = v.verify_stats(inp.parents, inp.tokens, inp.logits, inp.draft_probs, inp.temperature,
+                         inp.uniforms, _given(inp), debug=True)
+    torch.cuda.synchronize()
+    assert v.status() & ~16 == 0
+    v.close()
+    _check(inp, out)
+
+
+@pytest.mark.parametrize("path,V", [("cluster", 8008), ("persistent", 8008), ("two", 8005)])
+@pytest.mark.parametrize("value", [float("-inf"), float("inf")])
+def test_bf16_rows_without_a_normaliser(path, V, value):
+    """A row the traversal needs without a finite logit, or with +inf, makes its tree
+    invalid and no other."""
+    import paper_2505_12398_gb300 as tv
+    inp = _inputs(6, V, torch.bfloat16, 1.0)
+    clean = _run(inp, path)
+    if value < 0:
+        inp.logits[2, 0] = value
+    else:
+        inp.logits[2, 0, V - 3] = value
+    R = inp.parents.shape[1]
+    v = tv.Verifier(V, R - 1, 6, "bf16", path="auto" if path == "two" else path)
+    out = v.verify(inp.parents, inp.tokens, inp.logits, inp.draft_probs, 1.0, inp.uniforms)
+    torch.cuda.synchronize()
+    assert v.status() & ~16 == 64
+    v.close()
+    assert int(out[1][2]) == -1 and int(out[2][2]) == -1 and (out[0][2] == -1).all()
+    keep = [0, 1, 3, 4, 5]
+    for x, y in zip(out[:3], clean):
+        assert torch.equal(x[keep], y[keep])

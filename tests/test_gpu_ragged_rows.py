@@ -80,4 +80,8 @@ def test_rows_without_a_normaliser(B, V, dtype):
     assert status == 0
     first = int((inp.parents[1] == 0).nonzero()[0])
     assert int(inp.tokens[1, 1]) == int(inp.tokens[1, first])
-    assert int(out[1][1]) >= 0
+    inp.logits = lg
+    par, tok, lgn, dp, un = to_numpy_inputs(inp, trees=[1])
+    _, _, _, det = verify_batch(par, tok, lgn, dp, inp.temperature, un, keep_cdf=True)
+    summ = compare_batch(det, *[x[1:2].cpu().numpy() for x in out])
+    assert not summ["bad"], summ["bad"]
