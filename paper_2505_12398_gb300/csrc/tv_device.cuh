@@ -32,21 +32,21 @@ __device__ __forceinline__ float ex2(float x) {
   return y;
 }
 
-// 2^E for E = d c with c = c_hi + c_lo and d = d_hi + d_lo (see above).
+// 2^E for E = d c with c = c_hi + c_lo and d = d_hi + d_lo (see above), d <= 0.  Below
+// the normal range, for d = -inf and for NaN the weight is exactly 0, at any
+// temperature (masked and padding elements, read as -inf, contribute nothing): the
+// comparison takes out whatever the bits below it hold.
 __device__ __forceinline__ float exp2_split(float d, float d_lo, float c_hi, float c_lo) {
-  d = fmaxf(d, -1.0e4f);                      // -inf / NaN logits -> weight ~0
   const float e_hi = d * c_hi;
   float e_lo = fmaf(d, c_hi, -e_hi);          // exact error of the product
   e_lo = fmaf(d, c_lo, e_lo);
   e_lo = fmaf(d_lo, c_hi, e_lo);
   const float t = e_hi + 12582912.f;          // 1.5 * 2^23: round to integer
   const float nf = t - 12582912.f;
-  int ni = __float_as_int(t) - 0x4B400000;
   const float f = (e_hi - nf) + e_lo;         // e_hi - nf is exact
-  const float r = ex2(f);
-  // below the normal range the weight is taken as exactly 0 (this also makes
-  // padding elements, read as -inf, contribute nothing)
-  return (ni < -125) ? 0.f : __int_as_float(__float_as_int(r) + (ni << 23));
+  // bits(2^f) + n * 2^23, n = bits(t) - bits(1.5 * 2^23), in modular arithmetic
+  const uint32_t r = __float_as_uint(ex2(f)) + (__float_as_uint(t) << 23) - (0x4B400000u << 23);
+  return t >= 12582912.f - 125.f ? __uint_as_float(r) : 0.f;
 }
 
 // 2^E for E = d c, by a first-order correction of ex2.approx(E_hi) with the
@@ -58,12 +58,11 @@ __device__ __forceinline__ float exp2_split(float d, float d_lo, float c_hi, flo
 // (numerator and normaliser of the same distribution) or only decides
 // near-ties (the bonus draw).
 __device__ __forceinline__ float exp2_corrected(float d, float c_hi, float c_lo) {
-  d = fmaxf(d, -1.0e4f);
   const float e_hi = d * c_hi;
   float e_lo = fmaf(d, c_hi, -e_hi);
   e_lo = fmaf(d, c_lo, e_lo);
   const float r = ex2(e_hi);
-  return fmaf(r, e_lo * 0.6931471805599453f, r);
+  return fmaxf(fmaf(r, e_lo * 0.6931471805599453f, r), 0.f);   // (d = -inf and NaN: 0)
 }
 
 // ---- packed-pair (float2) forms for the bf16 hot loops (sm_100+ f32x2) ----
@@ -90,15 +89,11 @@ __device__ __forceinline__ float2 exp2_corrected_x2(float2 d, float2 c_hi, float
   return __ffma2_rn(r, t, r);
 }
 
-// exp2_split on a pair, with the same results (0 below the normal range), for any d <= 0:
-// the comparison takes out whatever the bits below it hold, also where |E| is so
-// large that e_lo alone passes 2 (a masked logit at a temperature under 2e-4), for d
-// = -inf and for NaN.  kLow: d + d_lo.
-// The hot loops of fp32 logits are bound by their arithmetic: in pairs, with the
-// clamp of d left to the caller's of v, persistent kernel: 60-node trees, V = 151936, B =
-// 256 966 -> 886 us, V = 128256, B = 64 472 -> 439 us, 26-node trees, V = 151936, B = 512
-// 1239 -> 1125 us; cluster kernel: V = 32000, B = 64 177 -> 167 us, 1024 chains of 8 730
-// -> 642 us.
+// exp2_split on a pair, with the same results; kLow: d + d_lo.
+// The hot loops of fp32 logits are bound by their arithmetic: in pairs, persistent
+// kernel: 60-node trees, V = 151936, B = 256 966 -> 886 us, V = 128256, B = 64 472 -> 439
+// us, 26-node trees, V = 151936, B = 512 1239 -> 1125 us; cluster kernel: V = 32000, B =
+// 64 177 -> 167 us, 1024 chains of 8 730 -> 642 us.
 template <bool kLow = false>
 __device__ __forceinline__ float2 exp2_split_zero_x2(float2 d, float2 c_hi, float2 c_lo,
                                                      float2 d_lo = make_float2(0.f, 0.f)) {
@@ -109,7 +104,6 @@ __device__ __forceinline__ float2 exp2_split_zero_x2(float2 d, float2 c_hi, floa
   const float2 t = __fadd2_rn(e_hi, make_float2(12582912.f, 12582912.f));
   const float2 nf = __fadd2_rn(t, make_float2(-12582912.f, -12582912.f));
   const float2 f = __fadd2_rn(__fadd2_rn(e_hi, make_float2(-nf.x, -nf.y)), e_lo);
-  // bits(2^f) + n * 2^23, n = bits(t) - bits(1.5 * 2^23), in modular arithmetic
   const uint32_t k = 0u - (0x4B400000u << 23);
   const float r0 = __uint_as_float(__float_as_uint(ex2(f.x)) + (__float_as_uint(t.x) << 23) + k);
   const float r1 = __uint_as_float(__float_as_uint(ex2(f.y)) + (__float_as_uint(t.y) << 23) + k);
@@ -191,7 +185,6 @@ struct F32Logits {
   static constexpr int kBytes = 4;
   // 2^((v - m) c) with the rounding error of v - m carried along (two-sum)
   __device__ static __forceinline__ float exp_rel(float v, float m, float c_hi, float c_lo) {
-    v = fmaxf(v, m - 1.0e4f);                 // -inf / NaN: finite, weight ~0
     const float d = v - m;
     const float bb = d - v;
     const float d_lo = (v - (d - bb)) + (-m - bb);
@@ -200,8 +193,6 @@ struct F32Logits {
   // exp_rel of two logits, the same results
   __device__ static __forceinline__ float2 exp_rel_x2(float2 v, float m, float2 c_hi,
                                                       float2 c_lo) {
-    const float least = m - 1.0e4f;
-    v = make_float2(fmaxf(v.x, least), fmaxf(v.y, least));
     const float2 nm = make_float2(-m, -m);
     const float2 d = __fadd2_rn(v, nm);
     const float2 bb = __fadd2_rn(d, make_float2(-v.x, -v.y));

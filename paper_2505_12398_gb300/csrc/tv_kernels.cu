@@ -110,13 +110,6 @@ __global__ void __launch_bounds__(kStatsThreads, kStatsThreads == 256 ? 6 - L::k
       if (x >= end) break;
       float2 t[4];
       L::block_exp(v[u], m, ch, cl, t);
-      if (edge) {              // (-inf has a weight at a high temperature)
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          if (x + 2 * k < sh || x + 2 * k >= end) t[k].x = 0.f;
-          if (x + 2 * k + 1 < sh || x + 2 * k + 1 >= end) t[k].y = 0.f;
-        }
-      }
       const float2 p = __fadd2_rn(__fadd2_rn(t[0], t[1]), __fadd2_rn(t[2], t[3]));
       acc.add(p.x + p.y);
     }

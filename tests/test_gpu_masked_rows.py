@@ -154,3 +154,12 @@ def test_bf16_rows_without_a_normaliser(path, V, value):
     keep = [0, 1, 3, 4, 5]
     for x, y in zip(out[:3], clean):
         assert torch.equal(x[keep], y[keep])
+
+
+@pytest.mark.parametrize("path,V", [("cluster", 8008), ("persistent", 8008), ("two", 8005)])
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+def test_masked_logits_at_a_high_temperature(path, V, dtype):
+    """Nor does a masked token weigh anything where a bound on the distance to the row's
+    maximum, 1e4 say, would leave it e^-5."""
+    inp = _inputs(8, V, dtype, 2000.0, seed=V % 1000)
+    _check(inp, _run(inp, path))
