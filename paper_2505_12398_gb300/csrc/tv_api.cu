@@ -25,9 +25,7 @@ struct tv_handle {
   int max_batch = 0;
   tv_dtype dtype = TV_BF16;
   unsigned flags = 0;
-  int sm_count = 0;
-  int smem_per_sm = 0;
-  int smem_per_block = 0;
+  TreeDevice dev;
   int force_ncw = 0, force_c = 0, force_stages = 0;   // tuning override (TV_FUSED_PLAN)
   int flow_force[5] = {0, 0, 0, 0, 0};                 // tuning override (TV_FLOW_PLAN)
   // device workspace
@@ -66,7 +64,7 @@ enum Path { kPathTwo = 0, kPathCluster = 1, kPathPersistent = 2 };
 size_t logit_bytes(const tv_handle* h) { return h->dtype == TV_BF16 ? 2 : 4; }
 
 FlowPlan flow_plan(const tv_handle* h, int R, int B) {
-  return tv_flow_plan(R, B, h->vocab, h->smem_per_sm, h->smem_per_block, h->flow_force[0],
+  return tv_flow_plan(R, B, h->vocab, h->dev.smem_per_sm, h->dev.smem_per_block, h->flow_force[0],
                       h->flow_force[1],
                       h->flow_force[2], h->flow_force[3], h->flow_force[4]);
 }
@@ -102,8 +100,7 @@ bool prefer_cluster(int V, int B, int R) {
 // The path of a call, and the cluster kernel's plan (also for the two-kernel
 // path, whose last kernel it is).
 Path choose_path(const tv_handle* h, int B, int R, FusedPlan* plan) {
-  *plan = tv_fused_plan(B, R, h->vocab, (int)logit_bytes(h), h->smem_per_sm, h->smem_per_block,
-                        h->force_ncw, h->force_c, h->force_stages);
+  *plan = tv_fused_plan(B, R, h->vocab, (int)logit_bytes(h), h->dev, h->force_ncw, h->force_c, h->force_stages);
   if ((h->vocab % 8) != 0 || (h->flags & TV_FLAG_UNFUSED)) return kPathTwo;
   if (h->flags & TV_FLAG_CLUSTER) return plan->ok ? kPathCluster : kPathTwo;
   if (!h->flow_ws || !flow_plan(h, R, B).ok) return kPathTwo;
@@ -297,9 +294,9 @@ int verify_impl(tv_handle* h, int B, int N, const int32_t* parents, const int32_
     f.epoch = ++h->epoch;
     f.withhold_tree = h->withhold_tree;
     h->withhold_tree = -1;
-    rc = tv_launch_flow(a, f, bf16, fp, h->sm_count, st, ev);
+    rc = tv_launch_flow(a, f, bf16, fp, h->dev.sm_count, st, ev);
   } else {
-    rc = tv_launch_all(a, bf16, plan, st, ev);
+    rc = tv_launch_all(a, bf16, plan, h->dev.sm_count, st, ev);
   }
   if (rc == TV_OK && h->timing) h->timed_call = true;
   return rc;
@@ -340,9 +337,6 @@ int tv_create(tv_handle** out, int device, int vocab, int max_nodes, int max_bat
   h->max_batch = max_batch;
   h->dtype = logit_dtype;
   h->flags = flags;
-  h->sm_count = prop.multiProcessorCount;
-  h->smem_per_sm = (int)prop.sharedMemPerMultiprocessor;
-  h->smem_per_block = (int)prop.sharedMemPerBlockOptin;
   // TV_FUSED_PLAN="ncw,cluster,stages" overrides the fused kernel's launch
   // shape (tuning only; invalid values are ignored)
   if (const char* env = std::getenv("TV_FUSED_PLAN"))
@@ -353,7 +347,8 @@ int tv_create(tv_handle** out, int device, int vocab, int max_nodes, int max_bat
     std::sscanf(env, "%d,%d,%d,%d,%d", &h->flow_force[0], &h->flow_force[1], &h->flow_force[2],
                 &h->flow_force[3], &h->flow_force[4]);
   DeviceGuard guard(device);
-  if (!guard.ok()) {
+  if (!guard.ok() || !tv_tree_device(device, &h->dev)) {
+    cudaGetLastError();
     delete h;
     return TV_ERR_CUDA;
   }
@@ -639,7 +634,7 @@ int tv_draft_children(tv_handle* h, int B, int N, const int32_t* parents,
   DeviceGuard guard(h->device);
   if (!guard.ok()) return TV_ERR_CUDA;
   const int rc = tv_launch_draft(parents, draft_probs, uniforms, out_tokens, B, N, h->vocab,
-                                 h->sm_count, h->status,
+                                 h->dev.sm_count, h->status,
                                  static_cast<cudaStream_t>(cuda_stream));
   return rc == 0 ? TV_OK : TV_ERR_CUDA;
 }

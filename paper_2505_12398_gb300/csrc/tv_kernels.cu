@@ -166,8 +166,8 @@ void launch_stats(const TravArgs& a, cudaStream_t stream) {
 }
 
 template <typename L>
-int launch_typed(const TravArgs& a, int logit_is_bf16, const FusedPlan& plan, cudaStream_t stream,
-                 cudaEvent_t* ev) {
+int launch_typed(const TravArgs& a, int logit_is_bf16, const FusedPlan& plan, int sm_count,
+                 cudaStream_t stream, cudaEvent_t* ev) {
   if (ev && cudaEventRecord(ev[0], stream) != cudaSuccess) return -5;
   if (ev && cudaEventRecord(ev[1], stream) != cudaSuccess) return -5;
   // Few rows: more threads on each, as long as every thread has a block or more.
@@ -191,7 +191,7 @@ int launch_typed(const TravArgs& a, int logit_is_bf16, const FusedPlan& plan, cu
   // are free first (119 -> 126 us at B = 32, V = 32003, 449 -> 463 us at B = 256);
   // single CTAs do not: 170 -> 165 us at B = 512, V = 4001, 774 -> 767 us at B = 600, V
   // = 32003.
-  const bool dependent = ev == nullptr && (plan.C == 1 || a.B * plan.C <= 152);
+  const bool dependent = ev == nullptr && (plan.C == 1 || (long)a.B * plan.C <= sm_count);
   if (tv_launch_tree(t, logit_is_bf16, plan, stream, dependent) != 0) return -5;
   if (ev && cudaEventRecord(ev[3], stream) != cudaSuccess) return -5;
   return 0;
@@ -199,9 +199,9 @@ int launch_typed(const TravArgs& a, int logit_is_bf16, const FusedPlan& plan, cu
 
 }  // namespace
 
-int tv_launch_all(const TravArgs& a, int logit_is_bf16, const FusedPlan& plan,
+int tv_launch_all(const TravArgs& a, int logit_is_bf16, const FusedPlan& plan, int sm_count,
                   cudaStream_t stream, cudaEvent_t* events) {
   if (!plan.ok) return -5;
-  return logit_is_bf16 ? launch_typed<tvk::Bf16Logits>(a, 1, plan, stream, events)
-                       : launch_typed<tvk::F32Logits>(a, 0, plan, stream, events);
+  return logit_is_bf16 ? launch_typed<tvk::Bf16Logits>(a, 1, plan, sm_count, stream, events)
+                       : launch_typed<tvk::F32Logits>(a, 0, plan, sm_count, stream, events);
 }

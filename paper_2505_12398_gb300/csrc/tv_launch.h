@@ -40,15 +40,24 @@ size_t tv_leaf_bonus_smem_bytes(int V);
 
 // Launch plan of the fused kernel: cluster size, ring stages, shared memory.
 struct FusedPlan {
-  int ncw = 8;       // consumer warps per CTA (4 or 8)
+  int ncw = 8;       // consumer warps per CTA (4, 8 or 16)
   int C = 1;
   int stages = 0;
   size_t smem = 0;
   bool ok = false;
 };
 
-FusedPlan tv_fused_plan(int B, int R, int V, int logit_bytes, int smem_per_sm,
-                        int smem_per_block, int force_ncw, int force_c, int force_stages);
+// What a device gives the cluster kernel.
+struct TreeDevice {
+  int sm_count = 0;
+  int smem_per_sm = 0, smem_per_block = 0;
+  int max_cluster = 1;           // CTAs of a whole SM each that a cluster may have
+};
+// Of the current device (asked once per device); false on a CUDA error.
+bool tv_tree_device(int device, TreeDevice* out);
+
+FusedPlan tv_fused_plan(int B, int R, int V, int logit_bytes, const TreeDevice& dev,
+                        int force_ncw, int force_c, int force_stages);
 
 // Queues the fused kernel (one cluster of plan.C CTAs per tree; any V).  With
 // `events`, events[0..2] are recorded before and events[3] after it.
@@ -68,7 +77,7 @@ bool tv_tree_fits(int R, int V, size_t smem_per_block);
 // `plan`); 0 on success, TV_ERR_CUDA otherwise.  With `events` non-null,
 // events[0..3] are recorded before the first kernel, between the kernels and
 // after the last one.
-int tv_launch_all(const TravArgs& a, int logit_is_bf16, const FusedPlan& plan,
+int tv_launch_all(const TravArgs& a, int logit_is_bf16, const FusedPlan& plan, int sm_count,
                   cudaStream_t stream, cudaEvent_t* events);
 
 // ---- persistent load-balanced kernel (tv_flow.cu) ----

@@ -42,12 +42,10 @@ static __device__ __align__(256) unsigned char g_tv_scratch[kScratchBytes];
 
 std::mutex g_setup_mutex;
 void* g_scratch_addr[kMaxDevices] = {};
-int g_sm_count[kMaxDevices] = {};
-int g_smem_optin[kMaxDevices] = {};
-int g_smem_sm[kMaxDevices] = {};
+TreeDevice g_dev[kMaxDevices];
 
 // Once per device, with that device current: the array's device address and
-// the two device properties the launch needs.
+// the device properties the launch needs.
 int setup_device(int device) {
   std::lock_guard<std::mutex> lock(g_setup_mutex);
   if (g_scratch_addr[device]) return TV_OK;
@@ -56,20 +54,16 @@ int setup_device(int device) {
     cudaGetLastError();
     return TV_ERR_CUDA;
   }
-  int sms = 0, smem = 0, smem_sm = 0, major = 0;
-  if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess ||
-      cudaDeviceGetAttribute(&smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, device) !=
-          cudaSuccess ||
-      cudaDeviceGetAttribute(&smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, device) !=
-          cudaSuccess ||
-      cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, device) != cudaSuccess) {
+  int major = 0;
+  if (cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, device) != cudaSuccess) {
     cudaGetLastError();
     return TV_ERR_CUDA;
   }
   if (major < 10) return TV_ERR_DEVICE;
-  g_sm_count[device] = sms;
-  g_smem_optin[device] = smem;
-  g_smem_sm[device] = smem_sm;
+  if (!tv_tree_device(device, &g_dev[device])) {
+    cudaGetLastError();
+    return TV_ERR_CUDA;
+  }
   g_scratch_addr[device] = ptr;
   return TV_OK;
 }
@@ -106,7 +100,7 @@ extern "C" int tv_verify_batch_noalloc(int device, int B, int N, int vocab, tv_d
     return TV_ERR_CUDA;
   }
   int rc = setup_device(device);
-  if (rc == TV_OK && !tv_tree_fits(N + 1, vocab, (size_t)g_smem_optin[device]))
+  if (rc == TV_OK && !tv_tree_fits(N + 1, vocab, (size_t)g_dev[device].smem_per_block))
     rc = TV_ERR_VOCAB;
   if (rc == TV_OK) {
     unsigned char* base = static_cast<unsigned char*>(g_scratch_addr[device]);
@@ -143,8 +137,9 @@ extern "C" int tv_verify_batch_noalloc(int device, int B, int N, int vocab, tv_d
       a.stats_given = 0;
       a.exact_exp = 0;
       const FusedPlan plan = tv_fused_plan(B, N + 1, vocab, logit_dtype == TV_BF16 ? 2 : 4,
-                                           g_smem_sm[device], g_smem_optin[device], 0, 0, 0);
-      rc = tv_launch_all(a, logit_dtype == TV_BF16 ? 1 : 0, plan, st, nullptr);
+                                           g_dev[device], 0, 0, 0);
+      rc = tv_launch_all(a, logit_dtype == TV_BF16 ? 1 : 0, plan, g_dev[device].sm_count, st,
+                         nullptr);
     }
   }
   if (prev != device) cudaSetDevice(prev);

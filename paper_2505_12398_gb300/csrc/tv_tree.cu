@@ -55,6 +55,9 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <algorithm>
+#include <mutex>
+
 #include "tv_control.cuh"
 #include "tv_device.cuh"
 #include "tv_launch.h"
@@ -1260,6 +1263,8 @@ __global__ void __launch_bounds__(TreeCta<L, NCW, kExact>::kThreads, 16 / NCW)
 
 namespace {
 
+constexpr int kStaticBytes = 1536;   // at least the kernel's static shared memory
+
 size_t tree_cta_bytes(int ncw, int lb, int C, int stages, int R, int V) {
   using namespace tvk::fused;
   return (size_t)stages * tree_stage_bytes(ncw, lb) + (size_t)2 * exchange_slots(C, ncw) * 8 +
@@ -1270,9 +1275,9 @@ size_t tree_cta_bytes(int ncw, int lb, int C, int stages, int R, int V) {
 int stages_for(int ncw, int lb, int C, int per_sm, int R, int V, int smem_per_sm,
                int smem_per_block) {
   using namespace tvk::fused;
-  const long reserve = 1024 + 1536;   // per-CTA system reserve and static shared memory
+  const long reserve = 1024 + kStaticBytes;   // (1024: the system's own, per CTA)
   long per_cta = (long)smem_per_sm / per_sm - reserve;
-  if (per_cta > smem_per_block - 1536) per_cta = smem_per_block - 1536;
+  if (per_cta > smem_per_block - kStaticBytes) per_cta = smem_per_block - kStaticBytes;
   const long st = (per_cta - (long)tree_cta_bytes(ncw, lb, C, 0, R, V)) /
                   tree_stage_bytes(ncw, lb);
   return (int)(st > kTreeMaxStages ? kTreeMaxStages : st);
@@ -1280,10 +1285,12 @@ int stages_for(int ncw, int lb, int C, int per_sm, int R, int V, int smem_per_sm
 
 }  // namespace
 
-FusedPlan tv_fused_plan(int B, int R, int V, int logit_bytes, int smem_per_sm,
-                        int smem_per_block, int force_ncw, int force_c, int force_stages) {
+FusedPlan tv_fused_plan(int batch, int R, int V, int logit_bytes, const TreeDevice& dev,
+                        int force_ncw, int force_c, int force_stages) {
   using namespace tvk::fused;
   FusedPlan p;
+  // (the batches below are those of 152 SMs)
+  const long B = (long)batch * 152 / dev.sm_count;
   // Few trees: as many SMs per tree as keep all trees in one wave (152 SMs, two
   // CTAs of 8 consumer warps or one of 16 on each; clusters do not cross a GPC,
   // so about 8 clusters of 16 whole SMs fit), down to slices of 1000 tokens, below
@@ -1310,13 +1317,15 @@ FusedPlan tv_fused_plan(int B, int R, int V, int logit_bytes, int smem_per_sm,
   else if (V <= 12288) ncw = 4;
   while (C > 1 && V / C < 1000) C /= 2;
   while (C < 8 && tree_tiles(V, C) * 8 > 32768) C *= 2;   // bonus tiles' shared memory
+  C = std::min(C, dev.max_cluster);
   if (force_ncw == 4 || force_ncw == 8 || force_ncw == 16) ncw = force_ncw;
   int per_sm = 16 / ncw;
-  if (force_c == 1 || force_c == 2 || force_c == 4 || force_c == 8 || force_c == 16) C = force_c;
-  int stages = stages_for(ncw, logit_bytes, C, per_sm, R, V, smem_per_sm, smem_per_block);
+  if (force_c == 1 || force_c == 2 || force_c == 4 || force_c == 8 || force_c == 16)
+    C = std::min(force_c, dev.max_cluster);
+  int stages = stages_for(ncw, logit_bytes, C, per_sm, R, V, dev.smem_per_sm, dev.smem_per_block);
   while (stages < 3 && per_sm > 1) {
     --per_sm;
-    stages = stages_for(ncw, logit_bytes, C, per_sm, R, V, smem_per_sm, smem_per_block);
+    stages = stages_for(ncw, logit_bytes, C, per_sm, R, V, dev.smem_per_sm, dev.smem_per_block);
   }
   if (force_stages >= 2 && force_stages <= kTreeMaxStages && force_stages < stages)
     stages = force_stages;
@@ -1324,7 +1333,7 @@ FusedPlan tv_fused_plan(int B, int R, int V, int logit_bytes, int smem_per_sm,
   p.C = C;
   p.stages = stages;
   p.smem = stages >= 0 ? tree_cta_bytes(ncw, logit_bytes, C, stages, R, V) : 0;
-  p.ok = stages >= 2 && p.smem + 1536 <= (size_t)smem_per_block;
+  p.ok = stages >= 2 && p.smem + kStaticBytes <= (size_t)dev.smem_per_block;
   return p;
 }
 
@@ -1371,6 +1380,60 @@ cudaError_t launch_ncw(const TravArgs& a, const FusedPlan& plan, cudaStream_t st
 }
 
 }  // namespace
+
+// The largest cluster of CTAs that fill an SM each, so that one of any plan's shape
+// fits: 16 CTAs is more than a device has to hold (their SMs must share a GPC), and a
+// device with few SMs may not hold 8 either.
+bool tv_tree_device(int device, TreeDevice* out) {
+  constexpr int kDevices = 64;
+  static std::mutex mutex;
+  static TreeDevice known[kDevices];
+  if (device < 0 || device >= kDevices) return false;
+  std::lock_guard<std::mutex> lock(mutex);
+  TreeDevice& d = known[device];
+  if (d.sm_count == 0) {
+    using T = tvk::fused::TreeCta<tvk::Bf16Logits, 16, false>;
+    auto k = tvk::fused::tv_tree_kernel<tvk::Bf16Logits, 16, false>;
+    TreeDevice q;
+    int sms = 0;
+    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess ||
+        cudaDeviceGetAttribute(&q.smem_per_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor,
+                               device) != cudaSuccess ||
+        cudaDeviceGetAttribute(&q.smem_per_block, cudaDevAttrMaxSharedMemoryPerBlockOptin,
+                               device) != cudaSuccess)
+      return false;
+    const int smem = q.smem_per_block - kStaticBytes;
+    if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess ||
+        cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)
+      return false;
+    for (int C = 16; C > 1; C /= 2) {
+      cudaLaunchConfig_t cfg = {};
+      cfg.gridDim = dim3((unsigned)C, 1, 1);
+      cfg.blockDim = dim3(T::kThreads, 1, 1);
+      cfg.dynamicSmemBytes = (size_t)smem;
+      cudaLaunchAttribute attr[1];
+      attr[0].id = cudaLaunchAttributeClusterDimension;
+      attr[0].val.clusterDim.x = (unsigned)C;
+      attr[0].val.clusterDim.y = 1;
+      attr[0].val.clusterDim.z = 1;
+      cfg.attrs = attr;
+      cfg.numAttrs = 1;
+      int active = 0;
+      if (cudaOccupancyMaxActiveClusters(&active, k, &cfg) != cudaSuccess) {
+        cudaGetLastError();
+        active = 0;
+      }
+      if (active > 0) {
+        q.max_cluster = C;
+        break;
+      }
+    }
+    q.sm_count = sms;
+    d = q;
+  }
+  *out = d;
+  return true;
+}
 
 int tv_launch_tree(const TravArgs& a, int logit_is_bf16, const FusedPlan& plan,
                    cudaStream_t stream, bool dependent) {
