@@ -1319,13 +1319,20 @@ FusedPlan tv_fused_plan(int batch, int R, int V, int logit_bytes, const TreeDevi
   while (C < 8 && tree_tiles(V, C) * 8 > 32768) C *= 2;   // bonus tiles' shared memory
   C = std::min(C, dev.max_cluster);
   if (force_ncw == 4 || force_ncw == 8 || force_ncw == 16) ncw = force_ncw;
-  int per_sm = 16 / ncw;
   if (force_c == 1 || force_c == 2 || force_c == 4 || force_c == 8 || force_c == 16)
     C = std::min(force_c, dev.max_cluster);
-  int stages = stages_for(ncw, logit_bytes, C, per_sm, R, V, dev.smem_per_sm, dev.smem_per_block);
-  while (stages < 3 && per_sm > 1) {
-    --per_sm;
-    stages = stages_for(ncw, logit_bytes, C, per_sm, R, V, dev.smem_per_sm, dev.smem_per_block);
+  auto fit = [&] {
+    int st = 0;
+    for (int per_sm = 16 / ncw; per_sm > 0 && st < 3; --per_sm)
+      st = stages_for(ncw, logit_bytes, C, per_sm, R, V, dev.smem_per_sm, dev.smem_per_block);
+    return st;
+  };
+  int stages = fit();
+  // the largest trees of the longest rows (from 1016 nodes of 4.0 million tokens, fp32):
+  // shorter slices, whose bonus tiles leave room for the ring
+  while (stages < 2 && C < 8 && C < dev.max_cluster) {
+    C *= 2;
+    stages = fit();
   }
   if (force_stages >= 2 && force_stages <= kTreeMaxStages && force_stages < stages)
     stages = force_stages;

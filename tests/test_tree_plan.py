@@ -66,3 +66,17 @@ def test_batches_count_against_the_sms(plans):
     whole = plans([(2 * B, 61, 128256, 2, 152, 16) for B in BATCHES])
     half = plans([(B, 61, 128256, 2, 76, 16) for B in BATCHES])
     assert whole == half
+
+
+def test_every_size_taken_has_a_plan(plans):
+    """The largest trees and vocabularies the entry points accept: two ring stages at
+    least, whatever the batch."""
+    cases = []
+    for R in (1, 2, 200, 500, 800, 1000, 1016, 1024):
+        room = (SMEM_BLOCK - 64 - 97 * R) // 8 * 256     # the largest vocabulary accepted
+        for V in [1, 1000, 262144] + [room * k // 64 for k in range(16, 65)]:
+            cases += [(B, R, V, lb, 152, most) for B in BATCHES for lb in (2, 4)
+                      for most in (16, 8)]
+    got = plans(cases)
+    assert all(p[5] for p in got)
+    assert [c for c, p in zip(cases, got) if not p[4] or p[2] < 2] == []
