@@ -351,9 +351,9 @@ int tv_last_phase_ms(tv_handle* h, float* ms);
 /*
  * tv_launch_shape -- how a call with these B and N would run on this handle:
  * *path = 0 for the two-kernel path, 1 for the cluster-per-tree kernel, 2
- * for the persistent kernel; *cluster = CTAs per tree (cluster path; 1
- * otherwise), *warps = consumer warps per CTA, *stages = ring stages (0 for
- * the two-kernel path).  Any output pointer may be NULL.
+ * for the persistent kernel; *cluster = CTAs per tree (1 for the persistent
+ * kernel), *warps = consumer warps per CTA, *stages = ring stages, of the
+ * traversal's kernel.  Any output pointer may be NULL.
  * Errors: TV_ERR_INVALID_ARG, TV_ERR_CAPACITY.
  */
 int tv_launch_shape(tv_handle* h, int B, int N, int* path, int* cluster, int* warps,

@@ -698,11 +698,11 @@ int tv_launch_shape(tv_handle* h, int B, int N, int* path, int* cluster, int* wa
   FusedPlan plan;
   const Path p = choose_path(h, B, N + 1, &plan);
   if (path) *path = (int)p;
-  if (cluster) *cluster = (p == kPathCluster) ? plan.C : 1;
   const FlowPlan fp = flow_plan(h, N + 1, B);
-  if (warps) *warps = (p == kPathCluster) ? plan.ncw : (p == kPathPersistent ? fp.ncw : 16);
-  if (stages)
-    *stages = (p == kPathCluster) ? plan.stages : (p == kPathPersistent ? fp.stages : 0);
+  const bool persistent = p == kPathPersistent;   // (else the cluster kernel traverses)
+  if (cluster) *cluster = persistent ? 1 : plan.C;
+  if (warps) *warps = persistent ? fp.ncw : plan.ncw;
+  if (stages) *stages = persistent ? fp.stages : plan.stages;
   return TV_OK;
 }
 

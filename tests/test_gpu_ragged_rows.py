@@ -25,7 +25,11 @@ def test_against_oracle(V, dtype, T, shape, monkeypatch):
     inp = make_inputs(w, seed=V, device="cuda")
     B, R = inp.parents.shape
     v = tv.Verifier(V, R - 1, B, "bf16" if dtype == torch.bfloat16 else "fp32")
-    assert v.launch_shape(B, R - 1)[0] == 0
+    code, C, ncw, stages = v.launch_shape(B, R - 1)
+    assert code == 0 and stages >= 2
+    if shape:
+        want = [int(x) for x in shape.split(",")]
+        assert [ncw, C] == want[:2] and want[2] in (0, stages)
     out = v.verify(inp.parents, inp.tokens, inp.logits, inp.draft_probs, inp.temperature,
                    inp.uniforms, debug=True)
     torch.cuda.synchronize()
