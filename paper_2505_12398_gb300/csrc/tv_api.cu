@@ -604,7 +604,7 @@ int tv_lm_head(tv_handle* h, int M, int K, const void* hidden, const void* weigh
   if (!guard.ok()) return TV_ERR_CUDA;
   if (!h->lmh_part) {   // sized for the handle's limits, once
     const size_t need =
-        tv_lm_head_scratch(h->max_batch * (h->max_nodes + 1), h->vocab) * sizeof(float2);
+        tv_lm_head_scratch((size_t)h->max_batch * (h->max_nodes + 1), h->vocab) * sizeof(float2);
     if (need == 0 || cudaMalloc(&h->lmh_part, need) != cudaSuccess) {
       cudaGetLastError();
       h->lmh_part = nullptr;

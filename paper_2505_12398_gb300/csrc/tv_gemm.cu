@@ -60,6 +60,7 @@
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
+#include <limits.h>
 #include <stdint.h>
 
 #include <algorithm>
@@ -670,7 +671,7 @@ GemmDevice g_gemm[kGemmDevices];
 // of 256 columns 196 us, 8 of 224 205, 14 of 128 292, the same columns each); on
 // single SMs W's bytes from HBM bound the kernel and 64 fits (M = 61, V = 128256:
 // 4 waves of 224 165 us, 5 of 176 167, 6 of 144 168, 4 of 256 169, 8 of 128 175).
-int tile_width(int m_tiles, int V, int units, bool pair, int extra) {
+int tile_width(size_t m_tiles, int V, int units, bool pair, int extra) {
   const int unit = pair ? 32 : 16;
   int best = tvk::gemm::kBN;
   long best_cost = 0;
@@ -750,18 +751,18 @@ bool gemm_device(int device, GemmDevice* out) {
 namespace {
 
 // One row tile: single SMs, bound by W's bytes; more: SM pairs.
-bool pairs_for(int M) { return M > tvk::gemm::kBM; }
+bool pairs_for(size_t M) { return M > tvk::gemm::kBM; }
 
-int width_for(int M, int V, const GemmDevice& g) {
+int width_for(size_t M, int V, const GemmDevice& g) {
   const bool pair = pairs_for(M);
-  const int tile_rows = pair ? 2 * tvk::gemm::kBM : tvk::gemm::kBM;
+  const size_t tile_rows = pair ? 2 * tvk::gemm::kBM : tvk::gemm::kBM;
   return tile_width((M + tile_rows - 1) / tile_rows, V, pair ? g.pairs : g.sms, pair,
                     pair ? 256 : 64);
 }
 
 }  // namespace
 
-size_t tv_lm_head_scratch(int rows, int V) {
+size_t tv_lm_head_scratch(size_t rows, int V) {
   using namespace tvk::gemm;
   int device = 0;
   GemmDevice g;
@@ -771,11 +772,13 @@ size_t tv_lm_head_scratch(int rows, int V) {
     return 0;
   }
   // the most any call of up to `rows` rows takes (the width depends on its row
-  // tiles only)
+  // tiles only; a call's rows are an int)
+  rows = std::min<size_t>(rows, INT_MAX);
   size_t most = 0;
-  for (int M = std::min(rows, kBM);; M = std::min(rows, (M / (2 * kBM) + 1) * 2 * kBM)) {
+  for (size_t M = std::min<size_t>(rows, kBM);;
+       M = std::min<size_t>(rows, (M / (2 * kBM) + 1) * 2 * kBM)) {
     const int bn = width_for(M, V, g);
-    most = std::max(most, (size_t)M * ((V + bn - 1) / bn));
+    most = std::max(most, M * ((V + bn - 1) / bn));
     if (M >= rows) return most;
   }
 }

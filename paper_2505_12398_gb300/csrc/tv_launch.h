@@ -144,7 +144,7 @@ int tv_launch_flow(const TravArgs& a, FlowArgs f, int logit_is_bf16, const FlowP
 
 // Partial normalisers (float2) that calls of up to `rows` rows need on the current
 // device; 0 on a CUDA error.
-size_t tv_lm_head_scratch(int rows, int V);
+size_t tv_lm_head_scratch(size_t rows, int V);
 // logits[M][V] (bf16) = hidden[M][K] x weight[V][K]^T (bf16) on the tensor
 // cores, and row_stats[M] = (max, sum of 2^((l - max) (c_hi + c_lo))) of the
 // stored logits.  part holds tv_lm_head_scratch(M, V) entries.  Requires K % 64

@@ -37,3 +37,20 @@ def test_exact_operands_at_tile_edges(M, K, V):
     st = st.cpu().numpy().astype(np.float64)
     assert np.array_equal(st[:, 0], m)
     assert np.max(np.abs(st[:, 1] - s) / s) < 1e-5   # the parity bar of the normalisers
+
+
+def test_handle_of_more_rows_than_an_int_counts():
+    """2^31 rows of 8 tokens: 16 GiB of row statistics and of scratch on the handle, a call of
+    a few rows as on any other."""
+    import paper_2505_12398_gb300 as tv
+    if torch.cuda.mem_get_info()[0] < 64 << 30:
+        pytest.skip("not enough free device memory")
+    g = torch.Generator().manual_seed(5)
+    H = (torch.randint(-8, 9, (5, 64), generator=g).float() / 16).to(torch.bfloat16)
+    W = (torch.randint(-8, 9, (8, 64), generator=g).float() / 16).to(torch.bfloat16)
+    v = tv.Verifier(8, 1023, 1 << 21, "bf16", path="three")
+    lg, _ = v.lm_head(H.cuda(), W.cuda(), 1.0)
+    torch.cuda.synchronize()
+    v.close()
+    ref = lmhead.to_bf16(lmhead.logits(H.float().numpy(), W.float().numpy()))
+    assert np.array_equal(lg.float().cpu().numpy().astype(np.float64), ref)
