@@ -44,6 +44,7 @@ struct FusedPlan {
   int C = 1;
   int stages = 0;
   size_t smem = 0;
+  size_t smem_most = 0;   // the most any plan of the device has
   bool ok = false;
 };
 

@@ -1340,7 +1340,8 @@ FusedPlan tv_fused_plan(int batch, int R, int V, int logit_bytes, const TreeDevi
   p.C = C;
   p.stages = stages;
   p.smem = stages >= 0 ? tree_cta_bytes(ncw, logit_bytes, C, stages, R, V) : 0;
-  p.ok = stages >= 2 && p.smem + kStaticBytes <= (size_t)dev.smem_per_block;
+  p.smem_most = (size_t)(dev.smem_per_block - kStaticBytes);
+  p.ok = stages >= 2 && p.smem <= p.smem_most;
   return p;
 }
 
@@ -1350,7 +1351,10 @@ template <typename L, int NCW, bool kExact>
 cudaError_t launch_one(const TravArgs& a, const FusedPlan& plan, cudaStream_t stream,
                        bool dependent) {
   auto k = tvk::fused::tv_tree_kernel<L, NCW, kExact>;
-  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)plan.smem);
+  // (the kernel's limit, the same at every launch: another thread may be about to launch
+  // with more shared memory than this plan has)
+  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)plan.smem_most);
   if (e != cudaSuccess) return e;
   if (plan.C > 8) {
     e = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
