@@ -415,14 +415,14 @@ struct TreeCta {
     return false;
   }
 
-  // Row normalisers: this warp's group takes every g-th row.
+  // Row normalisers: this warp's group takes every g-th row.  (Rows of whole blocks:
+  // with V % 8 != 0 the normalisers are given and no such job is posted.)
   __device__ bool sum_rows(const TreeJob& job, int wid, int lane) {
     const float c_hi = a.c_hi, c_lo = a.c_lo;
     const int n_rows = job.n_rows, total = job.total, xb = job.xb;
     uint32_t ph = job.ph;
     const int g = row_groups(n_rows, max_groups), group = wid % g, sub = wid / g, nsub = NCW / g;
     const bool reuse = total > n_stages;       // stages are filled more than once
-    const bool ragged = (a.V & 7) != 0;
     int st = 0, q = 0;
     for (int r = 0; r < n_rows; ++r) {
       const Slice sl(row0 + job.rows[r], a.V, v0, v1);
@@ -440,33 +440,29 @@ struct TreeCta {
           const int hop = nsub * kTileElems;
           int t0 = sub * kTileElems;
           // two whole tiles at a time: their chains of dependent operations overlap
-          if (!ragged) {
-            for (; t0 + hop + kTileElems <= n; t0 += 2 * hop) {
-              float v[2][8], t[2][8];
-              lds_logits<L>(lb + t0 + lane * kChunk, v[0]);
-              lds_logits<L>(lb + t0 + hop + lane * kChunk, v[1]);
-              const float cm = fmaxf(max8(v[0]), max8(v[1]));
-              if (cm > m_run) {
-                if (m_run != TV_NEG_INF) {
-                  const float sc = L::exp_rel(m_run, cm, c_hi, c_lo);
-                  acc.s *= sc;
-                  acc.c *= sc;
-                }
-                m_run = cm;
+          for (; t0 + hop + kTileElems <= n; t0 += 2 * hop) {
+            float v[2][8], t[2][8];
+            lds_logits<L>(lb + t0 + lane * kChunk, v[0]);
+            lds_logits<L>(lb + t0 + hop + lane * kChunk, v[1]);
+            const float cm = fmaxf(max8(v[0]), max8(v[1]));
+            if (cm > m_run) {
+              if (m_run != TV_NEG_INF) {
+                const float sc = L::exp_rel(m_run, cm, c_hi, c_lo);
+                acc.s *= sc;
+                acc.c *= sc;
               }
-              exp8<L, false>(v[0], m_run, c_hi, c_lo, t[0]);
-              exp8<L, false>(v[1], m_run, c_hi, c_lo, t[1]);
-              acc.add(sum8(t[0]));
-              acc.add(sum8(t[1]));
+              m_run = cm;
             }
+            exp8<L, false>(v[0], m_run, c_hi, c_lo, t[0]);
+            exp8<L, false>(v[1], m_run, c_hi, c_lo, t[1]);
+            acc.add(sum8(t[0]));
+            acc.add(sum8(t[1]));
           }
           for (; t0 < n; t0 += hop) {
             const int e0 = t0 + lane * kChunk;
             if (e0 >= n) continue;
-            const int lo = sl.sh - (x + e0), hi = sl.n - (x + e0);
-            const bool edge = ragged && (lo > 0 || hi < 8);
             float v[8], t[8];
-            stage_logits(lb, e0, true, edge, lo, hi, v);
+            lds_logits<L>(lb + e0, v);
             const float cm = max8(v);
             if (cm > m_run) {
               if (m_run != TV_NEG_INF) {
@@ -477,7 +473,6 @@ struct TreeCta {
               m_run = cm;
             }
             exp8<L, false>(v, m_run, c_hi, c_lo, t);
-            zero_outside(edge, lo, hi, t);
             acc.add(sum8(t));
           }
         }
