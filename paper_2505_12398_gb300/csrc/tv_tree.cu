@@ -1290,18 +1290,21 @@ FusedPlan tv_fused_plan(int batch, int R, int V, int logit_bytes, const TreeDevi
   // CTAs of 8 consumer warps or one of 16 on each; clusters do not cross a GPC,
   // so about 8 clusters of 16 whole SMs fit), down to slices of 1000 tokens, below
   // which a job is all latency.  Measured (us; 60-node trees; ncw x C):
-  //   V = 128256, B = 1: 16x16 112, 8x16 118, 16x8 132, 8x8 151, 4x8 212
-  //   V = 128256, B = 16: 8x16 144, 16x8 160, 8x8 188, 16x16 218, 4x8 267
+  //   V = 262144, B = 1: 16x16 71, 8x16 82, 16x8 94, 8x8 109; B = 4: 92, 106, 126, 144
+  //   V = 151936, B = 1: 8x16 79, 16x16 80, 16x8 93, 8x8 101
+  //   V = 128256, B = 1: 8x16 68, 16x16 70, 16x8 82, 8x8 82; B = 4: 98, 102, 118, 120
+  //   V = 128256, B = 16: 8x16 128, 16x8 144, 8x8 147, 4x8 194, 16x16 207
   //   V = 128256, B = 48: 4x8 215, 8x4 218, 16x4 220, 8x8 221; B = 64: 8x4 239, 4x8
   //   240, 8x8 287; B = 128: 8x2 419, 8x4 424, 4x4 429
   //   V = 262144, B = 32: 8x8 255, 4x8 341, 16x4 346, 8x4 364
-  //   V = 32000, B = 1: 8x16 63, 8x8 65, 4x8 71; B = 16: 8x8 120, 4x8 124, 8x16 143
+  //   V = 32000, B = 1: 8x16 56, 8x8 57, 4x8 58; B = 16: 4x8 101, 8x8 102, 8x16 106
   //   V = 32000, B = 64: 8x4 149, 4x8 154, 8x8 160; B = 128: 4x4 191, 8x2 192, 8x4 212
   //   V = 32000, B = 200: 8x2 230, 4x4 255, 4x2 280; B = 256: 4x2 250, 8x1 260, 8x2 261;
   //   B = 512: 4x2 386, 8x1 388, 8x2 399; B = 1024: 4x2 661, 8x1 662, 4x1 727, 8x2 731
   //   V = 16384, B = 300: 4x2 195, 8x1 200, 8x2 232; B = 1024: 8x1 470, 4x1 479
   //   V = 4000, B = 512: 4x1 183, 8x1 235; V = 8000, B = 1024 (26 nodes): 4x1 258, 8x1 308
-  // (B = 1 and 16 before the consumers took a chunk's tiles together)
+  // (16 consumer warps pay from between V = 151936 and 262144 on; from 98304, where they
+  // are taken, to there they are 1 to 4 % behind)
   int ncw = 8, C = 1;
   if (V > 98304 && B <= 4) ncw = 16, C = 16;
   else if (B <= 8 || (V > 98304 && B <= 16)) C = 16;

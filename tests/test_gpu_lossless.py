@@ -96,7 +96,7 @@ def chi2_p(obs, exp):
                                           ([-1, 0, 1, 2], 8, "persistent"),
                                           ([-1, 0, 0, 1, 1, 2, 2], 8, "cluster")])
 def test_kernel_output_law_is_target(tv, shape, V, path):
-    """V = 3 and 4 take the three-kernel path (V % 8 != 0); V = 8 runs the
+    """V = 3 and 4 take the two-kernel path (V % 8 != 0); V = 8 runs the
     persistent kernel and the cluster kernel."""
     obs, exp = z_counts(tv, shape, V, 1_000_000, seed=V * 17 + len(shape), path=path)
     assert chi2_p(obs, exp) > 1e-3

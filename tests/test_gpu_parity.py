@@ -155,9 +155,10 @@ def test_persistent_launch_shapes(tv, plan, monkeypatch):
 @pytest.mark.parametrize("V,N,want", [(32000, 60, 1), (49152, 127, 1), (32000, 200, 2),
                                        (50000, 60, 2), (128256, 60, 2), (1003, 60, 0)])
 def test_auto_path_choice(tv, V, N, want):
-    """A handle that picks its path itself: the cluster kernel for short rows
-    (V <= 49152, N + 1 <= 128), the persistent kernel otherwise, the
-    three-kernel path when V % 8 != 0 (tv_launch_shape's path codes 1, 2, 0)."""
+    """A handle that picks its path itself, 64 trees: the cluster kernel for short rows
+    (V <= 49152, N + 1 <= 128; fewer trees than 64 take it for longer ones too), the
+    persistent kernel otherwise, the two-kernel path when V % 8 != 0 (tv_launch_shape's
+    path codes 1, 2, 0)."""
     v = tv.Verifier(V, N, 64, "bf16")
     path, _, _, _ = v.launch_shape(64, N)
     v.close()
@@ -168,7 +169,7 @@ def test_auto_path_choice(tv, V, N, want):
 @pytest.mark.parametrize("path", ["persistent", "cluster"])
 def test_default_launch_shapes(tv, batch, path):
     """Batch sizes that select different default cluster shapes (clusters of
-    8, 8 and 1 CTA, 4 or 8 consumer warps) and, for the persistent kernel,
+    16, 16, 4, 2 and 1 CTA, 4 or 8 consumer warps) and, for the persistent kernel,
     fewer and more trees than CTAs."""
     w = get_workload("eagle_v32k", batch=batch)
     inp = make_inputs(w, seed=batch, device="cuda")

@@ -4,7 +4,7 @@ Some callers cannot allocate device memory (a serving process whose pool
 reserved the device up front and forbids new allocations, an embedding whose
 allocator owns the whole device).  This entry point keeps its
 scratch in a fixed static device array instead of a handle's workspace.  Its
-results must equal those of the handle-based three-kernel path (the same
+results must equal those of the handle-based two-kernel path (the same
 kernels run on the same inputs), call after call: the shared array keeps the
 previous call's contents and every call must clear what it needs.
 
