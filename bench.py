@@ -906,8 +906,9 @@ def main_lmhead(args, world, rank, local_rank):
     gemm_tflops = flops / (gemm_ms / 1e3) / 1e12
     ver_gbs = trav_bytes / (ver_ms / 1e3) / 1e9
     ms_step = total_ms_max / args.steps
+    ver_kernel = "tv_flow_kernel" if v.launch_shape(B, N)[0] == 2 else "tv_tree_kernel"
     phases = {"lm_head_kernel+lm_head_merge_kernel": round(gemm_ms, 6),
-              "tv_flow_kernel (given normalisers)": round(ver_ms, 6)}
+              f"{ver_kernel} (given normalisers)": round(ver_ms, 6)}
     if full:
         phases = {"tv_draft_kernel": round(draft_ms, 6), **phases}
     line = {
@@ -930,7 +931,7 @@ def main_lmhead(args, world, rank, local_rank):
                      "frac": round(gemm_tflops / peak, 4), "peak_kind": peak_kind + " (burst)",
                      "flops_per_launch": flops,
                      "traffic": kernel_traffic(w.name, B, "lmhead")},
-        "roofline_verify": {"bound": "hbm", "kernel": "tv_flow_kernel",
+        "roofline_verify": {"bound": "hbm", "kernel": ver_kernel,
                             "achieved": round(ver_gbs, 2), "peak": hbm, "unit": "GB/s",
                             "frac": round(ver_gbs / hbm, 4), "peak_kind": hbm_kind,
                             "bytes_per_launch": trav_bytes},
