@@ -14,9 +14,9 @@
 // groups of row tiles holding 32 MiB of H, row tile fastest inside a group, so
 // that the CTAs running at the same time share W tiles through L2 while the
 // group's H stays resident.  One group (976 x 4096 x 128256) reads W and H from HBM once,
-// 1.11 GB; two (7808 rows) do not reach that, 7.55 GB for 2.2: the 2 GB of logits pass
-// through the same L2.  The tensor cores bound that size all the same (1.01 of the
-// burst rate, at 1.8 TB/s read).
+// 1.11 GB; two (7808 rows) do not reach their 2.2 GB, 4.7 and 7.6 GB in two captures: the
+// 2 GB of logits pass through the same L2.  The tensor cores bound that size all the
+// same (1.01 of the burst rate, at up to 1.8 TB/s read).
 //   * SM pairs (tcgen05 cta_group::2; more than 128 rows): the two CTAs of a
 //     cluster own a 256 x bn tile, each holding 128 rows of H and bn / 2 of the
 //     tile's W rows in its shared memory; the leader issues the MMAs of both.
